@@ -50,10 +50,11 @@ struct fem_ctx {
     int32_t next_id = 1;
     uint32_t *d_err = nullptr;    // device error word
     uint32_t *d_small = nullptr;  // 64 device words for counters
-    uint32_t *h_small = nullptr;  // 64 pinned host words
+    uint32_t *h_small = nullptr;  // kSmallWords pinned host words
     // device address of h_small[kPubWord..kPubWord+1], written by the compaction and scan
     // kernels (count and error word); null where pinned memory is not mapped
     uint32_t *d_pub = nullptr;
+    uint32_t *d_plan = nullptr;  // the same of h_small[kPlanWord ..], written by the plan kernels
     uint32_t pub_seq = 0;  // sequence number of the last publishing launch
     // mapped pinned words a load's read-back is published to ([0] error word, [1] last
     // time, [2..258) type counts, [kLoadSeq] sequence number) and their device address
@@ -92,6 +93,7 @@ struct fem_ctx {
     // always do; count_any measures it): where it does not, the latest-chain kernels
     // would find few prefixes to share
     bool clustered = true;
+    bool hits_busy = false;  // a count over hit tables is being planned or run
     cudaEvent_t tev[2] = {nullptr, nullptr};
 };
 
@@ -121,6 +123,9 @@ enum { W_COUNT0 = 0, W_COUNT1 = 1, W_COUNT2 = 2, W_INFO = 8 /* 3 words */ };
 // first of the three pinned host words the kernels publish counts to
 constexpr uint32_t kPubWord = 48;
 constexpr uint32_t kLoadSeq = 2 + 256;  // the load read-back's sequence word
+// first of the mapped host words a plan is published to (plan words, error word, sequence)
+constexpr uint32_t kPlanWord = 64;
+constexpr uint32_t kSmallWords = kPlanWord + PLAN_WORDS + 2;
 
 size_t stream_bytes(const StreamDev &s) {
     if (!s.t) return 0;
@@ -130,10 +135,22 @@ size_t stream_bytes(const StreamDev &s) {
 
 void free_stream_buffers(StreamDev &s);
 
-// Room for `bytes` more under the context's memory budget: over budget, the buffers
-// kept from freed streams are released first; FEM_ENOMEM if it still does not fit.
+// Gives the hit tables' memory back (cudaFree waits for the work that reads them).
+void release_hits(fem_ctx *c) {
+    for (auto &kv : c->bufs) {
+        if (kv.first.compare(0, 4, "hit_") != 0 || !kv.second.p) continue;
+        cudaFree(kv.second.p);
+        c->mem_used -= std::min(kv.second.cap, c->mem_used);
+        kv.second = DevBuf{};
+    }
+}
+
+// Room for `bytes` more under the context's memory budget: over budget, the hit tables of
+// earlier calls and the buffers kept from freed streams are released first; FEM_ENOMEM if
+// it still does not fit.
 int reserve(fem_ctx *c, size_t bytes) {
     if (!c->mem_budget) return FEM_OK;
+    if (c->mem_used + bytes > c->mem_budget && !c->hits_busy) release_hits(c);
     while (c->mem_used + bytes > c->mem_budget && !c->pool.empty()) {
         c->mem_used -= std::min(stream_bytes(c->pool.front()), c->mem_used);
         free_stream_buffers(c->pool.front());
@@ -833,6 +850,263 @@ int count_pass(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
     return count_finish(c, s, pl, e, st);
 }
 
+// Segments of a hit-table pass over m candidates: about four 128-thread blocks for each
+// place on the GPU (the episodes' hits differ, so blocks end at different times), but of
+// eight slabs or more (a segment first goes through the window before it) unless that
+// would leave SMs without a block.  And segments whose tables stay in a part of the L2
+// cache while the blocks of all candidates, which run next to each other, read them (the
+// hour-long recording, 481 KB a slab: 168 ms with 240 segments,
+// 300 with eight).
+constexpr uint64_t kHitSegmentBytes = 24ull << 20;
+uint32_t hit_segments(const fem_ctx *c, uint32_t n_slabs, uint32_t n_chunks, uint32_t m,
+                      uint64_t slab_bytes) {
+    if (n_slabs < 2) return 1;
+    if (c->cfg.segments) return std::min(c->cfg.segments, std::max(n_chunks, 1u));
+    const uint64_t tiles = (m + 127) / 128, wave = (uint64_t)c->sm_count * 6;
+    const uint64_t P4 = (4 * wave + tiles - 1) / tiles, P1 = (wave + tiles - 1) / tiles;
+    const uint64_t longest = std::max<uint64_t>(16, kHitSegmentBytes / std::max<uint64_t>(slab_bytes, 1));
+    const uint64_t P = std::max(std::min<uint64_t>(P4, n_slabs / 8), std::min<uint64_t>(P1, n_slabs / 2));
+    return (uint32_t)std::min<uint64_t>(std::max<uint64_t>({1, P, (n_slabs + longest - 1) / longest}), 65535);
+}
+
+int count_grouped(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
+                  uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out, cudaStream_t st);
+
+// Launch a hit-table pass over p.m candidates (and its stitch when segmented).
+int hits_launch(fem_ctx *c, const StreamDev &s, uint32_t group, CountParams &p, uint32_t classes,
+                const char *tables, cudaStream_t st) {
+    const uint32_t P = hit_segments(c, p.hits.n_slabs, s.n_chunks, p.m, p.hits.slab_bytes);
+    p.cps = (p.hits.n_slabs + P - 1) / P;
+    p.P = (p.hits.n_slabs + p.cps - 1) / p.cps;
+    p.hit_classes = classes;
+    if (p.P > 1) RET(dbuf(c, tables, (size_t)p.P * p.m * classes, &p.tables));
+    CK(launch_hit_count(group, p.P > 1, p, st));
+    if (p.P > 1) CK(launch_stitch(p.tables, p.m, p.P, p.out, p.redo, c->d_err, st, classes));
+    return FEM_OK;
+}
+
+// Recount what a hit-table pass flagged: with all the class slots the kernel can use, then
+// by the per-thread kernels.
+int hits_finish(fem_ctx *c, const StreamDev &s, uint32_t group, const CountParams &p, int pass,
+                uint32_t e, cudaStream_t st) {
+    uint32_t *ridx, *rg, *rout, *scratch, r, er;
+    RET(dbuf(c, "hit_idx", p.m, &ridx));
+    RET(dbuf(c, "redo_scratch", compact_scratch_words(p.m), &scratch));
+    CK(launch_compact(nullptr, p.redo, 0, p.m, ridx, c->d_small + W_COUNT2, scratch, st, pub_of(c)));
+    RET(read_count_err(c, c->d_small + W_COUNT2, &r, &er, st));
+    if (r == 0) return FEM_OK;
+    if (std::getenv("FEM_DEBUG"))
+        std::fprintf(stderr, "fem: hit-table pass %d m=%u P=%u: %u episodes recounted (err %#x)\n", pass,
+                     p.m, p.P, r, e);
+    RET(dbuf(c, "hit_gather", r, &rg));
+    RET(dbuf(c, "hit_out", r, &rout));
+    CK(launch_compose_idx(p.gather, ridx, r, rg, st));
+    CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+    CountParams q = p;
+    q.gather = rg;
+    q.m = r;
+    q.out = rout;
+    RET(dbuf(c, "hit_redo", r, &q.redo));
+    CK(cudaMemsetAsync(q.redo, 0, r, st));
+    RET(hits_launch(c, s, group, q, S_RECOUNT, "redo_tables", st));
+    RET(read_err(c, st, &e));
+    RET(err_status(e));
+    if (e & ERR_CAP) {
+        CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+        RET(count_grouped(c, s, p.cands, rg, r, p.ivl, p.n_ivl, pass, rout, st));
+    }
+    CK(launch_scatter_u32(rout, ridx, r, p.out, st));
+    return FEM_OK;
+}
+
+// Count a candidate set over hit tables: all lengths, in an order of their own.  *done =
+// false, with nothing counted, where they do not apply: repeated types in the set, a
+// measured launch shape, or events too dense for the tables' words.
+int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
+               uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
+               cudaStream_t st, bool *done) {
+    *done = false;
+    uint64_t max_hi = 0;
+    for (const fem_interval &iv : c->ivl_host) max_hi = std::max<uint64_t>(max_hi, iv.hi_us);
+    PlanArgs a{};
+    a.cands = cands;
+    a.gather = gather;
+    a.m = m;
+    a.K = s.K;
+    a.n_ivl = nI;
+    a.parts = std::min(nI, PLAN_PARTS);
+    a.cfirst = s.cfirst;
+    a.t = s.t;
+    a.n_chunks = s.n_chunks;
+    a.n = s.n;
+    a.err = c->d_err;
+    const uint32_t bins = plan_bins(s.K, a.parts), tri = s.K * s.K * nI;
+    const size_t max_slabs = (size_t)s.n_chunks * 64 + 1;
+    uint32_t *order, *g2, *tmp;
+    uint8_t *redo;
+    RET(dbuf(c, "hit_plan", PLAN_WORDS + (size_t)bins + tri, &a.words));
+    a.hist = a.words + PLAN_WORDS;
+    a.edge_id = a.hist + bins;
+    RET(dbuf(c, "hit_plan_slabs", s.n_chunks + 2 * max_slabs, &a.parts_of));
+    a.begin = a.parts_of + s.n_chunks;
+    a.t0 = a.begin + max_slabs;
+    RET(dbuf(c, "hit_plan_bin", m, &a.bin));
+    RET(dbuf(c, "hit_plan_rank", m, &a.rank));
+    RET(dbuf(c, "hit_plan_order", m, &order));
+    RET(dbuf(c, "hit_plan_gather", m, &g2));
+    RET(dbuf(c, "hit_plan_out", m, &tmp));
+    RET(dbuf(c, "hit_plan_redo", m, &redo));
+    const uint32_t seq = ++c->pub_seq;
+    CK(launch_plan(a, s, order, g2, Publish{c->d_plan, c->d_err, seq}, st));
+    CK(cudaMemsetAsync(redo, 0, m, st));
+    const volatile uint32_t *w = c->h_small + kPlanWord;
+    RET(wait_seq(w + PLAN_WORDS + 1, seq, st));
+    RET(err_status(w[PLAN_WORDS]));
+    if (w[PLAN_REP]) return FEM_OK;
+    // the events before a slab are kept from its chunk and the one before
+    if (s.n_chunks > 1 && (uint64_t)(uint32_t)~w[PLAN_SPAN] <= max_hi) return FEM_OK;
+    uint32_t group_m[PLAN_GROUPS] = {};
+    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
+        if (!w[N - 1]) continue;
+        if (!c->tune.empty() &&
+            c->tune.count(tune_key((int)N, pass, true, w[N - 1], s.n_chunks, s.K)))
+            return FEM_OK;
+        group_m[plan_group(N, m)] += w[N - 1];
+    }
+    // short episodes, few of them for the stream's type pairs: the tables cost more than the
+    // per-thread machine's count (533 episodes of two and three nodes, 22 types, 360,000
+    // events: 0.66 against 0.61 ms for two passes; from four nodes on the tables were the
+    // faster at every size tried)
+    uint32_t longest = 0;
+    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N)
+        if (w[N - 1]) longest = N;
+    if (longest <= 3 && (uint64_t)m * longest < 5ull * s.K * s.K && (uint64_t)s.n * s.K > 4000000) return FEM_OK;
+    HitTables h{};
+    h.n_slabs = w[PLAN_SLABS], h.n_edges = w[PLAN_EDGES];
+    h.types = (s.K + 15) & ~15u;
+    h.edge_id = a.edge_id, h.begin = a.begin, h.t0 = a.t0;
+    HitBuild b{};
+    b.bev = s.bev, b.boff = s.boff, b.offs = s.offs, b.K = s.K, b.types = h.types;
+    b.ivl = d_ivl, b.n_ivl = nI, b.n_edges = h.n_edges;
+    b.max_words = CHUNK / 32 / w[PLAN_PARTS_MIN];
+    b.edge_id = a.edge_id, b.begin = a.begin, b.err = c->d_err;
+    // hits: at most one per edge and event of its last type, K n_edges / K per event on
+    // average; as many as events lie in the intervals at the stream's mean rate, and half
+    // again (the table grows when they are more)
+    double per_event = 0;
+    for (const fem_interval &iv : c->ivl_host)
+        per_event += (double)(iv.hi_us - (pass == FEM_PASS_EXACT ? iv.lo_us : 0u)) * (double)s.n /
+                     (double)std::max(s.t_max, 1u);
+    per_event *= (double)h.n_edges / tri;
+    uint64_t hits = (uint64_t)(1.5 * per_event * (double)s.n) + 4096;
+    hits = std::min<uint64_t>(hits, (uint64_t)s.n * (h.n_edges / s.K + 1));
+    uint32_t *words;
+    auto tables = [&]() -> int {
+        RET(dbuf(c, "hit_edges", (size_t)h.n_slabs * h.n_edges, &b.edge));
+        RET(dbuf(c, "hit_counts", (size_t)h.n_slabs * h.types, &b.count));
+        RET(dbuf(c, "hit_places", (size_t)h.n_slabs * h.types, &b.place));
+        RET(dbuf(c, "hit_index", s.n, &b.index));
+        RET(dbuf(c, "hit_words", 2, &words));
+        RET(dbuf(c, "hit_ranges", hits, &b.range));
+        b.capacity = c->bufs["hit_ranges"].cap / sizeof(uint32_t);
+        return FEM_OK;
+    };
+    for (;;) {
+        if (hits > 0xFFFFFFF0ull) return FEM_OK;
+        RET(tables());
+        b.used = reinterpret_cast<unsigned long long *>(words);
+        CK(cudaMemsetAsync(b.used, 0, 8, st));
+        CK(launch_hit_build(pass, h.n_slabs, b, c->sm_count, st));
+        h.slab_bytes = (uint64_t)h.n_edges * 8 + hits * 4 / std::max(h.n_slabs, 1u);
+        h.edge = b.edge, h.range = b.range, h.count = b.count, h.place = b.place, h.index = b.index;
+        CountParams part[PLAN_GROUPS]{};
+        uint32_t off = 0;
+        for (uint32_t g = 0; g < PLAN_GROUPS; ++g) {
+            if (!group_m[g]) continue;
+            CountParams &p = part[g];
+            p.cfirst = s.cfirst;
+            p.t = s.t;
+            p.n_chunks = s.n_chunks;
+            p.n = s.n;
+            p.K = s.K;
+            p.cands = cands;
+            p.gather = g2 + off;
+            p.m = group_m[g];
+            p.ivl = d_ivl;
+            p.n_ivl = nI;
+            p.out = tmp + off;
+            p.redo = redo + off;
+            p.err = c->d_err;
+            p.hits = h;
+            RET(hits_launch(c, s, g, p, S_MAX, "tables", st));
+            off += p.m;
+        }
+        uint32_t e, used;
+        CK(launch_scatter_u32(tmp, order, m, out, st));
+        CK(launch_publish_count(b.used, pub_of(c), st));
+        RET(read_count_err(c, nullptr, &used, &e, st));
+        RET(err_status(e));
+        if (e & ERR_DENSE) {
+            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+            return FEM_OK;
+        }
+        if (used > b.capacity) {  // more hits than the table held: a larger one
+            hits = used;
+            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+            CK(cudaMemsetAsync(redo, 0, m, st));
+            continue;
+        }
+        if (e & ERR_CAP) {
+            for (uint32_t g = 0; g < PLAN_GROUPS; ++g)
+                if (part[g].m) RET(hits_finish(c, s, g, part[g], pass, e, st));
+            CK(launch_scatter_u32(tmp, order, m, out, st));
+            CK(cudaStreamSynchronize(st));
+        }
+        *done = true;
+        return FEM_OK;
+    }
+}
+
+// Whether a set may be counted over hit tables: no configured kernel or ring size, no more
+// type pairs and intervals than are worth a table, and on average no more events of a type
+// in an interval than a word is for.
+constexpr uint32_t kHitMaxEdges = 1u << 18;
+bool hits_eligible(const fem_ctx *c, const StreamDev &s, uint32_t nI) {
+    uint64_t max_hi = 0;
+    for (const fem_interval &iv : c->ivl_host) max_hi = std::max<uint64_t>(max_hi, iv.hi_us);
+    return !c->cfg.kernel && !c->cfg.ring_capacity && c->d_plan && s.n_chunks && nI &&
+           (uint64_t)s.K * s.K * nI <= kHitMaxEdges &&
+           (double)s.n * (double)max_hi <= 8.0 * s.K * (double)std::max(s.t_max, 1u);
+}
+
+// Validate a candidate set (optionally gathered): the words of launch_validate_cands.
+int validate(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
+             uint32_t m, uint32_t nI, uint32_t *info, cudaStream_t st) {
+    CK(cudaMemsetAsync(c->d_small + W_INFO, 0, 3 * sizeof(uint32_t), st));
+    CK(launch_validate_cands(cands, gather, m, s.K, nI, c->d_small + W_INFO, c->d_err, st));
+    uint32_t e;
+    if (c->d_plan) {
+        const uint32_t seq = ++c->pub_seq;
+        CK(launch_publish_info(c->d_small + W_INFO, Publish{c->d_plan, c->d_err, seq}, st));
+        const volatile uint32_t *w = c->h_small + kPlanWord;
+        RET(wait_seq(w + 4, seq, st));
+        for (uint32_t k = 0; k < 3; ++k) info[k] = w[k];
+        e = w[3];
+    } else {
+        RET(read_words(c, c->d_small + W_INFO, 3, info, st));
+        RET(read_err(c, st, &e));
+    }
+    return err_status(e);
+}
+
+// Sets in runs of shared prefixes (at least four candidates long on average) are for the
+// latest-chain kernels.
+bool in_runs(const uint32_t *info, uint32_t m) { return (uint64_t)m >= 4ull * ((uint64_t)info[2] + 1); }
+
+int count_validated(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
+                    uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
+                    const uint32_t *info, cudaStream_t st);
+
 // Validate a candidate set (optionally gathered) and count it with `pass`,
 // grouping candidates by length.  out[i] is the count of candidate i of the
 // (gathered) set.
@@ -840,20 +1114,52 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
               uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
               cudaStream_t st) {
     if (m == 0) return FEM_OK;
-    CK(cudaMemsetAsync(c->d_small + W_INFO, 0, 3 * sizeof(uint32_t), st));
-    CK(launch_validate_cands(cands, gather, m, s.K, nI, c->d_small + W_INFO, c->d_err, st));
-    uint32_t info[3], e;
-    RET(read_words(c, c->d_small + W_INFO, 3, info, st));
-    RET(read_err(c, st, &e));
-    RET(err_status(e));
+    uint32_t info[3];
+    bool hits = hits_eligible(c, s, nI), known = false;
+    // a small set goes to the hit tables without a look at its runs (their plan validates
+    // too, and saves it a wait)
+    if (!hits || m >= 256) {
+        RET(validate(c, s, cands, gather, m, nI, info, st));
+        known = true;
+        hits = hits && !info[1] && !in_runs(info, m);
+    }
+    if (hits) {
+        bool done = false;
+        c->hits_busy = true;
+        const int rc = count_hits(c, s, cands, gather, m, d_ivl, nI, pass, out, st, &done);
+        c->hits_busy = false;
+        if (rc == FEM_ENOMEM) {  // no room beside the stream: the other kernels
+            release_hits(c);
+            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+        } else {
+            RET(rc);
+        }
+        if (done) return FEM_OK;
+    }
+    if (!known) RET(validate(c, s, cands, gather, m, nI, info, st));
+    return count_validated(c, s, cands, gather, m, d_ivl, nI, pass, out, info, st);
+}
+
+// The same by the other counting kernels, one length after the other.
+int count_grouped(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
+                  uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
+                  cudaStream_t st) {
+    if (m == 0) return FEM_OK;
+    uint32_t info[3];
+    RET(validate(c, s, cands, gather, m, nI, info, st));
+    return count_validated(c, s, cands, gather, m, d_ivl, nI, pass, out, info, st);
+}
+
+int count_validated(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
+                    uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
+                    const uint32_t *info, cudaStream_t st) {
     const uint32_t lens = info[0];
-    // runs of shared prefixes at least four candidates long on average
     struct Clustered {
         fem_ctx *c;
         bool saved;
         ~Clustered() { c->clustered = saved; }
     } restore{c, c->clustered};
-    c->clustered = (uint64_t)m >= 4ull * ((uint64_t)info[2] + 1);
+    c->clustered = in_runs(info, m);
     if (info[1] && info[1] < m) {
         // distinct-type and repeated-type episodes mixed: count each part on its own
         // (repeated types run with one segment), then put the counts back in place
@@ -987,7 +1293,7 @@ int fem_create(fem_ctx **out, int device, size_t mem_budget_bytes) {
         cudaStreamCreateWithFlags(&c->own, cudaStreamNonBlocking) != cudaSuccess ||
         cudaMalloc(&c->d_err, sizeof(uint32_t)) != cudaSuccess ||
         cudaMalloc(&c->d_small, 64 * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMallocHost(&c->h_small, 64 * sizeof(uint32_t)) != cudaSuccess ||
+        cudaMallocHost(&c->h_small, kSmallWords * sizeof(uint32_t)) != cudaSuccess ||
         cudaMallocHost(&c->h_load, (kLoadSeq + 1) * sizeof(uint32_t)) != cudaSuccess ||
         cudaMallocHost(&c->h_ivl, (FEM_MAX_INTERVALS + 1) * sizeof(fem_interval)) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ivl_ev, cudaEventDisableTiming) != cudaSuccess ||
@@ -1014,13 +1320,14 @@ int fem_create(fem_ctx **out, int device, size_t mem_budget_bytes) {
         }
     }
     cudaMemset(c->d_err, 0, sizeof(uint32_t));
-    std::memset(c->h_small, 0, 64 * sizeof(uint32_t));  // no stale sequence number
+    std::memset(c->h_small, 0, kSmallWords * sizeof(uint32_t));  // no stale sequence number
     std::memset(c->h_load, 0, (kLoadSeq + 1) * sizeof(uint32_t));
     {
         void *dp = nullptr, *dl = nullptr;
         if (cudaHostGetDevicePointer(&dp, c->h_small, 0) == cudaSuccess && dp &&
             cudaHostGetDevicePointer(&dl, c->h_load, 0) == cudaSuccess && dl) {
             c->d_pub = static_cast<uint32_t *>(dp) + kPubWord;
+            c->d_plan = static_cast<uint32_t *>(dp) + kPlanWord;
             c->d_load = static_cast<uint32_t *>(dl);
         }
         cudaGetLastError();

@@ -1,0 +1,498 @@
+// fem_hits.cu -- the hit tables of a stream and an edge set, the launches of the counting
+// kernels that read them, and the plan both need: the candidates checked and ordered, the
+// edges they use numbered, the stream cut into slabs.
+#include <mutex>
+
+#include "fem_hits.cuh"
+
+namespace fem {
+
+namespace {
+
+// Exclusive sum of one value per thread over a block of 1024; *total = the sum.
+__device__ __forceinline__ uint32_t block_scan_1024(uint32_t v, uint32_t *total) {
+    __shared__ uint32_t wsum[33];
+    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t inc = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= (uint32_t)d) inc += y;
+    }
+    __syncthreads();
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    if (w == 0) {
+        const uint32_t x = wsum[lane];
+        uint32_t s = x;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, s, d);
+            if (lane >= (uint32_t)d) s += y;
+        }
+        wsum[lane] = s - x;
+        if (lane == 31) wsum[32] = s;
+    }
+    __syncthreads();
+    *total = wsum[32];
+    return wsum[w] + inc - v;
+}
+
+// Exclusive sums of f(w[i]) over i < n by one block of 1024: g(i, w[i], sum before i) for
+// every i, *total = the whole sum.  A warp takes a run of words and goes through it 32 at
+// a time, twice.
+template <typename F, typename G>
+__device__ __forceinline__ void scan_words(const uint32_t *w, uint32_t n, uint32_t *total, F &&f, G &&g) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t per = ((n + 31) / 32 + 31) & ~31u, lo = min(warp * per, n), hi = min(lo + per, n);
+    uint32_t sum = 0;
+#pragma unroll 4
+    for (uint32_t i = lo + lane; i < hi; i += 32) sum += f(w[i]);
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    uint32_t at = block_scan_1024(lane == 0 ? sum : 0u, total);
+    at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll 4
+    for (uint32_t i0 = lo; i0 < hi; i0 += 32) {
+        const uint32_t i = i0 + lane, v = i < hi ? w[i] : 0u, x = i < hi ? f(v) : 0u;
+        uint32_t inc = x;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= (uint32_t)d) inc += y;
+        }
+        if (i < hi) g(i, v, at + inc - x);
+        at += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    __syncthreads();
+}
+
+// Bin of a valid candidate: the launch that counts it (plan_group), the places of its last
+// three intervals in the set (in `parts` parts each, the last first: the longest work
+// first), its last type.
+__device__ __forceinline__ uint32_t plan_bin(const fem_episode &e, const PlanArgs &a) {
+    const uint32_t N = e.len;
+    uint32_t bin = plan_group(N, a.m);
+    for (uint32_t k = 1; k <= 3; ++k)
+        bin = bin * a.parts + (N > k ? a.parts - 1u - e.ivl[N - 1 - k] * a.parts / a.n_ivl : 0u);
+    return bin * a.K + e.types[N - 1];
+}
+
+// Each candidate's bin and its place in the bin (the order within a bin is arbitrary: a
+// candidate's count does not depend on it), the bins' sizes, the edges in use, and the
+// plan words: per length 1..8 the candidates, [PLAN_REP] those with a repeated type,
+// [PLAN_SPAN] 2^32 - 1 less the least time that a chunk spans.
+__global__ void __launch_bounds__(256) k_plan_bins(const PlanArgs a) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t rep = 0, bad = 0, len = 0;
+    if (i < a.m) {
+        const fem_episode e = a.cands[a.gather ? a.gather[i] : i];
+        const uint32_t N = e.len;
+        if (N < 1 || N > FEM_MAX_LEN) {
+            bad = ERR_BADEP;
+        } else {
+            for (uint32_t k = 0; k < N; ++k)
+                if (e.types[k] >= a.K) bad = ERR_BADEP;
+            for (uint32_t k = 0; k + 1 < N; ++k)
+                if (e.ivl[k] >= a.n_ivl) bad = ERR_BADEP;
+            for (uint32_t x = 0; x < N; ++x)
+                for (uint32_t y = x + 1; y < N; ++y)
+                    if (e.types[x] == e.types[y]) rep = 1;
+        }
+        if (!bad) {
+            len = N;
+            const uint32_t bin = plan_bin(e, a);
+            a.bin[i] = bin;
+            a.rank[i] = atomicAdd(&a.hist[bin], 1u);
+            if (!rep)
+                for (uint32_t k = 0; k + 1 < N; ++k)
+                    a.edge_id[(e.types[k] * a.K + e.types[k + 1]) * a.n_ivl + e.ivl[k]] = 1u;
+        }
+    }
+    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
+        const uint32_t k = __popc(__ballot_sync(0xffffffffu, len == N));
+        if (k && (threadIdx.x & 31) == 0) atomicAdd(&a.words[N - 1], k);
+    }
+    rep = __reduce_add_sync(0xffffffffu, rep);
+    bad = __reduce_or_sync(0xffffffffu, bad);
+    if ((threadIdx.x & 31) == 0) {
+        if (rep) atomicAdd(&a.words[PLAN_REP], rep);
+        if (bad) atomicOr(a.err, bad);
+    }
+    // the least span, over the whole grid
+    uint32_t span = 0;
+    for (uint32_t c = i + 1; c < a.n_chunks; c += gridDim.x * blockDim.x)
+        span = max(span, ~(a.cfirst[c] - a.cfirst[c - 1]));
+    span = __reduce_max_sync(0xffffffffu, span);
+    if (span && (threadIdx.x & 31) == 0) atomicMax(&a.words[PLAN_SPAN], span);
+}
+
+// Slabs per chunk: the fewest equal parts (a power of two) in none of which a type has
+// more than 32 events.  One block per chunk, a warp per type.
+__global__ void __launch_bounds__(256) k_hit_cuts(const uint2 *bev, const uint16_t *boff, uint32_t offs,
+                                                  uint32_t K, uint32_t *parts_of) {
+    __shared__ uint32_t need;
+    const uint32_t c = blockIdx.x, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) need = 1;
+    __syncthreads();
+    const uint16_t *off = boff + (uint64_t)c * offs;
+    const uint2 *ev = bev + (uint64_t)c * CHUNK;
+    for (uint32_t b = threadIdx.x >> 5; b < K; b += blockDim.x >> 5) {
+        const uint32_t g0 = off[b], g1 = off[b + 1];
+        // a part holds more than 32 of the type iff two of its events 32 apart lie in it: the
+        // parts must be finer than the highest bit in which their places differ
+        uint32_t q = 1;
+        for (uint32_t j = g0 + lane; j + 32 < g1; j += 32) {
+            const uint32_t x = ev[j].y ^ ev[j + 32].y;  // not zero
+            q = max(q, CHUNK >> (31 - __clz(x)));       // parts of half the size of that bit's
+        }
+        q = __reduce_max_sync(0xffffffffu, q);
+        if (lane == 0 && q > 1) atomicMax(&need, q);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) parts_of[c] = need;
+}
+
+// One block of 1024: the bins' and the edges' numbers scanned in place (an edge in use
+// gets its number, the others none), the slabs' first events and times, and everything
+// the host plans with published.
+__global__ void __launch_bounds__(1024) k_plan_scan(const PlanArgs a, uint32_t bins, uint32_t edges,
+                                                    Publish pub) {
+    const uint32_t tid = threadIdx.x;
+    uint32_t total, n_edges, n_slabs, per;
+    scan_words(a.hist, bins, &total, [](uint32_t v) { return v; },
+               [&](uint32_t i, uint32_t, uint32_t at) { a.hist[i] = at; });
+    scan_words(a.edge_id, edges, &n_edges, [](uint32_t v) { return v; },
+               [&](uint32_t i, uint32_t v, uint32_t at) { a.edge_id[i] = v ? at : ~0u; });
+    {
+        per = (a.n_chunks + 1023) / 1024;
+        const uint32_t lo = min(tid * per, a.n_chunks), hi = min(lo + per, a.n_chunks);
+        auto slabs = [&](uint32_t c) {  // (the last chunk's parts end with the stream)
+            const uint32_t q = a.parts_of[c], size = CHUNK / q;
+            const uint64_t left = a.n - (uint64_t)c * CHUNK;
+            return left >= CHUNK ? q : (uint32_t)((left + size - 1) / size);
+        };
+        uint32_t v = 0;
+        for (uint32_t c = lo; c < hi; ++c) v += slabs(c);
+        uint32_t at = block_scan_1024(v, &n_slabs);
+        for (uint32_t c = lo; c < hi; ++c) {
+            const uint32_t q = slabs(c), size = CHUNK / a.parts_of[c];
+            for (uint32_t k = 0; k < q; ++k, ++at) {
+                a.begin[at] = c * CHUNK + k * size;
+                a.t0[at] = a.t[c * CHUNK + k * size];
+            }
+        }
+        if (tid == 0) a.begin[n_slabs] = (uint32_t)a.n, a.t0[n_slabs] = 0xFFFFFFFFu;
+    }
+    // the largest slab (the fewest parts of a chunk)
+    uint32_t fewest = HIT_PARTS;
+    for (uint32_t c = tid; c < a.n_chunks; c += 1024) fewest = min(fewest, a.parts_of[c]);
+    fewest = __reduce_min_sync(0xffffffffu, fewest);
+    __shared__ uint32_t least;
+    if (tid == 0) least = HIT_PARTS;
+    __syncthreads();
+    if ((tid & 31) == 0) atomicMin(&least, fewest);
+    __syncthreads();
+    if (tid == 0) {
+        volatile uint32_t *h = pub.host;
+        for (uint32_t k = 0; k < PLAN_EDGES; ++k) h[k] = a.words[k];
+        h[PLAN_PARTS_MIN] = least;
+        h[PLAN_EDGES] = n_edges;
+        h[PLAN_SLABS] = n_slabs;
+        h[PLAN_WORDS] = *reinterpret_cast<const volatile uint32_t *>(pub.err);
+        __threadfence_system();
+        h[PLAN_WORDS + 1] = pub.seq;
+    }
+}
+
+// order[slot] = i and gather[slot] = candidate record of i, by the scanned bins
+__global__ void __launch_bounds__(256) k_plan_place(const PlanArgs a, uint32_t *order,
+                                                    uint32_t *gather) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= a.m || (*a.err & ERR_BADEP)) return;
+    const uint32_t s = a.hist[a.bin[i]] + a.rank[i];
+    order[s] = i;
+    gather[s] = a.gather ? a.gather[i] : i;
+}
+
+// The words of k_validate_cands and the error word, published.
+__global__ void k_publish_info(const uint32_t *info, Publish pub) {
+    volatile uint32_t *h = pub.host;
+    for (uint32_t k = 0; k < 3; ++k) h[k] = info[k];
+    h[3] = *reinterpret_cast<const volatile uint32_t *>(pub.err);
+    __threadfence_system();
+    h[4] = pub.seq;
+}
+
+// (a count above 32 bits as 2^32 - 1)
+__global__ void k_publish_count(const unsigned long long *src, Publish pub) {
+    volatile uint32_t *h = pub.host;
+    const unsigned long long v = *reinterpret_cast<const volatile unsigned long long *>(src);
+    h[0] = v > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)v;
+    h[1] = *reinterpret_cast<const volatile uint32_t *>(pub.err);
+    __threadfence_system();
+    h[2] = pub.seq;
+}
+
+// The hit tables of one slab (a block; of a few slabs several, which share the types).  Every type's events in the slab and the 32
+// before it go into shared memory as rank rows (rank 32 is the slab's first; the types'
+// own order in the chunk gives the ranks), with a bit per position of the slab and, per
+// 32 positions, the events before them, so that the number of a type's events before any
+// event of the slab is two reads and a popc.  Then a warp takes a type y, a lane its event
+// r, and goes through the other types x: the x events before the lane's event as far back
+// as the longest interval reaches, a few steps down the row, give the ranges of four
+// intervals at once; a ballot per interval is the edge's mask.  Ranges are written to room
+// that a warp reserves in the table for many edges at a time.  (A thread per edge, merging
+// the edge's two rows, left three of four lanes idle: 1.15 ms for the 387,000 events of 64
+// types at 50 Hz and all 16,128 edges; a thread per event and earlier event, 1.04 ms.)
+constexpr uint32_t HIT_ROOM = 2048;  // ranges a warp reserves at a time
+
+template <int PASS>
+__global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build(const HitBuild b) {
+    const uint32_t T = HIT_BUILD_T, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr uint32_t NW = HIT_BUILD_T / 32, WORDS = CHUNK / 32;
+    const uint32_t s = blockIdx.x, K = b.K;
+    uint32_t *rt = reinterpret_cast<uint32_t *>(fem_hit_smem);  // times by rank [K][HIT_ROW]
+    uint32_t *bits = rt + K * HIT_ROW;                          // [K][slab words]
+    const uint32_t begin = b.begin[s], end = b.begin[s + 1], c = begin / CHUNK;
+    const uint32_t p0 = begin % CHUNK, p1 = p0 + (end - begin);  // the slab's places in its chunk
+    const uint32_t words = (end - begin + 31) / 32;
+    uint16_t *rp = reinterpret_cast<uint16_t *>(bits + K * b.max_words);  // positions by rank [K][HIT_ROW]
+    uint16_t *place = rp + K * HIT_ROW;                          // [K]
+    uint8_t *before = reinterpret_cast<uint8_t *>(place + K);    // events before a word [K][words]
+    uint8_t *hist = before + K * b.max_words;                    // events before the slab [K]
+    uint8_t *num = hist + K;                                     // events in the slab [K]
+    const uint32_t origin = c * CHUNK - CHUNK;                   // index of position 0 (modulo 2^32)
+    const uint16_t *off = b.boff + (uint64_t)c * b.offs;
+    const uint2 *ev = b.bev + (uint64_t)c * CHUNK;
+    for (uint32_t i = tid; i < K * words; i += T) bits[i] = 0;
+    __syncthreads();
+    for (uint32_t x = warp; x < K; x += NW) {
+        const uint32_t g0 = off[x], g1 = off[x + 1];
+        uint32_t a = g0, z = g0;  // the type's first event in the slab and past its last
+        for (uint32_t j0 = g0; j0 < g1; j0 += 32) {
+            const uint32_t j = j0 + lane, y = j < g1 ? ev[j].y : ~0u;
+            a += __popc(__ballot_sync(0xffffffffu, y < p0));
+            z += __popc(__ballot_sync(0xffffffffu, y < p1));
+        }
+        const uint32_t n = z - a, own = min(a - g0, 32u);
+        if (lane < n) {
+            const uint2 e = ev[a + lane];
+            rt[x * HIT_ROW + 32 + lane] = e.x;
+            rp[x * HIT_ROW + 32 + lane] = (uint16_t)(CHUNK + e.y);
+            atomicOr(&bits[x * words + ((e.y - p0) >> 5)], 1u << ((e.y - p0) & 31));
+        }
+        uint32_t h = own;  // earlier ones: of this chunk, then of the chunk before
+        if (lane < own) {
+            const uint2 e = ev[a - 1 - lane];
+            rt[x * HIT_ROW + 31 - lane] = e.x;
+            rp[x * HIT_ROW + 31 - lane] = (uint16_t)(CHUNK + e.y);
+        }
+        if (own < 32 && c > 0) {
+            const uint32_t f0 = off[(int)x - (int)b.offs], f1 = off[(int)x + 1 - (int)b.offs];
+            const uint32_t more = min(f1 - f0, 32u - own);
+            if (lane < more) {
+                const uint2 e = *(ev - CHUNK + (f1 - 1 - lane));
+                rt[x * HIT_ROW + 31 - own - lane] = e.x;
+                rp[x * HIT_ROW + 31 - own - lane] = (uint16_t)e.y;
+            }
+            h += more;
+        }
+        if (lane == 0) hist[x] = (uint8_t)h, num[x] = (uint8_t)n, b.count[(uint64_t)s * b.types + x] = (uint8_t)n;
+        __syncwarp();
+        uint32_t sum = 0;
+        for (uint32_t w0 = 0; w0 < words; w0 += 32) {
+            const uint32_t v = w0 + lane < words ? __popc(bits[x * words + w0 + lane]) : 0u;
+            uint32_t inc = v;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= (uint32_t)d) inc += y;
+            }
+            if (w0 + lane < words) before[x * words + w0 + lane] = (uint8_t)(sum + inc - v);
+            sum += __shfl_sync(0xffffffffu, inc, 31);
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {  // where each type's events start in the slab's list
+        uint32_t carry = 0;
+        for (uint32_t x0 = 0; x0 < K; x0 += 32) {
+            const uint32_t v = x0 + lane < K ? num[x0 + lane] : 0u;
+            uint32_t inc = v;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= (uint32_t)d) inc += y;
+            }
+            if (x0 + lane < K) {
+                place[x0 + lane] = (uint16_t)(carry + inc - v);
+                b.place[(uint64_t)s * b.types + x0 + lane] = (uint16_t)(carry + inc - v);
+            }
+            carry += __shfl_sync(0xffffffffu, inc, 31);
+        }
+    }
+    __syncthreads();
+    bool dense = false;
+    uint32_t at = 0, left = 0;  // the warp's room in the table of ranges
+    constexpr int U = 4;        // intervals taken at once
+    for (uint32_t u0 = 0; u0 < b.n_ivl; u0 += U) {
+        // a gap lies in interval u iff gap - from[u] <= wide[u] (unsigned); the relaxed pass
+        // takes any gap up to hi
+        uint32_t from[U], wide[U], far = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint2 v = b.ivl[min(u0 + u, b.n_ivl - 1)];  // (past the set: one not looked at)
+            from[u] = PASS == FEM_PASS_EXACT ? v.x + 1u : 0u;
+            wide[u] = v.y - from[u];
+            far = max(far, v.y);
+        }
+        for (uint32_t y = blockIdx.y * NW + warp; y < K; y += NW * gridDim.y) {
+            const uint32_t n = num[y];
+            const bool mine = lane < n;
+            const uint32_t t = mine ? rt[y * HIT_ROW + 32 + lane] : 0u;
+            const uint32_t pos = mine ? rp[y * HIT_ROW + 32 + lane] : CHUNK + p0;
+            if (mine && u0 == 0) b.index[begin + place[y] + lane] = (uint16_t)(origin + pos);
+            const uint32_t q = pos - CHUNK - p0, w = q >> 5, below = (1u << (q & 31)) - 1u;
+            const uint32_t before_me = (1u << lane) - 1u;
+            // lane u of four holds the number of edge (x, u0 + u, y), asked for an x ahead
+            const uint32_t *ids = b.edge_id + y * b.n_ivl + u0 + (lane & (U - 1));
+            const bool iv = lane < U && u0 + lane < b.n_ivl;
+            uint32_t next = iv ? __ldg(ids) : ~0u;
+            for (uint32_t x = 0; x < K; ++x) {
+                const uint32_t id = next;
+                if (x + 1 < K && iv) next = __ldg(ids + (x + 1) * K * b.n_ivl);
+                const uint32_t wanted = __ballot_sync(0xffffffffu, id != ~0u);
+                if (!wanted || x == y) continue;  // no edge in use
+                const uint32_t *tx = rt + x * HIT_ROW;
+                const uint32_t low = 32u - hist[x];
+                // x's events before the lane's event have the ranks below k; those in interval
+                // u are m_u from a_u on
+                uint32_t a[U] = {}, m[U] = {};
+                if (mine) {
+                    uint32_t k = 32u + before[x * words + w] + __popc(bits[x * words + w] & below);
+                    const uint32_t k0 = k;
+                    for (; k > low; --k) {
+                        const uint32_t gap = t - tx[k - 1];
+                        if (gap > far) break;
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (gap - from[u] <= wide[u]) a[u] = k - 1, ++m[u];
+                    }
+                    // older events than the 32 kept may lie in an interval, or more than a range
+                    // can say
+                    dense = dense || (k == 0 && k0 > 0) || k0 - k > 32;
+                }
+                uint32_t mask[U], total = 0;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    mask[u] = __ballot_sync(0xffffffffu, m[u] != 0);
+                    if (!((wanted >> u) & 1u)) mask[u] = 0;
+                    total += __popc(mask[u]);
+                }
+                if (total > left) {  // the same in every lane
+                    unsigned long long g = 0;
+                    if (lane == 0) g = atomicAdd(b.used, (unsigned long long)HIT_ROOM);
+                    g = __shfl_sync(0xffffffffu, g, 0);
+                    left = g + HIT_ROOM <= b.capacity ? HIT_ROOM : 0u;
+                    at = (uint32_t)g;
+                    if (total > left) total = mask[0] = mask[1] = mask[2] = mask[3] = 0;  // (the host sees it)
+                }
+                left -= total;
+                uint2 own = make_uint2(mask[0], at);  // lane u's edge
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (u > 0 && lane == (uint32_t)u) own = make_uint2(mask[u], at);
+                    if (!mask[u]) continue;  // uniform
+                    if ((mask[u] >> lane) & 1u)
+                        b.range[at + __popc(mask[u] & before_me)] =
+                            hit_pack(a[u], m[u], origin + rp[x * HIT_ROW + a[u] + m[u] - 1]);
+                    at += __popc(mask[u]);
+                }
+                if (id != ~0u) b.edge[(uint64_t)s * b.n_edges + id] = own;
+            }
+        }
+    }
+    if (dense) atomicOr(b.err, ERR_DENSE);
+}
+
+template <int NMAX, bool MC>
+cudaError_t count_run(const CountParams &p, cudaStream_t st) {
+    constexpr uint32_t T = 128;
+    const size_t sm = (size_t)hit_shared(NMAX) * 64 * T * 2;
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(once, [sm] {
+        attr_err = cudaFuncSetAttribute(k_hit_count<NMAX, MC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)sm);
+    });
+    if (attr_err != cudaSuccess) return attr_err;
+    k_hit_count<NMAX, MC><<<dim3((p.m + T - 1) / T, p.P), T, sm, st>>>(p);
+    note_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+uint32_t plan_bins(uint32_t K, uint32_t parts) { return PLAN_GROUPS * K * parts * parts * parts; }
+
+cudaError_t launch_plan(const PlanArgs &a, const StreamDev &s, uint32_t *order, uint32_t *gather,
+                        Publish pub, cudaStream_t st) {
+    const uint32_t bins = plan_bins(a.K, a.parts), edges = a.K * a.K * a.n_ivl, blocks = (a.m + 255) / 256;
+    cudaError_t e = cudaMemsetAsync(a.words, 0, (PLAN_WORDS + (size_t)bins + edges) * 4, st);
+    if (e != cudaSuccess) return e;
+    k_plan_bins<<<blocks, 256, 0, st>>>(a);
+    k_hit_cuts<<<s.n_chunks, 256, 0, st>>>(s.bev, s.boff, s.offs, s.K, a.parts_of);
+    k_plan_scan<<<1, 1024, 0, st>>>(a, bins, edges, pub);
+    k_plan_place<<<blocks, 256, 0, st>>>(a, order, gather);
+    note_launch(4);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_publish_info(const uint32_t *info, Publish pub, cudaStream_t st) {
+    k_publish_info<<<1, 1, 0, st>>>(info, pub);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_publish_count(const unsigned long long *src, Publish pub, cudaStream_t st) {
+    k_publish_count<<<1, 1, 0, st>>>(src, pub);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
+                             cudaStream_t st) {
+    if (n_slabs == 0) return cudaSuccess;
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(once, [] {
+        for (auto *k : {k_hit_build<FEM_PASS_RELAXED>, k_hit_build<FEM_PASS_EXACT>})
+            if (attr_err == cudaSuccess)
+                attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+    });
+    if (attr_err != cudaSuccess) return attr_err;
+    const size_t K = b.K;
+    const size_t sm = K * (HIT_ROW * 6 + b.max_words * 5 + 4) + 16;
+    if (sm > 224 * 1024) return cudaErrorInvalidConfiguration;
+    // a few slabs: their types shared among several blocks, for about three per SM
+    constexpr uint32_t NW = HIT_BUILD_T / 32;
+    uint32_t split = 1;
+    while (split < 8 && split * NW < b.K && 2 * split * n_slabs <= 3 * (uint32_t)sm_count) split *= 2;
+    (pass == FEM_PASS_RELAXED ? k_hit_build<FEM_PASS_RELAXED>
+                              : k_hit_build<FEM_PASS_EXACT>)<<<dim3(n_slabs, split), HIT_BUILD_T, sm, st>>>(b);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hit_count(uint32_t group, bool mc, const CountParams &p, cudaStream_t st) {
+    if (p.m == 0) return cudaSuccess;
+    switch (group) {
+        case 0: return mc ? count_run<2, true>(p, st) : count_run<2, false>(p, st);
+        case 1: return mc ? count_run<3, true>(p, st) : count_run<3, false>(p, st);
+        case 2: return mc ? count_run<4, true>(p, st) : count_run<4, false>(p, st);
+        case 3: return mc ? count_run<5, true>(p, st) : count_run<5, false>(p, st);
+        case 4: return mc ? count_run<8, true>(p, st) : count_run<8, false>(p, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace fem

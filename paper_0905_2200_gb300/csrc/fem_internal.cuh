@@ -38,6 +38,7 @@ constexpr uint32_t ERR_TYPE = 16u;
 constexpr uint32_t ERR_TABLE = 32u;        // transfer table missing a class (internal)
 constexpr uint32_t ERR_CLASS = 64u;        // more entry classes than table slots (host retries)
 constexpr uint32_t ERR_NODES = 128u;       // a latest-chain block's prefix tables overflowed (host retries)
+constexpr uint32_t ERR_DENSE = 256u;       // hit tables: too many events of a type in an interval
 // any capacity guard: the flagged episodes are recounted by the host
 constexpr uint32_t ERR_CAP = ERR_RING | ERR_TABLE | ERR_CLASS | ERR_NODES;
 
@@ -65,6 +66,20 @@ struct StreamDev {
     mutable uint64_t ring_gen = 0;
     mutable std::string ring_ivl;
     mutable bool ring_singles = false, ring_clusters = false;
+};
+
+// The hit tables of a stream, an edge set and a pass (fem_hits.cuh).
+struct HitTables {
+    const uint32_t *edge_id;  // number of edge (type, next type, interval)
+    const uint32_t *begin;    // [n_slabs + 1] first event of each slab
+    const uint32_t *t0;       // [n_slabs + 1] its time
+    const uint2 *edge;        // [n_slabs][n_edges] mask of the next type's events, first range
+    const uint32_t *range;    // per hit its range (hit_pack)
+    const uint8_t *count;     // [n_slabs][types] events of a type in a slab
+    const uint16_t *place;    // [n_slabs][types] where they start in the slab's list
+    const uint16_t *index;    // per slab its events by type: low half of their index
+    uint32_t n_slabs, n_edges, types;
+    uint64_t slab_bytes;      // (host) about the bytes of a slab's masks and ranges
 };
 
 // Arguments of the counting kernels (one pass over one candidate set).
@@ -96,6 +111,9 @@ struct CountParams {
     uint32_t state_stride;      // words per candidate: 1 + (N-1) relaxed, 1 + (N-1)(1 + 2R) exact
     // (level-2 pair kernel) frequent types f of a level-2 set of f (f - 1) n_ivl candidates
     uint32_t pair_types;
+    // (hit-table kernels) the tables, entry-class slots per transfer table
+    HitTables hits;
+    uint32_t hit_classes;
 };
 
 // MapConcatenate as printed (fem_literal.cu): time segments (tau[p], tau[p+1]]
@@ -240,6 +258,63 @@ cudaError_t count_set_smem_limits();
 cudaError_t launch_chain(int N, int pass, bool mc, uint32_t threads, const CountParams &p,
                          cudaStream_t st);
 size_t chain_smem_bytes(int N, bool mc, uint32_t threads, uint32_t offs);
+// fem_hits.cu: the same passes over hit tables (distinct types, lengths 1..8, one segment
+// or MapConcatenate over runs of slabs).  group: the episodes' plan_group
+cudaError_t launch_hit_count(uint32_t group, bool mc, const CountParams &p, cudaStream_t st);
+struct HitBuild {
+    const uint2 *bev;
+    const uint16_t *boff;
+    uint32_t offs, K, types;
+    uint32_t max_words;           // 32-event words of the largest slab
+    const uint2 *ivl;
+    uint32_t n_ivl, n_edges;
+    const uint32_t *edge_id, *begin;
+    uint2 *edge;
+    uint32_t *range;
+    unsigned long long capacity;  // hits the range table holds
+    unsigned long long *used;     // hits found (zeroed by the caller); beyond it nothing is written
+    uint8_t *count;
+    uint16_t *place, *index;
+    uint32_t *err;                // ERR_DENSE
+};
+cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
+                             cudaStream_t st);
+// What a count over hit tables is planned with: the candidates checked and put in the
+// order they run best in (by group, last three intervals, last type), the edges they use
+// numbered, the stream cut into slabs.  words, hist and edge_id are one block of PLAN_WORDS
+// + plan_bins(K, parts) + K K n_ivl words.
+constexpr uint32_t PLAN_PARTS = 4, PLAN_GROUPS = 5, PLAN_FINE = 8192;
+constexpr uint32_t PLAN_REP = 8, PLAN_SPAN = 9, PLAN_EDGES = 10, PLAN_SLABS = 11, PLAN_PARTS_MIN = 12,
+                   PLAN_WORDS = 13;
+// The launch that counts an episode of N nodes of a set of m: lengths 1-2, 3, 4, 5 and
+// 6-8, since registers and shared memory grow with the length; small sets, whose launches
+// are short, in three (1-3, 4-5, 6-8).
+__host__ __device__ inline uint32_t plan_group(uint32_t N, uint32_t m) {
+    if (N > 5) return 4;
+    if (m < PLAN_FINE) return N <= 3 ? 1 : 3;
+    return N <= 2 ? 0 : N - 2;
+}
+struct PlanArgs {
+    const fem_episode *cands;
+    const uint32_t *gather;
+    uint32_t m, K, n_ivl;
+    uint32_t parts;          // parts of the interval set (at most PLAN_PARTS, n_ivl)
+    const uint32_t *cfirst, *t;
+    uint32_t n_chunks;
+    uint64_t n;
+    uint32_t *words, *hist, *edge_id, *bin, *rank;
+    uint32_t *parts_of, *begin, *t0;  // per chunk its slabs; per slab its first event and time
+    uint32_t *err;
+};
+uint32_t plan_bins(uint32_t K, uint32_t parts);
+struct Publish;
+// order[slot] = the candidate's place in the set, gather[slot] = its record; publishes
+// the plan words, the error word and the sequence number (PLAN_WORDS + 2 words)
+cudaError_t launch_plan(const PlanArgs &a, const StreamDev &s, uint32_t *order, uint32_t *gather,
+                        Publish pub, cudaStream_t st);
+// info[0 .. 3) of launch_validate_cands, the error word and the sequence number (5 words)
+cudaError_t launch_publish_info(const uint32_t *info, Publish pub, cudaStream_t st);
+cudaError_t launch_publish_count(const unsigned long long *src, Publish pub, cudaStream_t st);
 // fem_windows.cu: window-based frequency, one thread per episode (distinct types)
 struct WindowParams {
     const uint2 *bev;

@@ -1,0 +1,108 @@
+"""The hit-table counting kernels (fem_hits.cu) against the oracle, element by element, at the
+places where they can go wrong: types with more events in a slab than a word holds (the
+slabs shrink to 32 events), equal times across slab and chunk ends, every length 1-8 with one
+segment up to more segments than chunks, overlapping intervals and more than four of them,
+256 types, windows denser than the tables' words (counted by the other kernels), more hits
+than the table was sized for, and a memory budget without room for the tables."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0905_2200_gb300 import fem, synth
+from tests.gpu_common import I_MS4, assert_counts_equal, ctx_fixture, oracle_counts
+
+pytestmark = pytest.mark.gpu
+PASSES = (fem.PASS_RELAXED, fem.PASS_EXACT)
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = ctx_fixture()
+    yield c
+    fem.fem_destroy(c)
+
+
+@pytest.fixture(autouse=True)
+def _reset_config(ctx):
+    yield
+    fem.fem_set_config(ctx, reset=True)
+
+
+def stream(seed, n, K, skew=0.0, tie=0.3, gap=400):
+    """n events of K types, gaps up to `gap` us, a share `tie` of equal times; type 0 takes
+    `skew` of the events."""
+    rng = np.random.default_rng(seed)
+    g = rng.integers(1, gap + 1, n)
+    g[rng.random(n) < tie] = 0
+    ty = rng.integers(0, K, n)
+    ty[rng.random(n) < skew] = 0
+    return ty.astype(np.uint8), np.cumsum(g).astype(np.uint32)
+
+
+def check(ctx, ty, t, K, cands, I, segments=(0,), what=""):
+    sid = fem.fem_load_stream(ctx, ty, t, K)
+    L, E, iv = cands
+    rec = fem.pack_episodes(L, E, iv)
+    for p in PASSES:
+        want = oracle_counts(ty, t, L, E, iv, I, p)
+        for seg in segments:
+            fem.fem_set_config(ctx, segments=seg)
+            assert_counts_equal(fem.fem_count_candidates(ctx, sid, rec, I, p), want,
+                                f"{what} pass {p} segments {seg}")
+    fem.fem_free_stream(ctx, sid)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 2047, 2048, 2049, 4096, 9000])
+def test_sizes_and_segments(ctx, n):
+    ty, t = stream(n, n, 12)
+    cands = synth.random_candidates(n, 240, 12, [1, 2, 3, 4, 5, 6, 7, 8], 4)
+    check(ctx, ty, t, 12, cands, I_MS4, (0, 1, 2, 7, 50), f"n {n}")
+
+
+@pytest.mark.parametrize("K,skew", [(2, 0.0), (5, 0.95), (40, 0.6)])
+def test_skewed_types(ctx, K, skew):
+    """A type with most of the events: up to 64 slabs per chunk."""
+    ty, t = stream(K, 7000, K, skew, gap=3000)
+    I = np.array([[0, 3000], [1000, 9000]], np.uint32)
+    check(ctx, ty, t, K, synth.random_candidates(K, 150, K, [2, min(3, K)], 2), I, (0, 3), "skewed")
+
+
+@pytest.mark.parametrize("K", [64, 256])
+def test_overlapping_intervals(ctx, K):
+    I = np.array([[0, 30000], [10000, 12000], [5000, 60000]] + ([[0, 1], [59999, 60000], [7, 9000]]
+                                                               if K == 64 else []), np.uint32)
+    ty, t = stream(K, 12000, K, gap=900)
+    check(ctx, ty, t, K, synth.random_candidates(K, 500, K, [2, 3, 5], len(I)), I, (0, 4), f"K {K}")
+
+
+def test_windows_denser_than_a_word(ctx):
+    ty, t = stream(1, 6000, 3, gap=60)
+    I = np.array([[0, 2000], [500, 9000]], np.uint32)  # up to 100 events of a type
+    check(ctx, ty, t, 3, synth.random_candidates(1, 60, 3, [2, 3], 2), I, (0, 2), "dense")
+
+
+def test_more_hits_than_estimated(ctx):
+    """Bursts in a quiet stream: far more hits than its mean rate gives, and entry classes
+    past eight."""
+    ty, t = synth.sparse_bursts(seed=5, n_types=16, base_hz=0.5, duration_s=200.0, n_bursts=40)
+    I = np.array([[0, 2000], [2000, 20000]], np.uint32)
+    check(ctx, ty, t, 16, synth.random_candidates(2, 700, 16, [2, 3, 4, 5], 2), I, (0, 1, 5), "bursts")
+
+
+def test_no_room_for_the_tables():
+    ty, t = stream(9, 20000, 32, gap=1500)
+    L, E, iv = synth.random_candidates(9, 300, 32, [2, 3, 4], 4)
+    rec = fem.pack_episodes(L, E, iv)
+    for budget in (600 << 10, 4 << 20):
+        c = fem.fem_create(0, mem_budget_bytes=budget)
+        try:
+            sid = fem.fem_load_stream(c, ty, t, 32)
+            for p in PASSES:
+                assert_counts_equal(fem.fem_count_candidates(c, sid, rec, I_MS4, p),
+                                    oracle_counts(ty, t, L, E, iv, I_MS4, p), f"budget {budget}")
+            assert fem.fem_mem_usage(c)[0] <= budget
+            # the tables make room for a stream
+            other = fem.fem_load_stream(c, ty[:5000], t[:5000], 32)
+            fem.fem_free_stream(c, other)
+        finally:
+            fem.fem_destroy(c)
