@@ -872,12 +872,17 @@ uint32_t hit_segments(const fem_ctx *c, uint32_t n_slabs, uint32_t n_chunks, uin
 int count_grouped(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
                   uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out, cudaStream_t st);
 
-// Launch a hit-table pass over p.m candidates (and its stitch when segmented).
-int hits_launch(fem_ctx *c, const StreamDev &s, uint32_t group, CountParams &p, uint32_t classes,
-                const char *tables, cudaStream_t st) {
+// Set a hit-table pass's segments.
+void hits_segments(const fem_ctx *c, const StreamDev &s, CountParams &p) {
     const uint32_t P = hit_segments(c, p.hits.n_slabs, s.n_chunks, p.m, p.hits.slab_bytes);
     p.cps = (p.hits.n_slabs + P - 1) / P;
     p.P = (p.hits.n_slabs + p.cps - 1) / p.cps;
+}
+
+// Launch a hit-table pass over p.m candidates (and its stitch when segmented).
+int hits_launch(fem_ctx *c, const StreamDev &s, uint32_t group, CountParams &p, uint32_t classes,
+                const char *tables, cudaStream_t st) {
+    hits_segments(c, s, p);
     p.hit_classes = classes;
     if (p.P > 1) RET(dbuf(c, tables, (size_t)p.P * p.m * classes, &p.tables));
     CK(launch_hit_count(group, p.P > 1, p, st));
@@ -919,13 +924,24 @@ int hits_finish(fem_ctx *c, const StreamDev &s, uint32_t group, const CountParam
     return FEM_OK;
 }
 
-// Count a candidate set over hit tables: all lengths, in an order of their own.  *done =
-// false, with nothing counted, where they do not apply: repeated types in the set, a
-// measured launch shape, or events too dense for the tables' words.
-int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
-               uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
-               cudaStream_t st, bool *done) {
-    *done = false;
+// A set planned for hit tables, and the tables.
+struct HitPlan {
+    uint32_t *order = nullptr, *gather = nullptr;  // slot -> place in the set, candidate record
+    uint32_t group_m[PLAN_GROUPS] = {};            // candidates per launch, in slot order
+    uint32_t len_m[FEM_MAX_LEN + 1] = {};          // candidates per length
+    HitTables h{};
+    HitBuild b{};
+    uint64_t hits = 0;  // the range table's size
+};
+
+// Plan a set (checked and ordered, its edges numbered, the stream cut) and size its tables.
+// *ok = false where tables do not apply: repeated types, or a stream whose chunks do not
+// span the longest interval (the events before a slab are kept from its chunk and the one
+// before).
+int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
+              uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, cudaStream_t st, HitPlan *pl,
+              bool *ok) {
+    *ok = false;
     uint64_t max_hi = 0;
     for (const fem_interval &iv : c->ivl_host) max_hi = std::max<uint64_t>(max_hi, iv.hi_us);
     PlanArgs a{};
@@ -942,8 +958,6 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
     a.err = c->d_err;
     const uint32_t bins = plan_bins(s.K, a.parts), tri = s.K * s.K * nI;
     const size_t max_slabs = (size_t)s.n_chunks * 64 + 1;
-    uint32_t *order, *g2, *tmp;
-    uint8_t *redo;
     RET(dbuf(c, "hit_plan", PLAN_WORDS + (size_t)bins + tri, &a.words));
     a.hist = a.words + PLAN_WORDS;
     a.edge_id = a.hist + bins;
@@ -952,117 +966,175 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
     a.t0 = a.begin + max_slabs;
     RET(dbuf(c, "hit_plan_bin", m, &a.bin));
     RET(dbuf(c, "hit_plan_rank", m, &a.rank));
-    RET(dbuf(c, "hit_plan_order", m, &order));
-    RET(dbuf(c, "hit_plan_gather", m, &g2));
-    RET(dbuf(c, "hit_plan_out", m, &tmp));
-    RET(dbuf(c, "hit_plan_redo", m, &redo));
+    RET(dbuf(c, "hit_plan_order", m, &pl->order));
+    RET(dbuf(c, "hit_plan_gather", m, &pl->gather));
     const uint32_t seq = ++c->pub_seq;
-    CK(launch_plan(a, s, order, g2, Publish{c->d_plan, c->d_err, seq}, st));
-    CK(cudaMemsetAsync(redo, 0, m, st));
+    CK(launch_plan(a, s, pl->order, pl->gather, Publish{c->d_plan, c->d_err, seq}, st));
     const volatile uint32_t *w = c->h_small + kPlanWord;
     RET(wait_seq(w + PLAN_WORDS + 1, seq, st));
     RET(err_status(w[PLAN_WORDS]));
     if (w[PLAN_REP]) return FEM_OK;
-    // the events before a slab are kept from its chunk and the one before
     if (s.n_chunks > 1 && (uint64_t)(uint32_t)~w[PLAN_SPAN] <= max_hi) return FEM_OK;
-    uint32_t group_m[PLAN_GROUPS] = {};
     for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
-        if (!w[N - 1]) continue;
-        if (!c->tune.empty() &&
-            c->tune.count(tune_key((int)N, pass, true, w[N - 1], s.n_chunks, s.K)))
-            return FEM_OK;
-        group_m[plan_group(N, m)] += w[N - 1];
+        pl->len_m[N] = w[N - 1];
+        pl->group_m[plan_group(N, m)] += w[N - 1];
     }
-    // short episodes, few of them for the stream's type pairs: the tables cost more than the
-    // per-thread machine's count (533 episodes of two and three nodes, 22 types, 360,000
-    // events: 0.66 against 0.61 ms for two passes; from four nodes on the tables were the
-    // faster at every size tried)
-    uint32_t longest = 0;
-    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N)
-        if (w[N - 1]) longest = N;
-    if (longest <= 3 && (uint64_t)m * longest < 5ull * s.K * s.K && (uint64_t)s.n * s.K > 4000000) return FEM_OK;
-    HitTables h{};
+    HitTables &h = pl->h;
     h.n_slabs = w[PLAN_SLABS], h.n_edges = w[PLAN_EDGES];
     h.types = (s.K + 15) & ~15u;
     h.edge_id = a.edge_id, h.begin = a.begin, h.t0 = a.t0;
-    HitBuild b{};
+    HitBuild &b = pl->b;
     b.bev = s.bev, b.boff = s.boff, b.offs = s.offs, b.K = s.K, b.types = h.types;
     b.ivl = d_ivl, b.n_ivl = nI, b.n_edges = h.n_edges;
     b.max_words = CHUNK / 32 / w[PLAN_PARTS_MIN];
     b.edge_id = a.edge_id, b.begin = a.begin, b.err = c->d_err;
-    // hits: at most one per edge and event of its last type, K n_edges / K per event on
-    // average; as many as events lie in the intervals at the stream's mean rate, and half
-    // again (the table grows when they are more)
+    // hits: as many as events lie in the intervals at the stream's mean rate, and half again
+    // (the table grows when they are more), at most one per edge and event of its last type
     double per_event = 0;
     for (const fem_interval &iv : c->ivl_host)
         per_event += (double)(iv.hi_us - (pass == FEM_PASS_EXACT ? iv.lo_us : 0u)) * (double)s.n /
                      (double)std::max(s.t_max, 1u);
     per_event *= (double)h.n_edges / tri;
-    uint64_t hits = (uint64_t)(1.5 * per_event * (double)s.n) + 4096;
-    hits = std::min<uint64_t>(hits, (uint64_t)s.n * (h.n_edges / s.K + 1));
-    uint32_t *words;
-    auto tables = [&]() -> int {
-        RET(dbuf(c, "hit_edges", (size_t)h.n_slabs * h.n_edges, &b.edge));
-        RET(dbuf(c, "hit_counts", (size_t)h.n_slabs * h.types, &b.count));
-        RET(dbuf(c, "hit_places", (size_t)h.n_slabs * h.types, &b.place));
-        RET(dbuf(c, "hit_index", s.n, &b.index));
-        RET(dbuf(c, "hit_words", 2, &words));
-        RET(dbuf(c, "hit_ranges", hits, &b.range));
-        b.capacity = c->bufs["hit_ranges"].cap / sizeof(uint32_t);
+    pl->hits = std::min<uint64_t>((uint64_t)(1.5 * per_event * (double)s.n) + 65536,
+                                  (uint64_t)s.n * (h.n_edges / s.K + 1) + 65536);
+    *ok = true;
+    return FEM_OK;
+}
+
+// The tables' memory and their build.
+int hits_build(fem_ctx *c, const StreamDev &s, int pass, HitPlan *pl, cudaStream_t st) {
+    HitBuild &b = pl->b;
+    HitTables &h = pl->h;
+    RET(dbuf(c, "hit_edges", (size_t)h.n_slabs * h.n_edges, &b.edge));
+    RET(dbuf(c, "hit_counts", (size_t)h.n_slabs * h.types, &b.count));
+    RET(dbuf(c, "hit_places", (size_t)h.n_slabs * h.types, &b.place));
+    RET(dbuf(c, "hit_index", s.n, &b.index));
+    RET(dbuf(c, "hit_used", 1, &b.used));
+    RET(dbuf(c, "hit_ranges", pl->hits, &b.range));
+    b.capacity = std::min<uint64_t>(c->bufs["hit_ranges"].cap / sizeof(uint32_t), 0xFFFFFFF0ull);
+    CK(cudaMemsetAsync(b.used, 0, 8, st));
+    CK(launch_hit_build(pass, h.n_slabs, b, c->sm_count, st));
+    h.slab_bytes = (uint64_t)h.n_edges * 8 + pl->hits * 4 / std::max(h.n_slabs, 1u);
+    h.edge = b.edge, h.range = b.range, h.count = b.count, h.place = b.place, h.index = b.index;
+    return FEM_OK;
+}
+
+// The kernel arguments of launch g (candidates from slot `off` on).
+CountParams hits_params(fem_ctx *c, const StreamDev &s, const HitPlan &pl, const fem_episode *cands,
+                        uint32_t g, uint32_t off) {
+    CountParams p{};
+    p.cfirst = s.cfirst;
+    p.t = s.t;
+    p.n_chunks = s.n_chunks;
+    p.n = s.n;
+    p.K = s.K;
+    p.cands = cands;
+    p.gather = pl.gather + off;
+    p.m = pl.group_m[g];
+    p.ivl = pl.b.ivl;
+    p.n_ivl = pl.b.n_ivl;
+    p.err = c->d_err;
+    p.hits = pl.h;
+    return p;
+}
+
+// What became of the launches over the tables: *e the error word (capacity guards), *again
+// when the tables held too few hits (pl->hits is then what they need), *dense when events
+// were too dense for them.  The error word is cleared where nothing was counted.
+int hits_check(fem_ctx *c, HitPlan *pl, uint32_t *e, bool *again, bool *dense, cudaStream_t st) {
+    uint32_t used;
+    CK(launch_publish_count(pl->b.used, pub_of(c), st));
+    RET(read_count_err(c, nullptr, &used, e, st));
+    RET(err_status(*e));
+    *dense = (*e & ERR_DENSE) != 0 || used > 0xF0000000u;
+    *again = !*dense && used > pl->b.capacity;
+    if (*again) pl->hits = used;
+    if (*again || *dense) CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+    return FEM_OK;
+}
+
+// Count a candidate set over hit tables: all lengths, in an order of their own.  *done =
+// false, with nothing counted, where they do not apply.
+int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
+               uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
+               cudaStream_t st, bool *done) {
+    *done = false;
+    HitPlan pl;
+    bool ok;
+    RET(hits_plan(c, s, cands, gather, m, d_ivl, nI, pass, st, &pl, &ok));
+    if (!ok) return FEM_OK;
+    // short episodes, few of them for the stream's type pairs: the tables cost more than the
+    // per-thread machine's count (533 episodes of two and three nodes, 22 types, 360,000
+    // events: 0.66 against 0.61 ms for two passes; from four nodes on the tables were the
+    // faster at every size tried)
+    uint32_t longest = 0;
+    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
+        if (!pl.len_m[N]) continue;
+        longest = N;
+        // (a shape measured for the other kernels)
+        if (c->tune.count(tune_key((int)N, pass, true, pl.len_m[N], s.n_chunks, s.K))) return FEM_OK;
+    }
+    if (longest <= 3 && (uint64_t)m * longest < 5ull * s.K * s.K && (uint64_t)s.n * s.K > 4000000)
         return FEM_OK;
-    };
+    uint32_t *tmp;
+    uint8_t *redo;
+    RET(dbuf(c, "hit_plan_out", m, &tmp));
+    RET(dbuf(c, "hit_plan_redo", m, &redo));
     for (;;) {
-        if (hits > 0xFFFFFFF0ull) return FEM_OK;
-        RET(tables());
-        b.used = reinterpret_cast<unsigned long long *>(words);
-        CK(cudaMemsetAsync(b.used, 0, 8, st));
-        CK(launch_hit_build(pass, h.n_slabs, b, c->sm_count, st));
-        h.slab_bytes = (uint64_t)h.n_edges * 8 + hits * 4 / std::max(h.n_slabs, 1u);
-        h.edge = b.edge, h.range = b.range, h.count = b.count, h.place = b.place, h.index = b.index;
+        CK(cudaMemsetAsync(redo, 0, m, st));
+        RET(hits_build(c, s, pass, &pl, st));
         CountParams part[PLAN_GROUPS]{};
         uint32_t off = 0;
         for (uint32_t g = 0; g < PLAN_GROUPS; ++g) {
-            if (!group_m[g]) continue;
-            CountParams &p = part[g];
-            p.cfirst = s.cfirst;
-            p.t = s.t;
-            p.n_chunks = s.n_chunks;
-            p.n = s.n;
-            p.K = s.K;
-            p.cands = cands;
-            p.gather = g2 + off;
-            p.m = group_m[g];
-            p.ivl = d_ivl;
-            p.n_ivl = nI;
-            p.out = tmp + off;
-            p.redo = redo + off;
-            p.err = c->d_err;
-            p.hits = h;
-            RET(hits_launch(c, s, g, p, S_MAX, "tables", st));
-            off += p.m;
+            if (!pl.group_m[g]) continue;
+            part[g] = hits_params(c, s, pl, cands, g, off);
+            part[g].out = tmp + off;
+            part[g].redo = redo + off;
+            RET(hits_launch(c, s, g, part[g], S_MAX, "tables", st));
+            off += part[g].m;
         }
-        uint32_t e, used;
-        CK(launch_scatter_u32(tmp, order, m, out, st));
-        CK(launch_publish_count(b.used, pub_of(c), st));
-        RET(read_count_err(c, nullptr, &used, &e, st));
-        RET(err_status(e));
-        if (e & ERR_DENSE) {
-            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
-            return FEM_OK;
-        }
-        if (used > b.capacity) {  // more hits than the table held: a larger one
-            hits = used;
-            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
-            CK(cudaMemsetAsync(redo, 0, m, st));
-            continue;
-        }
+        uint32_t e;
+        bool again, dense;
+        CK(launch_scatter_u32(tmp, pl.order, m, out, st));
+        RET(hits_check(c, &pl, &e, &again, &dense, st));
+        if (dense) return FEM_OK;
+        if (again) continue;
         if (e & ERR_CAP) {
             for (uint32_t g = 0; g < PLAN_GROUPS; ++g)
                 if (part[g].m) RET(hits_finish(c, s, g, part[g], pass, e, st));
-            CK(launch_scatter_u32(tmp, order, m, out, st));
+            CK(launch_scatter_u32(tmp, pl.order, m, out, st));
             CK(cudaStreamSynchronize(st));
         }
         *done = true;
+        return FEM_OK;
+    }
+}
+
+// The window-based frequency of a set over exact-pass hit tables (*done as above).
+int windows_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, uint32_t m,
+                 const uint2 *d_ivl, uint32_t nI, uint32_t window_us, uint64_t *out,
+                 cudaStream_t st, bool *done) {
+    *done = false;
+    HitPlan pl;
+    bool ok;
+    RET(hits_plan(c, s, cands, nullptr, m, d_ivl, nI, FEM_PASS_EXACT, st, &pl, &ok));
+    if (!ok) return FEM_OK;
+    for (;;) {
+        CK(cudaMemsetAsync(out, 0, (size_t)m * 8, st));
+        RET(hits_build(c, s, FEM_PASS_EXACT, &pl, st));
+        uint32_t off = 0;
+        for (uint32_t g = 0; g < PLAN_GROUPS; ++g) {
+            if (!pl.group_m[g]) continue;
+            CountParams p = hits_params(c, s, pl, cands, g, off);
+            hits_segments(c, s, p);
+            CK(launch_hit_windows(g, p, pl.order + off, window_us, out, st));
+            off += p.m;
+        }
+        uint32_t e;
+        bool again, dense;
+        RET(hits_check(c, &pl, &e, &again, &dense, st));
+        if (again) continue;
+        *done = !dense;
         return FEM_OK;
     }
 }
@@ -1841,28 +1913,38 @@ int fem_count_windows(fem_ctx *c, int32_t id, const fem_episode *cands, uint32_t
     }
     uint64_t *dout = counts_out;
     if (!counts_on_device) RET(dbuf(c, "win_out", m, &dout));
-    CK(cudaMemsetAsync(c->d_small + W_INFO, 0, 3 * sizeof(uint32_t), st));
-    CK(launch_validate_cands(dc, nullptr, m, s->K, nI, c->d_small + W_INFO, c->d_err, st));
     uint32_t info[3], e;
-    RET(read_words(c, c->d_small + W_INFO, 3, info, st));
-    RET(read_err(c, st, &e));
-    RET(err_status(e));
+    RET(validate(c, *s, dc, nullptr, m, nI, info, st));
     if (info[1]) return FEM_EINVAL;  // distinct types only
-    WindowParams p{};
-    p.bev = s->bev;
-    p.boff = s->boff;
-    p.offs = s->offs;
-    p.n = s->n;
-    p.cands = dc;
-    p.m = m;
-    p.ivl = d_ivl;
-    p.w = window_us;
-    p.out = dout;
-    p.err = c->d_err;
-    CK(launch_count_windows(p, info[0], st));
-    RET(read_err(c, st, &e));
-    if (e & ERR_RING) return FEM_EOVERFLOW;
-    RET(err_status(e));
+    bool done = false;
+    if (hits_eligible(c, *s, nI)) {
+        c->hits_busy = true;
+        const int rc = windows_hits(c, *s, dc, m, d_ivl, nI, window_us, dout, st, &done);
+        c->hits_busy = false;
+        if (rc == FEM_ENOMEM) {  // no room beside the stream: the kernel without tables
+            release_hits(c);
+            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+        } else {
+            RET(rc);
+        }
+    }
+    if (!done) {
+        WindowParams p{};
+        p.bev = s->bev;
+        p.boff = s->boff;
+        p.offs = s->offs;
+        p.n = s->n;
+        p.cands = dc;
+        p.m = m;
+        p.ivl = d_ivl;
+        p.w = window_us;
+        p.out = dout;
+        p.err = c->d_err;
+        CK(launch_count_windows(p, info[0], st));
+        RET(read_err(c, st, &e));
+        if (e & ERR_RING) return FEM_EOVERFLOW;
+        RET(err_status(e));
+    }
     if (!counts_on_device) {
         CK(cudaMemcpyAsync(counts_out, dout, (size_t)m * 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));

@@ -414,18 +414,13 @@ __global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build(const HitBuild b) {
     if (dense) atomicOr(b.err, ERR_DENSE);
 }
 
-template <int NMAX, bool MC>
-cudaError_t count_run(const CountParams &p, cudaStream_t st) {
+// Launch kernel `k` over p.m candidates in blocks of 128.
+template <int NMAX, typename Kernel, typename... Args>
+cudaError_t run(Kernel k, cudaStream_t st, const CountParams &p, Args... args) {
     constexpr uint32_t T = 128;
-    const size_t sm = (size_t)hit_shared(NMAX) * 64 * T * 2;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [sm] {
-        attr_err = cudaFuncSetAttribute(k_hit_count<NMAX, MC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)sm);
-    });
-    if (attr_err != cudaSuccess) return attr_err;
-    k_hit_count<NMAX, MC><<<dim3((p.m + T - 1) / T, p.P), T, sm, st>>>(p);
+    constexpr size_t sm = (size_t)hit_shared(NMAX) * 64 * T * 2;  // at most 48 KB: no opt-in
+    static_assert(sm <= 48 * 1024, "dynamic shared memory without an attribute");
+    k<<<dim3((p.m + T - 1) / T, p.P), T, sm, st>>>(p, args...);
     note_launch();
     return cudaGetLastError();
 }
@@ -486,11 +481,23 @@ cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int 
 cudaError_t launch_hit_count(uint32_t group, bool mc, const CountParams &p, cudaStream_t st) {
     if (p.m == 0) return cudaSuccess;
     switch (group) {
-        case 0: return mc ? count_run<2, true>(p, st) : count_run<2, false>(p, st);
-        case 1: return mc ? count_run<3, true>(p, st) : count_run<3, false>(p, st);
-        case 2: return mc ? count_run<4, true>(p, st) : count_run<4, false>(p, st);
-        case 3: return mc ? count_run<5, true>(p, st) : count_run<5, false>(p, st);
-        case 4: return mc ? count_run<8, true>(p, st) : count_run<8, false>(p, st);
+#define FEM_CASE(g, n) \
+    case g: return mc ? run<n>(k_hit_count<n, true>, st, p) : run<n>(k_hit_count<n, false>, st, p);
+        FEM_CASE(0, 2) FEM_CASE(1, 3) FEM_CASE(2, 4) FEM_CASE(3, 5) FEM_CASE(4, 8)
+#undef FEM_CASE
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_hit_windows(uint32_t group, const CountParams &p, const uint32_t *order, uint32_t w,
+                               uint64_t *out, cudaStream_t st) {
+    if (p.m == 0) return cudaSuccess;
+    unsigned long long *o = reinterpret_cast<unsigned long long *>(out);
+    switch (group) {
+#define FEM_CASE(g, n) \
+    case g: return run<n>(k_hit_windows<n>, st, p, order, w, o);
+        FEM_CASE(0, 2) FEM_CASE(1, 3) FEM_CASE(2, 4) FEM_CASE(3, 5) FEM_CASE(4, 8)
+#undef FEM_CASE
         default: return cudaErrorInvalidValue;
     }
 }

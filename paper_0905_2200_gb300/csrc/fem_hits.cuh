@@ -64,39 +64,29 @@ __device__ __forceinline__ uint32_t hit_pack(uint32_t start, uint32_t len, uint3
 
 extern __shared__ __align__(128) uint8_t fem_hit_smem[];
 
-// Count one tile of candidates over segment `seg`.  NMAX: most nodes of an episode.
-// Shared memory: the chains' starts (low half) of the inner nodes' last 64 events,
-// [node][event & 63][thread]; of long episodes the later nodes', which few chains reach, are in local
-// memory (all of eight nodes' in shared memory left an SM two blocks).
-template <int NMAX, bool MC>
-__global__ void __launch_bounds__(128) k_hit_count(const CountParams p) {
-    const uint32_t T = blockDim.x, tid = threadIdx.x;
-    const uint32_t ci = blockIdx.x * T + tid, seg = blockIdx.y;
-    const HitTables &h = p.hits;
-    uint16_t *starts = reinterpret_cast<uint16_t *>(fem_hit_smem) + tid;
-    constexpr int SHARED = hit_shared(NMAX);
-    uint16_t deep[hit_inner(NMAX) > SHARED ? (hit_inner(NMAX) - SHARED) * 64 : 1];
-    auto start_of = [&](int d, uint32_t at) -> uint16_t & {
-        if (hit_inner(NMAX) <= SHARED || d <= SHARED) return starts[((uint32_t)(d - 1) * 64u + (at & 63u)) * T];
-        return deep[(uint32_t)(d - 1 - SHARED) * 64u + (at & 63u)];
-    };
-
-    // ------------------------------------------------------------ episode
-    bool ok = ci < p.m;
-    uint32_t N = 0, last = 0;
-    uint64_t W = 0;
+// One thread's episode going through the slabs.  NMAX: most nodes of an episode.  Shared
+// memory: the chains' starts (low half) of the inner nodes' last 64 events,
+// [node][event & 63][thread]; of long episodes the later nodes', which few chains reach,
+// are in local memory (all of eight nodes' in shared memory left an SM two blocks).
+template <int NMAX>
+struct HitEpisode {
+    uint32_t N, last;                 // nodes, last type
+    uint64_t W;                       // sum of hi
     uint32_t edge[NMAX], type[NMAX];  // edge d joins node d - 1 to node d
+
+    // The candidate of the thread's slot; false if there is none or it is malformed.
+    __device__ __forceinline__ bool load(const CountParams &p, uint32_t ci) {
+        N = 0, last = 0, W = 0;
 #pragma unroll
-    for (int d = 0; d < NMAX; ++d) edge[d] = 0, type[d] = 0;
-    if (ok) {
+        for (int d = 0; d < NMAX; ++d) edge[d] = 0, type[d] = 0;
+        if (ci >= p.m) return false;
         const uint4 v = reinterpret_cast<const uint4 *>(p.cands)[p.gather ? p.gather[ci] : ci];
         fem_episode rec;
         memcpy(&rec, &v, sizeof(rec));
-        N = rec.len;
-        ok = N >= 1 && N <= NMAX;
+        bool ok = rec.len >= 1 && rec.len <= NMAX;
 #pragma unroll
         for (int d = 0; d < NMAX; ++d) {
-            if (ok && d < (int)N) {
+            if (ok && d < (int)rec.len) {
                 type[d] = rec.types[d];
                 ok = type[d] < p.K;
                 last = type[d];
@@ -105,16 +95,133 @@ __global__ void __launch_bounds__(128) k_hit_count(const CountParams p) {
                     ok = iv < p.n_ivl;
                     if (ok) {
                         W += p.ivl[iv].y;
-                        edge[d] = h.edge_id[(type[d > 0 ? d - 1 : 0] * p.K + type[d]) * p.n_ivl + iv];
+                        edge[d] = p.hits.edge_id[(type[d > 0 ? d - 1 : 0] * p.K + type[d]) * p.n_ivl + iv];
                     }
                 }
             }
         }
-        if (!ok) {
-            atomicOr(p.err, ERR_BADEP);
-            N = 0;
+        if (ok) N = rec.len;
+        else atomicOr(p.err, ERR_BADEP);
+        return ok;
+    }
+
+    // Slabs [s_w, s1) (the same in every lane of the warp): slab(s) before each, then
+    // leaf(s, r, S) for every last-node event (the slab's r-th of its type) that a chain
+    // reaches, in order; S is the index of the latest chain's first event.
+    template <typename SLAB, typename LEAF>
+    __device__ __forceinline__ void walk(const HitTables &h, uint32_t s_w, uint32_t s1, SLAB &&slab,
+                                         LEAF &&leaf) const {
+        constexpr int SHARED = hit_shared(NMAX);
+        const uint32_t T = blockDim.x;
+        uint16_t *starts = reinterpret_cast<uint16_t *>(fem_hit_smem) + threadIdx.x;
+        uint16_t deep[hit_inner(NMAX) > SHARED ? (hit_inner(NMAX) - SHARED) * 64 : 1];
+        auto start_of = [&](int d, uint32_t at) -> uint16_t & {
+            if (hit_inner(NMAX) <= SHARED || d <= SHARED)
+                return starts[((uint32_t)(d - 1) * 64u + (at & 63u)) * T];
+            return deep[(uint32_t)(d - 1 - SHARED) * 64u + (at & 63u)];
+        };
+        // Per inner node: its admitted events among the 32 before the slab, and where the
+        // event 32 before the slab's first sits in `starts`.
+        uint32_t hist[NMAX], at[NMAX];
+#pragma unroll
+        for (int d = 0; d < NMAX; ++d) hist[d] = 0, at[d] = 0;
+        // An edge's mask is asked for a slab ahead, its first ranges before any edge's are
+        // used; in episodes of six or more nodes only the first edges', the others' when the
+        // node before has any admitted event, which is seldom so.
+        constexpr int MASKS = NMAX <= 5 ? NMAX : 4, HEADS = NMAX <= 5 ? NMAX : 3, G = 4;
+        uint2 nxt[MASKS];
+#pragma unroll
+        for (int d = 1; d < MASKS; ++d)
+            nxt[d] = d < (int)N ? h.edge[(uint64_t)s_w * h.n_edges + edge[d]] : make_uint2(0u, 0u);
+        for (uint32_t s = s_w; s < s1; ++s) {
+            uint2 now[MASKS];
+            uint32_t cn[NMAX];
+            const uint8_t *crow = h.count + (uint64_t)s * h.types;
+            const uint2 *erow = h.edge + (uint64_t)s * h.n_edges;
+#pragma unroll
+            for (int d = 1; d < NMAX; ++d) {
+                cn[d] = d + 1 < NMAX && d + 1 < (int)N ? crow[type[d]] : 0u;
+                if (d >= MASKS) continue;
+                now[d] = nxt[d];
+                if (s + 1 < s1 && d < (int)N) nxt[d] = erow[h.n_edges + edge[d]];
+            }
+            slab(s);
+            const uint32_t end = h.begin[s + 1];  // a low half names one of the 65,536 before it
+            uint32_t head[HEADS][G];
+#pragma unroll
+            for (int d = 1; d < HEADS; ++d) {
+                const uint32_t k = d < (int)N ? __popc(now[d].x) : 0u;
+#pragma unroll
+                for (int g = 0; g < G; ++g) head[d][g] = (uint32_t)g < k ? __ldg(h.range + now[d].y + g) : 0u;
+            }
+            uint64_t before = 0;  // admitted events of the node before
+#pragma unroll
+            for (int d = 1; d < NMAX; ++d) {
+                if (d >= (int)N) continue;
+                const bool is_leaf = d + 1 == (int)N;
+                uint32_t bits = 0, rg = 0, cur = 0, e4[G];
+                if (d == 1 || before) {
+                    const uint2 e = d < MASKS ? now[d < MASKS ? d : 0] : erow[edge[d]];
+                    bits = e.x, rg = e.y;
+                    const uint32_t k = __popc(bits);
+#pragma unroll
+                    for (int g = 0; g < G; ++g)
+                        e4[g] = d < HEADS ? head[d < HEADS ? d : 0][g]
+                                          : (uint32_t)g < k ? __ldg(h.range + rg + g) : 0u;
+                }
+                while (bits) {
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        if (!bits) break;
+                        const uint32_t r = __ffs(bits) - 1;
+                        bits &= bits - 1u;
+                        const uint32_t e = e4[g];
+                        uint32_t S = e >> 16;
+                        if (d > 1) {
+                            const uint32_t start = e & 63u, len = (e >> 6) & 63u;
+                            const uint32_t w = (uint32_t)(before >> start) & (0xFFFFFFFFu >> (32u - len));
+                            if (!w) continue;
+                            S = start_of(d - 1, at[d - 1] + start + 31u - (uint32_t)__clz(w));
+                        }
+                        if (!is_leaf) {
+                            cur |= 1u << r;
+                            if (d + 1 < NMAX) start_of(d, at[d] + 32u + r) = (uint16_t)S;
+                        } else {
+                            leaf(s, r, end - ((end - S) & 0xFFFFu));
+                        }
+                    }
+                    if (!bits) break;
+                    rg += G;
+                    const uint32_t k = __popc(bits);
+#pragma unroll
+                    for (int g = 0; g < G; ++g) e4[g] = (uint32_t)g < k ? __ldg(h.range + rg + g) : 0u;
+                }
+                if (!is_leaf) {
+                    before = (uint64_t)cur << 32 | hist[d];
+                    hist[d] = (uint32_t)(before >> cn[d]);
+                }
+            }
+#pragma unroll
+            for (int d = 1; d < NMAX; ++d) at[d] += cn[d];
         }
     }
+
+    // The index of the slab's r-th event of the last type.
+    __device__ __forceinline__ uint32_t index(const HitTables &h, uint32_t s, uint32_t r) const {
+        const uint32_t end = h.begin[s + 1];
+        const uint32_t i = h.index[h.begin[s] + h.place[(uint64_t)s * h.types + last] + r];
+        return end - ((end - i) & 0xFFFFu);
+    }
+};
+
+// Count one tile of candidates over segment `seg`.
+template <int NMAX, bool MC>
+__global__ void __launch_bounds__(128) k_hit_count(const CountParams p) {
+    const uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x, seg = blockIdx.y;
+    const HitTables &h = p.hits;
+    HitEpisode<NMAX> ep;
+    const bool ok = ep.load(p, ci);
+    const uint64_t W = ep.W;
 
     // ------------------------------------------------------------ segment and window
     const uint32_t s0 = seg * p.cps, s1 = min(s0 + p.cps, h.n_slabs);
@@ -208,106 +315,27 @@ __global__ void __launch_bounds__(128) k_hit_count(const CountParams p) {
     };
 
     // ------------------------------------------------------------ slabs
-    // Per inner node: its admitted events among the 32 before the slab, and where the
-    // event 32 before the slab's first sits in `starts`.
-    uint32_t hist[NMAX], at[NMAX];
-#pragma unroll
-    for (int d = 0; d < NMAX; ++d) hist[d] = 0, at[d] = 0;
-    if (N == 1) {
-        for (uint32_t s = s0; s < s1; ++s) cnt += h.count[(uint64_t)s * h.types + last];
-        N = 0;
+    if (ep.N == 1) {
+        for (uint32_t s = s0; s < s1; ++s) cnt += h.count[(uint64_t)s * h.types + ep.last];
+        ep.N = 0;
     }
-    // An edge's mask is asked for a slab ahead, its first ranges before any edge's are used;
-    // in episodes of six or more nodes only the first edges', the others' when the node
-    // before has any admitted event, which is seldom so.
-    constexpr int MASKS = NMAX <= 5 ? NMAX : 4, HEADS = NMAX <= 5 ? NMAX : 3, G = 4;
-    uint2 nxt[MASKS];
-#pragma unroll
-    for (int d = 1; d < MASKS; ++d)
-        nxt[d] = d < (int)N ? h.edge[(uint64_t)s_w * h.n_edges + edge[d]] : make_uint2(0u, 0u);
-    for (uint32_t s = s_w; s < s1; ++s) {
-        uint2 now[MASKS];
-        uint32_t cn[NMAX];
-        const uint8_t *crow = h.count + (uint64_t)s * h.types;
-        const uint2 *erow = h.edge + (uint64_t)s * h.n_edges;
-#pragma unroll
-        for (int d = 1; d < NMAX; ++d) {
-            cn[d] = d + 1 < NMAX && d + 1 < (int)N ? crow[type[d]] : 0u;
-            if (d >= MASKS) continue;
-            now[d] = nxt[d];
-            if (s + 1 < s1 && d < (int)N) nxt[d] = erow[h.n_edges + edge[d]];
-        }
-        if (MC && umask) merge_before(h.t0[s], s < s0);
-        const uint32_t end = h.begin[s + 1];  // an index's low half names one of the 65,536 before it
-        uint32_t head[HEADS][G];
-#pragma unroll
-        for (int d = 1; d < HEADS; ++d) {
-            const uint32_t k = d < (int)N ? __popc(now[d].x) : 0u;
-#pragma unroll
-            for (int g = 0; g < G; ++g) head[d][g] = (uint32_t)g < k ? __ldg(h.range + now[d].y + g) : 0u;
-        }
-        uint64_t before = 0;  // admitted events of the node before
-#pragma unroll
-        for (int d = 1; d < NMAX; ++d) {
-            if (d >= (int)N) continue;
-            const bool leaf = d + 1 == (int)N;
-            uint32_t bits = 0, rg = 0, cur = 0, e4[G];
-            if (d == 1 || before) {
-                const uint2 e = d < MASKS ? now[d < MASKS ? d : 0] : erow[edge[d]];
-                bits = e.x, rg = e.y;
-                const uint32_t k = __popc(bits);
-#pragma unroll
-                for (int g = 0; g < G; ++g)
-                    e4[g] = d < HEADS ? head[d < HEADS ? d : 0][g]
-                                      : (uint32_t)g < k ? __ldg(h.range + rg + g) : 0u;
+    ep.walk(
+        h, s_w, s1,
+        [&](uint32_t s) {
+            if (MC && umask) merge_before(h.t0[s], s < s0);
+        },
+        [&](uint32_t s, uint32_t r, uint32_t S) {
+            const bool slow = MC && (s < s0 || umask);
+            if (!slow && S < st) return;
+            const uint32_t gidx = ep.index(h, s, r);
+            if (slow) {
+                slow_event(gidx, S);
+            } else {
+                st = gidx + 1u;
+                ++cnt;
+                if (MC) c0_done = true;
             }
-            while (bits) {
-#pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    if (!bits) break;
-                    const uint32_t r = __ffs(bits) - 1;
-                    bits &= bits - 1u;
-                    const uint32_t e = e4[g];
-                    uint32_t S = e >> 16;
-                    if (d > 1) {
-                        const uint32_t start = e & 63u, len = (e >> 6) & 63u;
-                        const uint32_t w = (uint32_t)(before >> start) & (0xFFFFFFFFu >> (32u - len));
-                        if (!w) continue;
-                        S = start_of(d - 1, at[d - 1] + start + 31u - (uint32_t)__clz(w));
-                    }
-                    if (!leaf) {
-                        cur |= 1u << r;
-                        if (d + 1 < NMAX) start_of(d, at[d] + 32u + r) = (uint16_t)S;
-                        continue;
-                    }
-                    S = end - ((end - S) & 0xFFFFu);
-                    const bool slow = MC && (s < s0 || umask);
-                    if (!slow && S < st) continue;
-                    const uint32_t i =
-                        h.index[h.begin[s] + h.place[(uint64_t)s * h.types + last] + r];
-                    const uint32_t gidx = end - ((end - i) & 0xFFFFu);
-                    if (slow) {
-                        slow_event(gidx, S);
-                    } else {
-                        st = gidx + 1u;
-                        ++cnt;
-                        if (MC) c0_done = true;
-                    }
-                }
-                if (!bits) break;
-                rg += G;
-                const uint32_t k = __popc(bits);
-#pragma unroll
-                for (int g = 0; g < G; ++g) e4[g] = (uint32_t)g < k ? __ldg(h.range + rg + g) : 0u;
-            }
-            if (!leaf) {
-                before = (uint64_t)cur << 32 | hist[d];
-                hist[d] = (uint32_t)(before >> cn[d]);
-            }
-        }
-#pragma unroll
-        for (int d = 1; d < NMAX; ++d) at[d] += cn[d];
-    }
+        });
 
     // ------------------------------------------------------------ results
     if (ci >= p.m) return;
@@ -332,6 +360,55 @@ __global__ void __launch_bounds__(128) k_hit_count(const CountParams p) {
             tab[j] = e;
         }
     }
+}
+
+// Window-based frequency (fem_windows.cu) of one tile of candidates over segment `seg`: the
+// starts whose window holds a chain ending at last-node event j are (t[j] - w, t[S]], S the
+// latest chain's first event (the exact pass's chains).  The ranges' left ends increase, so
+// what is at or below the greatest right end so far is covered, and event j adds what lies
+// above it.  A segment finds that end from the last-node events of the w before it (an
+// earlier one's range ends before its own ranges begin), and the segments' sums add up: no
+// stitch.  One thread per episode walked the whole stream before (fem_windows.cu), few warps
+// and long chains of loads: 16,128 pairs on 406,000 events 15.5 ms, now 0.10 ms and 0.52
+// for the tables.
+template <int NMAX>
+__global__ void __launch_bounds__(128) k_hit_windows(const CountParams p, const uint32_t *order,
+                                                     uint32_t w, unsigned long long *out) {
+    const uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x, seg = blockIdx.y;
+    const HitTables &h = p.hits;
+    HitEpisode<NMAX> ep;
+    const bool ok = ep.load(p, ci);
+    const uint32_t s0 = seg * p.cps, s1 = min(s0 + p.cps, h.n_slabs);
+    uint32_t s_w = s0;
+    if (ok) {
+        // chains of the events of the w before the segment: none starts before back
+        const uint64_t t = h.t0[s0], reach = (uint64_t)w + ep.W;
+        const uint32_t back = t >= reach ? (uint32_t)(t - reach) : 0u;
+        while (s_w > 0 && h.t0[s_w] >= back) --s_w;
+    }
+    s_w = __reduce_min_sync(0xffffffffu, s_w);
+    int64_t covered = -0x7FFFFFFFFFFFFFFFll;
+    uint64_t sum = 0;
+    auto add = [&](uint32_t s, int64_t t, int64_t right) {
+        const int64_t left = t - (int64_t)w;  // starts left + 1 .. right
+        if (left >= right) return;            // the chain is longer than the window
+        if (s >= s0) sum += (uint64_t)max((int64_t)0, right - max(left, covered));
+        covered = max(covered, right);
+    };
+    if (ep.N == 1) {
+        for (uint32_t s = s_w; s < s1; ++s) {
+            const uint32_t n = h.count[(uint64_t)s * h.types + ep.last];
+            for (uint32_t r = 0; r < n; ++r) {
+                const int64_t t = p.t[ep.index(h, s, r)];
+                add(s, t, t);
+            }
+        }
+        ep.N = 0;
+    }
+    ep.walk(
+        h, s_w, s1, [](uint32_t) {},
+        [&](uint32_t s, uint32_t r, uint32_t S) { add(s, p.t[ep.index(h, s, r)], p.t[S]); });
+    if (ok && sum) atomicAdd(&out[order[ci]], (unsigned long long)sum);
 }
 
 }  // namespace fem

@@ -261,6 +261,10 @@ size_t chain_smem_bytes(int N, bool mc, uint32_t threads, uint32_t offs);
 // fem_hits.cu: the same passes over hit tables (distinct types, lengths 1..8, one segment
 // or MapConcatenate over runs of slabs).  group: the episodes' plan_group
 cudaError_t launch_hit_count(uint32_t group, bool mc, const CountParams &p, cudaStream_t st);
+// the window-based frequency over exact-pass tables: out[order[slot]] += candidate slot's
+// starts (out zeroed by the caller)
+cudaError_t launch_hit_windows(uint32_t group, const CountParams &p, const uint32_t *order, uint32_t w,
+                               uint64_t *out, cudaStream_t st);
 struct HitBuild {
     const uint2 *bev;
     const uint16_t *boff;

@@ -2,7 +2,9 @@
 // after Mannila et al.), with the episode's interval constraints: the number of
 // integer window starts s such that some occurrence lies inside [s, s + w).
 //
-// One thread per episode walks the bucketed stream (global memory, L2-resident for
+// Where the hit tables apply, k_hit_windows (fem_hits.cuh) counts over them.  This kernel
+// is for the rest: configured kernels, streams too dense for the tables' words, many type
+// pairs and intervals.  One thread per episode walks the bucketed stream (global memory, L2-resident for
 // the workloads here), merging its N type groups by local index.  For each event j
 // of node k it needs L_k(j), the latest first-node time over the chains ending at j:
 // the maximum of L_{k-1} over the node-(k-1) events i < j with lo < t[j] - t[i] <= hi.

@@ -106,3 +106,17 @@ def test_no_room_for_the_tables():
             fem.fem_free_stream(c, other)
         finally:
             fem.fem_destroy(c)
+
+
+@pytest.mark.parametrize("n,w_us", [(1, 5), (33, 900), (2049, 1), (7000, 2500), (9000, 400000)])
+@pytest.mark.parametrize("segments", [0, 1, 5, 60])
+def test_window_frequency(ctx, n, w_us, segments):
+    """Window frequencies over segments: windows shorter and longer than a segment, one event,
+    equal times at the cuts."""
+    ty, t = stream(n + 1, n, 9)
+    cands = synth.random_candidates(n, 150, 9, [1, 2, 3, 4, 6, 8], 4)
+    sid = fem.fem_load_stream(ctx, ty, t, 9)
+    fem.fem_set_config(ctx, segments=segments)
+    got = fem.fem_count_windows(ctx, sid, fem.pack_episodes(*cands), I_MS4, w_us)
+    assert_counts_equal(got, oracle.count_windows_batch(ty, t, *cands, I_MS4, w_us), "windows")
+    fem.fem_free_stream(ctx, sid)
