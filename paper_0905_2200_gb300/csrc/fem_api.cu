@@ -938,9 +938,11 @@ struct HitPlan {
 // *ok = false where tables do not apply: repeated types, or a stream whose chunks do not
 // span the longest interval (the events before a slab are kept from its chunk and the one
 // before).
+// alloc(name, words, &pointer) gives the plan's device memory.
+template <typename Alloc>
 int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
-              uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, cudaStream_t st, HitPlan *pl,
-              bool *ok) {
+              uint32_t m, bool fine, const uint2 *d_ivl, uint32_t nI, int pass, cudaStream_t st,
+              HitPlan *pl, bool *ok, Alloc &&alloc) {
     *ok = false;
     uint64_t max_hi = 0;
     for (const fem_interval &iv : c->ivl_host) max_hi = std::max<uint64_t>(max_hi, iv.hi_us);
@@ -951,6 +953,7 @@ int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     a.K = s.K;
     a.n_ivl = nI;
     a.parts = std::min(nI, PLAN_PARTS);
+    a.fine = fine;
     a.cfirst = s.cfirst;
     a.t = s.t;
     a.n_chunks = s.n_chunks;
@@ -958,16 +961,16 @@ int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     a.err = c->d_err;
     const uint32_t bins = plan_bins(s.K, a.parts), tri = s.K * s.K * nI;
     const size_t max_slabs = (size_t)s.n_chunks * 64 + 1;
-    RET(dbuf(c, "hit_plan", PLAN_WORDS + (size_t)bins + tri, &a.words));
+    RET(alloc("hit_plan", PLAN_WORDS + (size_t)bins + tri, &a.words));
     a.hist = a.words + PLAN_WORDS;
     a.edge_id = a.hist + bins;
-    RET(dbuf(c, "hit_plan_slabs", s.n_chunks + 2 * max_slabs, &a.parts_of));
+    RET(alloc("hit_plan_slabs", s.n_chunks + 2 * max_slabs, &a.parts_of));
     a.begin = a.parts_of + s.n_chunks;
     a.t0 = a.begin + max_slabs;
-    RET(dbuf(c, "hit_plan_bin", m, &a.bin));
-    RET(dbuf(c, "hit_plan_rank", m, &a.rank));
-    RET(dbuf(c, "hit_plan_order", m, &pl->order));
-    RET(dbuf(c, "hit_plan_gather", m, &pl->gather));
+    RET(alloc("hit_plan_bin", m, &a.bin));
+    RET(alloc("hit_plan_rank", m, &a.rank));
+    RET(alloc("hit_plan_order", m, &pl->order));
+    RET(alloc("hit_plan_gather", m, &pl->gather));
     const uint32_t seq = ++c->pub_seq;
     CK(launch_plan(a, s, pl->order, pl->gather, Publish{c->d_plan, c->d_err, seq}, st));
     const volatile uint32_t *w = c->h_small + kPlanWord;
@@ -977,7 +980,7 @@ int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     if (s.n_chunks > 1 && (uint64_t)(uint32_t)~w[PLAN_SPAN] <= max_hi) return FEM_OK;
     for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
         pl->len_m[N] = w[N - 1];
-        pl->group_m[plan_group(N, m)] += w[N - 1];
+        pl->group_m[plan_group(N, a.fine)] += w[N - 1];
     }
     HitTables &h = pl->h;
     h.n_slabs = w[PLAN_SLABS], h.n_edges = w[PLAN_EDGES];
@@ -988,15 +991,16 @@ int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     b.ivl = d_ivl, b.n_ivl = nI, b.n_edges = h.n_edges;
     b.max_words = CHUNK / 32 / w[PLAN_PARTS_MIN];
     b.edge_id = a.edge_id, b.begin = a.begin, b.err = c->d_err;
-    // hits: as many as events lie in the intervals at the stream's mean rate, and half again
-    // (the table grows when they are more), at most one per edge and event of its last type
+    // hits: as many as events lie in the intervals at the stream's mean rate, and a quarter
+    // more (the table grows when that is too few), at most one per edge and event of its last type
     double per_event = 0;
     for (const fem_interval &iv : c->ivl_host)
         per_event += (double)(iv.hi_us - (pass == FEM_PASS_EXACT ? iv.lo_us : 0u)) * (double)s.n /
                      (double)std::max(s.t_max, 1u);
     per_event *= (double)h.n_edges / tri;
-    pl->hits = std::min<uint64_t>((uint64_t)(1.5 * per_event * (double)s.n) + 65536,
-                                  (uint64_t)s.n * (h.n_edges / s.K + 1) + 65536);
+    pl->hits = std::min<uint64_t>((uint64_t)(1.25 * per_event * (double)s.n) + 65536,
+                                  (uint64_t)s.n * (h.n_edges / s.K + 1)) +
+               hit_slack(h.n_slabs);
     *ok = true;
     return FEM_OK;
 }
@@ -1048,7 +1052,7 @@ int hits_check(fem_ctx *c, HitPlan *pl, uint32_t *e, bool *again, bool *dense, c
     RET(err_status(*e));
     *dense = (*e & ERR_DENSE) != 0 || used > 0xF0000000u;
     *again = !*dense && used > pl->b.capacity;
-    if (*again) pl->hits = used;
+    if (*again) pl->hits = used + used / 16 + hit_slack(pl->h.n_slabs);
     if (*again || *dense) CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
     return FEM_OK;
 }
@@ -1061,7 +1065,8 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
     *done = false;
     HitPlan pl;
     bool ok;
-    RET(hits_plan(c, s, cands, gather, m, d_ivl, nI, pass, st, &pl, &ok));
+    RET(hits_plan(c, s, cands, gather, m, m >= PLAN_FINE, d_ivl, nI, pass, st, &pl, &ok,
+                  [&](const char *n, size_t w, uint32_t **p) { return dbuf(c, n, w, p); }));
     if (!ok) return FEM_OK;
     // short episodes, few of them for the stream's type pairs: the tables cost more than the
     // per-thread machine's count (533 episodes of two and three nodes, 22 types, 360,000
@@ -1117,7 +1122,8 @@ int windows_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, uint3
     *done = false;
     HitPlan pl;
     bool ok;
-    RET(hits_plan(c, s, cands, nullptr, m, d_ivl, nI, FEM_PASS_EXACT, st, &pl, &ok));
+    RET(hits_plan(c, s, cands, nullptr, m, m >= PLAN_FINE, d_ivl, nI, FEM_PASS_EXACT, st, &pl, &ok,
+                  [&](const char *n, size_t w, uint32_t **p) { return dbuf(c, n, w, p); }));
     if (!ok) return FEM_OK;
     for (;;) {
         CK(cudaMemsetAsync(out, 0, (size_t)m * 8, st));
@@ -2303,9 +2309,41 @@ struct BatchGroup {
 
 }  // namespace
 
+namespace {
+
+// A batch counted over hit tables: its candidates by stream, each stream's planned once
+// (order, edges, slabs), the tables built and the candidates counted in every run.  A part
+// is a stream's candidates of one launch group; slots are in part order.
+struct BatchHits {
+    uint32_t n_jobs = 0, m = 0, n_streams = 0, n_parts = 0, n_slabs = 0;
+    std::vector<HitBuild> build;            // per stream
+    std::vector<CountParams> parts;         // per part, relaxed pass
+    HitBuild *d_build = nullptr;
+    uint32_t *first = nullptr;              // first slab block of each stream
+    CountParams *rparts = nullptr, *xparts = nullptr;
+    uint32_t *part_off = nullptr;           // first slot of each part
+    struct Launch {
+        uint4 *list = nullptr;
+        uint32_t n_list = 0, n_items = 0;
+    };
+    Launch rel[PLAN_GROUPS], ex[PLAN_GROUPS];
+    fem_episode *cands = nullptr;
+    uint32_t *record = nullptr;             // slot -> candidate
+    uint32_t *cand_off = nullptr, *theta = nullptr;  // per job
+    BatchOut *outs = nullptr;
+    uint32_t *r = nullptr, *x = nullptr, *idx = nullptr, *gx = nullptr, *scratch = nullptr, *n_idx = nullptr;
+    uint8_t *flags = nullptr, *redo = nullptr, *xredo = nullptr;
+    unsigned long long *used = nullptr;     // hits found by either pass
+    uint64_t capacity = 0;
+};
+
+}  // namespace
+
 struct fem_batch {
     fem_ctx *ctx = nullptr;
     std::vector<fem_job> jobs;
+    bool over_hits = false;
+    BatchHits hits;
     std::vector<BatchGroup> groups;
     std::vector<void *> allocs;
     std::vector<size_t> alloc_bytes;
@@ -2388,8 +2426,35 @@ int batch_enqueue_group(fem_ctx *c, BatchGroup &g, cudaStream_t st) {
     return FEM_OK;
 }
 
+// The two-pass count of a batch over hit tables, enqueued without host round trips.
+int batch_enqueue_hits(fem_ctx *c, BatchHits &h, cudaStream_t st) {
+    CK(cudaMemsetAsync(h.used, 0, 16, st));
+    CK(cudaMemsetAsync(h.redo, 0, h.m, st));
+    CK(cudaMemsetAsync(h.xredo, 0, h.m, st));
+    // first pass: relaxed counts of every candidate (Algorithm 3)
+    CK(launch_hit_build_batch(FEM_PASS_RELAXED, h.build.data(), h.d_build, h.first, h.n_streams, h.n_slabs, st));
+    for (uint32_t g = 0; g < PLAN_GROUPS; ++g)
+        CK(launch_hit_count_batch(g, h.rparts, h.rel[g].list, h.rel[g].n_list, h.rel[g].n_items, st));
+    CK(launch_stitch_batch(h.rparts, h.part_off, h.n_parts, h.m, c->d_err, st, S_RECOUNT));
+    // elimination at each job's theta (Algorithm 4)
+    CK(launch_batch_keep_slots(h.r, h.record, h.cand_off, h.theta, h.n_jobs, h.m, h.flags, st));
+    CK(launch_compact(nullptr, h.flags, 0, h.m, h.idx, h.n_idx, h.scratch, st));
+    CK(launch_batch_pick(h.idx, h.n_idx, h.m, h.record, h.gx, st));
+    // second pass: exact counts of the survivors (Algorithm 1)
+    CK(launch_batch_exact_jobs(h.xparts, h.part_off, h.n_parts, h.idx, h.n_idx, h.x, st, h.gx));
+    CK(cudaMemcpyAsync(h.used + 1, h.used, 8, cudaMemcpyDeviceToDevice, st));
+    CK(cudaMemsetAsync(h.used, 0, 8, st));
+    CK(launch_hit_build_batch(FEM_PASS_EXACT, h.build.data(), h.d_build, h.first, h.n_streams, h.n_slabs, st));
+    for (uint32_t g = 0; g < PLAN_GROUPS; ++g)
+        CK(launch_hit_count_batch(g, h.xparts, h.ex[g].list, h.ex[g].n_list, h.ex[g].n_items, st));
+    CK(launch_stitch_batch(h.xparts, h.part_off, h.n_parts, h.m, c->d_err, st, S_RECOUNT));
+    CK(launch_batch_outputs(h.outs, h.cand_off, h.n_jobs, h.m, h.gx, h.n_idx, h.x, st));
+    return FEM_OK;
+}
+
 // The whole two-pass count of the batch, enqueued on st without host round trips.
 int batch_enqueue(fem_batch *b, cudaStream_t st) {
+    if (b->over_hits) return batch_enqueue_hits(b->ctx, b->hits, st);
     for (BatchGroup &g : b->groups) RET(batch_enqueue_group(b->ctx, g, st));
     return FEM_OK;
 }
@@ -2429,6 +2494,211 @@ int batch_tune(fem_batch *b, cudaStream_t st) {
         if (std::getenv("FEM_DEBUG"))
             std::fprintf(stderr, "fem: batch N=%d jobs=%u m=%u: %u chunks per item, T %u/%u, %.3f ms\n",
                          g.N, g.n_jobs, g.m, bc, br, bx, best);
+    }
+    return FEM_OK;
+}
+
+// Plans a batch over hit tables and runs it once; *ok = false, with its memory given back,
+// where tables do not apply to one of the streams or their memory would pass an eighth of
+// the device's (or the context's budget).
+int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
+    *ok = false;
+    fem_ctx *c = b->ctx;
+    BatchHits &h = b->hits;
+    const uint32_t nI = b->nI;
+    size_t free_bytes = 0, total_bytes = 0;
+    CK(cudaMemGetInfo(&free_bytes, &total_bytes));
+    const uint64_t most = std::min(total_bytes / 8, free_bytes / 2);
+    // the jobs by stream
+    std::vector<uint32_t> job, off{0};
+    std::vector<int32_t> streams;
+    for (uint32_t j = 0; j < b->jobs.size(); ++j)
+        if (b->jobs[j].m && std::find(streams.begin(), streams.end(), b->jobs[j].stream_id) == streams.end())
+            streams.push_back(b->jobs[j].stream_id);
+    std::vector<uint32_t> stream_off;
+    uint64_t m = 0;
+    for (int32_t id : streams) {
+        if (!hits_eligible(c, *find_stream(c, id), nI)) return FEM_OK;
+        stream_off.push_back((uint32_t)m);
+        for (uint32_t j = 0; j < b->jobs.size(); ++j) {
+            if (b->jobs[j].stream_id != id || !b->jobs[j].m) continue;
+            job.push_back(j);
+            m += b->jobs[j].m;
+            off.push_back((uint32_t)m);
+        }
+        if (m > 0x7FFFFFFFull) return FEM_OK;
+    }
+    if (m == 0) return FEM_OK;
+    h.m = (uint32_t)m, h.n_jobs = (uint32_t)job.size(), h.n_streams = (uint32_t)streams.size();
+    RET(balloc(b, m, &h.cands));
+    std::vector<uint32_t> theta(h.n_jobs), iota(m);
+    std::vector<BatchOut> outs(h.n_jobs);
+    for (uint32_t k = 0; k < h.n_jobs; ++k) {
+        const fem_job &jb = b->jobs[job[k]];
+        CK(cudaMemcpyAsync(h.cands + off[k], jb.cands, (size_t)jb.m * sizeof(fem_episode),
+                           cudaMemcpyDeviceToDevice, st));
+        theta[k] = jb.theta;
+        outs[k] = BatchOut{jb.exact_out, jb.survived_out};
+    }
+    // every candidate has its job's length (the counting kernels take any)
+    std::vector<fem_episode> host(m);
+    CK(cudaMemcpyAsync(host.data(), h.cands, m * sizeof(fem_episode), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    for (uint32_t k = 0; k < h.n_jobs; ++k)
+        for (uint32_t i = off[k]; i < off[k + 1]; ++i)
+            if (host[i].len != b->jobs[job[k]].len) return FEM_EINVAL;
+    for (uint32_t i = 0; i < m; ++i) iota[i] = i;
+    uint32_t *d_iota;
+    RET(balloc(b, m, &d_iota));
+    RET(balloc(b, m, &h.record));
+    RET(balloc(b, h.n_jobs + 1, &h.cand_off));
+    RET(balloc(b, h.n_jobs, &h.theta));
+    RET(balloc(b, h.n_jobs, &h.outs));
+    RET(balloc(b, m, &h.r));
+    RET(balloc(b, m, &h.x));
+    RET(balloc(b, m, &h.idx));
+    RET(balloc(b, m, &h.gx));
+    RET(balloc(b, compact_scratch_words(h.m), &h.scratch));
+    RET(balloc(b, 1, &h.n_idx));
+    RET(balloc(b, m, &h.flags));
+    RET(balloc(b, m, &h.redo));
+    RET(balloc(b, m, &h.xredo));
+    RET(balloc(b, 2, &h.used));
+    CK(cudaMemcpyAsync(d_iota, iota.data(), m * 4, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(h.cand_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(h.theta, theta.data(), theta.size() * 4, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(h.outs, outs.data(), outs.size() * sizeof(BatchOut), cudaMemcpyHostToDevice, st));
+    // per stream its plan; the bins and ranks are shared by the streams, one after the other
+    uint32_t *bin, *rank, *order;
+    RET(balloc(b, m, &bin));
+    RET(balloc(b, m, &rank));
+    RET(balloc(b, m, &order));
+    std::vector<uint32_t> first{0}, part_off;
+    std::vector<uint32_t> part_group;
+    uint64_t bytes = 0;
+    h.capacity = 0;
+    for (uint32_t k = 0; k < h.n_streams; ++k) {
+        const StreamDev &s = *find_stream(c, streams[k]);
+        const uint32_t s0 = stream_off[k], ms = (k + 1 < h.n_streams ? stream_off[k + 1] : h.m) - s0;
+        HitPlan pl;
+        bool fits;
+        RET(hits_plan(c, s, h.cands, d_iota + s0, ms, true, b->ivl, nI, FEM_PASS_RELAXED, st, &pl, &fits,
+                      [&](const char *n, size_t w, uint32_t **p) -> int {
+                          if (!std::strcmp(n, "hit_plan_bin")) return *p = bin, FEM_OK;
+                          if (!std::strcmp(n, "hit_plan_rank")) return *p = rank, FEM_OK;
+                          if (!std::strcmp(n, "hit_plan_order")) return *p = order, FEM_OK;
+                          if (!std::strcmp(n, "hit_plan_gather")) return *p = h.record + s0, FEM_OK;
+                          return balloc(b, w, p);
+                      }));
+        if (!fits) return FEM_OK;
+        bytes += (uint64_t)pl.h.n_slabs * (pl.h.n_edges * 8ull + pl.h.types * 3ull) + s.n * 2ull + pl.hits * 4ull;
+        if (bytes > most || h.capacity + pl.hits > 0xF0000000ull) return FEM_OK;
+        h.capacity += pl.hits;
+        HitBuild &hb = pl.b;
+        RET(balloc(b, (size_t)pl.h.n_slabs * pl.h.n_edges, &hb.edge));
+        RET(balloc(b, (size_t)pl.h.n_slabs * pl.h.types, &hb.count));
+        RET(balloc(b, (size_t)pl.h.n_slabs * pl.h.types, &hb.place));
+        RET(balloc(b, s.n, &hb.index));
+        hb.used = h.used;
+        pl.h.edge = hb.edge, pl.h.count = hb.count, pl.h.place = hb.place, pl.h.index = hb.index;
+        h.build.push_back(hb);
+        first.push_back(first.back() + pl.h.n_slabs);
+        uint32_t slot = s0;
+        for (uint32_t g = 0; g < PLAN_GROUPS; ++g) {
+            if (!pl.group_m[g]) continue;
+            CountParams p = hits_params(c, s, pl, h.cands, g, 0);
+            p.gather = h.record + slot;
+            p.out = h.r + slot;
+            p.redo = h.redo + slot;
+            p.hit_classes = S_RECOUNT;
+            part_off.push_back(slot);
+            part_group.push_back(g);
+            h.parts.push_back(p);
+            slot += p.m;
+        }
+    }
+    h.n_slabs = first.back();
+    h.n_parts = (uint32_t)h.parts.size();
+    part_off.push_back(h.m);
+    // segments: the same number of slabs for every item of a launch, for about four blocks
+    // for each place on the GPU (the exact pass, with fewer candidates, four times as many)
+    std::vector<CountParams> xp = h.parts;
+    uint64_t tab = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        uint64_t t = 0;
+        for (uint32_t g = 0; g < PLAN_GROUPS; ++g) {
+            uint64_t work = 0;
+            for (uint32_t q = 0; q < h.n_parts; ++q)
+                if (part_group[q] == g) work += (uint64_t)((h.parts[q].m + 127) / 128) * h.parts[q].hits.n_slabs;
+            const uint64_t blocks = (uint64_t)c->sm_count * 24 * (pass ? 4 : 1);
+            const uint32_t cps = (uint32_t)std::max<uint64_t>(8, (work + blocks - 1) / blocks);
+            std::vector<uint4> list;
+            uint32_t items = 0;
+            for (uint32_t q = 0; q < h.n_parts; ++q) {
+                if (part_group[q] != g) continue;
+                CountParams &p = pass ? xp[q] : h.parts[q];
+                const uint32_t P = (p.hits.n_slabs + cps - 1) / cps;
+                p.cps = (p.hits.n_slabs + P - 1) / P;
+                p.P = (p.hits.n_slabs + p.cps - 1) / p.cps;
+                p.tables = reinterpret_cast<uint4 *>(t);  // (an offset until they are allocated)
+                t += (uint64_t)p.P * p.m * S_RECOUNT;
+                const uint32_t tiles = (p.m + 127) / 128;
+                list.push_back(make_uint4(items, tiles, q, 0));
+                items += tiles * p.P;
+            }
+            BatchHits::Launch &l = pass ? h.ex[g] : h.rel[g];
+            l.n_list = (uint32_t)list.size(), l.n_items = items;
+            if (list.empty()) continue;
+            RET(balloc(b, list.size(), &l.list));
+            CK(cudaMemcpy(l.list, list.data(), list.size() * sizeof(uint4), cudaMemcpyHostToDevice));
+        }
+        tab = std::max(tab, t);
+    }
+    if (bytes + tab * sizeof(uint4) > most) return FEM_OK;
+    uint4 *tables;
+    RET(balloc(b, tab, &tables));
+    for (uint32_t q = 0; q < h.n_parts; ++q) {
+        h.parts[q].tables = tables + reinterpret_cast<uint64_t>(h.parts[q].tables);
+        xp[q].tables = tables + reinterpret_cast<uint64_t>(xp[q].tables);
+        xp[q].redo = h.xredo + part_off[q];
+        xp[q].m = 0;
+    }
+    RET(balloc(b, h.n_streams, &h.d_build));
+    RET(balloc(b, first.size(), &h.first));
+    RET(balloc(b, h.n_parts, &h.rparts));
+    RET(balloc(b, h.n_parts, &h.xparts));
+    RET(balloc(b, part_off.size(), &h.part_off));
+    CK(cudaMemcpy(h.first, first.data(), first.size() * 4, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(h.part_off, part_off.data(), part_off.size() * 4, cudaMemcpyHostToDevice));
+    // one run, in which the ranges may turn out to be more than estimated
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        uint32_t *range;
+        RET(balloc(b, h.capacity, &range));
+        for (HitBuild &hb : h.build) hb.range = range, hb.capacity = h.capacity;
+        for (uint32_t q = 0; q < h.n_parts; ++q) h.parts[q].hits.range = xp[q].hits.range = range;
+        CK(cudaMemcpy(h.d_build, h.build.data(), h.n_streams * sizeof(HitBuild), cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(h.rparts, h.parts.data(), h.n_parts * sizeof(CountParams), cudaMemcpyHostToDevice));
+        CK(cudaMemcpy(h.xparts, xp.data(), h.n_parts * sizeof(CountParams), cudaMemcpyHostToDevice));
+        CK(cudaMemsetAsync(c->d_err, 0, 4, st));
+        RET(batch_enqueue_hits(c, h, st));
+        unsigned long long used[2];
+        uint32_t e;
+        CK(cudaMemcpyAsync(used, h.used, 16, cudaMemcpyDeviceToHost, st));
+        RET(read_err(c, st, &e));
+        RET(err_status(e));
+        const uint64_t need = std::max(used[0], used[1]);
+        if (std::getenv("FEM_DEBUG"))
+            std::fprintf(stderr, "fem: batch tables %.2f GB, transfer tables %.2f GB, hits %llu of %llu, err %#x\n",
+                         bytes * 1e-9, tab * 16e-9, (unsigned long long)need, (unsigned long long)h.capacity, e);
+        if (e & ERR_DENSE) return FEM_OK;
+        if (need <= h.capacity) {
+            *ok = true;
+            return FEM_OK;
+        }
+        if (need > 0xF0000000ull || bytes + (tab * sizeof(uint4)) + need * 4 > most) return FEM_OK;
+        cfree(c, range, b->alloc_bytes.back());
+        b->allocs.pop_back(), b->alloc_bytes.pop_back();
+        h.capacity = need + need / 16 + hit_slack(h.n_slabs);
     }
     return FEM_OK;
 }
@@ -2473,7 +2743,27 @@ int fem_batch_create(fem_ctx *c, const fem_job *jobs, uint32_t n_jobs, const fem
     BRET(balloc(b, std::max<uint32_t>(nI, 1), &b->ivl));
     if (nI) BCK(cudaMemcpyAsync(b->ivl, I, nI * sizeof(uint2), cudaMemcpyHostToDevice, st));
 
-    for (int N = 1; N <= FEM_MAX_LEN; ++N) {
+    c->ivl_host.assign(I, I + nI);
+    {
+        const size_t kept = b->allocs.size();
+        c->hits_busy = true;
+        const int rch = batch_plan_hits(b, st, &b->over_hits);
+        c->hits_busy = false;
+        if (rch != FEM_OK && rch != FEM_ENOMEM) return fail(rch);
+        if (std::getenv("FEM_DEBUG"))
+            std::fprintf(stderr, "fem: batch of %u candidates, %u streams: %s (%u slabs, %llu hits' room)\n",
+                         b->hits.m, b->hits.n_streams, b->over_hits ? "over hit tables" : "per-thread kernels",
+                         b->hits.n_slabs, (unsigned long long)b->hits.capacity);
+        if (!b->over_hits) {  // the per-thread kernels: give the tables' memory back
+            cudaGetLastError();
+            BCK(cudaStreamSynchronize(st));
+            for (; b->allocs.size() > kept; b->allocs.pop_back(), b->alloc_bytes.pop_back())
+                cfree(c, b->allocs.back(), b->alloc_bytes.back());
+            b->hits = BatchHits{};
+            BCK(cudaMemsetAsync(c->d_err, 0, 4, st));
+        }
+    }
+    for (int N = 1; N <= FEM_MAX_LEN && !b->over_hits; ++N) {
         BatchGroup g;
         g.N = N;
         struct Ent {
@@ -2581,7 +2871,7 @@ int fem_batch_create(fem_ctx *c, const fem_job *jobs, uint32_t n_jobs, const fem
     }
     // measured shapes when tuning is on; one eager run (sets kernel attributes, checks
     // the inputs); then capture
-    if (c->tune_on) BRET(batch_tune(b, st));
+    if (c->tune_on && !b->over_hits) BRET(batch_tune(b, st));
     BRET(fem_batch_run(b, cuda_stream));
     BCK(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
     BCK(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -2622,7 +2912,16 @@ int fem_batch_run(fem_batch *b, void *cuda_stream) {
     uint32_t e;
     RET(read_err(c, st, &e));
     RET(err_status(e));
-    if (!(e & ERR_CAP)) return FEM_OK;
+    if (!(e & (ERR_CAP | ERR_DENSE))) return FEM_OK;
+    if (b->over_hits) {  // (more than 32 entry classes: seldom) every job on its own
+        std::vector<fem_interval> I(b->nI);
+        if (b->nI) CK(cudaMemcpy(I.data(), b->ivl, b->nI * sizeof(uint2), cudaMemcpyDeviceToHost));
+        for (const fem_job &jb : b->jobs)
+            if (jb.m)
+                RET(fem_count_two_pass(c, jb.stream_id, jb.cands, jb.m, 1, I.data(), b->nI, jb.theta,
+                                       jb.exact_out, jb.survived_out, 1, st));
+        return FEM_OK;
+    }
     // A capacity guard tripped somewhere: recount the affected jobs one at a time
     // with the single-recording path, which widens rings as needed.
     std::vector<fem_interval> I(b->nI);

@@ -119,27 +119,60 @@ cudaError_t launch_batch_keep_flags(const uint32_t *rel, const uint32_t *cand_of
     return cudaGetLastError();
 }
 
-// Exact-pass job j counts the survivors idx[s_j .. e_j) (global candidate indices,
-// ascending) of its candidate range [cand_off[j], cand_off[j+1]).
+__global__ void k_batch_keep_slots(const uint32_t *__restrict__ rel, const uint32_t *__restrict__ order,
+                                   const uint32_t *__restrict__ cand_off,
+                                   const uint32_t *__restrict__ theta, uint32_t n_jobs, uint32_t m,
+                                   uint8_t *__restrict__ flags) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
+        flags[i] = rel[i] >= theta[find_job(cand_off, n_jobs, order[i])];
+}
+
+cudaError_t launch_batch_keep_slots(const uint32_t *rel, const uint32_t *order,
+                                    const uint32_t *cand_off, const uint32_t *theta, uint32_t n_jobs,
+                                    uint32_t m, uint8_t *flags, cudaStream_t st) {
+    if (m == 0) return cudaSuccess;
+    k_batch_keep_slots<<<(uint32_t)std::min<uint64_t>((m + 255) / 256, 4096), 256, 0, st>>>(
+        rel, order, cand_off, theta, n_jobs, m, flags);
+    note_launch();
+    return cudaGetLastError();
+}
+
+__global__ void k_batch_pick(const uint32_t *__restrict__ idx, const uint32_t *__restrict__ n,
+                             const uint32_t *__restrict__ x, uint32_t *__restrict__ out) {
+    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < *n; k += gridDim.x * blockDim.x)
+        out[k] = x[idx[k]];
+}
+
+cudaError_t launch_batch_pick(const uint32_t *idx, const uint32_t *n, uint32_t m, const uint32_t *x,
+                              uint32_t *out, cudaStream_t st) {
+    if (m == 0) return cudaSuccess;
+    k_batch_pick<<<(uint32_t)std::min<uint64_t>((m + 255) / 256, 4096), 256, 0, st>>>(idx, n, x, out);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// Exact-pass job j counts the survivors idx[s_j .. e_j) (global candidate indices or slots,
+// ascending) of its range [cand_off[j], cand_off[j+1]); their records are gather[s_j ..].
 __global__ void k_batch_exact_jobs(CountParams *__restrict__ xjobs,
                                    const uint32_t *__restrict__ cand_off, uint32_t n_jobs,
                                    const uint32_t *__restrict__ idx,
-                                   const uint32_t *__restrict__ n_idx, uint32_t *__restrict__ ex) {
+                                   const uint32_t *__restrict__ n_idx, uint32_t *__restrict__ ex,
+                                   const uint32_t *gather) {
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_jobs) return;
     const uint32_t cnt = *n_idx;
     const uint32_t s = lower_bound_u32(idx, cnt, cand_off[j]);
     const uint32_t e = lower_bound_u32(idx, cnt, cand_off[j + 1]);
     xjobs[j].m = e - s;
-    xjobs[j].gather = idx + s;
+    xjobs[j].gather = gather + s;
     xjobs[j].out = ex + s;
 }
 
 cudaError_t launch_batch_exact_jobs(CountParams *xjobs, const uint32_t *cand_off, uint32_t n_jobs,
                                     const uint32_t *idx, const uint32_t *n_idx, uint32_t *ex,
-                                    cudaStream_t st) {
+                                    cudaStream_t st, const uint32_t *gather) {
     k_batch_exact_jobs<<<(n_jobs + 127) / 128, 128, 0, st>>>(xjobs, cand_off, n_jobs, idx, n_idx,
-                                                             ex);
+                                                             ex, gather ? gather : idx);
     note_launch();
     return cudaGetLastError();
 }

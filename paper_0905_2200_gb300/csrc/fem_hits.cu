@@ -1,6 +1,7 @@
 // fem_hits.cu -- the hit tables of a stream and an edge set, the launches of the counting
 // kernels that read them, and the plan both need: the candidates checked and ordered, the
 // edges they use numbered, the stream cut into slabs.
+#include <algorithm>
 #include <mutex>
 
 #include "fem_hits.cuh"
@@ -71,7 +72,7 @@ __device__ __forceinline__ void scan_words(const uint32_t *w, uint32_t n, uint32
 // first), its last type.
 __device__ __forceinline__ uint32_t plan_bin(const fem_episode &e, const PlanArgs &a) {
     const uint32_t N = e.len;
-    uint32_t bin = plan_group(N, a.m);
+    uint32_t bin = plan_group(N, a.fine);
     for (uint32_t k = 1; k <= 3; ++k)
         bin = bin * a.parts + (N > k ? a.parts - 1u - e.ivl[N - 1 - k] * a.parts / a.n_ivl : 0u);
     return bin * a.K + e.types[N - 1];
@@ -237,28 +238,33 @@ __global__ void k_publish_count(const unsigned long long *src, Publish pub) {
 // before it go into shared memory as rank rows (rank 32 is the slab's first; the types'
 // own order in the chunk gives the ranks), with a bit per position of the slab and, per
 // 32 positions, the events before them, so that the number of a type's events before any
-// event of the slab is two reads and a popc.  Then a warp takes a type y, a lane its event
-// r, and goes through the other types x: the x events before the lane's event as far back
-// as the longest interval reaches, a few steps down the row, give the ranges of four
-// intervals at once; a ballot per interval is the edge's mask.  Ranges are written to room
-// that a warp reserves in the table for many edges at a time.  (A thread per edge, merging
-// the edge's two rows, left three of four lanes idle: 1.15 ms for the 387,000 events of 64
-// types at 50 Hz and all 16,128 edges; a thread per event and earlier event, 1.04 ms.)
-constexpr uint32_t HIT_ROOM = 2048;  // ranges a warp reserves at a time
+// event of the slab is two reads and a popc.  Then a warp takes a pack of types with up to 32
+// events in all, a lane an event, and goes through the types x: the x events before the
+// lane's event as far back as the longest interval reaches, a few steps down the row, give
+// the ranges of four intervals at once; a ballot per interval holds the masks of up to 32
+// edges, of which each lane takes one.  Ranges are written to room that a warp reserves in
+// the table for many edges at a time.  What bounds it: warp issue slots.  Measured on the
+// 406,000 events of 64 types at 20 Hz, all 16,128 edges, exact pass: 467 us; one type a
+// warp 490 us (half the lanes idle), a thread per edge, merging its two rows, 983, a thread
+// per event and earlier event 526 (and 4500 on a bursting recording).
+constexpr int U = 4;                   // intervals taken at once
+constexpr uint32_t HIT_PACK = 32 / U;  // types a warp takes at once
 
 template <int PASS>
-__global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build(const HitBuild b) {
+__device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, uint32_t part, uint32_t parts) {
     const uint32_t T = HIT_BUILD_T, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr uint32_t NW = HIT_BUILD_T / 32, WORDS = CHUNK / 32;
-    const uint32_t s = blockIdx.x, K = b.K;
+    constexpr uint32_t NW = HIT_BUILD_T / 32;
+    const uint32_t K = b.K;
+    __shared__ uint32_t n_packs;
     uint32_t *rt = reinterpret_cast<uint32_t *>(fem_hit_smem);  // times by rank [K][HIT_ROW]
     uint32_t *bits = rt + K * HIT_ROW;                          // [K][slab words]
     const uint32_t begin = b.begin[s], end = b.begin[s + 1], c = begin / CHUNK;
     const uint32_t p0 = begin % CHUNK, p1 = p0 + (end - begin);  // the slab's places in its chunk
     const uint32_t words = (end - begin + 31) / 32;
     uint16_t *rp = reinterpret_cast<uint16_t *>(bits + K * b.max_words);  // positions by rank [K][HIT_ROW]
-    uint16_t *place = rp + K * HIT_ROW;                          // [K]
-    uint8_t *before = reinterpret_cast<uint8_t *>(place + K);    // events before a word [K][words]
+    uint16_t *place = rp + K * HIT_ROW;                          // [K + 1]
+    uint16_t *pack = place + K + 1;                              // first type of each pack, K
+    uint8_t *before = reinterpret_cast<uint8_t *>(pack + K + 1);  // events before a word [K][words]
     uint8_t *hist = before + K * b.max_words;                    // events before the slab [K]
     uint8_t *num = hist + K;                                     // events in the slab [K]
     const uint32_t origin = c * CHUNK - CHUNK;                   // index of position 0 (modulo 2^32)
@@ -329,11 +335,22 @@ __global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build(const HitBuild b) {
             }
             carry += __shfl_sync(0xffffffffu, inc, 31);
         }
+        if (lane == 0) {
+            place[K] = (uint16_t)carry;
+            // packs of consecutive types: up to 32 events of up to 8 types
+            uint32_t n = 0, y0 = 0;
+            for (uint32_t y = 0; y < K; ++y) {
+                if (y > y0 && (place[y + 1] - place[y0] > 32 || y - y0 == HIT_PACK)) pack[n++] = (uint16_t)y0, y0 = y;
+            }
+            pack[n++] = (uint16_t)y0;
+            pack[n] = (uint16_t)K;
+            n_packs = n;
+        }
     }
     __syncthreads();
     bool dense = false;
     uint32_t at = 0, left = 0;  // the warp's room in the table of ranges
-    constexpr int U = 4;        // intervals taken at once
+    bool full = false;          // the table has no more (the warp goes on to count its hits)
     for (uint32_t u0 = 0; u0 < b.n_ivl; u0 += U) {
         // a gap lies in interval u iff gap - from[u] <= wide[u] (unsigned); the relaxed pass
         // takes any gap up to hi
@@ -345,31 +362,41 @@ __global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build(const HitBuild b) {
             wide[u] = v.y - from[u];
             far = max(far, v.y);
         }
-        for (uint32_t y = blockIdx.y * NW + warp; y < K; y += NW * gridDim.y) {
-            const uint32_t n = num[y];
+        for (uint32_t k = part * NW + warp; k < n_packs; k += NW * parts) {
+            const uint32_t y0 = pack[k], types = pack[k + 1] - y0, base = place[y0];
+            // the lane's event: the pack's lane-th, of type y0 + g
+            const uint32_t n = place[y0 + types] - base;
             const bool mine = lane < n;
-            const uint32_t t = mine ? rt[y * HIT_ROW + 32 + lane] : 0u;
-            const uint32_t pos = mine ? rp[y * HIT_ROW + 32 + lane] : CHUNK + p0;
-            if (mine && u0 == 0) b.index[begin + place[y] + lane] = (uint16_t)(origin + pos);
+            uint32_t g = 0;
+            for (uint32_t j = 1; j < types; ++j) g += place[y0 + j] - base <= lane;
+            if (!mine) g = 0;
+            const uint32_t y = y0 + g, o = place[y] - base, r = lane - o;
+            const uint32_t t = mine ? rt[y * HIT_ROW + 32 + r] : 0u;
+            const uint32_t pos = mine ? rp[y * HIT_ROW + 32 + r] : CHUNK + p0;
+            if (mine && u0 == 0) b.index[begin + base + lane] = (uint16_t)(origin + pos);
             const uint32_t q = pos - CHUNK - p0, w = q >> 5, below = (1u << (q & 31)) - 1u;
-            const uint32_t before_me = (1u << lane) - 1u;
-            // lane u of four holds the number of edge (x, u0 + u, y), asked for an x ahead
-            const uint32_t *ids = b.edge_id + y * b.n_ivl + u0 + (lane & (U - 1));
-            const bool iv = lane < U && u0 + lane < b.n_ivl;
-            uint32_t next = iv ? __ldg(ids) : ~0u;
+            const uint32_t same_below = ((1u << lane) - 1u) & ~((1u << o) - 1u);
+            // the lane's edge: (x, u0 + eu, y0 + eg), its number asked for an x ahead; `ours`
+            // are the lanes of its last type's events
+            const uint32_t eg = lane / U, eu = lane % U;
+            const bool edge = eg < types && u0 + eu < b.n_ivl;
+            const uint32_t eo = edge ? place[y0 + eg] - base : 0u, en = edge ? num[y0 + eg] : 0u;
+            const uint32_t ours = en ? (0xFFFFFFFFu >> (32u - en)) << eo : 0u;
+            const uint32_t *ids = b.edge_id + (y0 + (edge ? eg : 0u)) * b.n_ivl + u0 + eu;
+            uint32_t next = edge ? __ldg(ids) : ~0u;
             for (uint32_t x = 0; x < K; ++x) {
                 const uint32_t id = next;
-                if (x + 1 < K && iv) next = __ldg(ids + (x + 1) * K * b.n_ivl);
+                if (x + 1 < K && edge) next = __ldg(ids + (x + 1) * K * b.n_ivl);
                 const uint32_t wanted = __ballot_sync(0xffffffffu, id != ~0u);
-                if (!wanted || x == y) continue;  // no edge in use
+                if (!wanted) continue;  // no edge in use
                 const uint32_t *tx = rt + x * HIT_ROW;
                 const uint32_t low = 32u - hist[x];
-                // x's events before the lane's event have the ranks below k; those in interval
-                // u are m_u from a_u on
+                // x's events before the lane's event have the ranks below k0; those in interval
+                // u are m[u] from a[u] on
                 uint32_t a[U] = {}, m[U] = {};
                 if (mine) {
-                    uint32_t k = 32u + before[x * words + w] + __popc(bits[x * words + w] & below);
-                    const uint32_t k0 = k;
+                    const uint32_t k0 = 32u + before[x * words + w] + __popc(bits[x * words + w] & below);
+                    uint32_t k = k0;
                     for (; k > low; --k) {
                         const uint32_t gap = t - tx[k - 1];
                         if (gap > far) break;
@@ -381,37 +408,85 @@ __global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build(const HitBuild b) {
                     // can say
                     dense = dense || (k == 0 && k0 > 0) || k0 - k > 32;
                 }
-                uint32_t mask[U], total = 0;
+                // the masks of the pack's edges, and their places in the table
+                uint32_t hits[U], mask = 0;
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    mask[u] = __ballot_sync(0xffffffffu, m[u] != 0);
-                    if (!((wanted >> u) & 1u)) mask[u] = 0;
-                    total += __popc(mask[u]);
+                    hits[u] = __ballot_sync(0xffffffffu, m[u] != 0);
+                    if (eu == (uint32_t)u) mask = hits[u] & ours;
                 }
+                if (id == ~0u) mask = 0;
+                const uint32_t c = __popc(mask);
+                uint32_t inc = c;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t v = __shfl_up_sync(0xffffffffu, inc, d);
+                    if (lane >= (uint32_t)d) inc += v;
+                }
+                const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
                 if (total > left) {  // the same in every lane
-                    unsigned long long g = 0;
-                    if (lane == 0) g = atomicAdd(b.used, (unsigned long long)HIT_ROOM);
-                    g = __shfl_sync(0xffffffffu, g, 0);
-                    left = g + HIT_ROOM <= b.capacity ? HIT_ROOM : 0u;
-                    at = (uint32_t)g;
-                    if (total > left) total = mask[0] = mask[1] = mask[2] = mask[3] = 0;  // (the host sees it)
+                    const uint32_t ask = full ? total : HIT_ROOM;
+                    unsigned long long v = 0;
+                    if (lane == 0) v = atomicAdd(b.used, (unsigned long long)ask);
+                    v = __shfl_sync(0xffffffffu, v, 0);
+                    full = full || v + ask > b.capacity;
+                    left = full ? 0u : HIT_ROOM;
+                    at = (uint32_t)v;
                 }
-                left -= total;
-                uint2 own = make_uint2(mask[0], at);  // lane u's edge
+                const bool room = total <= left;
+                const uint32_t out = at + inc - c;
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    if (u > 0 && lane == (uint32_t)u) own = make_uint2(mask[u], at);
-                    if (!mask[u]) continue;  // uniform
-                    if ((mask[u] >> lane) & 1u)
-                        b.range[at + __popc(mask[u] & before_me)] =
+                    const uint32_t at_u = __shfl_sync(0xffffffffu, out, g * U + u);
+                    if (m[u] && room && ((wanted >> (g * U + u)) & 1u))
+                        b.range[at_u + __popc(hits[u] & same_below)] =
                             hit_pack(a[u], m[u], origin + rp[x * HIT_ROW + a[u] + m[u] - 1]);
-                    at += __popc(mask[u]);
                 }
-                if (id != ~0u) b.edge[(uint64_t)s * b.n_edges + id] = own;
+                if (id != ~0u) b.edge[(uint64_t)s * b.n_edges + id] = make_uint2(room ? mask >> eo : 0u, out);
+                if (room) at += total, left -= total;
             }
         }
     }
     if (dense) atomicOr(b.err, ERR_DENSE);
+}
+
+template <int PASS>
+__global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build(const HitBuild b) {
+    hit_build_slab<PASS>(b, blockIdx.x, blockIdx.y, gridDim.y);
+}
+
+// The same for the streams of a batch: block i builds slab i - first[j] of stream j.
+template <int PASS>
+__global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build_batch(const HitBuild *__restrict__ streams,
+                                                                 const uint32_t *__restrict__ first,
+                                                                 uint32_t n_streams) {
+    __shared__ HitBuild b;
+    uint32_t lo = 0, hi = n_streams;
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (first[mid] <= blockIdx.x) lo = mid;
+        else hi = mid;
+    }
+    if (threadIdx.x == 0) b = streams[lo];
+    __syncthreads();
+    hit_build_slab<PASS>(b, blockIdx.x - first[lo], 0, 1);
+}
+
+size_t build_smem(const HitBuild &b) {
+    return (size_t)b.K * (HIT_ROW * 6 + b.max_words * 5 + 6) + 32;
+}
+
+cudaError_t build_limits() {
+    static std::once_flag once;
+    static cudaError_t err = cudaSuccess;
+    std::call_once(once, [] {
+        for (const void *k : {(const void *)k_hit_build<FEM_PASS_RELAXED>, (const void *)k_hit_build<FEM_PASS_EXACT>,
+                              (const void *)k_hit_build_batch<FEM_PASS_RELAXED>,
+                              (const void *)k_hit_build_batch<FEM_PASS_EXACT>})
+            if (err == cudaSuccess)
+                err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+    });
+    return err;
 }
 
 // Launch kernel `k` over p.m candidates in blocks of 128.
@@ -421,6 +496,23 @@ cudaError_t run(Kernel k, cudaStream_t st, const CountParams &p, Args... args) {
     constexpr size_t sm = (size_t)hit_shared(NMAX) * 64 * T * 2;  // at most 48 KB: no opt-in
     static_assert(sm <= 48 * 1024, "dynamic shared memory without an attribute");
     k<<<dim3((p.m + T - 1) / T, p.P), T, sm, st>>>(p, args...);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// (48 KB of starts and the shared parameters: past the default limit)
+template <int NMAX>
+cudaError_t run_batch(const CountParams *parts, const uint4 *list, uint32_t n_list, uint32_t n_items,
+                      cudaStream_t st) {
+    constexpr uint32_t T = 128;
+    constexpr int sm = hit_shared(NMAX) * 64 * (int)T * 2;
+    static std::once_flag once;
+    static cudaError_t err = cudaSuccess;
+    std::call_once(once, [] {
+        err = cudaFuncSetAttribute(k_hit_count_batch<NMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    });
+    if (err != cudaSuccess) return err;
+    k_hit_count_batch<NMAX><<<n_items, T, sm, st>>>(parts, list, n_list);
     note_launch();
     return cudaGetLastError();
 }
@@ -454,28 +546,51 @@ cudaError_t launch_publish_count(const unsigned long long *src, Publish pub, cud
     return cudaGetLastError();
 }
 
+uint64_t hit_slack(uint32_t n_slabs) { return (uint64_t)n_slabs * (HIT_BUILD_T / 32) * HIT_ROOM; }
+
 cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
                              cudaStream_t st) {
     if (n_slabs == 0) return cudaSuccess;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        for (auto *k : {k_hit_build<FEM_PASS_RELAXED>, k_hit_build<FEM_PASS_EXACT>})
-            if (attr_err == cudaSuccess)
-                attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
-    });
-    if (attr_err != cudaSuccess) return attr_err;
-    const size_t K = b.K;
-    const size_t sm = K * (HIT_ROW * 6 + b.max_words * 5 + 4) + 16;
+    const cudaError_t e = build_limits();
+    if (e != cudaSuccess) return e;
+    const size_t sm = build_smem(b);
     if (sm > 224 * 1024) return cudaErrorInvalidConfiguration;
-    // a few slabs: their types shared among several blocks, for about three per SM
+    // a few slabs: their types shared among several blocks, for about four per SM
     constexpr uint32_t NW = HIT_BUILD_T / 32;
     uint32_t split = 1;
-    while (split < 8 && split * NW < b.K && 2 * split * n_slabs <= 3 * (uint32_t)sm_count) split *= 2;
+    while (split < 8 && split * NW < b.K && split * n_slabs < 4 * (uint32_t)sm_count) split *= 2;
     (pass == FEM_PASS_RELAXED ? k_hit_build<FEM_PASS_RELAXED>
                               : k_hit_build<FEM_PASS_EXACT>)<<<dim3(n_slabs, split), HIT_BUILD_T, sm, st>>>(b);
     note_launch();
     return cudaGetLastError();
+}
+
+cudaError_t launch_hit_build_batch(int pass, const HitBuild *host, const HitBuild *streams,
+                                   const uint32_t *first, uint32_t n_streams, uint32_t n_slabs,
+                                   cudaStream_t st) {
+    if (n_slabs == 0) return cudaSuccess;
+    const cudaError_t e = build_limits();
+    if (e != cudaSuccess) return e;
+    size_t sm = 0;
+    for (uint32_t j = 0; j < n_streams; ++j) sm = std::max(sm, build_smem(host[j]));
+    if (sm > 224 * 1024) return cudaErrorInvalidConfiguration;
+    (pass == FEM_PASS_RELAXED
+         ? k_hit_build_batch<FEM_PASS_RELAXED>
+         : k_hit_build_batch<FEM_PASS_EXACT>)<<<n_slabs, HIT_BUILD_T, sm, st>>>(streams, first, n_streams);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_hit_count_batch(uint32_t group, const CountParams *parts, const uint4 *list,
+                                   uint32_t n_list, uint32_t n_items, cudaStream_t st) {
+    if (n_items == 0) return cudaSuccess;
+    switch (group) {
+#define FEM_CASE(g, n) \
+    case g: return run_batch<n>(parts, list, n_list, n_items, st);
+        FEM_CASE(0, 2) FEM_CASE(1, 3) FEM_CASE(2, 4) FEM_CASE(3, 5) FEM_CASE(4, 8)
+#undef FEM_CASE
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_hit_count(uint32_t group, bool mc, const CountParams &p, cudaStream_t st) {

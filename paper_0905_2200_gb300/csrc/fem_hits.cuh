@@ -49,7 +49,8 @@ namespace fem {
 constexpr uint32_t HIT_CLASSES = 32;   // most entry classes per table
 constexpr uint32_t HIT_PARTS = 64;     // most slabs per chunk (32 events each)
 constexpr uint32_t HIT_ROW = 65;       // words per type of a slab's rank tables (64 and a pad)
-constexpr uint32_t HIT_BUILD_T = 512;  // threads of a build block
+constexpr uint32_t HIT_BUILD_T = 256;  // threads of a build block
+constexpr uint32_t HIT_ROOM = 512;     // ranges a warp of it reserves at a time
 
 // inner nodes of an episode of up to nmax nodes, and those whose chains' starts are in
 // shared memory
@@ -216,8 +217,8 @@ struct HitEpisode {
 
 // Count one tile of candidates over segment `seg`.
 template <int NMAX, bool MC>
-__global__ void __launch_bounds__(128) k_hit_count(const CountParams p) {
-    const uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x, seg = blockIdx.y;
+__device__ __forceinline__ void hit_count_tile(const CountParams &p, uint32_t tile, uint32_t seg) {
+    const uint32_t ci = tile * blockDim.x + threadIdx.x;
     const HitTables &h = p.hits;
     HitEpisode<NMAX> ep;
     const bool ok = ep.load(p, ci);
@@ -360,6 +361,32 @@ __global__ void __launch_bounds__(128) k_hit_count(const CountParams p) {
             tab[j] = e;
         }
     }
+}
+
+template <int NMAX, bool MC>
+__global__ void __launch_bounds__(128) k_hit_count(const CountParams p) {
+    hit_count_tile<NMAX, MC>(p, blockIdx.x, blockIdx.y);
+}
+
+// The same for a batch: list[i] names a part (z) whose items are the blocks from list[i].x on,
+// the list[i].y tiles of a segment one after the other.  A part's candidate count may be
+// the device's (survivors); its items are for the most there can be.
+template <int NMAX>
+__global__ void __launch_bounds__(128) k_hit_count_batch(const CountParams *__restrict__ parts,
+                                                         const uint4 *__restrict__ list, uint32_t n_list) {
+    __shared__ CountParams p;
+    uint32_t lo = 0, hi = n_list;
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (list[mid].x <= blockIdx.x) lo = mid;
+        else hi = mid;
+    }
+    const uint4 e = list[lo];
+    const uint32_t r = blockIdx.x - e.x, tile = r % e.y;
+    if (tile * blockDim.x >= parts[e.z].m) return;  // uniform
+    if (threadIdx.x == 0) p = parts[e.z];
+    __syncthreads();
+    hit_count_tile<NMAX, true>(p, tile, r / e.y);
 }
 
 // Window-based frequency (fem_windows.cu) of one tile of candidates over segment `seg`: the

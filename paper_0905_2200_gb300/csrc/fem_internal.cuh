@@ -281,8 +281,18 @@ struct HitBuild {
     uint16_t *place, *index;
     uint32_t *err;                // ERR_DENSE
 };
+// ranges that a build of n_slabs slabs may reserve beyond its hits
+uint64_t hit_slack(uint32_t n_slabs);
 cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
                              cudaStream_t st);
+// for a batch: streams[j]'s slabs are blocks first[j] .. first[j + 1] (device arrays; host:
+// the same HitBuilds); entry i of a launch's list: part list[i].z's items are the blocks from
+// list[i].x on, list[i].y tiles per segment
+cudaError_t launch_hit_build_batch(int pass, const HitBuild *host, const HitBuild *streams,
+                                   const uint32_t *first, uint32_t n_streams, uint32_t n_slabs,
+                                   cudaStream_t st);
+cudaError_t launch_hit_count_batch(uint32_t group, const CountParams *parts, const uint4 *list,
+                                   uint32_t n_list, uint32_t n_items, cudaStream_t st);
 // What a count over hit tables is planned with: the candidates checked and put in the
 // order they run best in (by group, last three intervals, last type), the edges they use
 // numbered, the stream cut into slabs.  words, hist and edge_id are one block of PLAN_WORDS
@@ -290,12 +300,12 @@ cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int 
 constexpr uint32_t PLAN_PARTS = 4, PLAN_GROUPS = 5, PLAN_FINE = 8192;
 constexpr uint32_t PLAN_REP = 8, PLAN_SPAN = 9, PLAN_EDGES = 10, PLAN_SLABS = 11, PLAN_PARTS_MIN = 12,
                    PLAN_WORDS = 13;
-// The launch that counts an episode of N nodes of a set of m: lengths 1-2, 3, 4, 5 and
-// 6-8, since registers and shared memory grow with the length; small sets, whose launches
-// are short, in three (1-3, 4-5, 6-8).
-__host__ __device__ inline uint32_t plan_group(uint32_t N, uint32_t m) {
+// The launch that counts an episode of N nodes: lengths 1-2, 3, 4, 5 and 6-8, since
+// registers and shared memory grow with the length; small sets (below PLAN_FINE), whose
+// launches are short, in three (1-3, 4-5, 6-8).
+__host__ __device__ inline uint32_t plan_group(uint32_t N, bool fine) {
     if (N > 5) return 4;
-    if (m < PLAN_FINE) return N <= 3 ? 1 : 3;
+    if (!fine) return N <= 3 ? 1 : 3;
     return N <= 2 ? 0 : N - 2;
 }
 struct PlanArgs {
@@ -303,6 +313,7 @@ struct PlanArgs {
     const uint32_t *gather;
     uint32_t m, K, n_ivl;
     uint32_t parts;          // parts of the interval set (at most PLAN_PARTS, n_ivl)
+    bool fine;               // plan_group's
     const uint32_t *cfirst, *t;
     uint32_t n_chunks;
     uint64_t n;
@@ -342,7 +353,8 @@ cudaError_t launch_literal(const LiteralParams &p, uint32_t len_mask, uint32_t *
 // stitch of a batch: job_base[j] = first global episode slot of job j (n_jobs + 1
 // entries); slots >= a job's current m are skipped
 cudaError_t launch_stitch_batch(const CountParams *jobs, const uint32_t *job_base,
-                                uint32_t n_jobs, uint32_t slots, uint32_t *err, cudaStream_t st);
+                                uint32_t n_jobs, uint32_t slots, uint32_t *err, cudaStream_t st,
+                                uint32_t classes = S_MAX);
 cudaError_t launch_stitch(const uint4 *tables, uint32_t m, uint32_t P, uint32_t *out,
                           uint8_t *redo, uint32_t *err, cudaStream_t st,
                           uint32_t classes = S_MAX);
@@ -402,12 +414,19 @@ cudaError_t launch_repeat_flags(const fem_episode *c, const uint32_t *gather, ui
 cudaError_t launch_batch_items(const CountParams *jobs, uint32_t n_jobs, uint32_t T,
                                uint32_t *item_off, uint32_t *n_items, uint32_t cap, uint4 *items,
                                cudaStream_t st);
+// the same over slots of candidates order[slot]
+cudaError_t launch_batch_keep_slots(const uint32_t *rel, const uint32_t *order,
+                                    const uint32_t *cand_off, const uint32_t *theta, uint32_t n_jobs,
+                                    uint32_t m, uint8_t *flags, cudaStream_t st);
+// out[k] = x[idx[k]] for k < *n (at most m)
+cudaError_t launch_batch_pick(const uint32_t *idx, const uint32_t *n, uint32_t m, const uint32_t *x,
+                              uint32_t *out, cudaStream_t st);
 cudaError_t launch_batch_keep_flags(const uint32_t *rel, const uint32_t *cand_off,
                                     const uint32_t *theta, uint32_t n_jobs, uint32_t m,
                                     uint8_t *flags, cudaStream_t st);
 cudaError_t launch_batch_exact_jobs(CountParams *xjobs, const uint32_t *cand_off, uint32_t n_jobs,
                                     const uint32_t *idx, const uint32_t *n_idx, uint32_t *ex,
-                                    cudaStream_t st);
+                                    cudaStream_t st, const uint32_t *gather = nullptr);
 cudaError_t launch_batch_outputs(const BatchOut *outs, const uint32_t *cand_off, uint32_t n_jobs,
                                  uint32_t m, const uint32_t *idx, const uint32_t *n_idx,
                                  const uint32_t *ex, cudaStream_t st);

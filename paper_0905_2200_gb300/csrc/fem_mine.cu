@@ -205,6 +205,7 @@ __global__ void __launch_bounds__(256) k_stitch(const uint4 *__restrict__ tables
 }
 
 // One warp per episode slot of a batch of jobs (each job its own tables and outputs).
+template <int SMX>
 __global__ void __launch_bounds__(256) k_stitch_batch(const CountParams *__restrict__ jobs,
                                                       const uint32_t *__restrict__ job_base,
                                                       uint32_t n_jobs, uint32_t slots,
@@ -219,14 +220,18 @@ __global__ void __launch_bounds__(256) k_stitch_batch(const CountParams *__restr
     }
     const CountParams &p = jobs[lo];
     const uint32_t ci = e - job_base[lo];
-    stitch_one<S_MAX>(p.tables, p.m, p.P, ci, 32u, ci < p.m && p.P > 0, p.out, p.redo, err);
+    stitch_one<SMX>(p.tables, p.m, p.P, ci, 32u, ci < p.m && p.P > 0, p.out, p.redo, err);
 }
 
 cudaError_t launch_stitch_batch(const CountParams *jobs, const uint32_t *job_base,
-                                uint32_t n_jobs, uint32_t slots, uint32_t *err, cudaStream_t st) {
+                                uint32_t n_jobs, uint32_t slots, uint32_t *err, cudaStream_t st,
+                                uint32_t classes) {
     if (slots == 0 || n_jobs == 0) return cudaSuccess;
     const uint32_t blocks = (uint32_t)(((uint64_t)slots * 32 + 255) / 256);
-    k_stitch_batch<<<blocks, 256, 0, st>>>(jobs, job_base, n_jobs, slots, err);
+    if (classes == S_RECOUNT)
+        k_stitch_batch<S_RECOUNT><<<blocks, 256, 0, st>>>(jobs, job_base, n_jobs, slots, err);
+    else
+        k_stitch_batch<S_MAX><<<blocks, 256, 0, st>>>(jobs, job_base, n_jobs, slots, err);
     note_launch();
     return cudaGetLastError();
 }

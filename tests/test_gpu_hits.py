@@ -120,3 +120,45 @@ def test_window_frequency(ctx, n, w_us, segments):
     got = fem.fem_count_windows(ctx, sid, fem.pack_episodes(*cands), I_MS4, w_us)
     assert_counts_equal(got, oracle.count_windows_batch(ty, t, *cands, I_MS4, w_us), "windows")
     fem.fem_free_stream(ctx, sid)
+
+
+@pytest.mark.parametrize("dense", [False, True])
+def test_batch(ctx, dense):
+    """A batch over streams of 1 to several chunks: a bursting one (more hits than estimated),
+    interleaved jobs, lengths 1-8, and with `dense` a stream the tables do not fit, for which
+    the whole batch takes the other kernels."""
+    torch = pytest.importorskip("torch")
+    I = np.array([[0, 2000], [2000, 20000]], np.uint32)
+    streams = [synth.sparse_bursts(seed=5, n_types=16, base_hz=0.5, duration_s=200.0, n_bursts=20),
+               stream(3, 1, 16), stream(4, 6000, 16)]
+    if dense:
+        streams.append(stream(6, 6000, 16, gap=5))
+    sids = [fem.fem_load_stream(ctx, ty, t, 16) for ty, t in streams]
+    jobs, want = [], []
+    for n in (2, 5, 1, 8, 3):
+        for k, (ty, t) in enumerate(streams):
+            cands = synth.random_candidates(10 * n + k, 90 + 37 * k, 16, [n], 2)
+            theta = 2 + 5 * k
+            jobs.append(dict(stream_id=sids[k], len=n, theta=theta,
+                             cands=torch.from_numpy(fem.pack_episodes(*cands)).cuda(),
+                             exact_out=torch.zeros(len(cands[0]), dtype=torch.int32, device="cuda"),
+                             survived_out=torch.zeros(len(cands[0]), dtype=torch.uint8, device="cuda")))
+            keep = oracle_counts(ty, t, *cands, I, fem.PASS_RELAXED) >= theta
+            want.append((np.where(keep, oracle_counts(ty, t, *cands, I, fem.PASS_EXACT), 0), keep))
+    torch.cuda.synchronize()
+    b = fem.fem_batch_create(ctx, jobs, I)
+    for _ in range(2):
+        for j in jobs:
+            j["exact_out"].fill_(-1)
+        torch.cuda.synchronize()
+        fem.fem_batch_run(b)
+        for i, (j, (ex, keep)) in enumerate(zip(jobs, want)):
+            assert_counts_equal(j["exact_out"].cpu().numpy(), ex, f"job {i}")
+            assert_counts_equal(j["survived_out"].cpu().numpy(), keep.astype(np.uint8), f"job {i}")
+    fem.fem_batch_destroy(b)
+    jobs[0]["len"] = 3  # candidates of another length than the job's
+    with pytest.raises(fem.FemError) as e:
+        fem.fem_batch_create(ctx, jobs, I)
+    assert e.value.status == -1
+    for sid in sids:
+        fem.fem_free_stream(ctx, sid)
