@@ -73,8 +73,11 @@ def kernel_source_hash() -> str:
 
 
 def dom_kernel(level: int, ps: str, kind: int = 1) -> str:
-    """Name of the library's counting kernel for a (length, pass) launch; kind 3 is the
-    level-2 pair kernel, 2 the latest-chain kernel, 1 the per-thread machine."""
+    """Name of the library's counting kernel for a (length, pass) launch; kind 4 is over
+    hit tables (level 3 of a large search joined), 3 the level-2 pair kernel, 2 the
+    latest-chain kernel, 1 the per-thread machine."""
+    if kind == 4:
+        return "k_join" if level == 3 else "k_hit_count"
     if kind == 3:
         return "k_pairs_relaxed"
     if kind == 2:

@@ -87,11 +87,24 @@ typedef struct {
  * 2..8).  PAIRS (not a configuration value): fem_count_pairs_relaxed's kernel, one
  * thread counting every interval variant of an ordered type pair from one merge of the
  * two types' events; with AUTO also fem_mine_levelwise's level-2 relaxed pass over two
- * to four intervals.  AUTO: chosen by measurement when tuning is on; else CHAIN for the
- * exact pass over 256 or more candidates that come in runs of shared prefixes or over
- * at most 64 candidates of three or more nodes, CHAIN for the relaxed pass over 32,768
- * or more such candidates of three or more nodes (or at most 64), MACHINE otherwise. */
-enum { FEM_KERNEL_AUTO = 0, FEM_KERNEL_MACHINE = 1, FEM_KERNEL_CHAIN = 2, FEM_KERNEL_PAIRS = 3 };
+ * to four intervals.  HITS (not a configuration value): tables of every edge's (type,
+ * interval, next type) events with an event in the interval before them, built per slab of
+ * the stream, and episodes counted over them in 64-bit words of events; with AUTO the
+ * counts of sets that do not come in prefix runs, batches, window frequencies, and the
+ * levels of fem_mine_levelwise whose work is large for the stream's events times types
+ * (where a slab's words hold the events, K K n_intervals <= 262,144, and the tables fit
+ * beside the stream); level 3 over 40,000 or more candidates joins them all at once.  AUTO
+ * otherwise: chosen by measurement when tuning is on; else CHAIN for the exact pass over
+ * 256 or more candidates that come in runs of shared prefixes or over at most 64
+ * candidates of three or more nodes, CHAIN for the relaxed pass over 32,768 or more such
+ * candidates of three or more nodes (or at most 64), MACHINE otherwise. */
+enum {
+    FEM_KERNEL_AUTO = 0,
+    FEM_KERNEL_MACHINE = 1,
+    FEM_KERNEL_CHAIN = 2,
+    FEM_KERNEL_PAIRS = 3,
+    FEM_KERNEL_HITS = 4
+};
 
 /* Per-level record of the last fem_mine_levelwise call. */
 typedef struct {
@@ -113,7 +126,7 @@ typedef struct {
      * updates; the work measure of the counting kernels) */
     uint64_t touched_relaxed;
     uint64_t touched_exact;
-    /* counting kernel of each pass: FEM_KERNEL_MACHINE or FEM_KERNEL_CHAIN (0: none ran) */
+    /* counting kernel of each pass: FEM_KERNEL_MACHINE, _CHAIN, _PAIRS or _HITS (0: none ran) */
     uint32_t kernel_relaxed, kernel_exact;
 } fem_level_stats;
 

@@ -135,14 +135,18 @@ size_t stream_bytes(const StreamDev &s) {
 
 void free_stream_buffers(StreamDev &s);
 
-// Gives the hit tables' memory back (cudaFree waits for the work that reads them).
-void release_hits(fem_ctx *c) {
+// Gives the hit tables' memory back (cudaFree waits for the work that reads them); whether
+// there was any.
+bool release_hits(fem_ctx *c) {
+    bool any = false;
     for (auto &kv : c->bufs) {
         if (kv.first.compare(0, 4, "hit_") != 0 || !kv.second.p) continue;
         cudaFree(kv.second.p);
         c->mem_used -= std::min(kv.second.cap, c->mem_used);
         kv.second = DevBuf{};
+        any = true;
     }
+    return any;
 }
 
 // Room for `bytes` more under the context's memory budget: over budget, the hit tables of
@@ -166,7 +170,12 @@ int cmalloc(fem_ctx *c, void **p, size_t bytes) {
     if (cudaMalloc(p, bytes) != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
-        return FEM_ENOMEM;
+        // (the device is full: once more without the hit tables of earlier calls)
+        if (c->hits_busy || !release_hits(c) || cudaMalloc(p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            *p = nullptr;
+            return FEM_ENOMEM;
+        }
     }
     c->mem_used += bytes;
     return FEM_OK;
@@ -582,6 +591,7 @@ struct PassLaunch {
     uint32_t R = 1;
     int evset = 0;  // the kernel event set recorded around it
     bool pairs = false;  // the level-2 pair kernel
+    bool hits = false;   // over hit tables (finished when launched)
 };
 
 // Launch one counting pass over m candidates (all of length N) -> out[0..m)
@@ -736,9 +746,11 @@ int count_launch_pairs(fem_ctx *c, const StreamDev &s, const fem_episode *cands,
 // Kernel and stitch times of the last launched pass (its events have completed).
 void pass_info(fem_ctx *c, const PassLaunch &pl, PassInfo *info) {
     info->segments = pl.p.m ? pl.p.P : 0;
-    info->kernel = pl.p.m ? (pl.pairs ? FEM_KERNEL_PAIRS
-                                      : pl.chain ? FEM_KERNEL_CHAIN : FEM_KERNEL_MACHINE)
-                          : 0u;
+    info->kernel = !pl.p.m    ? 0u
+                   : pl.hits  ? FEM_KERNEL_HITS
+                   : pl.pairs ? FEM_KERNEL_PAIRS
+                   : pl.chain ? FEM_KERNEL_CHAIN
+                              : FEM_KERNEL_MACHINE;
     info->ms_kernel = info->ms_stitch = 0;
     if (!pl.p.m) return;
     cudaEventElapsedTime(&info->ms_kernel, c->kev[pl.evset][0], c->kev[pl.evset][1]);
@@ -1061,7 +1073,7 @@ int hits_check(fem_ctx *c, HitPlan *pl, uint32_t *e, bool *again, bool *dense, c
 // false, with nothing counted, where they do not apply.
 int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
                uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
-               cudaStream_t st, bool *done) {
+               cudaStream_t st, bool *done, uint32_t *segments = nullptr) {
     *done = false;
     HitPlan pl;
     bool ok;
@@ -1108,8 +1120,11 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
             for (uint32_t g = 0; g < PLAN_GROUPS; ++g)
                 if (part[g].m) RET(hits_finish(c, s, g, part[g], pass, e, st));
             CK(launch_scatter_u32(tmp, pl.order, m, out, st));
+            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));  // nothing is flagged any more
             CK(cudaStreamSynchronize(st));
         }
+        if (segments)
+            for (const CountParams &q : part) *segments = std::max(*segments, q.P);
         *done = true;
         return FEM_OK;
     }
@@ -1145,6 +1160,17 @@ int windows_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, uint3
     }
 }
 
+// The status of work over hit tables; where there was no room for them beside the stream,
+// their memory is given back and the other kernels count (nothing was).
+int or_no_room(fem_ctx *c, int rc, bool *done, cudaStream_t st) {
+    c->hits_busy = false;
+    if (rc != FEM_ENOMEM) return rc;
+    *done = false;
+    release_hits(c);
+    CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+    return FEM_OK;
+}
+
 // Whether a set may be counted over hit tables: no configured kernel or ring size, no more
 // type pairs and intervals than are worth a table, and on average no more events of a type
 // in an interval than a word is for.
@@ -1156,6 +1182,99 @@ bool hits_eligible(const fem_ctx *c, const StreamDev &s, uint32_t nI) {
            (uint64_t)s.K * s.K * nI <= kHitMaxEdges &&
            (double)s.n * (double)max_hi <= 8.0 * s.K * (double)std::max(s.t_max, 1u);
 }
+
+// One pass of level 3 over m candidates of the frequent pairs F, all pairs at once (k_join):
+// counts of cands[gather[i]] in out[i].  *done = false, with nothing counted, where the
+// tables do not apply; a plan made before is used again if its tables are still there.
+int join_pass(fem_ctx *c, const StreamDev &s, HitPlan *pl, bool planned, const fem_episode *F, uint32_t f,
+              const fem_episode *cands, const uint32_t *gather, uint32_t m, const uint2 *d_ivl,
+              uint32_t nI, int pass, uint32_t *out, cudaStream_t st, PassLaunch *pt, bool *done) {
+    *done = false;
+    *pt = PassLaunch{};
+    pt->N = 3, pt->pass = pass, pt->hits = true;
+    pt->p.m = m, pt->p.P = 1;
+    if (!planned || !c->bufs["hit_plan"].p) {
+        bool ok;
+        *pl = HitPlan{};
+        RET(hits_plan(c, s, F, nullptr, f, true, d_ivl, nI, pass, st, pl, &ok,
+                      [&](const char *name, size_t w, uint32_t **p) { return dbuf(c, name, w, p); }));
+        if (!ok) return FEM_OK;
+    }
+    const uint32_t slots = s.K * nI, n = (uint32_t)s.n;
+    uint32_t *cells, *len, *scratch;
+    JoinTables g{};
+    RET(dbuf(c, "hit_join_cells", (size_t)s.K * slots * slots, &cells));
+    RET(dbuf(c, "hit_join_ends", (size_t)s.K * slots, &g.ends));
+    RET(dbuf(c, "hit_join_begins", (size_t)s.K * slots, &g.begins));
+    RET(dbuf(c, "hit_join_sizes", (size_t)2 * s.K, &g.n_ends));
+    g.n_begins = g.n_ends + s.K;
+    RET(dbuf(c, "hit_join_rank", (size_t)s.K * pl->h.n_slabs, &g.rank));
+    RET(dbuf(c, "hit_join_off", (size_t)n + 1, &g.off));
+    RET(dbuf(c, "hit_join_len", n, &len));
+    RET(dbuf(c, "hit_join_scan", compact_scratch_words(n), &scratch));
+    pt->evset = c->kev_flip ^= 1;
+    cudaEvent_t *kev = c->kev[pt->evset];
+    for (;;) {
+        CK(cudaEventRecord(kev[0], st));
+        RET(hits_build(c, s, pass, pl, st));
+        RET(dbuf(c, "hit_join_list", pl->b.capacity, &g.list));
+        CK(launch_join(pl->h, g, s.hist, n, s.K, nI, len, scratch, cells, st));
+        CK(cudaEventRecord(kev[1], st));
+        CK(launch_join_gather(cells, cands, gather, m, s.K, nI, out, st));
+        CK(cudaEventRecord(kev[2], st));
+        uint32_t e;
+        bool again, dense;
+        RET(hits_check(c, pl, &e, &again, &dense, st));
+        if (dense) return FEM_OK;
+        if (again) continue;
+        *done = true;
+        return FEM_OK;
+    }
+}
+
+// A mining level's pass over hit tables (count_hits).
+int level_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather, uint32_t m,
+               int N, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out, cudaStream_t st,
+               PassLaunch *pt, bool *done) {
+    *pt = PassLaunch{};
+    pt->N = N, pt->pass = pass, pt->hits = true;
+    pt->p.m = m;
+    pt->evset = c->kev_flip ^= 1;
+    cudaEvent_t *kev = c->kev[pt->evset];
+    CK(cudaEventRecord(kev[0], st));
+    RET(count_hits(c, s, cands, gather, m, d_ivl, nI, pass, out, st, done, &pt->p.P));
+    CK(cudaEventRecord(kev[1], st));
+    CK(cudaEventRecord(kev[2], st));
+    return FEM_OK;
+}
+
+// Whether a mining level's pass over m candidates of N nodes goes over hit tables.  Tables
+// cost a plan, a build and their launches, about 100 us and 6 us for a million of (events x
+// types); for a million of (candidates x events of their types) they then count in 1.2 us
+// what the other kernels do in 1.9.  Those flag candidates with more than eight entry
+// classes for a recount, which costs another 100 to 2,000 us when it comes.  Measured (us,
+// before / over tables, recounts included): 22 candidates, 64 types, 406,000 events 86 /
+// 131; 7,896 there 354 / 458 (the line is at 15,700); 44,544 there 3,316 / 1,304; 26,115 of 19 types, 64,000 events
+// 643 / 340; 6,729 of 22 types, 147,000 events 1,614 / 328; 20 of 18 types, 6,200 events
+// 340 / 127.  At level 2 (every type pair or most of them) the line is lower: 239 pairs of
+// 16 types, 4,000 events 290 / 96; 810 of 18, 6,200 events 155 / 112; 952 of 19, 64,000
+// events 155 / 146; 1,397 of 39, 101,000 events 95 / 172; 6,593 of 61, 179,000 events
+// 145 / 192.  With a segment count configured, level 2 keeps its kernels.
+bool level_by_hits(const fem_ctx *c, const StreamDev &s, uint32_t N, uint32_t m, uint32_t nI) {
+    if (!hits_eligible(c, s, nI) || m == 0) return false;
+    const double cells = (double)s.n * s.K;
+    if (N == 2) return !c->cfg.segments && cells <= 1.5e6;
+    return 13 * cells <= 40e6 + (double)m * N * (double)s.n / s.K;
+}
+
+// Level 3 joins all pairs of frequent pairs from this many candidates on, with at most so
+// many cells of (pair, pair) counts (512 MB).  Its cost is that of the pairs: over tables by
+// candidate, 31,000 candidates of 29 types and 30,000 events take 256 us, 45,000 of 36 types
+// and 186,000 events 913, 76,000 of 46 types and 159,000 events 1,081; joined 210, 872 and
+// 696.  9,800 candidates of 22 types and 147,000 events are better counted one by one (456
+// against 899 us: a few hundred warps that walk the whole stream).
+constexpr uint32_t kJoinCandidates = 40000;
+constexpr uint64_t kJoinCells = 1ull << 27;
 
 // Validate a candidate set (optionally gathered): the words of launch_validate_cands.
 int validate(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
@@ -1205,13 +1324,7 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
         bool done = false;
         c->hits_busy = true;
         const int rc = count_hits(c, s, cands, gather, m, d_ivl, nI, pass, out, st, &done);
-        c->hits_busy = false;
-        if (rc == FEM_ENOMEM) {  // no room beside the stream: the other kernels
-            release_hits(c);
-            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
-        } else {
-            RET(rc);
-        }
+        RET(or_no_room(c, rc, &done, st));
         if (done) return FEM_OK;
     }
     if (!known) RET(validate(c, s, cands, gather, m, nI, info, st));
@@ -1312,8 +1425,11 @@ int alloc_stream(fem_ctx *c, StreamDev &s, size_t ne, size_t nc) {
                     cudaMalloc(&s.hist, 256 * 4) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
+        const uint32_t offs = s.offs;
         free_stream_buffers(s);
-        return FEM_ENOMEM;
+        if (c->hits_busy || !release_hits(c)) return FEM_ENOMEM;
+        s.offs = offs;  // (the device is full: once more without the hit tables of earlier calls)
+        return alloc_stream(c, s, ne, nc);
     }
     c->mem_used += bytes;
     return FEM_OK;
@@ -1926,13 +2042,7 @@ int fem_count_windows(fem_ctx *c, int32_t id, const fem_episode *cands, uint32_t
     if (hits_eligible(c, *s, nI)) {
         c->hits_busy = true;
         const int rc = windows_hits(c, *s, dc, m, d_ivl, nI, window_us, dout, st, &done);
-        c->hits_busy = false;
-        if (rc == FEM_ENOMEM) {  // no room beside the stream: the kernel without tables
-            release_hits(c);
-            CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
-        } else {
-            RET(rc);
-        }
+        RET(or_no_room(c, rc, &done, st));
     }
     if (!done) {
         WindowParams p{};
@@ -2108,7 +2218,7 @@ int fem_mine_levelwise_ex(fem_ctx *c, int32_t id, const fem_interval *I, uint32_
         if (done) CK(cudaEventRecord(done, st));
         uint32_t e;
         RET(read_count_err(c, c->d_small + word, kept, &e, st));
-        if (e & ERR_CAP) {
+        if ((e & ERR_CAP) && !pl.hits) {  // (tables: no flags left)
             RET(count_finish(c, s, pl, e, st));
             CK(launch_compact(vals, nullptr, theta, mm, idx, c->d_small + word, scratch, st,
                               pub_of(c)));
@@ -2116,19 +2226,38 @@ int fem_mine_levelwise_ex(fem_ctx *c, int32_t id, const fem_interval *I, uint32_
         }
         return err_status(e);
     };
+    fem_episode *F = nullptr;  // the level's frequent episodes
     for (uint32_t N = 2; N <= max_len && m > 0; ++N) {
         fem_level_stats ls{};
         ls.level = N;
         ls.candidates = m;
         uint32_t *rel, *idx_s, *ex, *idx_f, *fcnt, *scratch;
-        fem_episode *F;
         RETF(dbuf(c, "rel", m, &rel));
         RETF(dbuf(c, "idx_s", m, &idx_s));
         RETF(dbuf(c, "scratch", compact_scratch_words(m), &scratch));
         // first pass (Algorithm 3) on every candidate, then eliminate relaxed < theta
         PassLaunch plr;
         cudaEventRecord(c->ev[2], st);
-        if (repeats) {  // repeated types among the candidates: split and count (count_any)
+        bool joined = false, counted = false;
+        HitPlan hp;
+        if (N == 3 && !repeats && m >= kJoinCandidates && hits_eligible(c, s, nI) &&
+            (uint64_t)s.K * s.K * nI * s.K * nI <= kJoinCells &&
+            !c->tune.count(tune_key(3, FEM_PASS_RELAXED, true, m, s.n_chunks, s.K))) {
+            c->hits_busy = true;
+            const int rc = join_pass(c, s, &hp, false, F, staged_f[2], cands, nullptr, m, d_ivl, nI,
+                                     FEM_PASS_RELAXED, rel, st, &plr, &joined);
+            RETF(or_no_room(c, rc, &joined, st));
+            counted = joined;
+        } else if (!repeats && !(N == 2 && pairs_level2) && level_by_hits(c, s, N, m, nI)) {
+            c->hits_busy = true;
+            const int rc = level_hits(c, s, cands, nullptr, m, (int)N, d_ivl, nI, FEM_PASS_RELAXED, rel,
+                                      st, &plr, &counted);
+            RETF(or_no_room(c, rc, &counted, st));
+        }
+        if (!counted) plr = PassLaunch{};
+        if (counted) {
+            // (over hit tables)
+        } else if (repeats) {  // repeated types among the candidates: split and count (count_any)
             RETF(count_any(c, s, cands, nullptr, m, d_ivl, nI, FEM_PASS_RELAXED, rel, st));
         } else if (N == 2 && pairs_level2) {
             // every interval variant of an ordered type pair from one merge; the
@@ -2155,7 +2284,22 @@ int fem_mine_levelwise_ex(fem_ctx *c, int32_t id, const fem_interval *I, uint32_
         RETF(dbuf(c, "idx_f", ms, &idx_f));
         PassLaunch plx;
         cudaEventRecord(c->ev[6], st);
-        if (repeats)
+        counted = false;
+        if (joined && ms >= kJoinCandidates / 2) {
+            c->hits_busy = true;
+            const int rc = join_pass(c, s, &hp, true, F, staged_f[2], cands, idx_s, ms, d_ivl, nI,
+                                     FEM_PASS_EXACT, ex, st, &plx, &counted);
+            RETF(or_no_room(c, rc, &counted, st));
+        } else if (!repeats && level_by_hits(c, s, N, ms, nI)) {
+            c->hits_busy = true;
+            const int rc = level_hits(c, s, cands, idx_s, ms, (int)N, d_ivl, nI, FEM_PASS_EXACT, ex, st,
+                                      &plx, &counted);
+            RETF(or_no_room(c, rc, &counted, st));
+        }
+        if (!counted) plx = PassLaunch{};
+        if (counted)
+            ;  // (over hit tables)
+        else if (repeats)
             RETF(count_any(c, s, cands, idx_s, ms, d_ivl, nI, FEM_PASS_EXACT, ex, st));
         else
             RETF(count_launch(c, s, cands, idx_s, ms, (int)N, d_ivl, nI, FEM_PASS_EXACT, ex, true,

@@ -517,6 +517,94 @@ cudaError_t run_batch(const CountParams *parts, const uint4 *list, uint32_t n_li
     return cudaGetLastError();
 }
 
+// Per type: its pairs by slot, and where its events of a slab stand among all events by
+// type and then time.
+__global__ void __launch_bounds__(256) k_join_index(const HitTables h, const JoinTables g,
+                                                    const uint32_t *__restrict__ hist, uint32_t K,
+                                                    uint32_t n_ivl) {
+    const uint32_t b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t slots = K * n_ivl;
+    __shared__ uint32_t wsum[8];
+    auto scan = [&](uint32_t v, uint32_t *before, uint32_t *all) {  // over the block's threads
+        uint32_t inc = v;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= (uint32_t)d) inc += y;
+        }
+        __syncthreads();
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        *before = inc - v, *all = 0;
+        for (uint32_t w = 0; w < 8; ++w) {
+            if (w < warp) *before += wsum[w];
+            *all += wsum[w];
+        }
+    };
+    for (int side = 0; side < 2; ++side) {
+        uint32_t seen = 0;
+        for (uint32_t l0 = 0; l0 < slots; l0 += 256) {
+            const uint32_t l = l0 + tid;
+            const uint32_t id = l < slots ? h.edge_id[side ? b * slots + l : (l / n_ivl * K + b) * n_ivl + l % n_ivl] : ~0u;
+            uint32_t r, all;
+            scan(id != ~0u, &r, &all);
+            if (id != ~0u) (side ? g.begins : g.ends)[b * slots + seen + r] = make_uint2(id, l);
+            seen += all;
+        }
+        if (tid == 0) (side ? g.n_begins : g.n_ends)[b] = seen;
+    }
+    uint32_t base, r;
+    scan(tid < b ? hist[tid] : 0u, &r, &base);  // (at most 256 types)
+    for (uint32_t s0 = 0; s0 < h.n_slabs; s0 += 256) {
+        const uint32_t s = s0 + tid;
+        uint32_t all;
+        scan(s < h.n_slabs ? h.count[(uint64_t)s * h.types + b] : 0u, &r, &all);
+        if (s < h.n_slabs) g.rank[(uint64_t)b * h.n_slabs + s] = base + r;
+        base += all;
+    }
+}
+
+// The lists of a slab's events of a type (a warp; lane r: event r): their lengths, or
+// (FILL) their entries.
+template <bool FILL>
+__global__ void __launch_bounds__(256) k_join_list(const HitTables h, const JoinTables g, uint32_t K,
+                                                   uint32_t slots, uint32_t *__restrict__ len) {
+    const uint32_t lane = threadIdx.x & 31, unit = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const uint32_t s = unit / K, b = unit % K;
+    if (s >= h.n_slabs) return;
+    const uint32_t n = h.count[(uint64_t)s * h.types + b], n_first = g.n_ends[b];
+    if (n == 0) return;
+    const uint32_t at = g.rank[(uint64_t)b * h.n_slabs + s] + lane;
+    const uint2 *row = h.edge + (uint64_t)s * h.n_edges;
+    uint32_t o = FILL && lane < n ? g.off[at] : 0u;
+    for (uint32_t i0 = 0; i0 < n_first; i0 += 32) {
+        const uint2 e = i0 + lane < n_first ? row[g.ends[b * slots + i0 + lane].x] : make_uint2(0u, 0u);
+#pragma unroll
+        for (uint32_t k = 0; k < 32; ++k) {
+            const uint32_t mask = __shfl_sync(0xffffffffu, e.x, k);
+            if (FILL) {
+                const uint32_t from = __shfl_sync(0xffffffffu, e.y, k);
+                if ((mask >> lane) & 1u)
+                    g.list[o++] = (i0 + k) << 16 | h.range[from + __popc(mask & ((1u << lane) - 1u))] >> 16;
+            } else {
+                o += (mask >> lane) & 1u;
+            }
+        }
+    }
+    if (!FILL && lane < n) len[at] = o;
+}
+
+// out[i] = the joined count of candidate i (three nodes)
+__global__ void __launch_bounds__(256) k_join_gather(const uint32_t *cells, const fem_episode *cands,
+                                                      const uint32_t *gather, uint32_t m, uint32_t K,
+                                                      uint32_t n_ivl, uint32_t *out) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const fem_episode e = cands[gather ? gather[i] : i];
+    const uint64_t slots = K * n_ivl;
+    out[i] = cells[(e.types[1] * slots + e.types[2] * n_ivl + e.ivl[1]) * slots + e.types[0] * n_ivl + e.ivl[0]];
+}
+
 }  // namespace
 
 uint32_t plan_bins(uint32_t K, uint32_t parts) { return PLAN_GROUPS * K * parts * parts * parts; }
@@ -615,6 +703,39 @@ cudaError_t launch_hit_windows(uint32_t group, const CountParams &p, const uint3
 #undef FEM_CASE
         default: return cudaErrorInvalidValue;
     }
+}
+
+size_t join_smem(uint32_t slots) { return JOIN_QUEUE * sizeof(uint4) + (size_t)slots * sizeof(uint2); }
+
+cudaError_t launch_join(const HitTables &h, const JoinTables &g, const uint32_t *hist, uint32_t n, uint32_t K,
+                        uint32_t n_ivl, uint32_t *len, uint32_t *scratch, uint32_t *out, cudaStream_t st) {
+    static std::once_flag once;
+    static cudaError_t err = cudaSuccess;
+    std::call_once(once, [] {
+        err = cudaFuncSetAttribute(k_join, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+    });
+    if (err != cudaSuccess) return err;
+    const uint32_t slots = K * n_ivl, units = h.n_slabs * K;
+    k_join_index<<<K, 256, 0, st>>>(h, g, hist, K, n_ivl);
+    note_launch();
+    k_join_list<false><<<(units + 7) / 8, 256, 0, st>>>(h, g, K, slots, len);
+    note_launch();
+    if ((err = launch_exclusive_scan(len, n, g.off, g.off + n, scratch, st)) != cudaSuccess) return err;
+    k_join_list<true><<<(units + 7) / 8, 256, 0, st>>>(h, g, K, slots, nullptr);
+    note_launch();
+    // blocks of up to eight warps in about 48 KB
+    const uint32_t NW = (uint32_t)std::min<size_t>(8, std::max<size_t>(1, 48 * 1024 / join_smem(slots)));
+    k_join<<<dim3(K, (slots + NW - 1) / NW), NW * 32, NW * join_smem(slots), st>>>(h, g, n, K, n_ivl, out);
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_join_gather(const uint32_t *cells, const fem_episode *cands, const uint32_t *gather,
+                                uint32_t m, uint32_t K, uint32_t n_ivl, uint32_t *out, cudaStream_t st) {
+    if (m == 0) return cudaSuccess;
+    k_join_gather<<<(m + 255) / 256, 256, 0, st>>>(cells, cands, gather, m, K, n_ivl, out);
+    note_launch();
+    return cudaGetLastError();
 }
 
 }  // namespace fem

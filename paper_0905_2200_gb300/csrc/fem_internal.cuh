@@ -82,6 +82,15 @@ struct HitTables {
     uint64_t slab_bytes;      // (host) about the bytes of a slab's masks and ranges
 };
 
+// The lists of k_join; slots are (other type) n_ivl + interval.
+struct JoinTables {
+    uint2 *ends, *begins;         // [K][slots] the pairs that end / start with a type: edge, slot
+    uint32_t *n_ends, *n_begins;  // [K]
+    uint32_t *rank;               // [K][n_slabs] a slab's first event of a type, by type and time
+    uint32_t *off;                // [n + 1] first entry of an event's list, by type and time
+    uint32_t *list;               // pair (its place in `ends`) << 16 | low half of its first event's index
+};
+
 // Arguments of the counting kernels (one pass over one candidate set).
 struct CountParams {
     const uint2 *bev;
@@ -293,6 +302,15 @@ cudaError_t launch_hit_build_batch(int pass, const HitBuild *host, const HitBuil
                                    cudaStream_t st);
 cudaError_t launch_hit_count_batch(uint32_t group, const CountParams *parts, const uint4 *list,
                                    uint32_t n_list, uint32_t n_items, cudaStream_t st);
+// Level 3 of level-wise mining at once (k_join): the counts of every frequent pair followed
+// by every frequent pair (tables over exactly those edges) into
+// out[b][c n_ivl + u][a n_ivl + v] (unset where either pair is not frequent), and a
+// candidate set's counts out of them.  `len`: n words; `scratch`: of the scan.
+size_t join_smem(uint32_t slots);
+cudaError_t launch_join(const HitTables &h, const JoinTables &g, const uint32_t *hist, uint32_t n, uint32_t K,
+                        uint32_t n_ivl, uint32_t *len, uint32_t *scratch, uint32_t *out, cudaStream_t st);
+cudaError_t launch_join_gather(const uint32_t *cells, const fem_episode *cands, const uint32_t *gather,
+                                uint32_t m, uint32_t K, uint32_t n_ivl, uint32_t *out, cudaStream_t st);
 // What a count over hit tables is planned with: the candidates checked and put in the
 // order they run best in (by group, last three intervals, last type), the edges they use
 // numbered, the stream cut into slabs.  words, hist and edge_id are one block of PLAN_WORDS

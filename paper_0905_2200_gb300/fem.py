@@ -42,7 +42,7 @@ class fem_config(ctypes.Structure):
                 ("ring_capacity", ctypes.c_uint32), ("kernel", ctypes.c_uint32)]
 
 
-KERNEL_AUTO, KERNEL_MACHINE, KERNEL_CHAIN, KERNEL_PAIRS = 0, 1, 2, 3
+KERNEL_AUTO, KERNEL_MACHINE, KERNEL_CHAIN, KERNEL_PAIRS, KERNEL_HITS = 0, 1, 2, 3, 4
 
 
 class fem_level_stats(ctypes.Structure):

@@ -162,3 +162,62 @@ def test_batch(ctx, dense):
     assert e.value.status == -1
     for sid in sids:
         fem.fem_free_stream(ctx, sid)
+
+
+I_LONG = np.array([[0, 9000], [9000, 18000]], np.uint32)
+MINES = {  # events, types, theta, gap, share of type 0, intervals
+    "long lists, several chunks": (5000, 24, 3, 400, 0.0, I_LONG),
+    "one more than a chunk": (2049, 24, 3, 300, 0.0, I_LONG),
+    "one interval": (2500, 36, 2, 300, 0.0, np.array([[0, 9000]], np.uint32)),
+    "too dense for the tables": (3000, 24, 3, 400, 0.5, I_LONG),
+}
+
+
+@pytest.mark.parametrize("name", list(MINES))
+def test_mine_joined(ctx, name):
+    """Level 3 of mining over 40,000 or more candidates joins the lists of pairs: lists shorter
+    and longer than a warp's 64 entries, more hits in a slab than the queue holds, and a
+    stream that is too dense, for which the other kernels count."""
+    n, K, theta, gap, skew, I = MINES[name]
+    ty, t = stream(n + K, n, K, skew=skew, gap=gap)
+    sid = fem.fem_load_stream(ctx, ty, t, K)
+    got = fem.fem_mine_levelwise(ctx, sid, I, theta, 3)
+    stats = fem.fem_last_mine_stats(ctx)
+    fem.fem_free_stream(ctx, sid)
+    assert stats[1]["level"] == 3 and stats[1]["candidates"] >= 40000
+    assert (stats[1]["kernel_relaxed"] == fem.KERNEL_HITS) == ("dense" not in name)
+    assert got == oracle.mine(ty, t, K, I, theta, 3)
+
+
+def test_mine_levels_and_budgets(ctx):
+    """Levels 2-6 over hit tables equal the oracle's; under a memory budget whatever the
+    latest-chain kernels can mine is mined too, with or without room for the tables."""
+    ty, t = stream(77, 4000, 24, tie=0.0, gap=2000)
+    ty[:2400] = np.tile(np.arange(24, dtype=np.uint8), 100)  # long chains
+    sid = fem.fem_load_stream(ctx, ty, t, 24)
+    want = fem.fem_mine_levelwise(ctx, sid, I_MS4[:2], 40, 6)
+    assert want == oracle.mine(ty, t, 24, I_MS4[:2], 40, 6)
+    kinds = [s["kernel_exact"] for s in fem.fem_last_mine_stats(ctx)]
+    assert len(kinds) >= 3 and kinds.count(fem.KERNEL_HITS) >= 2
+    fem.fem_free_stream(ctx, sid)
+    mined = 0
+    for mb in (1, 2, 3, 4, 6, 9, 13, 20, 30, 45, 70):
+        c = fem.fem_create(0, mem_budget_bytes=mb << 20)
+        try:
+            try:
+                sid = fem.fem_load_stream(c, ty, t, 24)
+                fem.fem_set_config(c, kernel=fem.KERNEL_CHAIN)
+                fem.fem_mine_levelwise(c, sid, I_MS4[:2], 40, 6)
+            except fem.FemError as e:
+                assert e.status == -5
+                continue
+        finally:
+            fem.fem_destroy(c)
+        c = fem.fem_create(0, mem_budget_bytes=mb << 20)
+        try:
+            sid = fem.fem_load_stream(c, ty, t, 24)
+            assert fem.fem_mine_levelwise(c, sid, I_MS4[:2], 40, 6) == want
+            mined += 1
+        finally:
+            fem.fem_destroy(c)
+    assert mined >= 3
