@@ -246,6 +246,13 @@ cudaError_t launch_hist_add(const uint8_t *ty, uint64_t n, uint32_t K, int sign,
 // dst[idx[i]] = src[i] and flags[idx[i]] = 1 for i < *m_dev (grid sized for m_max)
 cudaError_t launch_scatter_dev(const uint32_t *src, const uint32_t *idx, const uint32_t *m_dev,
                                uint32_t m_max, uint32_t *dst, uint8_t *flags, cudaStream_t st);
+// flags[idx[i]] = 1 where slot i < *m_dev is flagged; out[idx[i]] = flags[idx[i]] = 0;
+// dst[i] = outer[inner[i]] for i < *m_dev
+cudaError_t launch_mark_flagged(const uint8_t *slot_flags, const uint32_t *idx, const uint32_t *m_dev,
+                                uint32_t m_max, uint8_t *flags, cudaStream_t st);
+cudaError_t launch_clear_at(const uint32_t *idx, uint32_t m, uint32_t *out, uint8_t *flags, cudaStream_t st);
+cudaError_t launch_compose_dev(const uint32_t *outer, const uint32_t *inner, const uint32_t *m_dev,
+                               uint32_t m_max, uint32_t *dst, cudaStream_t st);
 int fem_ctx_device(const fem_ctx *c);
 int fem_ctx_sms(const fem_ctx *c);
 // fem_count.cu
@@ -373,9 +380,10 @@ cudaError_t launch_literal(const LiteralParams &p, uint32_t len_mask, uint32_t *
 cudaError_t launch_stitch_batch(const CountParams *jobs, const uint32_t *job_base,
                                 uint32_t n_jobs, uint32_t slots, uint32_t *err, cudaStream_t st,
                                 uint32_t classes = S_MAX);
+// m_dev: stitch the first *m_dev slots only (tables laid out for m)
 cudaError_t launch_stitch(const uint4 *tables, uint32_t m, uint32_t P, uint32_t *out,
                           uint8_t *redo, uint32_t *err, cudaStream_t st,
-                          uint32_t classes = S_MAX);
+                          uint32_t classes = S_MAX, const uint32_t *m_dev = nullptr);
 // info[0] |= 1 << len of every candidate; info[1] += candidates with a repeated type;
 // info[2] += candidates whose length or prefix before the last node differs from the
 // previous candidate's (the number of prefix runs is info[2] + 1)

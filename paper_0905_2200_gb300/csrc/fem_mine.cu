@@ -197,11 +197,13 @@ __device__ void stitch_one(const uint4 *__restrict__ tables, uint32_t m, uint32_
 template <int SMX>
 __global__ void __launch_bounds__(256) k_stitch(const uint4 *__restrict__ tables, uint32_t m,
                                                 uint32_t P, uint32_t G, uint32_t *__restrict__ out,
-                                                uint8_t *__restrict__ redo, uint32_t *err) {
+                                                uint8_t *__restrict__ redo, uint32_t *err,
+                                                const uint32_t *__restrict__ m_dev) {
     const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x, lg = __ffs(G) - 1;
-    if (((gt & ~31u) >> lg) >= m) return;  // the whole warp is past the end
+    const uint32_t n = m_dev ? min(*m_dev, m) : m;
+    if (((gt & ~31u) >> lg) >= n) return;  // the whole warp is past the end
     const uint32_t ci = gt >> lg;
-    stitch_one<SMX>(tables, m, P, ci, G, ci < m, out, redo, err);
+    stitch_one<SMX>(tables, m, P, ci, G, ci < n, out, redo, err);
 }
 
 // One warp per episode slot of a batch of jobs (each job its own tables and outputs).
@@ -237,7 +239,8 @@ cudaError_t launch_stitch_batch(const CountParams *jobs, const uint32_t *job_bas
 }
 
 cudaError_t launch_stitch(const uint4 *tables, uint32_t m, uint32_t P, uint32_t *out,
-                          uint8_t *redo, uint32_t *err, cudaStream_t st, uint32_t classes) {
+                          uint8_t *redo, uint32_t *err, cudaStream_t st, uint32_t classes,
+                          const uint32_t *m_dev) {
     if (m == 0) return cudaSuccess;
     // lanes per episode: about four segments per lane, so that a short cut (the relaxed
     // passes' 20-odd segments) takes a quarter of a warp rather than a whole one
@@ -245,9 +248,9 @@ cudaError_t launch_stitch(const uint4 *tables, uint32_t m, uint32_t P, uint32_t 
     while (G < 32 && G * 4 < P) G <<= 1;
     const uint32_t blocks = (uint32_t)(((uint64_t)m * G + 255) / 256);
     if (classes == S_RECOUNT)
-        k_stitch<S_RECOUNT><<<blocks, 256, 0, st>>>(tables, m, P, G, out, redo, err);
+        k_stitch<S_RECOUNT><<<blocks, 256, 0, st>>>(tables, m, P, G, out, redo, err, m_dev);
     else if (classes == S_MAX)
-        k_stitch<S_MAX><<<blocks, 256, 0, st>>>(tables, m, P, G, out, redo, err);
+        k_stitch<S_MAX><<<blocks, 256, 0, st>>>(tables, m, P, G, out, redo, err, m_dev);
     else
         return cudaErrorInvalidValue;
     note_launch();
@@ -613,6 +616,51 @@ cudaError_t launch_scatter_dev(const uint32_t *src, const uint32_t *idx, const u
     if (m_max == 0) return cudaSuccess;
     const uint32_t blocks = (m_max + 255) / 256 < 2048 ? (m_max + 255) / 256 : 2048;
     k_scatter_dev<<<blocks, 256, 0, st>>>(src, idx, m_dev, m_max, dst, flags);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// flags[idx[i]] = 1 where slot i < *m_dev is flagged
+__global__ void k_mark_flagged(const uint8_t *__restrict__ slot_flags, const uint32_t *__restrict__ idx,
+                               const uint32_t *__restrict__ m_dev, uint32_t m_max,
+                               uint8_t *__restrict__ flags) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < min(*m_dev, m_max) && slot_flags[i]) flags[idx[i]] = 1;
+}
+
+cudaError_t launch_mark_flagged(const uint8_t *slot_flags, const uint32_t *idx, const uint32_t *m_dev,
+                                uint32_t m_max, uint8_t *flags, cudaStream_t st) {
+    if (m_max == 0) return cudaSuccess;
+    k_mark_flagged<<<(m_max + 255) / 256, 256, 0, st>>>(slot_flags, idx, m_dev, m_max, flags);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// out[idx[i]] = 0, flags[idx[i]] = 0
+__global__ void k_clear_at(const uint32_t *__restrict__ idx, uint32_t m, uint32_t *__restrict__ out,
+                           uint8_t *__restrict__ flags) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < m) out[idx[i]] = 0, flags[idx[i]] = 0;
+}
+
+cudaError_t launch_clear_at(const uint32_t *idx, uint32_t m, uint32_t *out, uint8_t *flags, cudaStream_t st) {
+    if (m == 0) return cudaSuccess;
+    k_clear_at<<<(m + 255) / 256, 256, 0, st>>>(idx, m, out, flags);
+    note_launch();
+    return cudaGetLastError();
+}
+
+// dst[i] = outer[inner[i]] for i < *m_dev
+__global__ void k_compose_dev(const uint32_t *__restrict__ outer, const uint32_t *__restrict__ inner,
+                              const uint32_t *__restrict__ m_dev, uint32_t m_max, uint32_t *__restrict__ dst) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < min(*m_dev, m_max)) dst[i] = outer[inner[i]];
+}
+
+cudaError_t launch_compose_dev(const uint32_t *outer, const uint32_t *inner, const uint32_t *m_dev,
+                               uint32_t m_max, uint32_t *dst, cudaStream_t st) {
+    if (m_max == 0) return cudaSuccess;
+    k_compose_dev<<<(m_max + 255) / 256, 256, 0, st>>>(outer, inner, m_dev, m_max, dst);
     note_launch();
     return cudaGetLastError();
 }

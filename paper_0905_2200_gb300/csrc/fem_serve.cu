@@ -10,6 +10,8 @@
 // submission, and an append waits for the requests still reading that partial
 // chunk, so a reader never sees a chunk being rewritten.
 #include <algorithm>
+#include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <new>
@@ -119,6 +121,12 @@ struct Request {
     fem_episode *h_cands = nullptr;
     cudaStream_t lane = nullptr;
     cudaEvent_t done = nullptr;
+    // a recount: its number (0: the first count), and the candidates it is over (none: all),
+    // sorted positions by length group, on the device at sub()
+    int attempt = 0;
+    uint32_t n_sub = 0;
+    std::vector<Group> sub_groups;
+    uint32_t *sub() const { return rel + (m + 1) / 2; }  // (rel, idx: halves are free then)
     bool in_flight = false, fresh = false, holds_slot = false;
     int status = FEM_OK;
     uint64_t first_event = 0;            // a standing request counts from here
@@ -230,12 +238,16 @@ uint32_t serve_threads(int N, int pass, uint32_t R, uint32_t offs, bool mc = fal
 // One-shot: Algorithm 4 over [ev_begin, ev_end) of the stream, per length group,
 // with every size on the device (no host round trip).  A group of few candidates runs
 // both passes over MapConcatenate segments of the range (the exact pass over the
-// survivors, whose number stays on the device).  attempt 0: the rule's segments, 8
+// survivors, whose number stays on the device).  Attempt 0: the rule's segments, 8
 // entry classes per table, exact lists of kServeRing clusters; attempt 1 (after a
-// capacity guard tripped): a quarter of the segments with 32 classes per table in the
-// same memory and lists of 32 clusters; attempt 2: one segment, lists of 128.
-int enqueue_oneshot(fem_server *v, Request &r, const StreamDev &s, int attempt) {
+// capacity guard tripped): 32 classes per table in the same memory (over all candidates: a
+// quarter of the segments) and lists of 32 clusters; attempt 2: one segment, lists of 128.
+// A recount is over the candidates that either pass flagged where they are at most half:
+// the others' results stand.
+int enqueue_oneshot(fem_server *v, Request &r, const StreamDev &s) {
     cudaStream_t st = r.lane;
+    const int attempt = r.attempt;
+    const bool sub = r.n_sub != 0;
     const uint32_t cr0 = (uint32_t)(r.ev_begin / CHUNK);
     const uint32_t cr1 = (uint32_t)((r.ev_end + CHUNK - 1) / CHUNK);
     const uint32_t nch = cr1 > cr0 ? cr1 - cr0 : 0u;
@@ -243,16 +255,22 @@ int enqueue_oneshot(fem_server *v, Request &r, const StreamDev &s, int attempt) 
     const uint32_t cls = attempt == 0 ? S_MAX : S_RECOUNT;
     // the stitch skips episodes flagged for a recount: no flag may survive from the
     // memory's last user
-    SCK(cudaMemsetAsync(r.redo, 0, r.m, st));
-    for (const Group &g : r.groups) {
+    SCK(cudaMemsetAsync(r.redo, 0, sub ? r.n_sub : r.m, st));
+    if (sub) SCK(launch_clear_at(r.sub(), r.n_sub, r.out, r.flags, st));
+    const std::vector<Group> &groups = sub ? r.sub_groups : r.groups;
+    for (const Group &g : groups) {
+        uint32_t *cnt = r.cnt + (&g - groups.data());
         CountParams p = base_params(s, r, g, FEM_PASS_RELAXED);
-        p.cands = r.cands + g.off;
+        p.cands = sub ? r.cands : r.cands + g.off;
+        p.gather = sub ? r.sub() + g.off : nullptr;
         p.m = g.m;
         p.out = r.rel + g.off;
         uint32_t P = attempt < 2 && r.tables
                          ? oneshot_segments(g.m, nch, fem_ctx_sms(v->ctx), v->cfg.mem_budget_bytes)
                          : 1u;
-        if (attempt == 1) P /= S_RECOUNT / S_MAX;  // the same table memory, 4x the slots
+        if (attempt == 1)  // the same table memory, 4x the slots
+            P = sub ? (uint32_t)std::min<uint64_t>(P, r.tab_items * S_MAX / ((uint64_t)g.m * cls))
+                    : P / (S_RECOUNT / S_MAX);
         if (P > 1) {
             const uint32_t cps = (nch + P - 1) / P;
             P = (nch + cps - 1) / cps;
@@ -269,19 +287,24 @@ int enqueue_oneshot(fem_server *v, Request &r, const StreamDev &s, int attempt) 
                          pcls));
         if (P > 1)
             SCK(launch_stitch(r.tables, g.m, P, r.rel + g.off, r.redo + g.off, r.err, st, pcls));
-        SCK(launch_compact(r.rel + g.off, nullptr, r.theta, g.m, r.idx + g.off,
-                           r.cnt + (&g - r.groups.data()), r.scratch, st));
+        SCK(launch_compact(r.rel + g.off, nullptr, r.theta, g.m, r.idx + g.off, cnt, r.scratch, st));
         // the exact pass over the survivors (their number stays on the device): a grid for
         // all g.m, the blocks past the survivors leave at once; with the relaxed pass's
-        // segments, so that a few survivors still spread over the GPU.  The stitch runs
-        // over g.m slots too; those past the survivors hold the relaxed pass's tables and
-        // their results are never scattered.
+        // segments, so that a few survivors still spread over the GPU.  Its flags go where
+        // the relaxed counts were: the two passes' flags say which candidates to recount.
+        uint32_t *survivors = r.idx + g.off;
+        if (sub) {
+            survivors = r.idx + (r.m + 1) / 2 + g.off;
+            SCK(launch_compose_dev(r.sub() + g.off, r.idx + g.off, cnt, g.m, survivors, st));
+        }
         CountParams x = base_params(s, r, g, FEM_PASS_EXACT);
-        x.cands = r.cands + g.off;
-        x.gather = r.idx + g.off;
+        x.cands = sub ? r.cands : r.cands + g.off;
+        x.gather = survivors;
         x.m = g.m;
-        x.m_dev = r.cnt + (&g - r.groups.data());
+        x.m_dev = cnt;
         x.out = r.ex + g.off;
+        x.redo = reinterpret_cast<uint8_t *>(r.rel + g.off);
+        SCK(cudaMemsetAsync(x.redo, 0, g.m, st));
         const bool xmc = P > 1 && count_config_supported(g.N, FEM_PASS_EXACT, true, R);
         if (xmc) {
             x.cps = p.cps;
@@ -292,11 +315,13 @@ int enqueue_oneshot(fem_server *v, Request &r, const StreamDev &s, int attempt) 
                          serve_threads(g.N, FEM_PASS_EXACT, R, s.offs, xmc, pcls), x, st,
                          xmc ? pcls : S_MAX));
         if (xmc)
-            SCK(launch_stitch(r.tables, g.m, P, r.ex + g.off, r.redo + g.off, r.err, st, pcls));
-        SCK(cudaMemsetAsync(r.out + g.off, 0, (size_t)g.m * 4, st));
-        SCK(cudaMemsetAsync(r.flags + g.off, 0, g.m, st));
-        SCK(launch_scatter_dev(r.ex + g.off, r.idx + g.off, x.m_dev, g.m, r.out + g.off,
-                               r.flags + g.off, st));
+            SCK(launch_stitch(r.tables, g.m, P, r.ex + g.off, x.redo, r.err, st, pcls, cnt));
+        if (!sub) {
+            SCK(cudaMemsetAsync(r.out + g.off, 0, (size_t)g.m * 4, st));
+            SCK(cudaMemsetAsync(r.flags + g.off, 0, g.m, st));
+        }
+        SCK(launch_scatter_dev(r.ex + g.off, survivors, cnt, g.m, sub ? r.out : r.out + g.off,
+                               sub ? r.flags : r.flags + g.off, st));
     }
     return FEM_OK;
 }
@@ -340,6 +365,37 @@ int finish_enqueue(fem_server *v, Request &r, ServeStream &ss) {
     }
     r.in_flight = true;
     return FEM_OK;
+}
+
+// A one-shot's next attempt, enqueued on its lane after a capacity guard tripped (the last
+// attempt has finished): over the candidates whose flags the first attempt left, or over all
+// where those are more than half, or the guard left none.
+int enqueue_recount(fem_server *v, Request &r, ServeStream &ss) {
+    cudaStream_t st = r.lane;
+    SCK(cudaStreamWaitEvent(st, ss.ingested, 0));  // (the range's last chunk may have moved)
+    if (r.attempt == 0) {
+        for (const Group &g : r.groups)
+            SCK(launch_mark_flagged(reinterpret_cast<uint8_t *>(r.rel + g.off), r.idx + g.off,
+                                    r.cnt + (&g - r.groups.data()), g.m, r.redo + g.off, st));
+        SCK(cudaMemcpyAsync(r.h_flags, r.redo, r.m, cudaMemcpyDeviceToHost, st));
+        SCK(cudaStreamSynchronize(st));
+        for (const Group &g : r.groups) {
+            Group q{g.N, r.n_sub, 0, 0};
+            for (uint32_t i = g.off; i < g.off + g.m && r.n_sub <= r.m / 2; ++i)
+                if (r.h_flags[i] && r.n_sub++ < r.m / 2) r.h_out[q.off + q.m++] = i;
+            if (q.m) r.sub_groups.push_back(q);
+        }
+        if (r.n_sub > r.m / 2) r.n_sub = 0;
+        if (r.n_sub)
+            SCK(cudaMemcpyAsync(r.sub(), r.h_out, r.n_sub * 4ull, cudaMemcpyHostToDevice, st));
+    }
+    ++r.attempt;
+    if (std::getenv("FEM_DEBUG"))
+        std::fprintf(stderr, "fem: serve recount %d of request %llu: %u of %u candidates\n", r.attempt,
+                     (unsigned long long)r.id, r.n_sub ? r.n_sub : r.m, r.m);
+    SCK(cudaMemsetAsync(r.err, 0, 4, st));
+    SRET(enqueue_oneshot(v, r, ss.s));
+    return finish_enqueue(v, r, ss);
 }
 
 // Return pinned staging buffers whose uploads have finished (all of them if wait).
@@ -637,7 +693,7 @@ int fem_server_submit(fem_server *v, int32_t sid, const fem_episode *cands, uint
     }
     if (s.t_max > kServeMaxTime) return fail(FEM_ERANGE);
     if (mode == FEM_REQ_ONESHOT) {
-        int rc = enqueue_oneshot(v, r, s, 0);
+        int rc = enqueue_oneshot(v, r, s);
         if (rc == FEM_OK) rc = finish_enqueue(v, r, ss);
         if (rc != FEM_OK) return fail(rc);
     } else {
@@ -680,21 +736,17 @@ int fem_server_poll(fem_server *v, uint64_t *done_ids, uint32_t cap, uint32_t *n
         else if (e & ERR_BADEP) r.status = FEM_EINVAL;
         else if ((e & (ERR_RING | ERR_CLASS | ERR_TABLE)) && r.mode == FEM_REQ_ONESHOT &&
                  r.status == FEM_OK) {
-            // a capacity guard tripped: recount with more entry classes per table, then
-            // in one segment with larger rings, synchronously on the request's lane
-            auto sit = v->streams.find(r.sid);
-            int rc = FEM_OK;
-            bool still = true;
-            for (int attempt = 1; attempt <= 2 && still && rc == FEM_OK; ++attempt) {
-                rc = cudaMemsetAsync(r.err, 0, 4, r.lane) == cudaSuccess ? FEM_OK : FEM_ECUDA;
-                if (rc == FEM_OK) rc = enqueue_oneshot(v, r, sit->second.s, attempt);
-                if (rc == FEM_OK) rc = finish_enqueue(v, r, sit->second);
-                if (rc == FEM_OK && cudaEventSynchronize(r.done) != cudaSuccess) rc = FEM_ECUDA;
-                still = (*r.h_err & (ERR_RING | ERR_CLASS | ERR_TABLE)) != 0;
+            // a capacity guard tripped: recount with more entry classes per table, then in one
+            // segment with larger rings, on the request's lane beside the others' work
+            if (r.attempt < 2) {
+                const int rc = enqueue_recount(v, r, v->streams.find(r.sid)->second);
+                if (rc == FEM_OK) continue;
+                cudaStreamSynchronize(r.lane);
+                r.in_flight = false;
+                r.status = rc;
+            } else {
+                r.status = FEM_EOVERFLOW;
             }
-            r.in_flight = false;
-            if (rc != FEM_OK) r.status = rc;
-            else if (still) r.status = FEM_EOVERFLOW;
         } else if (e & ERR_RING) {
             r.status = FEM_EOVERFLOW;  // a standing request's carried lists overflowed
         }
@@ -779,8 +831,9 @@ int fem_server_release(fem_server *v, uint64_t id) {
 int fem_server_drain(fem_server *v) {
     if (!v) return FEM_EINVAL;
     cudaSetDevice(v->device);
-    // finish in-flight work, then let standing requests catch up with the stream
-    for (int round = 0; round < 4; ++round) {
+    // finish in-flight work and its recounts, then let standing requests catch up with the
+    // stream
+    for (int round = 0; round < 8; ++round) {
         for (cudaStream_t s : v->lanes)
             if (cudaStreamSynchronize(s) != cudaSuccess) return FEM_ECUDA;
         if (cudaStreamSynchronize(v->ingest) != cudaSuccess) return FEM_ECUDA;
