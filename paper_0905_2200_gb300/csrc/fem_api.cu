@@ -1011,8 +1011,7 @@ int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
                      (double)std::max(s.t_max, 1u);
     per_event *= (double)h.n_edges / tri;
     pl->hits = std::min<uint64_t>((uint64_t)(1.25 * per_event * (double)s.n) + 65536,
-                                  (uint64_t)s.n * (h.n_edges / s.K + 1)) +
-               hit_slack(h.n_slabs);
+                                  (uint64_t)s.n * (h.n_edges / s.K + 1));
     *ok = true;
     return FEM_OK;
 }
@@ -1064,7 +1063,7 @@ int hits_check(fem_ctx *c, HitPlan *pl, uint32_t *e, bool *again, bool *dense, c
     RET(err_status(*e));
     *dense = (*e & ERR_DENSE) != 0 || used > 0xF0000000u;
     *again = !*dense && used > pl->b.capacity;
-    if (*again) pl->hits = used + used / 16 + hit_slack(pl->h.n_slabs);
+    if (*again) pl->hits = used + used / 16;
     if (*again || *dense) CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
     return FEM_OK;
 }
@@ -2842,7 +2841,7 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
         if (need > 0xF0000000ull || bytes + (tab * sizeof(uint4)) + need * 4 > most) return FEM_OK;
         cfree(c, range, b->alloc_bytes.back());
         b->allocs.pop_back(), b->alloc_bytes.pop_back();
-        h.capacity = need + need / 16 + hit_slack(h.n_slabs);
+        h.capacity = need + need / 16;
     }
     return FEM_OK;
 }

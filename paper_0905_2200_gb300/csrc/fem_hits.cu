@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(256) k_plan_bins(const PlanArgs a) {
             a.rank[i] = atomicAdd(&a.hist[bin], 1u);
             if (!rep)
                 for (uint32_t k = 0; k + 1 < N; ++k)
-                    a.edge_id[(e.types[k] * a.K + e.types[k + 1]) * a.n_ivl + e.ivl[k]] = 1u;
+                    a.edge_id[(e.types[k + 1] * a.K + e.types[k]) * a.n_ivl + e.ivl[k]] = 1u;
         }
     }
     for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
@@ -234,38 +234,38 @@ __global__ void k_publish_count(const unsigned long long *src, Publish pub) {
     h[2] = pub.seq;
 }
 
-// The hit tables of one slab (a block; of a few slabs several, which share the types).  Every type's events in the slab and the 32
-// before it go into shared memory as rank rows (rank 32 is the slab's first; the types'
-// own order in the chunk gives the ranks), with a bit per position of the slab and, per
-// 32 positions, the events before them, so that the number of a type's events before any
-// event of the slab is two reads and a popc.  Then a warp takes a pack of types with up to 32
-// events in all, a lane an event, and goes through the types x: the x events before the
-// lane's event as far back as the longest interval reaches, a few steps down the row, give
-// the ranges of four intervals at once; a ballot per interval holds the masks of up to 32
-// edges, of which each lane takes one.  Ranges are written to room that a warp reserves in
-// the table for many edges at a time.  What bounds it: warp issue slots.  Measured on the
-// 406,000 events of 64 types at 20 Hz, all 16,128 edges, exact pass: 467 us; one type a
-// warp 490 us (half the lanes idle), a thread per edge, merging its two rows, 983, a thread
-// per event and earlier event 526 (and 4500 on a bursting recording).
+// The hit tables of one slab (a block; of a few slabs several, which share the types).
+// Every type's events in the slab and the 32 before it go into shared memory as rank rows
+// (rank 32 is the slab's first; the types' own order in the chunk gives the ranks), with a
+// bit per position of the slab and, per 32 positions, the events before them, so that the
+// number of a type's events before any event of the slab is two reads and a popc.  Then a
+// warp takes a type y, a lane a type x: for each of y's events, the x events before it as far
+// back as the longest interval reaches, a few steps down the row, give the masks of four
+// edges.  The warp reserves room for its hits in the table, and the ranges are found again:
+// by each lane for its own hits where these are few, else event by event for all four
+// intervals.  What bounds it: issue slots, two thirds of them used, half the lanes in the
+// walks.  Measured on the 406,000 events of 64 types at 20 Hz, all 16,128 edges, exact pass:
+// 258 us (48 recordings, 16 to 64 types: 3.1 ms exact, 3.3 relaxed; bursts of 64 types,
+// 635 us).  Lanes on the events of a few y, all x one after the other, with ballots for the
+// masks: 467 us (3.6 and 3.5 ms; 671 us).  Masks first, then one reservation a block and the
+// ranges: 272 us (3.3 and 3.8 ms; 950 us).  Without the walk event by event, bursts take
+// 837 us.  A thread per edge, merging its two rows: 983 us.
 constexpr int U = 4;                   // intervals taken at once
-constexpr uint32_t HIT_PACK = 32 / U;  // types a warp takes at once
 
 template <int PASS>
 __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, uint32_t part, uint32_t parts) {
     const uint32_t T = HIT_BUILD_T, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr uint32_t NW = HIT_BUILD_T / 32;
     const uint32_t K = b.K;
-    __shared__ uint32_t n_packs;
     uint32_t *rt = reinterpret_cast<uint32_t *>(fem_hit_smem);  // times by rank [K][HIT_ROW]
     uint32_t *bits = rt + K * HIT_ROW;                          // [K][slab words]
     const uint32_t begin = b.begin[s], end = b.begin[s + 1], c = begin / CHUNK;
     const uint32_t p0 = begin % CHUNK, p1 = p0 + (end - begin);  // the slab's places in its chunk
-    const uint32_t words = (end - begin + 31) / 32;
-    uint16_t *rp = reinterpret_cast<uint16_t *>(bits + K * b.max_words);  // positions by rank [K][HIT_ROW]
+    const uint32_t words = ((end - begin + 31) / 32) | 1u;  // (an odd stride: no bank conflicts)
+    uint16_t *rp = reinterpret_cast<uint16_t *>(bits + K * (b.max_words | 1u));  // positions by rank [K][HIT_ROW]
     uint16_t *place = rp + K * HIT_ROW;                          // [K + 1]
-    uint16_t *pack = place + K + 1;                              // first type of each pack, K
-    uint8_t *before = reinterpret_cast<uint8_t *>(pack + K + 1);  // events before a word [K][words]
-    uint8_t *hist = before + K * b.max_words;                    // events before the slab [K]
+    uint8_t *before = reinterpret_cast<uint8_t *>(place + K + 1);  // events before a word [K][words]
+    uint8_t *hist = before + K * (b.max_words | 1u);                    // events before the slab [K]
     uint8_t *num = hist + K;                                     // events in the slab [K]
     const uint32_t origin = c * CHUNK - CHUNK;                   // index of position 0 (modulo 2^32)
     const uint16_t *off = b.boff + (uint64_t)c * b.offs;
@@ -335,22 +335,18 @@ __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, ui
             }
             carry += __shfl_sync(0xffffffffu, inc, 31);
         }
-        if (lane == 0) {
-            place[K] = (uint16_t)carry;
-            // packs of consecutive types: up to 32 events of up to 8 types
-            uint32_t n = 0, y0 = 0;
-            for (uint32_t y = 0; y < K; ++y) {
-                if (y > y0 && (place[y + 1] - place[y0] > 32 || y - y0 == HIT_PACK)) pack[n++] = (uint16_t)y0, y0 = y;
-            }
-            pack[n++] = (uint16_t)y0;
-            pack[n] = (uint16_t)K;
-            n_packs = n;
-        }
     }
     __syncthreads();
+    for (uint32_t x = warp; x < K && part == 0; x += NW)
+        if (lane < num[x]) b.index[begin + place[x] + lane] = (uint16_t)(origin + rp[x * HIT_ROW + 32 + lane]);
+    uint2 *const row = b.edge + (uint64_t)s * b.n_edges;
     bool dense = false;
-    uint32_t at = 0, left = 0;  // the warp's room in the table of ranges
-    bool full = false;          // the table has no more (the warp goes on to count its hits)
+    // x's events before event r of type y: those of ranks below k0
+    auto rank_of = [&](uint32_t x, uint32_t y, uint32_t r) {
+        const uint32_t q = rp[y * HIT_ROW + 32 + r] - CHUNK - p0, w = q >> 5;
+        return 32u + before[x * words + w] + __popc(bits[x * words + w] & ((1u << (q & 31)) - 1u));
+    };
+    const uint32_t groups = (K + 31) / 32;
     for (uint32_t u0 = 0; u0 < b.n_ivl; u0 += U) {
         // a gap lies in interval u iff gap - from[u] <= wide[u] (unsigned); the relaxed pass
         // takes any gap up to hi
@@ -362,88 +358,103 @@ __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, ui
             wide[u] = v.y - from[u];
             far = max(far, v.y);
         }
-        for (uint32_t k = part * NW + warp; k < n_packs; k += NW * parts) {
-            const uint32_t y0 = pack[k], types = pack[k + 1] - y0, base = place[y0];
-            // the lane's event: the pack's lane-th, of type y0 + g
-            const uint32_t n = place[y0 + types] - base;
-            const bool mine = lane < n;
-            uint32_t g = 0;
-            for (uint32_t j = 1; j < types; ++j) g += place[y0 + j] - base <= lane;
-            if (!mine) g = 0;
-            const uint32_t y = y0 + g, o = place[y] - base, r = lane - o;
-            const uint32_t t = mine ? rt[y * HIT_ROW + 32 + r] : 0u;
-            const uint32_t pos = mine ? rp[y * HIT_ROW + 32 + r] : CHUNK + p0;
-            if (mine && u0 == 0) b.index[begin + base + lane] = (uint16_t)(origin + pos);
-            const uint32_t q = pos - CHUNK - p0, w = q >> 5, below = (1u << (q & 31)) - 1u;
-            const uint32_t same_below = ((1u << lane) - 1u) & ~((1u << o) - 1u);
-            // the lane's edge: (x, u0 + eu, y0 + eg), its number asked for an x ahead; `ours`
-            // are the lanes of its last type's events
-            const uint32_t eg = lane / U, eu = lane % U;
-            const bool edge = eg < types && u0 + eu < b.n_ivl;
-            const uint32_t eo = edge ? place[y0 + eg] - base : 0u, en = edge ? num[y0 + eg] : 0u;
-            const uint32_t ours = en ? (0xFFFFFFFFu >> (32u - en)) << eo : 0u;
-            const uint32_t *ids = b.edge_id + (y0 + (edge ? eg : 0u)) * b.n_ivl + u0 + eu;
-            uint32_t next = edge ? __ldg(ids) : ~0u;
-            for (uint32_t x = 0; x < K; ++x) {
-                const uint32_t id = next;
-                if (x + 1 < K && edge) next = __ldg(ids + (x + 1) * K * b.n_ivl);
-                const uint32_t wanted = __ballot_sync(0xffffffffu, id != ~0u);
-                if (!wanted) continue;  // no edge in use
-                const uint32_t *tx = rt + x * HIT_ROW;
-                const uint32_t low = 32u - hist[x];
-                // x's events before the lane's event have the ranks below k0; those in interval
-                // u are m[u] from a[u] on
-                uint32_t a[U] = {}, m[U] = {};
-                if (mine) {
-                    const uint32_t k0 = 32u + before[x * words + w] + __popc(bits[x * words + w] & below);
+        for (uint32_t task = part * NW + warp; task < K * groups; task += NW * parts) {
+            const uint32_t y = task / groups, x = (task % groups) * 32 + lane, n = num[y];
+            uint32_t id[U], mask[U], any = 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                id[u] = x < K && u0 + u < b.n_ivl ? __ldg(b.edge_id + (y * K + x) * b.n_ivl + u0 + u) : ~0u;
+                any |= ~id[u];
+                mask[u] = 0;
+            }
+            if (!__any_sync(0xffffffffu, any != 0)) continue;  // no edge in use
+            const uint32_t *tx = rt + x * HIT_ROW, *ty = rt + y * HIT_ROW + 32;
+            const uint32_t low = any ? 32u - hist[x] : ~0u;  // (no edge: no event is looked at)
+            for (uint32_t r = 0; r < n && any; ++r) {
+                const uint32_t t = ty[r], k0 = rank_of(x, y, r);
+                uint32_t k = k0;
+                for (; k > low; --k) {
+                    const uint32_t gap = t - tx[k - 1];
+                    if (gap > far) break;
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (gap - from[u] <= wide[u]) mask[u] |= 1u << r;
+                }
+                // older events than the 32 kept may lie in an interval, or more than a range
+                // can say
+                dense = dense || (k == 0 && k0 > 0) || k0 - k > 32;
+            }
+            uint32_t c = 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (id[u] == ~0u) mask[u] = 0;
+                c += __popc(mask[u]);
+            }
+            uint32_t inc = c;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, inc, d);
+                if (lane >= (uint32_t)d) inc += v;
+            }
+            const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+            unsigned long long v = 0;
+            if (total) {
+                if (lane == 0) v = atomicAdd(b.used, (unsigned long long)total);
+                v = __shfl_sync(0xffffffffu, v, 0);
+            }
+            const bool room = v + total <= b.capacity;
+            uint32_t o = (uint32_t)v + inc - c, at = o;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (id[u] != ~0u) row[id[u]] = make_uint2(room ? mask[u] : 0u, at);
+                at += __popc(mask[u]);
+            }
+            if (!room) continue;
+            // the hits' ranges: where they are many for the events, event by event, with one
+            // walk for all intervals
+            if (__reduce_max_sync(0xffffffffu, c) > 2 * n) {
+                if (c == 0) continue;
+                uint32_t to[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) to[u] = o, o += __popc(mask[u]);
+                for (uint32_t r = 0; r < n; ++r) {
+                    const uint32_t t = ty[r], k0 = rank_of(x, y, r);
+                    uint32_t in[U] = {};
                     uint32_t k = k0;
-                    for (; k > low; --k) {
+                    for (uint32_t bit = 1; k > low; --k, bit <<= 1) {
                         const uint32_t gap = t - tx[k - 1];
                         if (gap > far) break;
 #pragma unroll
                         for (int u = 0; u < U; ++u)
-                            if (gap - from[u] <= wide[u]) a[u] = k - 1, ++m[u];
+                            if (gap - from[u] <= wide[u]) in[u] |= bit;  // (rank k0 - 1 - bit)
                     }
-                    // older events than the 32 kept may lie in an interval, or more than a range
-                    // can say
-                    dense = dense || (k == 0 && k0 > 0) || k0 - k > 32;
-                }
-                // the masks of the pack's edges, and their places in the table
-                uint32_t hits[U], mask = 0;
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    hits[u] = __ballot_sync(0xffffffffu, m[u] != 0);
-                    if (eu == (uint32_t)u) mask = hits[u] & ours;
+                    for (int u = 0; u < U; ++u) {
+                        if (!((mask[u] >> r) & 1u)) continue;
+                        const uint32_t m = __popc(in[u]), last = k0 - __ffs(in[u]);
+                        b.range[to[u]++] = hit_pack(last + 1 - m, m, origin + rp[x * HIT_ROW + last]);
+                    }
                 }
-                if (id == ~0u) mask = 0;
-                const uint32_t c = __popc(mask);
-                uint32_t inc = c;
+                continue;
+            }
+            // else each lane its own, one after the other
+            uint32_t u = 0, left = mask[0], f = from[0], wd = wide[0];
+            for (; c; --c) {
+                while (!left) {
+                    ++u;
 #pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const uint32_t v = __shfl_up_sync(0xffffffffu, inc, d);
-                    if (lane >= (uint32_t)d) inc += v;
+                    for (int j = 1; j < U; ++j)
+                        if (u == (uint32_t)j) left = mask[j], f = from[j], wd = wide[j];
                 }
-                const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
-                if (total > left) {  // the same in every lane
-                    const uint32_t ask = full ? total : HIT_ROOM;
-                    unsigned long long v = 0;
-                    if (lane == 0) v = atomicAdd(b.used, (unsigned long long)ask);
-                    v = __shfl_sync(0xffffffffu, v, 0);
-                    full = full || v + ask > b.capacity;
-                    left = full ? 0u : HIT_ROOM;
-                    at = (uint32_t)v;
-                }
-                const bool room = total <= left;
-                const uint32_t out = at + inc - c;
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const uint32_t at_u = __shfl_sync(0xffffffffu, out, g * U + u);
-                    if (m[u] && room && ((wanted >> (g * U + u)) & 1u))
-                        b.range[at_u + __popc(hits[u] & same_below)] =
-                            hit_pack(a[u], m[u], origin + rp[x * HIT_ROW + a[u] + m[u] - 1]);
-                }
-                if (id != ~0u) b.edge[(uint64_t)s * b.n_edges + id] = make_uint2(room ? mask >> eo : 0u, out);
-                if (room) at += total, left -= total;
+                const uint32_t r = __ffs(left) - 1u;
+                left &= left - 1u;
+                const uint32_t t = ty[r];
+                uint32_t k = rank_of(x, y, r), m = 0;
+                if (PASS == FEM_PASS_EXACT)
+                    while (t - tx[k - 1] - f > wd) --k;  // (too near; the mask says that one is not)
+                const uint32_t last = k - 1;
+                for (; k > low && t - tx[k - 1] - f <= wd; --k) ++m;
+                b.range[o++] = hit_pack(k, m, origin + rp[x * HIT_ROW + last]);
             }
         }
     }
@@ -473,7 +484,7 @@ __global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build_batch(const HitBuild 
 }
 
 size_t build_smem(const HitBuild &b) {
-    return (size_t)b.K * (HIT_ROW * 6 + b.max_words * 5 + 6) + 32;
+    return (size_t)b.K * (HIT_ROW * 6 + (b.max_words | 1u) * 5 + 4) + 32;
 }
 
 cudaError_t build_limits() {
@@ -545,7 +556,7 @@ __global__ void __launch_bounds__(256) k_join_index(const HitTables h, const Joi
         uint32_t seen = 0;
         for (uint32_t l0 = 0; l0 < slots; l0 += 256) {
             const uint32_t l = l0 + tid;
-            const uint32_t id = l < slots ? h.edge_id[side ? b * slots + l : (l / n_ivl * K + b) * n_ivl + l % n_ivl] : ~0u;
+            const uint32_t id = l < slots ? h.edge_id[side ? (l / n_ivl * K + b) * n_ivl + l % n_ivl : b * slots + l] : ~0u;
             uint32_t r, all;
             scan(id != ~0u, &r, &all);
             if (id != ~0u) (side ? g.begins : g.ends)[b * slots + seen + r] = make_uint2(id, l);
@@ -634,8 +645,6 @@ cudaError_t launch_publish_count(const unsigned long long *src, Publish pub, cud
     return cudaGetLastError();
 }
 
-uint64_t hit_slack(uint32_t n_slabs) { return (uint64_t)n_slabs * (HIT_BUILD_T / 32) * HIT_ROOM; }
-
 cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
                              cudaStream_t st) {
     if (n_slabs == 0) return cudaSuccess;
@@ -646,7 +655,7 @@ cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int 
     // a few slabs: their types shared among several blocks, for about four per SM
     constexpr uint32_t NW = HIT_BUILD_T / 32;
     uint32_t split = 1;
-    while (split < 8 && split * NW < b.K && split * n_slabs < 4 * (uint32_t)sm_count) split *= 2;
+    while (split < 8 && split * NW < b.K * ((b.K + 31) / 32) && split * n_slabs < 4 * (uint32_t)sm_count) split *= 2;
     (pass == FEM_PASS_RELAXED ? k_hit_build<FEM_PASS_RELAXED>
                               : k_hit_build<FEM_PASS_EXACT>)<<<dim3(n_slabs, split), HIT_BUILD_T, sm, st>>>(b);
     note_launch();

@@ -50,7 +50,6 @@ constexpr uint32_t HIT_CLASSES = 32;   // most entry classes per table
 constexpr uint32_t HIT_PARTS = 64;     // most slabs per chunk (32 events each)
 constexpr uint32_t HIT_ROW = 65;       // words per type of a slab's rank tables (64 and a pad)
 constexpr uint32_t HIT_BUILD_T = 256;  // threads of a build block
-constexpr uint32_t HIT_ROOM = 512;     // ranges a warp of it reserves at a time
 
 // inner nodes of an episode of up to nmax nodes, and those whose chains' starts are in
 // shared memory
@@ -96,7 +95,7 @@ struct HitEpisode {
                     ok = iv < p.n_ivl;
                     if (ok) {
                         W += p.ivl[iv].y;
-                        edge[d] = p.hits.edge_id[(type[d > 0 ? d - 1 : 0] * p.K + type[d]) * p.n_ivl + iv];
+                        edge[d] = p.hits.edge_id[(type[d] * p.K + type[d > 0 ? d - 1 : 0]) * p.n_ivl + iv];
                     }
                 }
             }

@@ -70,7 +70,7 @@ struct StreamDev {
 
 // The hit tables of a stream, an edge set and a pass (fem_hits.cuh).
 struct HitTables {
-    const uint32_t *edge_id;  // number of edge (type, next type, interval)
+    const uint32_t *edge_id;  // number of edge (next type, type, interval)
     const uint32_t *begin;    // [n_slabs + 1] first event of each slab
     const uint32_t *t0;       // [n_slabs + 1] its time
     const uint2 *edge;        // [n_slabs][n_edges] mask of the next type's events, first range
@@ -298,7 +298,6 @@ struct HitBuild {
     uint32_t *err;                // ERR_DENSE
 };
 // ranges that a build of n_slabs slabs may reserve beyond its hits
-uint64_t hit_slack(uint32_t n_slabs);
 cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
                              cudaStream_t st);
 // for a batch: streams[j]'s slabs are blocks first[j] .. first[j + 1] (device arrays; host:
