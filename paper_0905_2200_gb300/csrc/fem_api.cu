@@ -1299,6 +1299,16 @@ int validate(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uin
 // latest-chain kernels.
 bool in_runs(const uint32_t *info, uint32_t m) { return (uint64_t)m >= 4ull * ((uint64_t)info[2] + 1); }
 
+// Most of all pairs, exact, on a long stream: the latest-chain kernel looks every last-node
+// event up for each, the tables' cost is that of the stream.  Chain / tables, us: 16,128 pairs
+// of 64 types over 383,000 events 570 / 481, over 1.5 million 1,904 / 1,171, over 128,000
+// 240 / 269; 3,968 of 32 over 288,000 375 / 301; 2,208 of 24 over 864,000 476 / 411; 30% of
+// the 64 types' pairs over 383,000 events 228 / 272.  (Relaxed, the machine is the faster.)
+bool most_pairs(const StreamDev &s, const uint32_t *info, uint32_t m, uint32_t nI, int pass) {
+    return pass == FEM_PASS_EXACT && info[0] == 1u << 2 && 4ull * m >= 3ull * s.K * (s.K - 1) * nI &&
+           (double)m * (double)s.n >= 35e6 * s.K;
+}
+
 int count_validated(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
                     uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
                     const uint32_t *info, cudaStream_t st);
@@ -1317,7 +1327,7 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     if (!hits || m >= 256) {
         RET(validate(c, s, cands, gather, m, nI, info, st));
         known = true;
-        hits = hits && !info[1] && !in_runs(info, m);
+        hits = hits && !info[1] && (!in_runs(info, m) || most_pairs(s, info, m, nI, pass));
     }
     if (hits) {
         bool done = false;
