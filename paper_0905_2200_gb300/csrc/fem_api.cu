@@ -1285,9 +1285,9 @@ int validate(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uin
         const uint32_t seq = ++c->pub_seq;
         CK(launch_publish_info(c->d_small + W_INFO, Publish{c->d_plan, c->d_err, seq}, st));
         const volatile uint32_t *w = c->h_small + kPlanWord;
-        RET(wait_seq(w + 4, seq, st));
+        RET(wait_seq(w + PLAN_WORDS + 1, seq, st));
         for (uint32_t k = 0; k < 3; ++k) info[k] = w[k];
-        e = w[3];
+        e = w[PLAN_WORDS];
     } else {
         RET(read_words(c, c->d_small + W_INFO, 3, info, st));
         RET(read_err(c, st, &e));

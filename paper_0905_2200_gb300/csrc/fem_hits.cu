@@ -215,13 +215,14 @@ __global__ void __launch_bounds__(256) k_plan_place(const PlanArgs a, uint32_t *
     gather[s] = a.gather ? a.gather[i] : i;
 }
 
-// The words of k_validate_cands and the error word, published.
+// The words of k_validate_cands and the error word, published; the error word and the
+// sequence number where a plan's are, so that no other word is ever taken for the number.
 __global__ void k_publish_info(const uint32_t *info, Publish pub) {
     volatile uint32_t *h = pub.host;
     for (uint32_t k = 0; k < 3; ++k) h[k] = info[k];
-    h[3] = *reinterpret_cast<const volatile uint32_t *>(pub.err);
+    h[PLAN_WORDS] = *reinterpret_cast<const volatile uint32_t *>(pub.err);
     __threadfence_system();
-    h[4] = pub.seq;
+    h[PLAN_WORDS + 1] = pub.seq;
 }
 
 // (a count above 32 bits as 2^32 - 1)

@@ -221,3 +221,28 @@ def test_mine_levels_and_budgets(ctx):
         finally:
             fem.fem_destroy(c)
     assert mined >= 3
+
+
+@pytest.mark.parametrize("n5", range(60, 72))
+def test_many_calls(ctx, n5):
+    """Call after call in a new context: a set's count of one length passes the sequence number
+    of the words the host waits for, which must not be taken for it."""
+    torch = pytest.importorskip("torch")
+    ty, t = stream(5, 3000, 12)
+    parts = [synth.random_candidates(m, m, 12, [n], 4) for m, n in ((n5, 5), (127, 4), (120, 3))]
+    cands = tuple(np.concatenate(p) for p in zip(*parts))
+    keep = oracle_counts(ty, t, *cands, I_MS4, fem.PASS_RELAXED) >= 0
+    want = np.where(keep, oracle_counts(ty, t, *cands, I_MS4, fem.PASS_EXACT), 0)
+    rec = torch.from_numpy(fem.pack_episodes(*cands)).cuda()
+    ex = torch.zeros(len(keep), dtype=torch.int32, device="cuda")
+    kept = torch.zeros(len(keep), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    c = fem.fem_create(0)
+    try:
+        sid = fem.fem_load_stream(c, ty, t, 12)
+        for k in range(60):
+            fem.fem_count_two_pass(c, sid, rec, I_MS4, 0, ex, kept)
+            assert_counts_equal(ex.cpu().numpy(), want, f"call {k}")
+            assert_counts_equal(kept.cpu().numpy(), keep.astype(np.uint8), f"call {k}")
+    finally:
+        fem.fem_destroy(c)
