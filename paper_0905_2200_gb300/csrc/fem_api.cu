@@ -1068,6 +1068,18 @@ int hits_check(fem_ctx *c, HitPlan *pl, uint32_t *e, bool *again, bool *dense, c
     return FEM_OK;
 }
 
+// A few short episodes of many types on a long stream: the tables, whose cost is that of
+// events and types, cost more than the per-thread machine's count, whose is that of
+// segments and nodes (machine / tables, us: 571 episodes of five nodes, 57 types, 736,000
+// events 505 / 736; 266 of three and four, 53 types, 1.06 million, two passes 834 / 1,102;
+// 320 of three, 38 types, 353,000 285 / 296; 746 of five to seven, 49 types, 911,000, two
+// passes 3,224 / 1,572; 167 of four, 18 types, 635,000, two passes 968 / 706; 1,756 of two
+// to four, 60 types, 79,000, two passes 538 / 391)
+bool few_on_long(const StreamDev &s, uint32_t m, uint32_t longest) {
+    return (uint64_t)m * longest < 5ull * s.K * s.K && (uint64_t)s.K * s.K > 400ull * longest &&
+           (uint64_t)s.n * s.K > 10000000;
+}
+
 // Count a candidate set over hit tables: all lengths, in an order of their own.  *done =
 // false, with nothing counted, where they do not apply.
 int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
@@ -1079,10 +1091,6 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
     RET(hits_plan(c, s, cands, gather, m, m >= PLAN_FINE, d_ivl, nI, pass, st, &pl, &ok,
                   [&](const char *n, size_t w, uint32_t **p) { return dbuf(c, n, w, p); }));
     if (!ok) return FEM_OK;
-    // short episodes, few of them for the stream's type pairs: the tables cost more than the
-    // per-thread machine's count (533 episodes of two and three nodes, 22 types, 360,000
-    // events: 0.66 against 0.61 ms for two passes; from four nodes on the tables were the
-    // faster at every size tried)
     uint32_t longest = 0;
     for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
         if (!pl.len_m[N]) continue;
@@ -1090,8 +1098,7 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
         // (a shape measured for the other kernels)
         if (c->tune.count(tune_key((int)N, pass, true, pl.len_m[N], s.n_chunks, s.K))) return FEM_OK;
     }
-    if (longest <= 3 && (uint64_t)m * longest < 5ull * s.K * s.K && (uint64_t)s.n * s.K > 4000000)
-        return FEM_OK;
+    if (few_on_long(s, m, longest)) return FEM_OK;
     uint32_t *tmp;
     uint8_t *redo;
     RET(dbuf(c, "hit_plan_out", m, &tmp));
@@ -1255,14 +1262,14 @@ int level_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
 // before / over tables, recounts included): 22 candidates, 64 types, 406,000 events 86 /
 // 131; 7,896 there 354 / 458 (the line is at 15,700); 44,544 there 3,316 / 1,304; 26,115 of 19 types, 64,000 events
 // 643 / 340; 6,729 of 22 types, 147,000 events 1,614 / 328; 20 of 18 types, 6,200 events
-// 340 / 127.  At level 2 (every type pair or most of them) the line is lower: 239 pairs of
-// 16 types, 4,000 events 290 / 96; 810 of 18, 6,200 events 155 / 112; 952 of 19, 64,000
-// events 155 / 146; 1,397 of 39, 101,000 events 95 / 172; 6,593 of 61, 179,000 events
-// 145 / 192.  With a segment count configured, level 2 keeps its kernels.
+// 340 / 127.  At level 2 (every type pair or most of them) the other kernels fill the device
+// from about 1,000 candidates on: 239 pairs of 16 types, 4,000 events 290 / 96; 810 of 18,
+// 6,200 events 155 / 112; 952 of 19, 64,000 events 155 / 146; 1,397 of 39, 101,000 events
+// 95 / 172; 3,435 of 40, 20,000 events 104 / 144; 6,593 of 61, 179,000 events 145 / 192.  With a segment count configured, level 2 keeps its kernels.
 bool level_by_hits(const fem_ctx *c, const StreamDev &s, uint32_t N, uint32_t m, uint32_t nI) {
     if (!hits_eligible(c, s, nI) || m == 0) return false;
     const double cells = (double)s.n * s.K;
-    if (N == 2) return !c->cfg.segments && cells <= 1.5e6;
+    if (N == 2) return !c->cfg.segments && m <= 1000 && cells <= 1.5e6;
     return 13 * cells <= 40e6 + (double)m * N * (double)s.n / s.K;
 }
 
@@ -1328,6 +1335,9 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
         RET(validate(c, s, cands, gather, m, nI, info, st));
         known = true;
         hits = hits && !info[1] && (!in_runs(info, m) || most_pairs(s, info, m, nI, pass));
+        uint32_t longest = FEM_MAX_LEN;
+        while (longest > 1 && !(info[0] >> longest & 1u)) --longest;
+        hits = hits && !few_on_long(s, m, longest);
     }
     if (hits) {
         bool done = false;
