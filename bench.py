@@ -64,7 +64,7 @@ def kernel_source_hash() -> str:
               "fem_count_exact.cu", "fem_count_exact_n12.cu", "fem_count_exact_n34.cu",
               "fem_count_exact_n56.cu", "fem_count_exact_n78.cu", "fem_chain.cuh",
               "fem_chain_launch.cuh", "fem_chain_relaxed.cu", "fem_chain_exact.cu",
-              "fem_pairs.cu"):
+              "fem_pairs.cu", "fem_hits.cuh", "fem_hits.cu"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     with open(os.path.join(csrc, "fem_internal.cuh"), "rb") as fh:

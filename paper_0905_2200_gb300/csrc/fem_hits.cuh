@@ -25,13 +25,13 @@
 // per-thread machine spends 60 to 150 issue slots on every event of every node, and the cost
 // of an episode hardly grows with its length: a node after one without admitted events is
 // passed over.  Measured (two-pass and single-pass counts, start of the change -> now): an
-// hour of 64 types at 50 Hz, 100,000 episodes of 3-5 nodes, 331 -> 169 ms; 20,011 episodes
-// of 2-8 nodes on 196,000 events, 5.97 -> 1.59 ms; a bursting recording 47.8 -> 8.6 ms (no
+// hour of 64 types at 50 Hz, 100,000 episodes of 3-5 nodes, 332 -> 147 ms; 20,011 episodes
+// of 2-8 nodes on 196,000 events, 6.02 -> 1.56 ms; a bursting recording 31.4 -> 7.3 ms (no
 // rings, and twice the entry classes in the first try); 100 episodes on 3,400 events, 0.95 ->
 // 0.26 ms (all lengths planned in one host wait).  What bounds it: in the count, warp issue
 // slots (41-54% used at 15 to 31 warps per SM, a third to a half of the lanes active: lanes
 // wait for the one with the most hits, so the candidates are ordered by their last three
-// intervals) and the latency of the tables' L2 reads; in the build, issue slots (80% used).
+// intervals) and the latency of the tables' L2 reads; in the build, issue slots (two thirds used).
 //
 // MapConcatenate (template flag MC): the entry classes and transfer tables are those of
 // the other counting kernels, so the same stitch composes them; segments are runs of
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(128) k_hit_count_batch(const CountParams *__re
 // above it.  A segment finds that end from the last-node events of the w before it (an
 // earlier one's range ends before its own ranges begin), and the segments' sums add up: no
 // stitch.  One thread per episode walked the whole stream before (fem_windows.cu), few warps
-// and long chains of loads: 16,128 pairs on 406,000 events 15.5 ms, now 0.10 ms and 0.52
+// and long chains of loads: 16,128 pairs on 406,000 events 15.5 ms, now 0.10 ms and 0.26
 // for the tables.
 template <int NMAX>
 __global__ void __launch_bounds__(128) k_hit_windows(const CountParams p, const uint32_t *order,
@@ -449,10 +449,10 @@ __global__ void __launch_bounds__(128) k_hit_windows(const CountParams p, const 
 //
 // What bounds it: issue slots, about 12 for 32 entries, and the lists' latency.  Measured on
 // the deep search of 64 types, 300 s (2.4 million candidates from 12,400 frequent pairs):
-// 2.4 ms
-// relaxed and 1.2 ms exact, after 0.6 ms for the tables and lists.  A thread for each
-// (a, v, b) that looked at every hit of (b, u, c) took 7.3 ms: one in five admits it.  The latest-chain kernel, which looks up every
-// last-node event of every candidate: 31.2 ms relaxed and 15.1 ms exact.
+// 2.4 ms relaxed and 1.2 ms exact, after 0.4 ms for the tables and lists.  A thread for each
+// (a, v, b) that looked at every hit of (b, u, c) took 7.3 ms: one in five admits it.  The
+// latest-chain kernel, which looks up every last-node event of every candidate: 31.2 ms
+// relaxed and 15.1 ms exact.
 constexpr uint32_t JOIN_QUEUE = 64;  // hits a warp takes at a time, at least a slab's 32
 
 __global__ void __launch_bounds__(256) k_join(const HitTables h, const JoinTables g, uint32_t n_events,
