@@ -1429,27 +1429,30 @@ void free_stream_buffers(StreamDev &s) {
 }
 
 // Buffers for a stream of up to ne events in nc chunks (offs per chunk), charged to
-// the context's budget as one block.
+// the context's budget as one block.  Where this fails, s holds no buffers and is
+// otherwise as it was.
 int alloc_stream(fem_ctx *c, StreamDev &s, size_t ne, size_t nc) {
     StreamDev q;
     q.cap_events = ne, q.cap_chunks = nc, q.cap_offs = (uint32_t)(nc * s.offs);
     q.t = reinterpret_cast<uint32_t *>(1);  // stream_bytes of the capacities
     const size_t bytes = stream_bytes(q);
     RET(reserve(c, bytes));
-    s.cap_events = ne, s.cap_chunks = nc, s.cap_offs = q.cap_offs;
-    const bool ok = cudaMalloc(&s.t, ne * 4) == cudaSuccess && cudaMalloc(&s.type, ne) == cudaSuccess &&
-                    cudaMalloc(&s.bev, nc * CHUNK * 8) == cudaSuccess &&
-                    cudaMalloc(&s.boff, nc * s.offs * 2) == cudaSuccess &&
-                    cudaMalloc(&s.cfirst, (nc + 1) * 4) == cudaSuccess &&
-                    cudaMalloc(&s.hist, 256 * 4) == cudaSuccess;
-    if (!ok) {
+    auto take = [&] {
+        q.t = nullptr;
+        if (cudaMalloc(&q.t, ne * 4) == cudaSuccess && cudaMalloc(&q.type, ne) == cudaSuccess &&
+            cudaMalloc(&q.bev, nc * CHUNK * 8) == cudaSuccess &&
+            cudaMalloc(&q.boff, nc * s.offs * 2) == cudaSuccess &&
+            cudaMalloc(&q.cfirst, (nc + 1) * 4) == cudaSuccess &&
+            cudaMalloc(&q.hist, 256 * 4) == cudaSuccess)
+            return true;
         cudaGetLastError();
-        const uint32_t offs = s.offs;
-        free_stream_buffers(s);
-        if (c->hits_busy || !release_hits(c)) return FEM_ENOMEM;
-        s.offs = offs;  // (the device is full: once more without the hit tables of earlier calls)
-        return alloc_stream(c, s, ne, nc);
-    }
+        free_stream_buffers(q);
+        return false;
+    };
+    // (the device is full: once more without the hit tables of earlier calls)
+    if (!take() && (c->hits_busy || !release_hits(c) || !take())) return FEM_ENOMEM;
+    s.t = q.t, s.type = q.type, s.bev = q.bev, s.boff = q.boff, s.cfirst = q.cfirst, s.hist = q.hist;
+    s.cap_events = ne, s.cap_chunks = nc, s.cap_offs = (uint32_t)(nc * s.offs);
     c->mem_used += bytes;
     return FEM_OK;
 }

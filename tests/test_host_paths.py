@@ -1,0 +1,65 @@
+"""Host code of the library where calls of the runtime fail: every fault is the fake
+runtime's (host_cuda.c), no GPU is needed."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_0905_2200_gb300 import fem
+from tests.host_cuda import PLAN_EDGES, PLAN_PARTS_MIN, PLAN_SLABS, Host
+
+vp = ctypes.c_void_p
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    return Host(str(tmp_path_factory.mktemp("host_cuda")))
+
+
+@pytest.fixture()
+def ctx(host):
+    host.plan = {2: 40, PLAN_EDGES: 50, PLAN_SLABS: 1, PLAN_PARTS_MIN: 1}  # 40 of three nodes
+    host.error = 0
+    c = vp()
+    assert host.lib.fem_create(ctypes.byref(c), 0, ctypes.c_size_t(0)) == 0
+    yield c
+    assert host.lib.fem_destroy(c) == 0
+
+
+def load(host, ctx, n, K):
+    """A stream of n events a millisecond apart; its id."""
+    ty = (np.arange(n) % K).astype(np.uint8)
+    t = (1000 * np.arange(n)).astype(np.uint32)
+    sid = ctypes.c_int32()
+    assert host.lib.fem_load_stream(ctx, ty.ctypes.data_as(vp), t.ctypes.data_as(vp), ctypes.c_uint64(n), K, 0,
+                                    None, ctypes.byref(sid)) == 0
+    return sid
+
+
+def count(host, ctx, sid, m=40, pass_=1, K=8):
+    """A count of m candidates of three nodes; the kernels that it launched."""
+    rec = fem.pack_episodes(np.full(m, 3), np.tile([0, 1, 2] + [0] * 5, (m, 1)), np.zeros((m, 7), int))
+    I = np.array([[0, 4000]], np.uint32)
+    out = np.zeros(m, np.uint32)
+    at = len(host.launches)
+    rc = host.lib.fem_count_candidates(ctx, sid, rec.ctypes.data_as(vp), m, 0, I.ctypes.data_as(vp), 1, pass_,
+                                       out.ctypes.data_as(vp), 0, None)
+    assert rc == 0
+    return host.launches[at:]
+
+
+@pytest.mark.parametrize("failing", [1, 2, 6])
+def test_stream_loaded_after_the_tables_made_room(host, ctx, failing):
+    """The device is full when a stream is loaded, and the hit tables of an earlier count are
+    given up for it: the stream is then the one that was asked for."""
+    sid = load(host, ctx, 4000, 8)
+    assert any("k_hit_count" in k for k in count(host, ctx, sid))
+    at = len(host.launches)
+    host.number("host_fail_malloc").value = failing  # of the stream's six allocations
+    other = load(host, ctx, 50000, 8)
+    assert host.number("host_fail_malloc").value == 0
+    assert any("k_bucket" in k for k in host.launches[at:])
+    counts = np.full(8, 7, np.uint32)
+    assert host.lib.fem_type_counts(ctx, other, counts.ctypes.data_as(vp)) == 0
+    assert (counts == 0).all()  # (of all eight types; the fake runtime counts none)
+    assert any("k_hit_count" in k for k in count(host, ctx, other))
