@@ -432,7 +432,10 @@ __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, ui
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         if (!((mask[u] >> r) & 1u)) continue;
-                        const uint32_t m = __popc(in[u]), last = k0 - __ffs(in[u]);
+                        // (denser than a word, the tables are not counted with, but read they
+                        // are: past 32 events the range is the latest one's)
+                        const uint32_t w = in[u] ? in[u] : 1u;
+                        const uint32_t m = __popc(w), last = k0 - __ffs(w);
                         b.range[to[u]++] = hit_pack(last + 1 - m, m, origin + rp[x * HIT_ROW + last]);
                     }
                 }
@@ -455,7 +458,8 @@ __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, ui
                     while (t - tx[k - 1] - f > wd) --k;  // (too near; the mask says that one is not)
                 const uint32_t last = k - 1;
                 for (; k > low && t - tx[k - 1] - f <= wd; --k) ++m;
-                b.range[o++] = hit_pack(k, m, origin + rp[x * HIT_ROW + last]);
+                m = min(m, 32u);  // (more only where denser than a word)
+                b.range[o++] = hit_pack(last + 1 - m, m, origin + rp[x * HIT_ROW + last]);
             }
         }
     }

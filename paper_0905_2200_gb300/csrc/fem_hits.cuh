@@ -56,8 +56,10 @@ constexpr uint32_t HIT_BUILD_T = 256;  // threads of a build block
 __host__ __device__ constexpr int hit_inner(int nmax) { return nmax > 2 ? nmax - 2 : 0; }
 __host__ __device__ constexpr int hit_shared(int nmax) { return nmax <= 5 ? hit_inner(nmax) : 2; }
 
-// The stored form of a hit: bits 0-5 the first event of the range, 6-11 their number, from
-// bit 16 on the low half of the latest one's index in the stream.
+// The stored form of a hit: bits 0-5 the first event of the range, 6-11 their number (1 to
+// 32; start + number at most 64), from bit 16 on the low half of the latest one's index in
+// the stream.  That holds for every stored hit, also on streams too dense for the tables:
+// the host learns of those only after the kernels that read them have run.
 __device__ __forceinline__ uint32_t hit_pack(uint32_t start, uint32_t len, uint32_t latest) {
     return latest << 16 | len << 6 | start;
 }

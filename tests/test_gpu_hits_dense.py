@@ -1,0 +1,80 @@
+"""Streams that are sparse on average and, in a burst, denser than the hit tables' words: the
+tables are built and read before their build is found out, and the other kernels then count.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0905_2200_gb300 import fem, synth
+from tests.gpu_common import assert_counts_equal, ctx_fixture, oracle_counts
+
+pytestmark = pytest.mark.gpu
+PASSES = (fem.PASS_RELAXED, fem.PASS_EXACT)
+K = 16
+I = np.array([[0, 5000], [0, 10000], [100, 12000], [15000, 40000]], np.uint32)
+
+
+def burst_stream(seed, n=3000, seconds=10.0, bursts=2, first_us=0):
+    """n events of K types over `seconds`; in each burst 100 of type 0, 400 us apart, one of type
+    1 every 2 ms among them, and 20 of type 1 after them: 30 of type 0 in 12 ms, 100 in 40 ms,
+    and the last 32 of them all less than 15 ms before the first type 1 that follows."""
+    rng = np.random.default_rng(seed)
+    ty, t = [rng.integers(0, K, n)], [rng.integers(0, int(seconds * 1e6), n)]
+    for k in range(bursts):
+        at = int(seconds * 1e6 * (k + 0.5) / bursts)
+        ty += [np.zeros(100, int), np.ones(20, int), np.ones(20, int)]
+        t += [at + 400 * np.arange(100), at + 1001 + 2000 * np.arange(20),
+              at + 400 * 99 + 50 + 100 * np.arange(20)]
+    ty, t = np.concatenate(ty), np.concatenate(t)
+    order = np.argsort(t, kind="stable")
+    return ty[order].astype(np.uint8), (t[order] + first_us).astype(np.uint32)
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = ctx_fixture()
+    yield c
+    fem.fem_destroy(c)
+
+
+def with_edge(cands, ivl):
+    """The set with the candidates (0, I[0], 1) to (0, I[ivl], 1) first: with all four a type 1
+    after a burst has more hits than the events of its slab."""
+    L, E, iv = (a.copy() for a in cands)
+    k = ivl + 1
+    L[:k], E[:k], E[:k, 1], iv[:k, 0] = 2, 0, 1, np.arange(k)
+    return L, E, iv
+
+
+@pytest.mark.parametrize("first_us", [0, 70000])
+def test_windows(ctx, first_us):
+    """With the edges of the shorter intervals the other kernel counts; with the longest one its
+    lists run over, which is an error as it is without tables."""
+    ty, t = burst_stream(1, first_us=first_us)
+    sid = fem.fem_load_stream(ctx, ty, t, K)
+    L, E, iv = synth.random_candidates(1, 300, K - 2, [2, 3], 3)
+    E = np.where(np.arange(E.shape[1]) < L[:, None], E + 2, 0)
+    for ivl in (2, 3):
+        cands = with_edge((L, E, iv), ivl)
+        rec = fem.pack_episodes(*cands)
+        if ivl == 3:
+            with pytest.raises(fem.FemError) as e:
+                fem.fem_count_windows(ctx, sid, rec, I, 30000)
+            assert e.value.status == -9
+        else:
+            assert_counts_equal(fem.fem_count_windows(ctx, sid, rec, I, 30000),
+                                oracle.count_windows_batch(ty, t, *cands, I, 30000), "windows")
+    fem.fem_free_stream(ctx, sid)
+
+
+@pytest.mark.parametrize("m", [200, 700])
+def test_counts(ctx, m):
+    ty, t = burst_stream(2)
+    sid = fem.fem_load_stream(ctx, ty, t, K)
+    cands = with_edge(synth.random_candidates(2, m, K, [2, 3, 4], 4), 3)
+    rec = fem.pack_episodes(*cands)
+    for p in PASSES:
+        want = oracle_counts(ty, t, *cands, I, p)
+        for call in range(3):
+            assert_counts_equal(fem.fem_count_candidates(ctx, sid, rec, I, p), want, f"pass {p} call {call}")
+    fem.fem_free_stream(ctx, sid)
