@@ -2676,8 +2676,17 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     CK(cudaMemGetInfo(&free_bytes, &total_bytes));
     const uint64_t most = std::min(total_bytes / 8, free_bytes / 2);
     // the jobs by stream
-    std::vector<uint32_t> job, off{0};
+    std::vector<uint32_t> job, off{0}, theta, iota, first{0}, part_off, part_group;
     std::vector<int32_t> streams;
+    std::vector<BatchOut> outs;
+    std::vector<CountParams> xp;
+    std::vector<std::vector<uint4>> lists;
+    // every upload goes in st's order, before the kernels that read it; what is uploaded
+    // (declared above, or the batch's) lives until st has taken it
+    struct Drain {
+        cudaStream_t st;
+        ~Drain() { cudaStreamSynchronize(st); }
+    } drain{st};
     for (uint32_t j = 0; j < b->jobs.size(); ++j)
         if (b->jobs[j].m && std::find(streams.begin(), streams.end(), b->jobs[j].stream_id) == streams.end())
             streams.push_back(b->jobs[j].stream_id);
@@ -2697,8 +2706,7 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     if (m == 0) return FEM_OK;
     h.m = (uint32_t)m, h.n_jobs = (uint32_t)job.size(), h.n_streams = (uint32_t)streams.size();
     RET(balloc(b, m, &h.cands));
-    std::vector<uint32_t> theta(h.n_jobs), iota(m);
-    std::vector<BatchOut> outs(h.n_jobs);
+    theta.resize(h.n_jobs), iota.resize(m), outs.resize(h.n_jobs);
     for (uint32_t k = 0; k < h.n_jobs; ++k) {
         const fem_job &jb = b->jobs[job[k]];
         CK(cudaMemcpyAsync(h.cands + off[k], jb.cands, (size_t)jb.m * sizeof(fem_episode),
@@ -2739,8 +2747,6 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     RET(balloc(b, m, &bin));
     RET(balloc(b, m, &rank));
     RET(balloc(b, m, &order));
-    std::vector<uint32_t> first{0}, part_off;
-    std::vector<uint32_t> part_group;
     uint64_t bytes = 0;
     h.capacity = 0;
     for (uint32_t k = 0; k < h.n_streams; ++k) {
@@ -2788,7 +2794,7 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     part_off.push_back(h.m);
     // segments: the same number of slabs for every item of a launch, for about four blocks
     // for each place on the GPU (the exact pass, with fewer candidates, four times as many)
-    std::vector<CountParams> xp = h.parts;
+    xp = h.parts;
     uint64_t tab = 0;
     for (int pass = 0; pass < 2; ++pass) {
         uint64_t t = 0;
@@ -2816,7 +2822,8 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
             l.n_list = (uint32_t)list.size(), l.n_items = items;
             if (list.empty()) continue;
             RET(balloc(b, list.size(), &l.list));
-            CK(cudaMemcpy(l.list, list.data(), list.size() * sizeof(uint4), cudaMemcpyHostToDevice));
+            CK(cudaMemcpyAsync(l.list, list.data(), list.size() * sizeof(uint4), cudaMemcpyHostToDevice, st));
+            lists.push_back(std::move(list));
         }
         tab = std::max(tab, t);
     }
@@ -2834,17 +2841,17 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     RET(balloc(b, h.n_parts, &h.rparts));
     RET(balloc(b, h.n_parts, &h.xparts));
     RET(balloc(b, part_off.size(), &h.part_off));
-    CK(cudaMemcpy(h.first, first.data(), first.size() * 4, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(h.part_off, part_off.data(), part_off.size() * 4, cudaMemcpyHostToDevice));
+    CK(cudaMemcpyAsync(h.first, first.data(), first.size() * 4, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(h.part_off, part_off.data(), part_off.size() * 4, cudaMemcpyHostToDevice, st));
     // one run, in which the ranges may turn out to be more than estimated
     for (int attempt = 0; attempt < 2; ++attempt) {
         uint32_t *range;
         RET(balloc(b, h.capacity, &range));
         for (HitBuild &hb : h.build) hb.range = range, hb.capacity = h.capacity;
         for (uint32_t q = 0; q < h.n_parts; ++q) h.parts[q].hits.range = xp[q].hits.range = range;
-        CK(cudaMemcpy(h.d_build, h.build.data(), h.n_streams * sizeof(HitBuild), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(h.rparts, h.parts.data(), h.n_parts * sizeof(CountParams), cudaMemcpyHostToDevice));
-        CK(cudaMemcpy(h.xparts, xp.data(), h.n_parts * sizeof(CountParams), cudaMemcpyHostToDevice));
+        CK(cudaMemcpyAsync(h.d_build, h.build.data(), h.n_streams * sizeof(HitBuild), cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(h.rparts, h.parts.data(), h.n_parts * sizeof(CountParams), cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(h.xparts, xp.data(), h.n_parts * sizeof(CountParams), cudaMemcpyHostToDevice, st));
         CK(cudaMemsetAsync(c->d_err, 0, 4, st));
         RET(batch_enqueue_hits(c, h, st));
         unsigned long long used[2];

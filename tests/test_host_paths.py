@@ -63,3 +63,36 @@ def test_stream_loaded_after_the_tables_made_room(host, ctx, failing):
     assert host.lib.fem_type_counts(ctx, other, counts.ctypes.data_as(vp)) == 0
     assert (counts == 0).all()  # (of all eight types; the fake runtime counts none)
     assert any("k_hit_count" in k for k in count(host, ctx, other))
+
+
+class Job(ctypes.Structure):
+    _fields_ = fem.fem_job._fields_
+
+
+def batch_jobs(sids, m=40):
+    """One job of m candidates of three nodes per stream; the array and what it points to."""
+    rec = fem.pack_episodes(np.full(m, 3), np.tile([0, 1, 2] + [0] * 5, (m, 1)), np.zeros((m, 7), int))
+    out, kept = np.zeros((len(sids), m), np.uint32), np.zeros((len(sids), m), np.uint8)
+    jobs = (Job * len(sids))()
+    for k, sid in enumerate(sids):
+        jobs[k] = Job(sid.value, 3, m, rec.ctypes.data, 1, out[k].ctypes.data, kept[k].ctypes.data)
+    return jobs, (rec, out, kept)
+
+
+def create_batch(host, ctx, jobs):
+    I = np.array([[0, 4000]], np.uint32)
+    b = vp()
+    assert host.lib.fem_batch_create(ctx, jobs, len(jobs), I.ctypes.data_as(vp), 1, None, ctypes.byref(b)) == 0
+    return b
+
+
+def test_batch_uploads_in_its_streams_order(host, ctx):
+    """What the kernels of a batch read is uploaded on their stream: a plain copy from pageable
+    memory goes over the default stream, which a stream of the context's kind does not wait for."""
+    jobs, kept = batch_jobs([load(host, ctx, 4000, 8), load(host, ctx, 5000, 8)])
+    plain = host.number("host_plain_uploads", ctypes.c_uint64)
+    at, before = len(host.launches), plain.value
+    b = create_batch(host, ctx, jobs)
+    assert any("k_hit_count_batch" in k for k in host.launches[at:])
+    assert plain.value == before
+    assert host.lib.fem_batch_destroy(b) == 0
