@@ -729,12 +729,13 @@ cudaError_t launch_join(const HitTables &h, const JoinTables &g, const uint32_t 
         err = cudaFuncSetAttribute(k_join, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
     });
     if (err != cudaSuccess) return err;
+    cudaError_t e;
     const uint32_t slots = K * n_ivl, units = h.n_slabs * K;
     k_join_index<<<K, 256, 0, st>>>(h, g, hist, K, n_ivl);
     note_launch();
     k_join_list<false><<<(units + 7) / 8, 256, 0, st>>>(h, g, K, slots, len);
     note_launch();
-    if ((err = launch_exclusive_scan(len, n, g.off, g.off + n, scratch, st)) != cudaSuccess) return err;
+    if ((e = launch_exclusive_scan(len, n, g.off, g.off + n, scratch, st)) != cudaSuccess) return e;
     k_join_list<true><<<(units + 7) / 8, 256, 0, st>>>(h, g, K, slots, nullptr);
     note_launch();
     // blocks of up to eight warps in about 48 KB

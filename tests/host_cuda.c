@@ -13,7 +13,7 @@ enum { OK = 0, NO_MEMORY = 2, LAUNCH_FAILED = 719 };
 /* what a test sets and reads */
 void (*host_on_launch)(const char *name, void **args) = 0;
 int host_fail_malloc = 0;  /* fail the allocation so many calls ahead (1: the next) */
-int host_fail_launch = 0;  /* report this many launches to come as failed */
+int host_fail_launch = 0;  /* the same of launches (cudaGetLastError tells) */
 int host_device = 0, host_devices = 1;
 uint64_t host_mallocs = 0, host_attributes = 0, host_stream_uploads = 0, host_plain_uploads = 0;
 size_t host_bytes = 0;     /* device memory held */
@@ -51,7 +51,7 @@ int __cudaPopCallConfiguration(dim3_ *g, dim3_ *b, size_t *smem, void **st) {
 int __cudaGetKernel(const void **k, const void *stub) { return *k = stub, OK; }
 int __cudaLaunchKernel(const void *k, dim3_ g, dim3_ b, void **args, size_t smem, void *st) {
     (void)g, (void)b, (void)smem, (void)st;
-    if (host_fail_launch > 0) return --host_fail_launch, last_error = LAUNCH_FAILED;
+    if (host_fail_launch > 0 && --host_fail_launch == 0) return last_error = LAUNCH_FAILED;
     if (host_on_launch) host_on_launch(name_of(k), args);
     return OK;
 }

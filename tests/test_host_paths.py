@@ -96,3 +96,25 @@ def test_batch_uploads_in_its_streams_order(host, ctx):
     assert any("k_hit_count_batch" in k for k in host.launches[at:])
     assert plain.value == before
     assert host.lib.fem_batch_destroy(b) == 0
+
+
+def join(host):
+    """The launches of a level-3 join over one slab of 4 types; the status."""
+    fn = getattr(host.lib, "_ZN3fem11launch_joinERKNS_9HitTablesERKNS_10JoinTablesEPKjjjjPjS8_S8_P11CUstream_st")
+    h, g = (ctypes.c_uint32 * 64)(), (ctypes.c_uint32 * 64)()
+    ctypes.c_uint32.from_buffer(h, 64).value = 1  # n_slabs
+    words = (ctypes.c_uint32 * 4096)()
+    for k in range(0, 64, 2):
+        ctypes.c_uint64.from_buffer(g, 4 * k).value = ctypes.addressof(words)
+    return fn(h, g, words, 100, 4, 1, words, words, words, None)
+
+
+@pytest.mark.parametrize("failing", [1, 2, 3, 4, 5])
+def test_a_failed_join_is_not_remembered(host, failing):
+    """One of a join's launches (the third is its lists' scan) fails once: that call says so,
+    the next one runs."""
+    assert join(host) == 0
+    host.number("host_fail_launch").value = failing
+    assert join(host) == 719
+    assert host.number("host_fail_launch").value == 0
+    assert join(host) == 0
