@@ -2,7 +2,6 @@
 // instantiated per pass in fem_chain_relaxed.cu and fem_chain_exact.cu.
 #pragma once
 
-#include <mutex>
 
 #include "fem_chain.cuh"
 
@@ -11,13 +10,9 @@ namespace chain_detail {
 
 template <int N, int PASS, bool MC>
 cudaError_t run(const CountParams &p, uint32_t threads, cudaStream_t st) {
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(k_chain<N, PASS, MC>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    });
-    if (attr_err != cudaSuccess) return attr_err;
+    static std::atomic<uint64_t> set;
+    const cudaError_t e = smem_limit(set, (const void *)k_chain<N, PASS, MC>, 227 * 1024);
+    if (e != cudaSuccess) return e;
     if (threads < 32 || threads > 256 || threads % 32) return cudaErrorInvalidConfiguration;
     const size_t sm = 2 * (size_t)stage_bytes(p.offs) + 128 + ChainLayout<N, MC>::bytes(threads);
     if (sm > 227 * 1024) return cudaErrorInvalidConfiguration;

@@ -4,7 +4,6 @@
 #pragma once
 
 #include <algorithm>
-#include <mutex>
 #include <type_traits>
 
 #include "fem_count.cuh"
@@ -23,13 +22,9 @@ struct BatchArgs {
 
 template <int N, int PASS, bool MC, int R>
 cudaError_t run_batch(const BatchArgs &a, uint32_t threads, int sm_count, cudaStream_t st) {
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(count_batch_kernel<N, PASS, MC, R>(),
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    });
-    if (attr_err != cudaSuccess) return attr_err;
+    static std::atomic<uint64_t> set;
+    const cudaError_t e = smem_limit(set, (const void *)count_batch_kernel<N, PASS, MC, R>(), 200 * 1024);
+    if (e != cudaSuccess) return e;
     size_t sm = 2 * (size_t)a.SB + 128 + (N >= 3 ? (size_t)S_MAX * threads * 4u : 0);  // keys
     if (PASS == FEM_PASS_EXACT && N > 1) sm += (size_t)(N - 1) * R * threads * 8u;
     if (sm > 200 * 1024) return cudaErrorInvalidConfiguration;
@@ -64,13 +59,9 @@ cudaError_t run_batch_r(uint32_t R, const BatchArgs &a, uint32_t threads, int sm
 
 template <int N, int PASS, bool MC, int R, int SMX = S_MAX>
 cudaError_t run(const CountParams &p, uint32_t threads, cudaStream_t st) {
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(count_kernel<N, PASS, MC, R, SMX>(),
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    });
-    if (attr_err != cudaSuccess) return attr_err;
+    static std::atomic<uint64_t> set;
+    const cudaError_t e = smem_limit(set, (const void *)count_kernel<N, PASS, MC, R, SMX>(), 227 * 1024);
+    if (e != cudaSuccess) return e;
     const size_t sm = count_smem_bytes(N, PASS, MC, R, threads, p.offs, SMX);
     if (sm > 227 * 1024) return cudaErrorInvalidConfiguration;
     dim3 grid((p.m + threads - 1) / threads, p.P);

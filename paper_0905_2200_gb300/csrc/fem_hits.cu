@@ -2,7 +2,6 @@
 // kernels that read them, and the plan both need: the candidates checked and ordered, the
 // edges they use numbered, the stream cut into slabs.
 #include <algorithm>
-#include <mutex>
 
 #include "fem_hits.cuh"
 
@@ -488,21 +487,9 @@ __global__ void __launch_bounds__(HIT_BUILD_T) k_hit_build_batch(const HitBuild 
     hit_build_slab<PASS>(b, blockIdx.x - first[lo], 0, 1);
 }
 
+constexpr int kBuildSmem = 224 * 1024;
 size_t build_smem(const HitBuild &b) {
     return (size_t)b.K * (HIT_ROW * 6 + (b.max_words | 1u) * 5 + 4) + 32;
-}
-
-cudaError_t build_limits() {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        for (const void *k : {(const void *)k_hit_build<FEM_PASS_RELAXED>, (const void *)k_hit_build<FEM_PASS_EXACT>,
-                              (const void *)k_hit_build_batch<FEM_PASS_RELAXED>,
-                              (const void *)k_hit_build_batch<FEM_PASS_EXACT>})
-            if (err == cudaSuccess)
-                err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
-    });
-    return err;
 }
 
 // Launch kernel `k` over p.m candidates in blocks of 128.
@@ -522,12 +509,9 @@ cudaError_t run_batch(const CountParams *parts, const uint4 *list, uint32_t n_li
                       cudaStream_t st) {
     constexpr uint32_t T = 128;
     constexpr int sm = hit_shared(NMAX) * 64 * (int)T * 2;
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        err = cudaFuncSetAttribute(k_hit_count_batch<NMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    });
-    if (err != cudaSuccess) return err;
+    static std::atomic<uint64_t> set;
+    const cudaError_t e = smem_limit(set, (const void *)k_hit_count_batch<NMAX>, sm);
+    if (e != cudaSuccess) return e;
     k_hit_count_batch<NMAX><<<n_items, T, sm, st>>>(parts, list, n_list);
     note_launch();
     return cudaGetLastError();
@@ -653,16 +637,17 @@ cudaError_t launch_publish_count(const unsigned long long *src, Publish pub, cud
 cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
                              cudaStream_t st) {
     if (n_slabs == 0) return cudaSuccess;
-    const cudaError_t e = build_limits();
-    if (e != cudaSuccess) return e;
     const size_t sm = build_smem(b);
-    if (sm > 224 * 1024) return cudaErrorInvalidConfiguration;
+    if (sm > kBuildSmem) return cudaErrorInvalidConfiguration;
+    static std::atomic<uint64_t> set[2];
+    const auto kernel = pass == FEM_PASS_RELAXED ? k_hit_build<FEM_PASS_RELAXED> : k_hit_build<FEM_PASS_EXACT>;
+    const cudaError_t e = smem_limit(set[pass == FEM_PASS_RELAXED], (const void *)kernel, kBuildSmem);
+    if (e != cudaSuccess) return e;
     // a few slabs: their types shared among several blocks, for about four per SM
     constexpr uint32_t NW = HIT_BUILD_T / 32;
     uint32_t split = 1;
     while (split < 8 && split * NW < b.K * ((b.K + 31) / 32) && split * n_slabs < 4 * (uint32_t)sm_count) split *= 2;
-    (pass == FEM_PASS_RELAXED ? k_hit_build<FEM_PASS_RELAXED>
-                              : k_hit_build<FEM_PASS_EXACT>)<<<dim3(n_slabs, split), HIT_BUILD_T, sm, st>>>(b);
+    kernel<<<dim3(n_slabs, split), HIT_BUILD_T, sm, st>>>(b);
     note_launch();
     return cudaGetLastError();
 }
@@ -671,14 +656,15 @@ cudaError_t launch_hit_build_batch(int pass, const HitBuild *host, const HitBuil
                                    const uint32_t *first, uint32_t n_streams, uint32_t n_slabs,
                                    cudaStream_t st) {
     if (n_slabs == 0) return cudaSuccess;
-    const cudaError_t e = build_limits();
-    if (e != cudaSuccess) return e;
     size_t sm = 0;
     for (uint32_t j = 0; j < n_streams; ++j) sm = std::max(sm, build_smem(host[j]));
-    if (sm > 224 * 1024) return cudaErrorInvalidConfiguration;
-    (pass == FEM_PASS_RELAXED
-         ? k_hit_build_batch<FEM_PASS_RELAXED>
-         : k_hit_build_batch<FEM_PASS_EXACT>)<<<n_slabs, HIT_BUILD_T, sm, st>>>(streams, first, n_streams);
+    if (sm > kBuildSmem) return cudaErrorInvalidConfiguration;
+    static std::atomic<uint64_t> set[2];
+    const auto kernel =
+        pass == FEM_PASS_RELAXED ? k_hit_build_batch<FEM_PASS_RELAXED> : k_hit_build_batch<FEM_PASS_EXACT>;
+    const cudaError_t e = smem_limit(set[pass == FEM_PASS_RELAXED], (const void *)kernel, kBuildSmem);
+    if (e != cudaSuccess) return e;
+    kernel<<<n_slabs, HIT_BUILD_T, sm, st>>>(streams, first, n_streams);
     note_launch();
     return cudaGetLastError();
 }
@@ -723,13 +709,9 @@ size_t join_smem(uint32_t slots) { return JOIN_QUEUE * sizeof(uint4) + (size_t)s
 
 cudaError_t launch_join(const HitTables &h, const JoinTables &g, const uint32_t *hist, uint32_t n, uint32_t K,
                         uint32_t n_ivl, uint32_t *len, uint32_t *scratch, uint32_t *out, cudaStream_t st) {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        err = cudaFuncSetAttribute(k_join, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
-    });
-    if (err != cudaSuccess) return err;
-    cudaError_t e;
+    static std::atomic<uint64_t> set;
+    cudaError_t e = smem_limit(set, (const void *)k_join, 224 * 1024);
+    if (e != cudaSuccess) return e;
     const uint32_t slots = K * n_ivl, units = h.n_slabs * K;
     k_join_index<<<K, 256, 0, st>>>(h, g, hist, K, n_ivl);
     note_launch();

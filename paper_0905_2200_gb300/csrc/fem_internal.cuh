@@ -13,6 +13,7 @@
 // (TMA) copy; each thread then walks only the groups of its episode's types.
 #pragma once
 
+#include <atomic>
 #include <string>
 
 #include <cuda_runtime.h>
@@ -253,6 +254,18 @@ cudaError_t launch_mark_flagged(const uint8_t *slot_flags, const uint32_t *idx, 
 cudaError_t launch_clear_at(const uint32_t *idx, uint32_t m, uint32_t *out, uint8_t *flags, cudaStream_t st);
 cudaError_t launch_compose_dev(const uint32_t *outer, const uint32_t *inner, const uint32_t *m_dev,
                                uint32_t m_max, uint32_t *dst, cudaStream_t st);
+// A kernel's limit of dynamic shared memory, set on the current device (where it holds for
+// this device only) unless `set`, the kernel's own, has the device's bit.
+inline cudaError_t smem_limit(std::atomic<uint64_t> &set, const void *kernel, int bytes) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+    if (set.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) set.fetch_or(bit, std::memory_order_release);
+    return e;
+}
 int fem_ctx_device(const fem_ctx *c);
 int fem_ctx_sms(const fem_ctx *c);
 // fem_count.cu

@@ -305,17 +305,10 @@ cudaError_t launch_pairs_relaxed(const CountParams &p, uint32_t threads, cudaStr
     if (threads < 32 || threads > 256 || threads % 32) return cudaErrorInvalidConfiguration;
     const bool mc = p.P > 1;
     const size_t sm = pairs_smem_bytes(mc, threads, p.offs);
-    static bool attr_set[2] = {false, false};
-    if (!attr_set[mc]) {
-        const cudaError_t e = mc ? cudaFuncSetAttribute(k_pairs_relaxed<true>,
-                                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        227 * 1024)
-                                 : cudaFuncSetAttribute(k_pairs_relaxed<false>,
-                                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                        227 * 1024);
-        if (e != cudaSuccess) return e;
-        attr_set[mc] = true;
-    }
+    static std::atomic<uint64_t> set[2];
+    const cudaError_t e = smem_limit(
+        set[mc], mc ? (const void *)k_pairs_relaxed<true> : (const void *)k_pairs_relaxed<false>, 227 * 1024);
+    if (e != cudaSuccess) return e;
     const uint32_t n_pairs = p.pair_types * (p.pair_types - 1);
     dim3 grid((n_pairs + threads - 1) / threads, mc ? p.P : 1);
     if (mc) k_pairs_relaxed<true><<<grid, threads, sm, st>>>(p);

@@ -118,3 +118,28 @@ def test_a_failed_join_is_not_remembered(host, failing):
     assert join(host) == 719
     assert host.number("host_fail_launch").value == 0
     assert join(host) == 0
+
+
+def test_shared_memory_limits_on_each_device(host):
+    """A kernel's limit holds on the device that it was set on: the first launch on another
+    device sets it there too, the second does not."""
+    attributes = host.number("host_attributes", ctypes.c_uint64)
+    host.number("host_devices").value = 2
+
+    def work(device):
+        before, c = attributes.value, vp()
+        assert host.lib.fem_create(ctypes.byref(c), device, ctypes.c_size_t(0)) == 0
+        jobs, kept = batch_jobs([load(host, c, 4000, 8)])
+        assert host.lib.fem_batch_destroy(create_batch(host, c, jobs)) == 0
+        assert join(host) == 0
+        assert host.lib.fem_destroy(c) == 0
+        return attributes.value - before
+
+    try:
+        work(0)
+        assert work(0) == 0
+        assert work(1) >= 4  # two builds, a batch's count, the join
+        assert work(1) == 0
+    finally:
+        host.number("host_devices").value = 1
+        host.rt.cudaSetDevice(0)
