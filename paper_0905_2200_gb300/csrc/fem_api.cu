@@ -2499,6 +2499,8 @@ struct BatchHits {
     BatchOut *outs = nullptr;
     uint32_t *r = nullptr, *x = nullptr, *idx = nullptr, *gx = nullptr, *scratch = nullptr, *n_idx = nullptr;
     uint8_t *flags = nullptr, *redo = nullptr, *xredo = nullptr;
+    std::vector<uint32_t> job;              // the batch's job of each job here
+    uint8_t *marks = nullptr;               // per job: to be recounted
     unsigned long long *used = nullptr;     // hits found by either pass
     uint64_t capacity = 0;
 };
@@ -2676,7 +2678,7 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     CK(cudaMemGetInfo(&free_bytes, &total_bytes));
     const uint64_t most = std::min(total_bytes / 8, free_bytes / 2);
     // the jobs by stream
-    std::vector<uint32_t> job, off{0}, theta, iota, first{0}, part_off, part_group;
+    std::vector<uint32_t> &job = h.job, off{0}, theta, iota, first{0}, part_off, part_group;
     std::vector<int32_t> streams;
     std::vector<BatchOut> outs;
     std::vector<CountParams> xp;
@@ -2738,6 +2740,7 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     RET(balloc(b, m, &h.redo));
     RET(balloc(b, m, &h.xredo));
     RET(balloc(b, 2, &h.used));
+    RET(balloc(b, h.n_jobs, &h.marks));
     CK(cudaMemcpyAsync(d_iota, iota.data(), m * 4, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(h.cand_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(h.theta, theta.data(), theta.size() * 4, cudaMemcpyHostToDevice, st));
@@ -3086,13 +3089,22 @@ int fem_batch_run(fem_batch *b, void *cuda_stream) {
     RET(read_err(c, st, &e));
     RET(err_status(e));
     if (!(e & (ERR_CAP | ERR_DENSE))) return FEM_OK;
-    if (b->over_hits) {  // (more than 32 entry classes: seldom) every job on its own
+    if (b->over_hits) {  // (more than 32 entry classes: seldom) the jobs with such candidates
+        BatchHits &h = b->hits;
         std::vector<fem_interval> I(b->nI);
+        std::vector<uint8_t> marks(h.n_jobs);
         if (b->nI) CK(cudaMemcpy(I.data(), b->ivl, b->nI * sizeof(uint2), cudaMemcpyDeviceToHost));
-        for (const fem_job &jb : b->jobs)
-            if (jb.m)
-                RET(fem_count_two_pass(c, jb.stream_id, jb.cands, jb.m, 1, I.data(), b->nI, jb.theta,
-                                       jb.exact_out, jb.survived_out, 1, st));
+        CK(cudaMemsetAsync(h.marks, 0, h.n_jobs, st));
+        CK(launch_batch_flagged_jobs(h.redo, h.xredo, h.record, h.idx, h.n_idx, h.m, h.part_off, h.n_parts,
+                                     h.cand_off, h.n_jobs, h.marks, st));
+        CK(cudaMemcpyAsync(marks.data(), h.marks, h.n_jobs, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        for (uint32_t k = 0; k < h.n_jobs; ++k) {
+            if (!marks[k] && !(e & ERR_DENSE)) continue;
+            const fem_job &jb = b->jobs[h.job[k]];
+            RET(fem_count_two_pass(c, jb.stream_id, jb.cands, jb.m, 1, I.data(), b->nI, jb.theta,
+                                   jb.exact_out, jb.survived_out, 1, st));
+        }
         return FEM_OK;
     }
     // A capacity guard tripped somewhere: recount the affected jobs one at a time

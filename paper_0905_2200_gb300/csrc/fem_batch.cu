@@ -177,6 +177,34 @@ cudaError_t launch_batch_exact_jobs(CountParams *xjobs, const uint32_t *cand_off
     return cudaGetLastError();
 }
 
+// marks[j] = 1 for every job j with a candidate that either pass flagged: the first by slot,
+// the second by survivor i of its part (the survivors idx are slots, ascending)
+__global__ void k_batch_flagged_jobs(const uint8_t *__restrict__ redo, const uint8_t *__restrict__ xredo,
+                                     const uint32_t *__restrict__ record, const uint32_t *__restrict__ idx,
+                                     const uint32_t *__restrict__ n_idx, uint32_t m,
+                                     const uint32_t *__restrict__ part_off, uint32_t n_parts,
+                                     const uint32_t *__restrict__ cand_off, uint32_t n_jobs,
+                                     uint8_t *__restrict__ marks) {
+    const uint32_t cnt = *n_idx;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
+        if (redo[i]) marks[find_job(cand_off, n_jobs, record[i])] = 1;
+        if (i >= cnt) continue;
+        const uint32_t slot = idx[i], off = part_off[find_job(part_off, n_parts, slot)];
+        if (xredo[off + i - lower_bound_u32(idx, cnt, off)]) marks[find_job(cand_off, n_jobs, record[slot])] = 1;
+    }
+}
+
+cudaError_t launch_batch_flagged_jobs(const uint8_t *redo, const uint8_t *xredo, const uint32_t *record,
+                                      const uint32_t *idx, const uint32_t *n_idx, uint32_t m,
+                                      const uint32_t *part_off, uint32_t n_parts, const uint32_t *cand_off,
+                                      uint32_t n_jobs, uint8_t *marks, cudaStream_t st) {
+    if (m == 0) return cudaSuccess;
+    k_batch_flagged_jobs<<<(uint32_t)std::min<uint64_t>((m + 255) / 256, 4096), 256, 0, st>>>(
+        redo, xredo, record, idx, n_idx, m, part_off, n_parts, cand_off, n_jobs, marks);
+    note_launch();
+    return cudaGetLastError();
+}
+
 // Zero every job's outputs, then write the exact count and survived flag of each
 // survivor (idx ascending, ex in the same order).
 __global__ void k_batch_zero_out(const BatchOut *__restrict__ outs,

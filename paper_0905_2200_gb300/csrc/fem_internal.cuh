@@ -465,6 +465,11 @@ cudaError_t launch_batch_keep_flags(const uint32_t *rel, const uint32_t *cand_of
 cudaError_t launch_batch_exact_jobs(CountParams *xjobs, const uint32_t *cand_off, uint32_t n_jobs,
                                     const uint32_t *idx, const uint32_t *n_idx, uint32_t *ex,
                                     cudaStream_t st, const uint32_t *gather = nullptr);
+// marks[j] (zeroed) = 1 for every job with a candidate that either pass flagged
+cudaError_t launch_batch_flagged_jobs(const uint8_t *redo, const uint8_t *xredo, const uint32_t *record,
+                                      const uint32_t *idx, const uint32_t *n_idx, uint32_t m,
+                                      const uint32_t *part_off, uint32_t n_parts, const uint32_t *cand_off,
+                                      uint32_t n_jobs, uint8_t *marks, cudaStream_t st);
 cudaError_t launch_batch_outputs(const BatchOut *outs, const uint32_t *cand_off, uint32_t n_jobs,
                                  uint32_t m, const uint32_t *idx, const uint32_t *n_idx,
                                  const uint32_t *ex, cudaStream_t st);
