@@ -2708,7 +2708,7 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     if (m == 0) return FEM_OK;
     h.m = (uint32_t)m, h.n_jobs = (uint32_t)job.size(), h.n_streams = (uint32_t)streams.size();
     RET(balloc(b, m, &h.cands));
-    theta.resize(h.n_jobs), iota.resize(m), outs.resize(h.n_jobs);
+    theta.resize(h.n_jobs), outs.resize(h.n_jobs);
     for (uint32_t k = 0; k < h.n_jobs; ++k) {
         const fem_job &jb = b->jobs[job[k]];
         CK(cudaMemcpyAsync(h.cands + off[k], jb.cands, (size_t)jb.m * sizeof(fem_episode),
@@ -2716,16 +2716,27 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
         theta[k] = jb.theta;
         outs[k] = BatchOut{jb.exact_out, jb.survived_out};
     }
-    // every candidate has its job's length (the counting kernels take any)
-    std::vector<fem_episode> host(m);
-    CK(cudaMemcpyAsync(host.data(), h.cands, m * sizeof(fem_episode), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    for (uint32_t k = 0; k < h.n_jobs; ++k)
-        for (uint32_t i = off[k]; i < off[k + 1]; ++i)
-            if (host[i].len != b->jobs[job[k]].len) return FEM_EINVAL;
-    for (uint32_t i = 0; i < m; ++i) iota[i] = i;
+    // every candidate has its job's length (the counting kernels take any); in pieces, whatever
+    // the batch's size is on the host
     uint32_t *d_iota;
     RET(balloc(b, m, &d_iota));
+    {
+        constexpr uint32_t PIECE = 1u << 16;
+        std::vector<fem_episode> host(std::min<uint64_t>(m, PIECE));
+        iota.resize(host.size());
+        uint32_t k = 0;
+        for (uint32_t i0 = 0; i0 < m; i0 += PIECE) {
+            const uint32_t n = std::min<uint32_t>(PIECE, (uint32_t)m - i0);
+            CK(cudaMemcpyAsync(host.data(), h.cands + i0, n * sizeof(fem_episode), cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            for (uint32_t i = 0; i < n; ++i) {
+                while (i0 + i >= off[k + 1]) ++k;
+                if (host[i].len != b->jobs[job[k]].len) return FEM_EINVAL;
+                iota[i] = i0 + i;
+            }
+            CK(cudaMemcpyAsync(d_iota + i0, iota.data(), n * 4, cudaMemcpyHostToDevice, st));
+        }
+    }
     RET(balloc(b, m, &h.record));
     RET(balloc(b, h.n_jobs + 1, &h.cand_off));
     RET(balloc(b, h.n_jobs, &h.theta));
@@ -2741,7 +2752,6 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     RET(balloc(b, m, &h.xredo));
     RET(balloc(b, 2, &h.used));
     RET(balloc(b, h.n_jobs, &h.marks));
-    CK(cudaMemcpyAsync(d_iota, iota.data(), m * 4, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(h.cand_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(h.theta, theta.data(), theta.size() * 4, cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(h.outs, outs.data(), outs.size() * sizeof(BatchOut), cudaMemcpyHostToDevice, st));

@@ -15,10 +15,16 @@ void (*host_on_launch)(const char *name, void **args) = 0;
 int host_fail_malloc = 0;  /* fail the allocation so many calls ahead (1: the next) */
 int host_fail_launch = 0;  /* the same of launches (cudaGetLastError tells) */
 int host_device = 0, host_devices = 1;
+size_t host_new_max = 0;   /* the largest piece of host memory that the library took by `new` */
 uint64_t host_mallocs = 0, host_attributes = 0, host_stream_uploads = 0, host_plain_uploads = 0;
 size_t host_bytes = 0;     /* device memory held */
 size_t host_total = (size_t)256 << 30;
 static int last_error = OK;
+
+void *__wrap__Znwm(size_t n) {
+    if (n > host_new_max) host_new_max = n;
+    return malloc(n ? n : 1);
+}
 
 /* kernels by the address of their stub */
 static struct { const void *stub; const char *name; } fn[8192];

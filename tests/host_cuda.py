@@ -29,7 +29,8 @@ def link(tmp):
         pytest.skip("the build's objects are not kept here")
     rt, lib = os.path.join(tmp, "libhostcuda.so"), os.path.join(tmp, "libfem_host.so")
     subprocess.check_call(["gcc", "-shared", "-fPIC", "-O1", "-o", rt, os.path.join(HERE, "host_cuda.c")])
-    subprocess.check_call(["g++", "-shared", "-o", lib] + objs + [rt, f"-Wl,-rpath,{tmp}"])
+    subprocess.check_call(["g++", "-shared", "-o", lib] + objs +
+                          [rt, f"-Wl,-rpath,{tmp}", "-Wl,--wrap=_Znwm"])
     return lib, rt
 
 

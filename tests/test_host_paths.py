@@ -143,3 +143,22 @@ def test_shared_memory_limits_on_each_device(host):
     finally:
         host.number("host_devices").value = 1
         host.rt.cudaSetDevice(0)
+
+
+@pytest.mark.parametrize("m", [300000, 65536, 65537])
+def test_batch_of_many_candidates_on_the_host(host, ctx, m):
+    """Creating a batch takes little host memory whatever the number of its candidates (none of
+    it can be refused across the C boundary), and every candidate's length is looked at."""
+    host.plan[2] = m
+    sid = load(host, ctx, 4000, 8)
+    jobs, kept = batch_jobs([sid, sid], m)
+    taken = host.number("host_new_max", ctypes.c_size_t)
+    taken.value = 0
+    b = create_batch(host, ctx, jobs)
+    assert 0 < taken.value <= 2 << 20
+    assert host.lib.fem_batch_destroy(b) == 0
+    for at in (0, 65535, m - 1):
+        kept[0][at, 15] = 2
+        I = np.array([[0, 4000]], np.uint32)
+        assert host.lib.fem_batch_create(ctx, jobs, 2, I.ctypes.data_as(vp), 1, None, ctypes.byref(vp())) == -1
+        kept[0][at, 15] = 3
