@@ -80,7 +80,8 @@ __device__ __forceinline__ uint32_t plan_bin(const fem_episode &e, const PlanArg
 // Each candidate's bin and its place in the bin (the order within a bin is arbitrary: a
 // candidate's count does not depend on it), the bins' sizes, the edges in use, and the
 // plan words: per length 1..8 the candidates, [PLAN_REP] those with a repeated type,
-// [PLAN_SPAN] 2^32 - 1 less the least time that a chunk spans.
+// [PLAN_SPAN] 2^32 - 1 less the least time that a chunk spans (and of k_plan_scan [PLAN_DENSE]:
+// an edge in use leads from a type too dense for the tables).
 __global__ void __launch_bounds__(256) k_plan_bins(const PlanArgs a) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t rep = 0, bad = 0, len = 0;
@@ -127,9 +128,13 @@ __global__ void __launch_bounds__(256) k_plan_bins(const PlanArgs a) {
 }
 
 // Slabs per chunk: the fewest equal parts (a power of two) in none of which a type has
-// more than 32 events.  One block per chunk, a warp per type.
+// more than 32 events.  One block per chunk, a warp per type.  Types with more than 32 events
+// of the chunk in the longest interval are told too: their tables would be too dense (all
+// but certainly: it takes an event of the edge's next type at the right time), and the set
+// need not wait for the build to find out.
 __global__ void __launch_bounds__(256) k_hit_cuts(const uint2 *bev, const uint16_t *boff, uint32_t offs,
-                                                  uint32_t K, uint32_t *parts_of) {
+                                                  uint32_t K, uint32_t *parts_of, uint32_t max_hi,
+                                                  uint32_t *dense) {
     __shared__ uint32_t need;
     const uint32_t c = blockIdx.x, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) need = 1;
@@ -140,13 +145,17 @@ __global__ void __launch_bounds__(256) k_hit_cuts(const uint2 *bev, const uint16
         const uint32_t g0 = off[b], g1 = off[b + 1];
         // a part holds more than 32 of the type iff two of its events 32 apart lie in it: the
         // parts must be finer than the highest bit in which their places differ
-        uint32_t q = 1;
+        uint32_t q = 1, span = ~0u;
         for (uint32_t j = g0 + lane; j + 32 < g1; j += 32) {
-            const uint32_t x = ev[j].y ^ ev[j + 32].y;  // not zero
-            q = max(q, CHUNK >> (31 - __clz(x)));       // parts of half the size of that bit's
+            const uint2 e = ev[j], f = ev[j + 32];
+            const uint32_t x = e.y ^ f.y;          // not zero
+            q = max(q, CHUNK >> (31 - __clz(x)));  // parts of half the size of that bit's
+            span = min(span, f.x - e.x);
         }
         q = __reduce_max_sync(0xffffffffu, q);
+        span = __reduce_min_sync(0xffffffffu, span);
         if (lane == 0 && q > 1) atomicMax(&need, q);
+        if (lane == 0 && span <= max_hi) atomicMin(&dense[b], max_hi);
     }
     __syncthreads();
     if (threadIdx.x == 0) parts_of[c] = need;
@@ -187,15 +196,22 @@ __global__ void __launch_bounds__(1024) k_plan_scan(const PlanArgs a, uint32_t b
     uint32_t fewest = HIT_PARTS;
     for (uint32_t c = tid; c < a.n_chunks; c += 1024) fewest = min(fewest, a.parts_of[c]);
     fewest = __reduce_min_sync(0xffffffffu, fewest);
-    __shared__ uint32_t least;
-    if (tid == 0) least = HIT_PARTS;
+    __shared__ uint32_t least, dense;
+    if (tid == 0) least = HIT_PARTS, dense = 0;
     __syncthreads();
     if ((tid & 31) == 0) atomicMin(&least, fewest);
-    __syncthreads();
+    // whether an edge in use leads from a type that is too dense (else none is told)
+    if (__syncthreads_or(tid < a.K && a.dense[tid] <= a.max_hi)) {
+        for (uint32_t i = tid; i < edges; i += 1024)
+            if (a.edge_id[i] != ~0u && a.dense[i / a.n_ivl % a.K] <= a.max_hi) dense = 1;
+        __syncthreads();
+        if (!dense && tid < a.K) a.dense[tid] = ~0u;
+    }
     if (tid == 0) {
         volatile uint32_t *h = pub.host;
         for (uint32_t k = 0; k < PLAN_EDGES; ++k) h[k] = a.words[k];
         h[PLAN_PARTS_MIN] = least;
+        h[PLAN_DENSE] = dense;
         h[PLAN_EDGES] = n_edges;
         h[PLAN_SLABS] = n_slabs;
         h[PLAN_WORDS] = *reinterpret_cast<const volatile uint32_t *>(pub.err);
@@ -216,9 +232,9 @@ __global__ void __launch_bounds__(256) k_plan_place(const PlanArgs a, uint32_t *
 
 // The words of k_validate_cands and the error word, published; the error word and the
 // sequence number where a plan's are, so that no other word is ever taken for the number.
-__global__ void k_publish_info(const uint32_t *info, Publish pub) {
+__global__ void k_publish_info(const uint32_t *info, uint32_t n, Publish pub) {
     volatile uint32_t *h = pub.host;
-    for (uint32_t k = 0; k < 3; ++k) h[k] = info[k];
+    for (uint32_t k = 0; k < n; ++k) h[k] = info[k];
     h[PLAN_WORDS] = *reinterpret_cast<const volatile uint32_t *>(pub.err);
     __threadfence_system();
     h[PLAN_WORDS + 1] = pub.seq;
@@ -340,7 +356,6 @@ __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, ui
     for (uint32_t x = warp; x < K && part == 0; x += NW)
         if (lane < num[x]) b.index[begin + place[x] + lane] = (uint16_t)(origin + rp[x * HIT_ROW + 32 + lane]);
     uint2 *const row = b.edge + (uint64_t)s * b.n_edges;
-    bool dense = false;
     // x's events before event r of type y: those of ranks below k0
     auto rank_of = [&](uint32_t x, uint32_t y, uint32_t r) {
         const uint32_t q = rp[y * HIT_ROW + 32 + r] - CHUNK - p0, w = q >> 5;
@@ -370,6 +385,7 @@ __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, ui
             if (!__any_sync(0xffffffffu, any != 0)) continue;  // no edge in use
             const uint32_t *tx = rt + x * HIT_ROW, *ty = rt + y * HIT_ROW + 32;
             const uint32_t low = any ? 32u - hist[x] : ~0u;  // (no edge: no event is looked at)
+            bool dense = false;
             for (uint32_t r = 0; r < n && any; ++r) {
                 const uint32_t t = ty[r], k0 = rank_of(x, y, r);
                 uint32_t k = k0;
@@ -384,6 +400,7 @@ __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, ui
                 // can say
                 dense = dense || (k == 0 && k0 > 0) || k0 - k > 32;
             }
+            if (dense) atomicOr(b.err, ERR_DENSE), atomicMin(&b.dense[x], far);
             uint32_t c = 0;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -462,7 +479,6 @@ __device__ __forceinline__ void hit_build_slab(const HitBuild &b, uint32_t s, ui
             }
         }
     }
-    if (dense) atomicOr(b.err, ERR_DENSE);
 }
 
 template <int PASS>
@@ -615,15 +631,16 @@ cudaError_t launch_plan(const PlanArgs &a, const StreamDev &s, uint32_t *order, 
     cudaError_t e = cudaMemsetAsync(a.words, 0, (PLAN_WORDS + (size_t)bins + edges) * 4, st);
     if (e != cudaSuccess) return e;
     k_plan_bins<<<blocks, 256, 0, st>>>(a);
-    k_hit_cuts<<<s.n_chunks, 256, 0, st>>>(s.bev, s.boff, s.offs, s.K, a.parts_of);
+    k_hit_cuts<<<s.n_chunks, 256, 0, st>>>(s.bev, s.boff, s.offs, s.K, a.parts_of, a.max_hi, a.dense);
     k_plan_scan<<<1, 1024, 0, st>>>(a, bins, edges, pub);
     k_plan_place<<<blocks, 256, 0, st>>>(a, order, gather);
     note_launch(4);
     return cudaGetLastError();
 }
 
-cudaError_t launch_publish_info(const uint32_t *info, Publish pub, cudaStream_t st) {
-    k_publish_info<<<1, 1, 0, st>>>(info, pub);
+cudaError_t launch_publish_info(const uint32_t *info, uint32_t n, Publish pub, cudaStream_t st) {
+    if (n > PLAN_WORDS) return cudaErrorInvalidValue;
+    k_publish_info<<<1, 1, 0, st>>>(info, n, pub);
     note_launch();
     return cudaGetLastError();
 }

@@ -221,8 +221,11 @@ template <int NMAX, bool MC>
 __device__ __forceinline__ void hit_count_tile(const CountParams &p, uint32_t tile, uint32_t seg) {
     const uint32_t ci = tile * blockDim.x + threadIdx.x;
     const HitTables &h = p.hits;
+    // tables that are too dense (the build before said so) are not worth a count
+    const uint32_t e0 = *reinterpret_cast<const volatile uint32_t *>(p.err);
     HitEpisode<NMAX> ep;
     const bool ok = ep.load(p, ci);
+    if (e0 & ERR_DENSE) return;
     const uint64_t W = ep.W;
 
     // ------------------------------------------------------------ segment and window
@@ -404,8 +407,10 @@ __global__ void __launch_bounds__(128) k_hit_windows(const CountParams p, const 
                                                      uint32_t w, unsigned long long *out) {
     const uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x, seg = blockIdx.y;
     const HitTables &h = p.hits;
+    const uint32_t e0 = *reinterpret_cast<const volatile uint32_t *>(p.err);
     HitEpisode<NMAX> ep;
     const bool ok = ep.load(p, ci);
+    if (e0 & ERR_DENSE) return;  // (as in hit_count_tile)
     const uint32_t s0 = seg * p.cps, s1 = min(s0 + p.cps, h.n_slabs);
     uint32_t s_w = s0;
     if (ok) {
@@ -459,6 +464,7 @@ constexpr uint32_t JOIN_QUEUE = 64;  // hits a warp takes at a time, at least a 
 
 __global__ void __launch_bounds__(256) k_join(const HitTables h, const JoinTables g, uint32_t n_events,
                                               uint32_t K, uint32_t n_ivl, uint32_t *__restrict__ out) {
+    if (*g.err & ERR_DENSE) return;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NW = blockDim.x / 32;
     const uint32_t slots = K * n_ivl, b = blockIdx.x, second = blockIdx.y * NW + warp;
     if (second >= g.n_begins[b]) return;  // (warps are on their own)

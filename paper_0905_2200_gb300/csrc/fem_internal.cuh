@@ -15,6 +15,7 @@
 
 #include <atomic>
 #include <string>
+#include <vector>
 
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -67,6 +68,10 @@ struct StreamDev {
     mutable uint64_t ring_gen = 0;
     mutable std::string ring_ivl;
     mutable bool ring_singles = false, ring_clusters = false;
+    // per type the shortest interval found to hold more of its events than a hit table's
+    // word (2^32 - 1: none; empty: none of any type).  Appended events make no interval
+    // emptier, so what was found stays true of a stream as long as it lives.
+    mutable std::vector<uint32_t> dense_hi;
 };
 
 // The hit tables of a stream, an edge set and a pass (fem_hits.cuh).
@@ -90,6 +95,7 @@ struct JoinTables {
     uint32_t *rank;               // [K][n_slabs] a slab's first event of a type, by type and time
     uint32_t *off;                // [n + 1] first entry of an event's list, by type and time
     uint32_t *list;               // pair (its place in `ends`) << 16 | low half of its first event's index
+    const uint32_t *err;          // ERR_DENSE: nothing is joined
 };
 
 // Arguments of the counting kernels (one pass over one candidate set).
@@ -309,6 +315,7 @@ struct HitBuild {
     uint8_t *count;
     uint16_t *place, *index;
     uint32_t *err;                // ERR_DENSE
+    uint32_t *dense;              // per type the shortest reach that was too dense, lowered
 };
 // ranges that a build of n_slabs slabs may reserve beyond its hits
 cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
@@ -336,7 +343,7 @@ cudaError_t launch_join_gather(const uint32_t *cells, const fem_episode *cands, 
 // + plan_bins(K, parts) + K K n_ivl words.
 constexpr uint32_t PLAN_PARTS = 4, PLAN_GROUPS = 5, PLAN_FINE = 8192;
 constexpr uint32_t PLAN_REP = 8, PLAN_SPAN = 9, PLAN_EDGES = 10, PLAN_SLABS = 11, PLAN_PARTS_MIN = 12,
-                   PLAN_WORDS = 13;
+                   PLAN_DENSE = 13, PLAN_WORDS = 14;
 // The launch that counts an episode of N nodes: lengths 1-2, 3, 4, 5 and 6-8, since
 // registers and shared memory grow with the length; small sets (below PLAN_FINE), whose
 // launches are short, in three (1-3, 4-5, 6-8).
@@ -356,6 +363,8 @@ struct PlanArgs {
     uint64_t n;
     uint32_t *words, *hist, *edge_id, *bin, *rank;
     uint32_t *parts_of, *begin, *t0;  // per chunk its slabs; per slab its first event and time
+    uint32_t max_hi;                  // the longest interval
+    uint32_t *dense;                  // HitBuild::dense, lowered where [PLAN_DENSE] is set
     uint32_t *err;
 };
 uint32_t plan_bins(uint32_t K, uint32_t parts);
@@ -364,8 +373,9 @@ struct Publish;
 // the plan words, the error word and the sequence number (PLAN_WORDS + 2 words)
 cudaError_t launch_plan(const PlanArgs &a, const StreamDev &s, uint32_t *order, uint32_t *gather,
                         Publish pub, cudaStream_t st);
-// info[0 .. 3) of launch_validate_cands, the error word and the sequence number (5 words)
-cudaError_t launch_publish_info(const uint32_t *info, Publish pub, cudaStream_t st);
+// the first n words (at most PLAN_WORDS) of launch_validate_cands, and where a plan's are the
+// error word and the sequence number
+cudaError_t launch_publish_info(const uint32_t *info, uint32_t n, Publish pub, cudaStream_t st);
 cudaError_t launch_publish_count(const unsigned long long *src, Publish pub, cudaStream_t st);
 // fem_windows.cu: window-based frequency, one thread per episode (distinct types)
 struct WindowParams {
@@ -398,10 +408,11 @@ cudaError_t launch_stitch(const uint4 *tables, uint32_t m, uint32_t P, uint32_t 
                           uint32_t classes = S_MAX, const uint32_t *m_dev = nullptr);
 // info[0] |= 1 << len of every candidate; info[1] += candidates with a repeated type;
 // info[2] += candidates whose length or prefix before the last node differs from the
-// previous candidate's (the number of prefix runs is info[2] + 1)
+// previous candidate's (the number of prefix runs is info[2] + 1); with types, info[3 .. 11)
+// |= a bit for the type of every node but the last
 cudaError_t launch_validate_cands(const fem_episode *c, const uint32_t *gather, uint32_t m,
                                   uint32_t K, uint32_t n_ivl, uint32_t *info, uint32_t *err,
-                                  cudaStream_t st);
+                                  cudaStream_t st, bool types = false);
 cudaError_t launch_len_flags(const fem_episode *c, const uint32_t *gather, uint32_t m, uint32_t N,
                              uint8_t *flags, cudaStream_t st);
 // dst[i] = outer ? outer[inner[i]] : inner[i]

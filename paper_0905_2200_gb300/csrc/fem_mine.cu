@@ -259,11 +259,12 @@ cudaError_t launch_stitch(const uint4 *tables, uint32_t m, uint32_t P, uint32_t 
 
 // ------------------------------------------------------------------ candidate validation
 // info[0] |= 1 << len for every candidate; info[1] += candidates with a repeated type.
+template <bool TYPES>
 __global__ void k_validate_cands(const fem_episode *__restrict__ c, const uint32_t *gather,
                                  uint32_t m, uint32_t K, uint32_t n_ivl, uint32_t *info,
                                  uint32_t *err) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t lenbit = 0, rep = 0, bad = 0, brk = 0;
+    uint32_t lenbit = 0, rep = 0, bad = 0, brk = 0, types[TYPES ? 8 : 1] = {};
     if (i < m) {
         const fem_episode e = ld_ep(c, gather ? gather[i] : i);
         const uint32_t N = e.len;
@@ -285,6 +286,19 @@ __global__ void k_validate_cands(const fem_episode *__restrict__ c, const uint32
             for (uint32_t a = 0; a < N; ++a)
                 for (uint32_t b2 = a + 1; b2 < N; ++b2)
                     if (e.types[a] == e.types[b2]) rep = 1;
+            if (TYPES) {
+                for (uint32_t k = 0; k + 1 < N; ++k)
+#pragma unroll
+                    for (uint32_t w = 0; w < 8; ++w)
+                        if (e.types[k] >> 5 == w) types[w] |= 1u << (e.types[k] & 31u);
+            }
+        }
+    }
+    if (TYPES) {
+#pragma unroll
+        for (uint32_t w = 0; w < 8; ++w) {
+            const uint32_t v = __reduce_or_sync(0xffffffffu, types[w]);
+            if ((threadIdx.x & 31) == 0 && v) atomicOr(&info[3 + w], v);
         }
     }
     lenbit = __reduce_or_sync(0xffffffffu, lenbit);
@@ -301,9 +315,10 @@ __global__ void k_validate_cands(const fem_episode *__restrict__ c, const uint32
 
 cudaError_t launch_validate_cands(const fem_episode *c, const uint32_t *gather, uint32_t m,
                                   uint32_t K, uint32_t n_ivl, uint32_t *info, uint32_t *err,
-                                  cudaStream_t st) {
+                                  cudaStream_t st, bool types) {
     if (m == 0) return cudaSuccess;
-    k_validate_cands<<<(m + 255) / 256, 256, 0, st>>>(c, gather, m, K, n_ivl, info, err);
+    (types ? k_validate_cands<true> : k_validate_cands<false>)<<<(m + 255) / 256, 256, 0, st>>>(
+        c, gather, m, K, n_ivl, info, err);
     note_launch();
     return cudaGetLastError();
 }

@@ -78,3 +78,66 @@ def test_counts(ctx, m):
         for call in range(3):
             assert_counts_equal(fem.fem_count_candidates(ctx, sid, rec, I, p), want, f"pass {p} call {call}")
     fem.fem_free_stream(ctx, sid)
+
+
+@pytest.fixture()
+def told(monkeypatch, capfd):
+    """What became of the hit tables since the last look, one word each."""
+    monkeypatch.setenv("FEM_DEBUG", "1")
+
+    def look():
+        return [x.split(": ")[-1] for x in capfd.readouterr().err.splitlines() if "hit tables of" in x]
+
+    return look
+
+
+@pytest.mark.parametrize("m", [100, 700])
+def test_a_dense_type_is_remembered(ctx, told, m):
+    """Tables that turned out too dense are not built again for sets with an edge from that type
+    and an interval as long, also after events were appended; other sets still go over them."""
+    ty, t = burst_stream(3)
+    sid = fem.fem_load_stream(ctx, ty, t, K)
+    L, E, iv = synth.random_candidates(3, m, K - 2, [2, 3], 4)
+    quiet = L, np.where(np.arange(E.shape[1]) < L[:, None], E + 2, 0).astype(np.uint8), iv
+    dense = with_edge(quiet, 3)
+
+    def counts(cands, intervals=I):
+        told()
+        for p in PASSES:
+            assert_counts_equal(fem.fem_count_candidates(ctx, sid, fem.pack_episodes(*cands), intervals, p),
+                                oracle_counts(ty, t, *cands, intervals, p), f"pass {p}")
+        return told()
+
+    assert counts(dense) == ["too dense"]
+    assert counts(dense) == []
+    assert counts(quiet) == ["counted"] * 2
+    assert counts(dense, I // 4) == ["counted"] * 2  # up to 25 of type 0 in the longest
+    more = np.arange(200, dtype=np.uint32) * 30000 + t[-1] + 1
+    for k in range(3):  # (the stream's buffers grow)
+        fem.fem_append_stream(ctx, sid, np.full(200, 2 + k, np.uint8), more)
+        ty, t = np.append(ty, np.full(200, 2 + k, np.uint8)), np.append(t, more)
+        more = more + np.uint32(7_000_000)
+        assert counts(dense) == [] and counts(quiet) == ["counted"] * 2
+    assert fem.fem_count_windows(ctx, sid, fem.pack_episodes(*quiet), I, 9000).sum() > 0
+    assert told() == ["counted"]
+    with pytest.raises(fem.FemError):
+        fem.fem_count_windows(ctx, sid, fem.pack_episodes(*dense), I, 9000)
+    assert told() == []
+    fem.fem_free_stream(ctx, sid)
+
+
+def test_mining_a_dense_stream(ctx, told):
+    ty, t = burst_stream(4)
+    sid = fem.fem_load_stream(ctx, ty, t, K)
+    want = oracle.mine(ty, t, K, I[:2], 20, 4)
+    long = np.array([[0, 5000], [0, 40000]], np.uint32)
+    for intervals, first, second in ((I[:2], None, None), (long, 1, 0)):
+        for expected in (first, second):
+            got = fem.fem_mine_levelwise(ctx, sid, intervals, 20, 4)
+            assert got == (want if expected is None else oracle.mine(ty, t, K, intervals, 20, 4))
+            words = told()
+            if expected is None:
+                assert set(words) == {"counted"}
+            else:
+                assert words == ["too dense"] * expected
+    fem.fem_free_stream(ctx, sid)
