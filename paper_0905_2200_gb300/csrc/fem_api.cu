@@ -58,7 +58,8 @@ struct fem_ctx {
     uint32_t *d_plan = nullptr;  // the same of h_small[kPlanWord ..], written by the plan kernels
     uint32_t pub_seq = 0;  // sequence number of the last publishing launch
     // mapped pinned words a load's read-back is published to ([0] error word, [1] last
-    // time, [2..258) type counts, [kLoadSeq] sequence number) and their device address
+    // time, [2..258) type counts, [258] first time, [kLoadSeq] sequence number) and their
+    // device address
     uint32_t *h_load = nullptr, *d_load = nullptr;
     // pinned staging of an interval set (so that its upload is asynchronous), and the
     // event after the last upload from it (the next one waits for that copy to leave)
@@ -123,7 +124,7 @@ void report_cuda(cudaError_t e, int line) {
 enum { W_COUNT0 = 0, W_COUNT1 = 1, W_COUNT2 = 2, W_INFO = 8 /* 11 words */ };
 // first of the three pinned host words the kernels publish counts to
 constexpr uint32_t kPubWord = 48;
-constexpr uint32_t kLoadSeq = 2 + 256;  // the load read-back's sequence word
+constexpr uint32_t kLoadSeq = 2 + 256 + 1;  // the load read-back's sequence word
 // first of the mapped host words a plan is published to (plan words, error word, sequence)
 constexpr uint32_t kPlanWord = 64;
 constexpr uint32_t kSmallWords = kPlanWord + PLAN_WORDS + 2;
@@ -1038,7 +1039,7 @@ int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     double per_event = 0;
     for (const fem_interval &iv : c->ivl_host)
         per_event += (double)(iv.hi_us - (pass == FEM_PASS_EXACT ? iv.lo_us : 0u)) * (double)s.n /
-                     (double)std::max(s.t_max, 1u);
+                     (double)std::max(s.t_max - s.t_min, 1u);
     per_event *= (double)h.n_edges / tri;
     pl->hits = std::min<uint64_t>((uint64_t)(1.25 * per_event * (double)s.n) + 65536,
                                   (uint64_t)s.n * (h.n_edges / s.K + 1));
@@ -1221,7 +1222,7 @@ bool hits_eligible(const fem_ctx *c, const StreamDev &s, uint32_t nI) {
     for (const fem_interval &iv : c->ivl_host) max_hi = std::max<uint64_t>(max_hi, iv.hi_us);
     return !c->cfg.kernel && !c->cfg.ring_capacity && c->d_plan && s.n_chunks && nI &&
            (uint64_t)s.K * s.K * nI <= kHitMaxEdges &&
-           (double)s.n * (double)max_hi <= 8.0 * s.K * (double)std::max(s.t_max, 1u);
+           (double)s.n * (double)max_hi <= 8.0 * s.K * (double)std::max(s.t_max - s.t_min, 1u);
 }
 
 // One pass of level 3 over m candidates of the frequent pairs F, all pairs at once (k_join):
@@ -1761,24 +1762,25 @@ int fem_load_stream(fem_ctx *c, const uint8_t *types, const uint32_t *t_us, uint
         if (c->d_load) {
             const uint32_t seq = ++c->pub_seq;
             if (launch_publish_load(c->d_err, n ? s.t + (n - 1) : nullptr, s.hist, n_types,
-                                    c->d_load, kLoadSeq, seq, st) != cudaSuccess) {
+                                    c->d_load, kLoadSeq, seq, s.t, st) != cudaSuccess) {
                 rc = FEM_ECUDA;
                 break;
             }
             if ((rc = wait_seq(c->h_load + kLoadSeq, seq, st)) != FEM_OK) break;
             const volatile uint32_t *hv = c->h_load;
             if ((rc = err_status(hv[0])) != FEM_OK) break;
-            if (n) s.t_max = hv[1];
+            if (n) s.t_max = hv[1], s.t_min = hv[kLoadSeq - 1];
             hist_host.assign(n_types, 0);
             for (uint32_t a = 0; a < n_types; ++a) hist_host[a] = hv[2 + a];
             break;
         }
         void *hp;
-        if ((rc = pinbuf(c, 0, (2 + 256) * sizeof(uint32_t), st, &hp)) != FEM_OK) break;
+        if ((rc = pinbuf(c, 0, (3 + 256) * sizeof(uint32_t), st, &hp)) != FEM_OK) break;
         uint32_t *hw = static_cast<uint32_t *>(hp);
         if (cudaMemcpyAsync(hw, c->d_err, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             (n && cudaMemcpyAsync(hw + 1, s.t + (n - 1), 4, cudaMemcpyDeviceToHost, st) !=
                       cudaSuccess) ||
+            (n && cudaMemcpyAsync(hw + 258, s.t, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess) ||
             cudaMemcpyAsync(hw + 2, s.hist, n_types * 4, cudaMemcpyDeviceToHost, st) !=
                 cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) {
@@ -1786,7 +1788,7 @@ int fem_load_stream(fem_ctx *c, const uint8_t *types, const uint32_t *t_us, uint
             break;
         }
         if ((rc = err_status(hw[0])) != FEM_OK) break;
-        if (n) s.t_max = hw[1];
+        if (n) s.t_max = hw[1], s.t_min = hw[258];
         hist_host.assign(hw + 2, hw + 2 + n_types);
     } while (0);
     if (rc != FEM_OK) {
@@ -1814,7 +1816,7 @@ int fem_append_stream(fem_ctx *c, int32_t id, const uint8_t *types, const uint32
     if (n_new >= 0xFFFFFFF0ull) return FEM_EINVAL;
     cudaSetDevice(c->device);
     cudaStream_t st = pick(c, cuda_stream);
-    const uint32_t ch_old = s.n_chunks, K = s.K, t_max_old = s.t_max;
+    const uint32_t ch_old = s.n_chunks, K = s.K, t_min = s.t_min, t_max_old = s.t_max;
     const uint32_t ch_new = (uint32_t)((n_new + CHUNK - 1) / CHUNK);
     if (n_new > s.cap_events || ch_new > s.cap_chunks || (uint64_t)ch_new * s.offs > s.cap_offs) {
         // grow by half at least, keeping what is grouped already
@@ -1845,7 +1847,7 @@ int fem_append_stream(fem_ctx *c, int32_t id, const uint8_t *types, const uint32
         c->mem_used -= std::min(stream_bytes(s), c->mem_used);
         g.dense_hi = std::move(s.dense_hi);
         free_stream_buffers(s);
-        g.n = n_old, g.K = K, g.n_chunks = ch_old, g.t_max = t_max_old;
+        g.n = n_old, g.K = K, g.n_chunks = ch_old, g.t_min = t_min, g.t_max = t_max_old;
         s = g;
     }
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -1860,11 +1862,12 @@ int fem_append_stream(fem_ctx *c, int32_t id, const uint8_t *types, const uint32
     CK(launch_bucket_chunks(s, c0, ch_new, st, c->d_err));
     CK(launch_hist_add(s.type + n_old, n, s.K, +1, s.hist, st));
     void *hp;
-    RET(pinbuf(c, 0, (2 + 256) * sizeof(uint32_t), st, &hp));
+    RET(pinbuf(c, 0, (3 + 256) * sizeof(uint32_t), st, &hp));
     uint32_t *hw = static_cast<uint32_t *>(hp);
     CK(cudaMemcpyAsync(hw, c->d_err, 4, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(hw + 1, s.t + (n_new - 1), 4, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(hw + 2, s.hist, s.K * 4, cudaMemcpyDeviceToHost, st));
+    if (!n_old) CK(cudaMemcpyAsync(hw + 258, s.t, 4, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     const int rc = err_status(hw[0]);
     if (rc != FEM_OK) {
@@ -1879,6 +1882,7 @@ int fem_append_stream(fem_ctx *c, int32_t id, const uint8_t *types, const uint32
         return rc;
     }
     s.t_max = hw[1];
+    if (!n_old) s.t_min = hw[258];
     s.gen = c->next_gen++;
     c->hist_h[id].assign(hw + 2, hw + 2 + s.K);
     return FEM_OK;

@@ -56,7 +56,7 @@ struct StreamDev {
     uint32_t cap_offs = 0;
     uint64_t n = 0;
     uint32_t K = 0, n_chunks = 0, offs = 0;
-    uint32_t t_max = 0;
+    uint32_t t_min = 0, t_max = 0;  // first and last time
     uint32_t *t = nullptr;
     uint8_t *type = nullptr;
     uint2 *bev = nullptr;
@@ -229,10 +229,11 @@ cudaError_t launch_bucket_chunks(StreamDev &s, uint32_t c0, uint32_t c1, cudaStr
                                  uint32_t *d_err = nullptr);
 // hist[ty[i]] += sign (+1 or -1) for i < n
 // host[0] = *err, host[1] = *t_last (0 if null), host[2 .. 2 + K) = hist, then
-// host[seq_word] = seq (host: the device address of mapped pinned words)
+// host[seq_word - 1] = *t_first (0 if there is no last), host[seq_word] = seq (host: the device
+// address of mapped pinned words)
 cudaError_t launch_publish_load(const uint32_t *err, const uint32_t *t_last, const uint32_t *hist,
                                 uint32_t K, uint32_t *host, uint32_t seq_word, uint32_t seq,
-                                cudaStream_t st);
+                                const uint32_t *t_first, cudaStream_t st);
 // fem_pairs.cu: the relaxed pass of a level-2 set, all interval variants of an ordered
 // type pair in one thread (p.pair_types = f, p.n_ivl <= 4; P > 1: MapConcatenate tables)
 cudaError_t launch_pairs_relaxed(const CountParams &p, uint32_t threads, cudaStream_t st);

@@ -167,7 +167,7 @@ cudaError_t launch_hist_add(const uint8_t *ty, uint64_t n, uint32_t K, int sign,
 __global__ void __launch_bounds__(256) k_publish_load(const uint32_t *err, const uint32_t *t_last,
                                                       const uint32_t *hist, uint32_t K,
                                                       uint32_t *host, uint32_t seq_word,
-                                                      uint32_t seq) {
+                                                      uint32_t seq, const uint32_t *t_first) {
     __shared__ uint32_t hs[256];  // K <= 256
     for (uint32_t a = threadIdx.x; a < K; a += blockDim.x) hs[a] = hist[a];
     __syncthreads();
@@ -176,15 +176,16 @@ __global__ void __launch_bounds__(256) k_publish_load(const uint32_t *err, const
     for (uint32_t a = 0; a < K; ++a) h[2 + a] = hs[a];
     h[0] = *reinterpret_cast<const volatile uint32_t *>(err);
     h[1] = t_last ? *t_last : 0u;
+    h[seq_word - 1] = t_last ? *t_first : 0u;
     __threadfence_system();
     h[seq_word] = seq;
 }
 
 cudaError_t launch_publish_load(const uint32_t *err, const uint32_t *t_last, const uint32_t *hist,
                                 uint32_t K, uint32_t *host, uint32_t seq_word, uint32_t seq,
-                                cudaStream_t st) {
+                                const uint32_t *t_first, cudaStream_t st) {
     if (K > 256) return cudaErrorInvalidValue;
-    k_publish_load<<<1, 256, 0, st>>>(err, t_last, hist, K, host, seq_word, seq);
+    k_publish_load<<<1, 256, 0, st>>>(err, t_last, hist, K, host, seq_word, seq, t_first);
     note_launch();
     return cudaGetLastError();
 }

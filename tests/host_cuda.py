@@ -62,7 +62,8 @@ class Host:
             t_last, k, host = (arg(i, kind) for i, kind in
                                ((1, ctypes.POINTER(ctypes.c_uint32)), (3, ctypes.c_uint32),
                                 (4, ctypes.POINTER(ctypes.c_uint32))))
-            host[0], host[1] = 0, t_last[0] if t_last else 0
+            first = arg(7, ctypes.POINTER(ctypes.c_uint32))
+            host[0], host[1], host[258] = 0, t_last[0] if t_last else 0, first[0] if t_last else 0
             for a in range(k):
                 host[2 + a] = 0
             host[arg(5, ctypes.c_uint32)] = arg(6, ctypes.c_uint32)

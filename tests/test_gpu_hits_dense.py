@@ -141,3 +141,26 @@ def test_mining_a_dense_stream(ctx, told):
             else:
                 assert words == ["too dense"] * expected
     fem.fem_free_stream(ctx, sid)
+
+
+@pytest.mark.parametrize("appended", [False, True])
+def test_streams_that_start_late(ctx, told, appended):
+    """How dense a stream is, is told by the time from its first to its last event: an hour after
+    time 0 as at time 0, also where it was empty when it was loaded."""
+    rng = np.random.default_rng(8)
+    dense = rng.integers(0, 3, 6000).astype(np.uint8), np.cumsum(rng.integers(1, 60, 6000)).astype(np.uint32)
+    even = rng.integers(0, K, 60000).astype(np.uint8), np.cumsum(rng.integers(1, 700, 60000)).astype(np.uint32)
+    for (ty, t), types, ivls, words in ((dense, 3, np.array([[500, 9000]], np.uint32), []),
+                                        (even, K, I[2:3], ["counted"])):
+        cands = synth.random_candidates(8, 200, types, [2, 3], 1)
+        for first_us in (0, 3_600_000_000):
+            t1 = (t + np.uint32(first_us)).astype(np.uint32)
+            n0 = 0 if appended else len(t)
+            sid = fem.fem_load_stream(ctx, ty[:n0], t1[:n0], types)
+            if appended:
+                fem.fem_append_stream(ctx, sid, ty, t1)
+            told()
+            got = fem.fem_count_candidates(ctx, sid, fem.pack_episodes(*cands), ivls, 0)
+            assert told() == words
+            assert_counts_equal(got, oracle_counts(ty, t1, *cands, ivls, 0), f"from {first_us}")
+            fem.fem_free_stream(ctx, sid)
