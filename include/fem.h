@@ -135,9 +135,14 @@ typedef struct {
  * Context.  One per device; allocates its own device working memory: resident
  * streams (about 13 bytes per event plus 2 (K + 1) bytes per chunk of 2048 events),
  * per-call working buffers (kept and reused), and batches.  mem_budget_bytes bounds
- * that memory (0: no bound).  A call that would need more first releases the buffers
- * kept from freed streams and otherwise fails with FEM_ENOMEM, leaving the context
- * usable.  Serving (fem_server_*) has its own budget in fem_server_config.
+ * that memory (0: no bound).  A call that would need more first releases the hit tables
+ * (FEM_KERNEL_HITS) of earlier calls and the buffers kept from freed streams, and otherwise
+ * fails with FEM_ENOMEM, leaving the context usable; where the tables themselves find no
+ * room, the other kernels count.  Between calls a context keeps tables of at most a 16th of
+ * the device's memory (100,000 candidates on an hour of 64 types at 50 Hz: 10 GB); they are
+ * given back where one of the context's own allocations or fem_server_create needs the
+ * memory, and with fem_destroy.  fem_mem_usage tells what is held.  Serving (fem_server_*)
+ * has its own budget in fem_server_config.
  */
 int fem_create(fem_ctx **out, int device, size_t mem_budget_bytes);
 /* Device bytes the context holds now (*used_out) and its budget (*budget_out, 0 = none);

@@ -40,6 +40,7 @@ struct fem_ctx {
     // device memory the context holds for streams, working buffers and batches, and
     // the caller's bound on it (0: none)
     size_t mem_budget = 0, mem_used = 0;
+    size_t mem_device = 0;  // the device's memory
     cudaStream_t own = nullptr;
     fem_config cfg{};
     int sm_count = 152;
@@ -893,14 +894,27 @@ void hits_segments(const fem_ctx *c, const StreamDev &s, CountParams &p) {
     p.P = (p.hits.n_slabs + p.cps - 1) / p.cps;
 }
 
-// Launch a hit-table pass over p.m candidates (and its stitch when segmented).
+// Launch a hit-table pass over p.m candidates (and its stitch when segmented).  The transfer
+// tables (30 KB a candidate on the hour-long recording) take at most a 64th of the device's
+// memory: more candidates (145,000 there) are counted a part after the other, each with all
+// segments.
 int hits_launch(fem_ctx *c, const StreamDev &s, uint32_t group, CountParams &p, uint32_t classes,
                 const char *tables, cudaStream_t st) {
     hits_segments(c, s, p);
     p.hit_classes = classes;
-    if (p.P > 1) RET(dbuf(c, tables, (size_t)p.P * p.m * classes, &p.tables));
-    CK(launch_hit_count(group, p.P > 1, p, st));
-    if (p.P > 1) CK(launch_stitch(p.tables, p.m, p.P, p.out, p.redo, c->d_err, st, classes));
+    uint32_t step = p.m;
+    if (p.P > 1) {
+        const size_t each = (size_t)p.P * classes;
+        step = (uint32_t)std::min<size_t>(step, std::max<size_t>(128, c->mem_device / 64 / (each * sizeof(uint4)) / 128 * 128));
+        RET(dbuf(c, tables, each * step, &p.tables));
+    }
+    for (uint64_t off = 0; off < p.m; off += step) {
+        CountParams q = p;
+        q.gather += off, q.out += off, q.redo += off;
+        q.m = std::min(step, p.m - (uint32_t)off);
+        CK(launch_hit_count(group, q.P > 1, q, st));
+        if (q.P > 1) CK(launch_stitch(q.tables, q.m, q.P, q.out, q.redo, c->d_err, st, classes));
+    }
     return FEM_OK;
 }
 
@@ -927,7 +941,7 @@ int hits_finish(fem_ctx *c, const StreamDev &s, uint32_t group, const CountParam
     q.out = rout;
     RET(dbuf(c, "hit_redo", r, &q.redo));
     CK(cudaMemsetAsync(q.redo, 0, r, st));
-    RET(hits_launch(c, s, group, q, S_RECOUNT, "redo_tables", st));
+    RET(hits_launch(c, s, group, q, S_RECOUNT, "hit_redo_tables", st));
     RET(read_err(c, st, &e));
     RET(err_status(e));
     if (e & ERR_CAP) {
@@ -1149,7 +1163,7 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
             part[g] = hits_params(c, s, pl, cands, g, off);
             part[g].out = tmp + off;
             part[g].redo = redo + off;
-            RET(hits_launch(c, s, g, part[g], S_MAX, "tables", st));
+            RET(hits_launch(c, s, g, part[g], S_MAX, "hit_tables", st));
             off += part[g].m;
         }
         uint32_t e;
@@ -1203,9 +1217,15 @@ int windows_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, uint3
 }
 
 // The status of work over hit tables; where there was no room for them beside the stream,
-// their memory is given back and the other kernels count (nothing was).
+// their memory is given back and the other kernels count (nothing was).  So it is where they
+// are more than a 16th of the device's memory: no more is kept for the next call (the
+// hour-long recording's, 10 GB, are).
 int or_no_room(fem_ctx *c, int rc, bool *done, cudaStream_t st) {
     c->hits_busy = false;
+    size_t kept = 0;
+    for (const auto &kv : c->bufs)
+        if (kv.first.compare(0, 4, "hit_") == 0) kept += kv.second.cap;
+    if (kept > c->mem_device / 16) release_hits(c);
     if (rc != FEM_ENOMEM) return rc;
     *done = false;
     release_hits(c);
@@ -1508,6 +1528,7 @@ extern "C" {
 namespace fem {
 int fem_ctx_device(const fem_ctx *c) { return c->device; }
 int fem_ctx_sms(const fem_ctx *c) { return c->sm_count; }
+bool fem_ctx_release_hits(fem_ctx *c) { return release_hits(c); }
 }  // namespace fem
 
 extern "C" {
@@ -1576,6 +1597,12 @@ int fem_create(fem_ctx **out, int device, size_t mem_budget_bytes) {
             fem_destroy(c);
             return FEM_ECUDA;
         }
+    }
+    size_t mem_free = 0;
+    if (cudaMemGetInfo(&mem_free, &c->mem_device) != cudaSuccess) {
+        cudaGetLastError();
+        fem_destroy(c);
+        return FEM_ECUDA;
     }
     cudaMemset(c->d_err, 0, sizeof(uint32_t));
     cudaMemset(c->d_dense, 0xFF, 256 * sizeof(uint32_t));

@@ -275,6 +275,7 @@ inline cudaError_t smem_limit(std::atomic<uint64_t> &set, const void *kernel, in
 }
 int fem_ctx_device(const fem_ctx *c);
 int fem_ctx_sms(const fem_ctx *c);
+bool fem_ctx_release_hits(fem_ctx *c);  // the hit tables kept from earlier counts; whether any
 // fem_count.cu
 // classes: entry-class slots per transfer table (S_MAX; 2 S_MAX for the segmented recount,
 // relaxed or exact with ring_cap 32)

@@ -435,7 +435,9 @@ int fem_server_create(fem_ctx *ctx, const fem_server_config *cfg, fem_server **o
     if (!v->cfg.max_active) v->cfg.max_active = 64;
     if (!v->cfg.n_lanes) v->cfg.n_lanes = 8;
     cudaSetDevice(v->device);
-    bool ok = v->dev.init(v->cfg.mem_budget_bytes, false) &&
+    // (where the device is full, once more without the context's hit tables)
+    bool ok = (v->dev.init(v->cfg.mem_budget_bytes, false) ||
+               (fem_ctx_release_hits(ctx) && v->dev.init(v->cfg.mem_budget_bytes, false))) &&
               v->host.init(std::max<size_t>(v->cfg.mem_budget_bytes / 4, (size_t)64 << 20), true) &&
               cudaStreamCreateWithFlags(&v->ingest, cudaStreamNonBlocking) == cudaSuccess;
     for (uint32_t i = 0; ok && i < v->cfg.n_lanes; ++i) {

@@ -15,6 +15,7 @@ void (*host_on_launch)(const char *name, void **args) = 0;
 int host_fail_malloc = 0;  /* fail the allocation so many calls ahead (1: the next) */
 int host_fail_launch = 0;  /* the same of launches (cudaGetLastError tells) */
 int host_device = 0, host_devices = 1;
+size_t host_malloc_max = 0; /* the largest allocation of device memory */
 size_t host_new_max = 0;   /* the largest piece of host memory that the library took by `new` */
 uint64_t host_mallocs = 0, host_attributes = 0, host_stream_uploads = 0, host_plain_uploads = 0;
 size_t host_bytes = 0;     /* device memory held */
@@ -73,6 +74,7 @@ static int take(void **p, size_t n) {
 }
 int cudaMalloc(void **p, size_t n) {
     ++host_mallocs;
+    if (n > host_malloc_max) host_malloc_max = n;
     if (host_fail_malloc > 0 && --host_fail_malloc == 0) return last_error = NO_MEMORY;
     return take(p, n);
 }

@@ -73,7 +73,7 @@ class Host:
                 p.host[w] = self.plan.get(w, 0)
             p.host[PLAN_WORDS], p.host[PLAN_WORDS + 1] = 0, p.seq
         elif "k_publish_info" in name:
-            p = arg(1, Publish)
+            p = arg(2, Publish)
             for w in range(3):
                 p.host[w] = self.plan.get(("info", w), 0)
             p.host[PLAN_WORDS], p.host[PLAN_WORDS + 1] = 0, p.seq

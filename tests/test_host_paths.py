@@ -162,3 +162,63 @@ def test_batch_of_many_candidates_on_the_host(host, ctx, m):
         I = np.array([[0, 4000]], np.uint32)
         assert host.lib.fem_batch_create(ctx, jobs, 2, I.ctypes.data_as(vp), 1, None, ctypes.byref(vp())) == -1
         kept[0][at, 15] = 3
+
+
+def used(host, ctx):
+    n = ctypes.c_size_t()
+    assert host.lib.fem_mem_usage(ctx, ctypes.byref(n), None) == 0
+    return n.value
+
+
+def many(m, edges, slabs):
+    """The words of a plan, and of a validation, of m candidates of three nodes not in runs."""
+    return {2: m, PLAN_EDGES: edges, PLAN_SLABS: slabs, PLAN_PARTS_MIN: 1, ("info", 0): 8, ("info", 2): m}
+
+
+def context(host, budget=0):
+    c = vp()
+    assert host.lib.fem_create(ctypes.byref(c), 0, ctypes.c_size_t(budget)) == 0
+    return c
+
+
+def test_transfer_tables_are_bounded_in_bytes(host):
+    """Many candidates on a long stream: the tables between its segments take at most a 64th of
+    the device's memory, and no more than a 16th is kept in all."""
+    total, largest = host.number("host_total", ctypes.c_size_t), host.number("host_malloc_max", ctypes.c_size_t)
+    was, total.value = total.value, 16 << 30
+    host.error = 0
+    try:
+        c = context(host)
+        for slabs, edges in ((2000, 30000), (4000, 60000)):  # 0.5 and 1.9 GB of edges
+            host.plan = many(100000, edges, slabs)
+            sid = load(host, c, 4000, 8)
+            largest.value = 0
+            assert any("k_hit_count" in k for k in count(host, c, sid, 100000))
+            assert largest.value <= max(slabs * edges * 8, total.value // 64) + 4096
+            assert used(host, c) <= total.value // 16 + (16 << 20)
+        assert host.lib.fem_destroy(c) == 0
+    finally:
+        total.value = was
+
+
+def test_transfer_tables_make_room_for_a_stream(host):
+    """Under a budget a stream that fits beside the other one is loaded, whatever was counted
+    before."""
+    host.error = 0
+    host.plan = many(100000, 6000, 400)
+    c = context(host, 110 << 20)
+    sid = load(host, c, 4000, 8)
+    assert any("k_hit_count" in k for k in count(host, c, sid, 100000))
+    assert used(host, c) > 70 << 20
+    load(host, c, 4_000_000, 8)  # 55 MB
+    assert host.lib.fem_destroy(c) == 0
+
+
+def test_tables_make_room_for_a_server(host, ctx):
+    sid = load(host, ctx, 4000, 8)
+    assert any("k_hit_count" in k for k in count(host, ctx, sid))
+    v, before = vp(), used(host, ctx)
+    host.number("host_fail_malloc").value = 1
+    assert host.lib.fem_server_create(ctx, None, ctypes.byref(v)) == 0
+    assert used(host, ctx) < before
+    assert host.lib.fem_server_destroy(v) == 0
