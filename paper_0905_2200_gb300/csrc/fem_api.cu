@@ -3012,9 +3012,7 @@ int fem_batch_create(fem_ctx *c, const fem_job *jobs, uint32_t n_jobs, const fem
     c->ivl_host.assign(I, I + nI);
     {
         const size_t kept = b->allocs.size();
-        c->hits_busy = true;
         const int rch = batch_plan_hits(b, st, &b->over_hits);
-        c->hits_busy = false;
         if (rch != FEM_OK && rch != FEM_ENOMEM) return fail(rch);
         if (std::getenv("FEM_DEBUG"))
             std::fprintf(stderr, "fem: batch of %u candidates, %u streams: %s (%u slabs, %llu hits' room)\n",

@@ -44,6 +44,7 @@ class Host:
         self.launches = []
         self.plan = {}     # words of the next plans
         self.error = 0     # error word that the next counts publish
+        self.publish_seq = True  # else plans and validations publish it everywhere but in its place
         self.on_launch = ON_LAUNCH(self._launched)
         ctypes.c_void_p.in_dll(self.rt, "host_on_launch").value = ctypes.cast(self.on_launch,
                                                                               ctypes.c_void_p).value
@@ -69,14 +70,18 @@ class Host:
             host[arg(5, ctypes.c_uint32)] = arg(6, ctypes.c_uint32)
         elif "k_plan_scan" in name:
             p = arg(3, Publish)
-            for w in range(PLAN_WORDS):
-                p.host[w] = self.plan.get(w, 0)
-            p.host[PLAN_WORDS], p.host[PLAN_WORDS + 1] = 0, p.seq
+            self._words(p, PLAN_WORDS, self.plan)
         elif "k_publish_info" in name:
-            p = arg(2, Publish)
-            for w in range(3):
-                p.host[w] = self.plan.get(("info", w), 0)
-            p.host[PLAN_WORDS], p.host[PLAN_WORDS + 1] = 0, p.seq
+            self._words(arg(2, Publish), 3, {w: self.plan.get(("info", w), 0) for w in range(3)})
         elif "k_publish_count" in name:
             p = arg(1, Publish)
             p.host[0], p.host[1], p.host[2] = 0, self.error, p.seq
+
+    def _words(self, p, n, values):
+        if not self.publish_seq:
+            for w in range(PLAN_WORDS):
+                p.host[w] = p.seq
+            return
+        for w in range(n):
+            p.host[w] = values.get(w, 0)
+        p.host[PLAN_WORDS], p.host[PLAN_WORDS + 1] = 0, p.seq

@@ -222,3 +222,43 @@ def test_tables_make_room_for_a_server(host, ctx):
     assert host.lib.fem_server_create(ctx, None, ctypes.byref(v)) == 0
     assert used(host, ctx) < before
     assert host.lib.fem_server_destroy(v) == 0
+
+
+def test_tables_of_a_count_make_room_for_a_batch(host):
+    """A batch goes over hit tables of its own under a budget that the tables of an earlier count
+    would leave no room in."""
+    host.error = 0
+    host.plan = many(100000, 6000, 400)
+    c = context(host, 110 << 20)
+    sid = load(host, c, 4000, 8)
+    assert any("k_hit_count" in k for k in count(host, c, sid, 100000))
+    assert used(host, c) > 70 << 20
+    host.plan = many(40, 6000, 400)
+    jobs, kept = batch_jobs([sid, sid, sid])
+    at = len(host.launches)
+    b = create_batch(host, c, jobs)
+    assert any("k_hit_count_batch" in k for k in host.launches[at:])
+    assert host.lib.fem_batch_destroy(b) == 0
+    assert host.lib.fem_destroy(c) == 0
+
+
+def test_only_the_sequence_word_ends_a_wait(host, ctx):
+    """Whatever the published words are, also the sequence number that is waited for, the host
+    takes them when the word behind them says so and not before (here it never does)."""
+    sid = load(host, ctx, 4000, 8)
+    assert any("k_hit_count" in k for k in count(host, ctx, sid))
+    publish = host.publish_seq
+
+    def count_rc(m):
+        rec = fem.pack_episodes(np.full(m, 3), np.tile([0, 1, 2] + [0] * 5, (m, 1)), np.zeros((m, 7), int))
+        I, out = np.array([[0, 4000]], np.uint32), np.zeros(m, np.uint32)
+        return host.lib.fem_count_candidates(ctx, sid, rec.ctypes.data_as(vp), m, 0, I.ctypes.data_as(vp), 1, 0,
+                                             out.ctypes.data_as(vp), 0, None)
+
+    try:
+        host.publish_seq = False
+        assert count_rc(40) == -8   # the plan's words
+        assert count_rc(300) == -8  # a validation's
+    finally:
+        host.publish_seq = publish
+    assert count_rc(40) == 0
