@@ -989,11 +989,12 @@ bool known_dense(const fem_ctx *c, const StreamDev &s, const uint32_t *types) {
 // *ok = false where tables do not apply: repeated types, or a stream whose chunks do not
 // span the longest interval (the events before a slab are kept from its chunk and the one
 // before).
-// alloc(name, words, &pointer) gives the plan's device memory.
+// alloc(name, words, &pointer) gives the plan's device memory.  info: the words of a
+// validation (three of them).
 template <typename Alloc>
 int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
               uint32_t m, bool fine, const uint2 *d_ivl, uint32_t nI, int pass, cudaStream_t st,
-              HitPlan *pl, bool *ok, Alloc &&alloc) {
+              HitPlan *pl, bool *ok, Alloc &&alloc, uint32_t *info = nullptr) {
     *ok = false;
     uint64_t max_hi = 0;
     for (const fem_interval &iv : c->ivl_host) max_hi = std::max<uint64_t>(max_hi, iv.hi_us);
@@ -1005,6 +1006,7 @@ int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     a.n_ivl = nI;
     a.parts = std::min(nI, PLAN_PARTS);
     a.fine = fine;
+    a.runs = info != nullptr;
     a.cfirst = s.cfirst;
     a.t = s.t;
     a.n_chunks = s.n_chunks;
@@ -1029,12 +1031,19 @@ int hits_plan(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     const volatile uint32_t *w = c->h_small + kPlanWord;
     RET(wait_seq(w + PLAN_WORDS + 1, seq, st));
     RET(err_status(w[PLAN_WORDS]));
+    if (info) {
+        info[0] = 0, info[1] = w[PLAN_REP], info[2] = w[PLAN_RUNS];
+        for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N)
+            if (w[N - 1]) info[0] |= 1u << N;
+    }
+    const uint64_t span = (uint32_t)~w[PLAN_SPAN];
+    if (s.n_chunks > 1) s.least_span = std::min(s.least_span, span);
     if (w[PLAN_DENSE]) {
         if (std::getenv("FEM_DEBUG")) std::fprintf(stderr, "fem: hit tables of %u slabs: too dense\n", w[PLAN_SLABS]);
         return remember_dense(c, s, st);
     }
     if (w[PLAN_REP]) return FEM_OK;
-    if (s.n_chunks > 1 && (uint64_t)(uint32_t)~w[PLAN_SPAN] <= max_hi) return FEM_OK;
+    if (s.n_chunks > 1 && span <= max_hi) return FEM_OK;
     for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
         pl->len_m[N] = w[N - 1];
         pl->group_m[plan_group(N, a.fine)] += w[N - 1];
@@ -1134,12 +1143,12 @@ bool few_on_long(const StreamDev &s, uint32_t m, uint32_t longest) {
 // false, with nothing counted, where they do not apply.
 int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const uint32_t *gather,
                uint32_t m, const uint2 *d_ivl, uint32_t nI, int pass, uint32_t *out,
-               cudaStream_t st, bool *done, uint32_t *segments = nullptr) {
+               cudaStream_t st, bool *done, uint32_t *segments = nullptr, uint32_t *info = nullptr) {
     *done = false;
     HitPlan pl;
     bool ok;
     RET(hits_plan(c, s, cands, gather, m, m >= PLAN_FINE, d_ivl, nI, pass, st, &pl, &ok,
-                  [&](const char *n, size_t w, uint32_t **p) { return dbuf(c, n, w, p); }));
+                  [&](const char *n, size_t w, uint32_t **p) { return dbuf(c, n, w, p); }, info));
     if (!ok) return FEM_OK;
     uint32_t longest = 0;
     for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
@@ -1235,13 +1244,14 @@ int or_no_room(fem_ctx *c, int rc, bool *done, cudaStream_t st) {
 
 // Whether a set may be counted over hit tables: no configured kernel or ring size, no more
 // type pairs and intervals than are worth a table, and on average no more events of a type
-// in an interval than a word is for.
+// in an interval than a word is for; nor a stream known to have chunks shorter than an interval
+// (hits_plan).
 constexpr uint32_t kHitMaxEdges = 1u << 18;
 bool hits_eligible(const fem_ctx *c, const StreamDev &s, uint32_t nI) {
     uint64_t max_hi = 0;
     for (const fem_interval &iv : c->ivl_host) max_hi = std::max<uint64_t>(max_hi, iv.hi_us);
     return !c->cfg.kernel && !c->cfg.ring_capacity && c->d_plan && s.n_chunks && nI &&
-           (uint64_t)s.K * s.K * nI <= kHitMaxEdges &&
+           (uint64_t)s.K * s.K * nI <= kHitMaxEdges && (s.n_chunks == 1 || s.least_span > max_hi) &&
            (double)s.n * (double)max_hi <= 8.0 * s.K * (double)std::max(s.t_max - s.t_min, 1u);
 }
 
@@ -1391,8 +1401,11 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     uint32_t info[kInfoWords];
     bool hits = hits_eligible(c, s, nI), known = false;
     // a small set goes to the hit tables without a look at its runs (their plan validates
-    // too, and saves it a wait)
-    if (!hits || m >= 256 || !s.dense_hi.empty()) {
+    // too, and saves it a wait); where they turn out not to apply, the plan's words are the
+    // validation's (100 episodes with repeated types 338 us with a validation after the plan, 320
+    // so, 315 without tables; 200 of three nodes on 300,000 events 172, 127 and 141; 200 on a
+    // stream with chunks of 5 ms 513, 322 and 338)
+    if (!hits || m >= 256 || !s.dense_hi.empty() || few_on_long(s, m, FEM_MAX_LEN)) {
         RET(validate(c, s, cands, gather, m, nI, info, st));
         known = true;
         hits = hits && !info[1] && (!in_runs(info, m) || most_pairs(s, info, m, nI, pass));
@@ -1402,10 +1415,13 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     }
     if (hits) {
         bool done = false;
+        if (!known) info[0] = 0;
         c->hits_busy = true;
-        const int rc = count_hits(c, s, cands, gather, m, d_ivl, nI, pass, out, st, &done);
+        const int rc = count_hits(c, s, cands, gather, m, d_ivl, nI, pass, out, st, &done, nullptr,
+                                  known ? nullptr : info);
         RET(or_no_room(c, rc, &done, st));
         if (done) return FEM_OK;
+        known = known || info[0];  // (no plan was made where there was no room for it)
     }
     if (!known) RET(validate(c, s, cands, gather, m, nI, info, st));
     return count_validated(c, s, cands, gather, m, d_ivl, nI, pass, out, info, st);
@@ -1872,7 +1888,7 @@ int fem_append_stream(fem_ctx *c, int32_t id, const uint8_t *types, const uint32
             return FEM_ECUDA;
         }
         c->mem_used -= std::min(stream_bytes(s), c->mem_used);
-        g.dense_hi = std::move(s.dense_hi);
+        g.dense_hi = std::move(s.dense_hi), g.least_span = s.least_span;
         free_stream_buffers(s);
         g.n = n_old, g.K = K, g.n_chunks = ch_old, g.t_min = t_min, g.t_max = t_max_old;
         s = g;

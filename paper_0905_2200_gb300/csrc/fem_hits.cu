@@ -81,13 +81,19 @@ __device__ __forceinline__ uint32_t plan_bin(const fem_episode &e, const PlanArg
 // candidate's count does not depend on it), the bins' sizes, the edges in use, and the
 // plan words: per length 1..8 the candidates, [PLAN_REP] those with a repeated type,
 // [PLAN_SPAN] 2^32 - 1 less the least time that a chunk spans (and of k_plan_scan [PLAN_DENSE]:
-// an edge in use leads from a type too dense for the tables).
+// an edge in use leads from a type too dense for the tables), [PLAN_RUNS] where asked for.
 __global__ void __launch_bounds__(256) k_plan_bins(const PlanArgs a) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t rep = 0, bad = 0, len = 0;
+    uint32_t rep = 0, bad = 0, len = 0, brk = 0;
     if (i < a.m) {
         const fem_episode e = a.cands[a.gather ? a.gather[i] : i];
         const uint32_t N = e.len;
+        if (a.runs && i > 0) {  // a run of candidates sharing the prefix of a last node ends here
+            const fem_episode q = a.cands[a.gather ? a.gather[i - 1] : i - 1];
+            brk = q.len != N;
+            for (uint32_t k = 0; k + 1 < N && k < FEM_MAX_LEN; ++k) brk |= q.types[k] != e.types[k];
+            for (uint32_t k = 0; k + 2 < N && k < FEM_MAX_LEN - 1; ++k) brk |= q.ivl[k] != e.ivl[k];
+        }
         if (N < 1 || N > FEM_MAX_LEN) {
             bad = ERR_BADEP;
         } else {
@@ -115,8 +121,10 @@ __global__ void __launch_bounds__(256) k_plan_bins(const PlanArgs a) {
     }
     rep = __reduce_add_sync(0xffffffffu, rep);
     bad = __reduce_or_sync(0xffffffffu, bad);
+    brk = __reduce_add_sync(0xffffffffu, brk);
     if ((threadIdx.x & 31) == 0) {
         if (rep) atomicAdd(&a.words[PLAN_REP], rep);
+        if (brk) atomicAdd(&a.words[PLAN_RUNS], brk);
         if (bad) atomicOr(a.err, bad);
     }
     // the least span, over the whole grid
@@ -212,6 +220,7 @@ __global__ void __launch_bounds__(1024) k_plan_scan(const PlanArgs a, uint32_t b
         for (uint32_t k = 0; k < PLAN_EDGES; ++k) h[k] = a.words[k];
         h[PLAN_PARTS_MIN] = least;
         h[PLAN_DENSE] = dense;
+        h[PLAN_RUNS] = a.words[PLAN_RUNS];
         h[PLAN_EDGES] = n_edges;
         h[PLAN_SLABS] = n_slabs;
         h[PLAN_WORDS] = *reinterpret_cast<const volatile uint32_t *>(pub.err);

@@ -72,6 +72,9 @@ struct StreamDev {
     // word (2^32 - 1: none; empty: none of any type).  Appended events make no interval
     // emptier, so what was found stays true of a stream as long as it lives.
     mutable std::vector<uint32_t> dense_hi;
+    // the least time from a chunk's first event to the next one's, as far as it was looked at
+    // (likewise)
+    mutable uint64_t least_span = ~0ull;
 };
 
 // The hit tables of a stream, an edge set and a pass (fem_hits.cuh).
@@ -345,7 +348,7 @@ cudaError_t launch_join_gather(const uint32_t *cells, const fem_episode *cands, 
 // + plan_bins(K, parts) + K K n_ivl words.
 constexpr uint32_t PLAN_PARTS = 4, PLAN_GROUPS = 5, PLAN_FINE = 8192;
 constexpr uint32_t PLAN_REP = 8, PLAN_SPAN = 9, PLAN_EDGES = 10, PLAN_SLABS = 11, PLAN_PARTS_MIN = 12,
-                   PLAN_DENSE = 13, PLAN_WORDS = 14;
+                   PLAN_DENSE = 13, PLAN_RUNS = 14, PLAN_WORDS = 15;
 // The launch that counts an episode of N nodes: lengths 1-2, 3, 4, 5 and 6-8, since
 // registers and shared memory grow with the length; small sets (below PLAN_FINE), whose
 // launches are short, in three (1-3, 4-5, 6-8).
@@ -360,6 +363,7 @@ struct PlanArgs {
     uint32_t m, K, n_ivl;
     uint32_t parts;          // parts of the interval set (at most PLAN_PARTS, n_ivl)
     bool fine;               // plan_group's
+    bool runs;               // [PLAN_RUNS]: as info[2] of launch_validate_cands
     const uint32_t *cfirst, *t;
     uint32_t n_chunks;
     uint64_t n;

@@ -12,7 +12,7 @@ from paper_0905_2200_gb300 import build as fembuild
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 # words of a published plan (fem_internal.cuh)
-PLAN_EDGES, PLAN_SLABS, PLAN_PARTS_MIN, PLAN_WORDS = 10, 11, 12, 14
+PLAN_EDGES, PLAN_SLABS, PLAN_PARTS_MIN, PLAN_WORDS = 10, 11, 12, 15
 ON_LAUNCH = ctypes.CFUNCTYPE(None, ctypes.c_char_p, ctypes.POINTER(ctypes.c_void_p))
 
 
