@@ -161,8 +161,16 @@ int fem_set_config(fem_ctx *ctx, const fem_config *cfg);   /* NULL restores auto
  * the other block size), each a complete count with the same result, and caches
  * the fastest.  A class not cached and tuning off uses the rule.  An explicit
  * fem_set_config segment or block size overrides the cache.
+ * Where the rule takes the hit tables (FEM_KERNEL_HITS; they have no shape to choose), the
+ * count is timed over them and by the other kernels in their best shape, twice each, and the
+ * choice is cached under "distinct" 2 for sets that do not come in prefix runs (N = 0: several
+ * lengths) and 3 for fem_mine_levelwise's passes, "kernel" 4 for the tables.  A pass of
+ * fem_mine_levelwise whose class has a shape but no choice (a file of an earlier version)
+ * keeps that shape; other sets without a choice go by the rule.  Window frequencies are not
+ * tuned; a batch is where it does not go over the tables, when it is created.
  * fem_tune_save writes the cache as JSON lines
- *   {"key": "N/pass/distinct/log2m/log2chunks/K", "segments": P, "threads": T, "ms": t}
+ *   {"key": "N/pass/distinct/log2m/log2chunks/K", "segments": P, "threads": T, "ms": t,
+ *    "kernel": k}
  * and fem_tune_load merges such a file (FEM_EIO: cannot open/write; FEM_EINVAL:
  * a malformed line, nothing merged).  Host only, not thread safe per context.
  */

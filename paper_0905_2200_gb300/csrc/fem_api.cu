@@ -84,11 +84,11 @@ struct fem_ctx {
     cudaEvent_t kev[2][3] = {};
     int kev_flip = 0;
     // measured mapping choice: launch shape per (N, pass, distinct, log2 m,
-    // log2 chunks, K) class
+    // log2 chunks, K) class, and whether the class goes over hit tables
     struct Shape {
         uint32_t P, T;
         float ms;
-        uint32_t kernel;  // FEM_KERNEL_MACHINE or FEM_KERNEL_CHAIN
+        uint32_t kernel;  // FEM_KERNEL_MACHINE or FEM_KERNEL_CHAIN; a choice: _HITS or _MACHINE
     };
     std::map<std::string, Shape> tune;
     bool tune_on = false, tuning = false;
@@ -494,10 +494,13 @@ uint32_t chain_threads(uint32_t) { return 256u; }
 
 // The class a measured launch shape is kept for: counts of the same length,
 // pass and type structure, with m and the stream length in the same power-of-two
-// range and the same type count, map alike.
-std::string tune_key(int N, int pass, bool distinct, uint32_t m, uint32_t n_chunks, uint32_t K) {
+// range and the same type count, map alike.  Besides the shapes of the other kernels (distinct
+// types or not), the choice between these and the hit tables is kept, for sets that do not
+// come in runs (kind 2; N = 0: of several lengths) and for mining's levels (kind 3).
+constexpr int kTuneSet = 2, kTuneLevel = 3;
+std::string tune_key(int N, int pass, int kind, uint32_t m, uint32_t n_chunks, uint32_t K) {
     char b[96];
-    std::snprintf(b, sizeof(b), "%d/%d/%d/%u/%u/%u", N, pass, distinct ? 1 : 0, ceil_log2(m),
+    std::snprintf(b, sizeof(b), "%d/%d/%d/%u/%u/%u", N, pass, kind, ceil_log2(m),
                   ceil_log2(n_chunks), K);
     return b;
 }
@@ -1152,10 +1155,7 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
     if (!ok) return FEM_OK;
     uint32_t longest = 0;
     for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
-        if (!pl.len_m[N]) continue;
-        longest = N;
-        // (a shape measured for the other kernels)
-        if (c->tune.count(tune_key((int)N, pass, true, pl.len_m[N], s.n_chunks, s.K))) return FEM_OK;
+        if (pl.len_m[N]) longest = N;
     }
     if (few_on_long(s, m, longest)) return FEM_OK;
     uint32_t *tmp;
@@ -1253,6 +1253,45 @@ bool hits_eligible(const fem_ctx *c, const StreamDev &s, uint32_t nI) {
     return !c->cfg.kernel && !c->cfg.ring_capacity && c->d_plan && s.n_chunks && nI &&
            (uint64_t)s.K * s.K * nI <= kHitMaxEdges && (s.n_chunks == 1 || s.least_span > max_hi) &&
            (double)s.n * (double)max_hi <= 8.0 * s.K * (double)std::max(s.t_max - s.t_min, 1u);
+}
+
+// Whether a set that the rule sends over the hit tables goes there (*use): as measured for its
+// class, or, with tuning on and nothing measured, as two counts of either kind tell, each of
+// them complete (others(), tables(&done)).  The tables stay unless the other kernels are at
+// least 2% faster.  A configured launch shape leaves the rule's choice.
+template <typename Others, typename Tables>
+int tuned_route(fem_ctx *c, const std::string &key, cudaStream_t st, bool *use, Others &&others,
+                Tables &&tables) {
+    if (c->cfg.segments || c->cfg.threads_per_block) return FEM_OK;
+    auto it = c->tune.find(key);
+    if (it == c->tune.end() && c->tune_on && !c->tuning) {
+        float ms[2] = {-1.f, -1.f};  // (the first of the others also measures their shapes)
+        for (int k : {0, 1, 0, 1}) {
+            CK(cudaStreamSynchronize(st));
+            const auto t0 = std::chrono::steady_clock::now();
+            bool done = true;
+            const int rc = k ? tables(&done) : others();
+            if (rc == FEM_EOVERFLOW && !k) {  // (the others cannot count it at all)
+                CK(cudaMemsetAsync(c->d_err, 0, sizeof(uint32_t), st));
+                return FEM_OK;
+            }
+            RET(rc);
+            if (!done) {
+                *use = false;
+                return FEM_OK;
+            }
+            CK(cudaStreamSynchronize(st));
+            const float t = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();
+            if (ms[k] < 0 || t < ms[k]) ms[k] = t;
+        }
+        const bool hits = !(ms[0] < 0.98f * ms[1]);
+        it = c->tune.emplace(key, fem_ctx::Shape{1, 32, ms[hits], hits ? (uint32_t)FEM_KERNEL_HITS
+                                                                      : (uint32_t)FEM_KERNEL_MACHINE}).first;
+        if (std::getenv("FEM_DEBUG"))
+            std::fprintf(stderr, "fem: class %s: other kernels %.3f ms, tables %.3f ms\n", key.c_str(), ms[0], ms[1]);
+    }
+    if (it != c->tune.end()) *use = it->second.kernel == FEM_KERNEL_HITS;
+    return FEM_OK;
 }
 
 // One pass of level 3 over m candidates of the frequent pairs F, all pairs at once (k_join):
@@ -1405,7 +1444,8 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     // validation's (100 episodes with repeated types 338 us with a validation after the plan, 320
     // so, 315 without tables; 200 of three nodes on 300,000 events 172, 127 and 141; 200 on a
     // stream with chunks of 5 ms 513, 322 and 338)
-    if (!hits || m >= 256 || !s.dense_hi.empty() || few_on_long(s, m, FEM_MAX_LEN)) {
+    if (!hits || m >= 256 || !s.dense_hi.empty() || few_on_long(s, m, FEM_MAX_LEN) || c->tune_on ||
+        !c->tune.empty()) {
         RET(validate(c, s, cands, gather, m, nI, info, st));
         known = true;
         hits = hits && !info[1] && (!in_runs(info, m) || most_pairs(s, info, m, nI, pass));
@@ -1413,13 +1453,22 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
         while (longest > 1 && !(info[0] >> longest & 1u)) --longest;
         hits = hits && !few_on_long(s, m, longest) && !known_dense(c, s, info + 3);
     }
+    auto tables = [&](bool *done) {
+        c->hits_busy = true;
+        const int rc = count_hits(c, s, cands, gather, m, d_ivl, nI, pass, out, st, done, nullptr,
+                                  known ? nullptr : info);
+        return or_no_room(c, rc, done, st);
+    };
+    if (hits && known) {
+        const int N = __builtin_popcount(info[0]) == 1 ? __builtin_ctz(info[0]) : 0;
+        RET(tuned_route(c, tune_key(N, pass, kTuneSet, m, s.n_chunks, s.K), st, &hits,
+                        [&] { return count_validated(c, s, cands, gather, m, d_ivl, nI, pass, out, info, st); },
+                        tables));
+    }
     if (hits) {
         bool done = false;
         if (!known) info[0] = 0;
-        c->hits_busy = true;
-        const int rc = count_hits(c, s, cands, gather, m, d_ivl, nI, pass, out, st, &done, nullptr,
-                                  known ? nullptr : info);
-        RET(or_no_room(c, rc, &done, st));
+        RET(tables(&done));
         if (done) return FEM_OK;
         known = known || info[0];  // (no plan was made where there was no room for it)
     }
@@ -1728,7 +1777,9 @@ int fem_tune_load(fem_ctx *c, const char *path) {
         bool good = nf == 5 && P != 0 && T != 0 && T <= 256 && T % 8 == 0;
         if (good && close == ',') {  // with the kernel field
             good = std::sscanf(std::strstr(line, "\"ms\""), "\"ms\": %*f, \"kernel\": %u}", &K) == 1 &&
-                   (K == FEM_KERNEL_MACHINE || K == FEM_KERNEL_CHAIN);
+                   (K == FEM_KERNEL_MACHINE || K == FEM_KERNEL_CHAIN || K == FEM_KERNEL_HITS);
+            int kind = 0;  // (tables are a choice, not a shape)
+            if (K == FEM_KERNEL_HITS) good = good && std::sscanf(key, "%*d/%*d/%d", &kind) == 1 && kind >= kTuneSet;
         } else if (good) {
             good = close == '}';
         }
@@ -2355,19 +2406,42 @@ int fem_mine_levelwise_ex(fem_ctx *c, int32_t id, const fem_interval *I, uint32_
         bool joined = false, counted = false;
         HitPlan hp;
         auto tables = [&] { return !repeats && !known_dense(c, s, ftypes_h); };
-        if (N == 3 && tables() && m >= kJoinCandidates && hits_eligible(c, s, nI) &&
-            (uint64_t)s.K * s.K * nI * s.K * nI <= kJoinCells &&
-            !c->tune.count(tune_key(3, FEM_PASS_RELAXED, true, m, s.n_chunks, s.K))) {
+        // a pass over hit tables: the join of all pairs, or candidate by candidate
+        auto over_tables = [&](bool join, bool planned, const uint32_t *g, uint32_t mm, int pass, uint32_t *o,
+                               PassLaunch *pt, bool *done) {
             c->hits_busy = true;
-            const int rc = join_pass(c, s, &hp, false, F, staged_f[2], cands, nullptr, m, d_ivl, nI,
-                                     FEM_PASS_RELAXED, rel, st, &plr, &joined);
-            RETF(or_no_room(c, rc, &joined, st));
-            counted = joined;
-        } else if (tables() && !(N == 2 && pairs_level2) && level_by_hits(c, s, N, m, nI)) {
-            c->hits_busy = true;
-            const int rc = level_hits(c, s, cands, nullptr, m, (int)N, d_ivl, nI, FEM_PASS_RELAXED, rel,
-                                      st, &plr, &counted);
-            RETF(or_no_room(c, rc, &counted, st));
+            const int rc = join ? join_pass(c, s, &hp, planned, F, staged_f[2], cands, g, mm, d_ivl, nI, pass,
+                                            o, st, pt, done)
+                                : level_hits(c, s, cands, g, mm, (int)N, d_ivl, nI, pass, o, st, pt, done);
+            return or_no_room(c, rc, done, st);
+        };
+        // whether it runs, where the rule says so: not if a shape of the other kernels is cached
+        // for the class and no choice is; else as tuned_route finds
+        auto chosen = [&](bool join, bool planned, const uint32_t *g, uint32_t mm, int pass, uint32_t *o,
+                          bool *use) -> int {
+            *use = true;
+            const std::string key = tune_key((int)N, pass, kTuneLevel, mm, s.n_chunks, s.K);
+            if (!c->tune.count(key) && c->tune.count(tune_key((int)N, pass, 1, mm, s.n_chunks, s.K))) {
+                *use = false;
+                return FEM_OK;
+            }
+            return tuned_route(c, key, st, use,
+                               [&] {
+                                   return count_pass(c, s, cands, g, mm, (int)N, d_ivl, nI, pass, o, true, st,
+                                                     nullptr);
+                               },
+                               [&](bool *done) {
+                                   PassLaunch pt;
+                                   return over_tables(join, planned, g, mm, pass, o, &pt, done);
+                               });
+        };
+        bool use = false;
+        const bool join = N == 3 && m >= kJoinCandidates && hits_eligible(c, s, nI) &&
+                          (uint64_t)s.K * s.K * nI * s.K * nI <= kJoinCells;
+        if (tables() && (join || (!(N == 2 && pairs_level2) && level_by_hits(c, s, N, m, nI)))) {
+            RETF(chosen(join, false, nullptr, m, FEM_PASS_RELAXED, rel, &use));
+            if (use) RETF(over_tables(join, false, nullptr, m, FEM_PASS_RELAXED, rel, &plr, &counted));
+            joined = join && counted;
         }
         if (!counted) plr = PassLaunch{};
         if (counted) {
@@ -2400,16 +2474,10 @@ int fem_mine_levelwise_ex(fem_ctx *c, int32_t id, const fem_interval *I, uint32_
         PassLaunch plx;
         cudaEventRecord(c->ev[6], st);
         counted = false;
-        if (joined && ms >= kJoinCandidates / 2) {
-            c->hits_busy = true;
-            const int rc = join_pass(c, s, &hp, true, F, staged_f[2], cands, idx_s, ms, d_ivl, nI,
-                                     FEM_PASS_EXACT, ex, st, &plx, &counted);
-            RETF(or_no_room(c, rc, &counted, st));
-        } else if (tables() && level_by_hits(c, s, N, ms, nI)) {
-            c->hits_busy = true;
-            const int rc = level_hits(c, s, cands, idx_s, ms, (int)N, d_ivl, nI, FEM_PASS_EXACT, ex, st,
-                                      &plx, &counted);
-            RETF(or_no_room(c, rc, &counted, st));
+        const bool again = joined && ms >= kJoinCandidates / 2;
+        if (again || (tables() && level_by_hits(c, s, N, ms, nI))) {
+            RETF(chosen(again, true, idx_s, ms, FEM_PASS_EXACT, ex, &use));
+            if (use) RETF(over_tables(again, true, idx_s, ms, FEM_PASS_EXACT, ex, &plx, &counted));
         }
         if (!counted) plx = PassLaunch{};
         if (counted)
