@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -1130,16 +1131,70 @@ int hits_check(fem_ctx *c, const StreamDev &s, HitPlan *pl, uint32_t *e, bool *a
     return FEM_OK;
 }
 
-// A few short episodes of many types on a long stream: the tables, whose cost is that of
-// events and types, cost more than the per-thread machine's count, whose is that of
-// segments and nodes (machine / tables, us: 571 episodes of five nodes, 57 types, 736,000
-// events 505 / 736; 266 of three and four, 53 types, 1.06 million, two passes 834 / 1,102;
-// 320 of three, 38 types, 353,000 285 / 296; 746 of five to seven, 49 types, 911,000, two
-// passes 3,224 / 1,572; 167 of four, 18 types, 635,000, two passes 968 / 706; 1,756 of two
-// to four, 60 types, 79,000, two passes 538 / 391)
-bool few_on_long(const StreamDev &s, uint32_t m, uint32_t longest) {
-    return (uint64_t)m * longest < 5ull * s.K * s.K && (uint64_t)s.K * s.K > 400ull * longest &&
-           (uint64_t)s.n * s.K > 10000000;
+// What a count takes in microseconds, over hit tables and by the other kernels.  The tables'
+// cost is that of the edges a set may use (the plan numbers them), of events times types (the
+// build, whose blocks share an SM as their rank rows leave room) and of hits (build and count);
+// the other kernels' is that of a launch and a wait for each length, of events times nodes,
+// and of an event's look-back for every length.  Fits to 3,680 counts of 100 to 60,000 episodes
+// of one length (2 to 7) or several, on 500 to 3 million events of 8 to 200 types at 5 to 55
+// Hz, both passes by both ways: half of the estimates within 12%, nine of ten within 33
+// (tables) and 38%.  By the faster estimate 66 of those counts (and 19 of 400 others) take more
+// than 5% longer than by the other kernels, 1.7 (1.2) times at most; over tables wherever they
+// apply 1,604 would, up to 14 times (5,000 events of 128 types, 2,000 pairs, relaxed: 116 us
+// and 270).  Over the 400 others the counts are 1.68 times as fast as without tables.
+constexpr double kPlanEdgeUs = 1.05e-3;  // a plan, per type pair and interval
+double events_in_interval(const fem_ctx *c, const StreamDev &s) {  // of a type, in the longest
+    uint64_t max_hi = 0;
+    for (const fem_interval &iv : c->ivl_host) max_hi = std::max<uint64_t>(max_hi, iv.hi_us);
+    return (double)s.n * (double)max_hi / ((double)s.K * (double)std::max(s.t_max - s.t_min, 1u));
+}
+
+struct SetSize {  // candidates per length
+    double len_m[FEM_MAX_LEN + 1] = {};
+};
+SetSize equal_parts(uint32_t lens, uint32_t m) {  // of the lengths in a mask
+    SetSize z;
+    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N)
+        if (lens >> N & 1u) z.len_m[N] = (double)m / __builtin_popcount(lens);
+    return z;
+}
+
+double tables_us(const fem_ctx *c, const StreamDev &s, uint32_t nI, const SetSize &z, int pass) {
+    const bool x = pass == FEM_PASS_EXACT;
+    const double K = s.K, n = (double)s.n, pairs = K * K, in = events_in_interval(c, s);
+    double m = 0, nodes = 0;
+    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) m += z.len_m[N], nodes += N * z.len_m[N];
+    const double edges = nodes - m;  // (of all episodes, some of them the same)
+    const double used = std::min(1.0, edges / (pairs * nI)), groups = std::min(1.0, edges * std::min(K, 32.0) / pairs);
+    // blocks of a build on an SM (at least four by registers): 719 bytes a type (build_smem)
+    const double blocks = std::max(1.0, std::min(4.0, std::floor(232448.0 / (719 * K + 1024))));
+    return (x ? 147 : 156) + kPlanEdgeUs * pairs * nI +
+           4 / blocks * n * K * (3.1e-6 * groups + (x ? 1.65e-5 : 2.2e-5) * used * in) +
+           (x ? 1.05e-6 : 1.6e-6) * nodes * n / K * in + 7e-4 * m;
+}
+
+double others_us(const fem_ctx *c, const StreamDev &s, const SetSize &z, int pass) {
+    const bool x = pass == FEM_PASS_EXACT;
+    const double each = (double)s.n / s.K;  // events of a type
+    double us = 0;
+    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
+        const double m = z.len_m[N];
+        if (m <= 0) continue;
+        const double segments = std::max(1.0, std::min(c->sm_count * 2048.0 / m, (double)s.n / CHUNK));
+        us += (x ? 38 + 13.0 * N : 52 + 6.0 * N) + (s.n_chunks > 1 ? (x ? 32 : 41) : 0) +
+              (x ? 2.08e-6 : 5.95e-7) * m * N * N * each + (x ? 0.28 : 0.207) * N * each / segments;
+    }
+    return us;
+}
+
+// A set of fewer candidates is planned for the tables without a validation before (one wait
+// less where they do count it), unless the plan, whose edges are scanned by one block, costs
+// far more than that, or a mixed set of that size would not go over them.
+constexpr uint32_t kPlanFirst = 256;
+constexpr double kPlanUs = 20;  // a plan over a validation
+bool plan_first(const fem_ctx *c, const StreamDev &s, uint32_t m, uint32_t nI, int pass) {
+    const SetSize z = equal_parts(1u << 2 | 1u << 3 | 1u << 4, m);
+    return m < kPlanFirst && kPlanEdgeUs * s.K * s.K * nI < 25 && tables_us(c, s, nI, z, pass) < others_us(c, s, z, pass);
 }
 
 // Count a candidate set over hit tables: all lengths, in an order of their own.  *done =
@@ -1153,11 +1208,11 @@ int count_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
     RET(hits_plan(c, s, cands, gather, m, m >= PLAN_FINE, d_ivl, nI, pass, st, &pl, &ok,
                   [&](const char *n, size_t w, uint32_t **p) { return dbuf(c, n, w, p); }, info));
     if (!ok) return FEM_OK;
-    uint32_t longest = 0;
-    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) {
-        if (pl.len_m[N]) longest = N;
+    if (info) {  // (nothing was known of the set; the plan is made now, whichever way it goes)
+        SetSize z;
+        for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N) z.len_m[N] = pl.len_m[N];
+        if (others_us(c, s, z, pass) + kPlanUs + kPlanEdgeUs * s.K * s.K * nI < tables_us(c, s, nI, z, pass)) return FEM_OK;
     }
-    if (few_on_long(s, m, longest)) return FEM_OK;
     uint32_t *tmp;
     uint8_t *redo;
     RET(dbuf(c, "hit_plan_out", m, &tmp));
@@ -1442,16 +1497,15 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     // a small set goes to the hit tables without a look at its runs (their plan validates
     // too, and saves it a wait); where they turn out not to apply, the plan's words are the
     // validation's (100 episodes with repeated types 338 us with a validation after the plan, 320
-    // so, 315 without tables; 200 of three nodes on 300,000 events 172, 127 and 141; 200 on a
-    // stream with chunks of 5 ms 513, 322 and 338)
-    if (!hits || m >= 256 || !s.dense_hi.empty() || few_on_long(s, m, FEM_MAX_LEN) || c->tune_on ||
-        !c->tune.empty()) {
+    // so, 315 without tables; 200 on a stream with chunks of 5 ms 513, 322 and 338)
+    if (!hits || !plan_first(c, s, m, nI, pass) || !s.dense_hi.empty() || c->tune_on || !c->tune.empty()) {
         RET(validate(c, s, cands, gather, m, nI, info, st));
         known = true;
-        hits = hits && !info[1] && (!in_runs(info, m) || most_pairs(s, info, m, nI, pass));
-        uint32_t longest = FEM_MAX_LEN;
-        while (longest > 1 && !(info[0] >> longest & 1u)) --longest;
-        hits = hits && !few_on_long(s, m, longest) && !known_dense(c, s, info + 3);
+        hits = hits && !info[1] && !known_dense(c, s, info + 3);
+        if (hits && !most_pairs(s, info, m, nI, pass)) {
+            const SetSize z = equal_parts(info[0], m);
+            hits = (m < kPlanFirst || !in_runs(info, m)) && tables_us(c, s, nI, z, pass) < others_us(c, s, z, pass);
+        }
     }
     auto tables = [&](bool *done) {
         c->hits_busy = true;

@@ -29,7 +29,7 @@ CASES = {  # stream, types, candidates, launches more than with the per-thread k
     "repeated types": (lambda: stream(5, 6000, 16, gap=1500), 16,
                        lambda: repeated(synth.random_candidates(1, 100, 16, [2, 3], 4)), 2),
     "few on a long stream": (lambda: stream(6, 160000, 64, gap=1000), 64,
-                             lambda: synth.random_candidates(1, 200, 64, [3], 4), 0),
+                             lambda: synth.random_candidates(1, 200, 64, [3], 4), 2),
     "short chunks": (lambda: lumps(40000, 250), 250, lambda: synth.random_candidates(1, 200, 250, [3], 4), 0),
 }
 
