@@ -1187,6 +1187,21 @@ double others_us(const fem_ctx *c, const StreamDev &s, const SetSize &z, int pas
     return us;
 }
 
+// The same of window frequencies, whose other kernel has one thread per episode walk the whole
+// stream, one length after the other (us by that kernel / over tables: 2,000 pairs on 1,000
+// events of 64 types 110 / 137, of four nodes 160 / 144; pairs of 128 types on 1,000 events 93 /
+// 183, on 3,400 139 / 204, on 20,000 431 / 224; 100 pairs of 16 types on 100 events 87 / 108, on
+// 1,000 208 / 117).
+bool windows_over_tables(const StreamDev &s, uint32_t nI, uint32_t lens, uint32_t m) {
+    const double K = s.K, n = (double)s.n;
+    double others = 52;
+    uint32_t most = 1;
+    for (uint32_t N = 1; N <= FEM_MAX_LEN; ++N)
+        if (lens >> N & 1u) others += 20 + (0.7 + 0.1 * N) * N * n / K + 10.0 * s.n_chunks, most = N;
+    const double groups = std::min(1.0, (double)m * (most - 1) * std::min(K, 32.0) / (K * K));
+    return 108 + 0.6e-3 * K * K * nI + 3e-3 * K * K * groups + 4e-3 * m < others;
+}
+
 // A set of fewer candidates is planned for the tables without a validation before (one wait
 // less where they do count it), unless the plan, whose edges are scanned by one block, costs
 // far more than that, or a mixed set of that size would not go over them.
@@ -2257,11 +2272,14 @@ int fem_count_windows(fem_ctx *c, int32_t id, const fem_episode *cands, uint32_t
     RET(validate(c, *s, dc, nullptr, m, nI, info, st));
     if (info[1]) return FEM_EINVAL;  // distinct types only
     bool done = false;
-    if (hits_eligible(c, *s, nI) && !known_dense(c, *s, info + 3)) {
+    auto tables = [&]() -> int {
         c->hits_busy = true;
         const int rc = windows_hits(c, *s, dc, m, d_ivl, nI, window_us, dout, st, &done);
-        RET(or_no_room(c, rc, &done, st));
-    }
+        return or_no_room(c, rc, &done, st);
+    };
+    const bool eligible = hits_eligible(c, *s, nI) && !known_dense(c, *s, info + 3);
+    const bool first = eligible && windows_over_tables(*s, nI, info[0], m);
+    if (first) RET(tables());
     if (!done) {
         WindowParams p{};
         p.bev = s->bev;
@@ -2276,8 +2294,14 @@ int fem_count_windows(fem_ctx *c, int32_t id, const fem_episode *cands, uint32_t
         p.err = c->d_err;
         CK(launch_count_windows(p, info[0], st));
         RET(read_err(c, st, &e));
-        if (e & ERR_RING) return FEM_EOVERFLOW;
-        RET(err_status(e));
+        if (e & ERR_RING) {  // (its lists ran over: the tables, where they were not tried)
+            if (!eligible || first) return FEM_EOVERFLOW;
+            CK(cudaMemsetAsync(c->d_err, 0, 4, st));
+            RET(tables());
+            if (!done) return FEM_EOVERFLOW;
+        } else {
+            RET(err_status(e));
+        }
     }
     if (!counts_on_device) {
         CK(cudaMemcpyAsync(counts_out, dout, (size_t)m * 8, cudaMemcpyDeviceToHost, st));
