@@ -2905,6 +2905,49 @@ int batch_tune(fem_batch *b, cudaStream_t st) {
     return FEM_OK;
 }
 
+// Whether a batch of these jobs (and streams) is estimated to run faster over hit tables than by
+// the other kernels, in microseconds a run: over tables, building them for both passes (the
+// events times types of all streams, and a block's share where there are few slabs) and the
+// hits; by the others, per length a launch of items whose longest goes through 16 chunks,
+// and all events times nodes.  Fits to 260 batches of 1 to 48 jobs of 20 to 15,000
+// candidates on streams of 4 to 128 types, 3 s to 10 min: half of the estimates within 18 and
+// 28%, nine of ten within 55 and 95%; by them four batches take more than 5% longer than by the other
+// kernels, 1.6 times at most, where over tables 76 did, up to 13 times (32 jobs of 1,000
+// episodes of five nodes on 32 half-minutes of 128 types: 0.54 and 5.2 ms).
+bool batch_over_tables(const fem_ctx *c, const std::vector<fem_job> &jobs, uint32_t nI) {
+    struct Stream {
+        const StreamDev *s = nullptr;
+        double edges = 0;
+    };
+    std::map<int32_t, Stream> streams;
+    double hits = 0, m = 0, work = 0, longest[FEM_MAX_LEN + 1] = {};
+    for (const fem_job &jb : jobs) {
+        if (!jb.m) continue;
+        Stream &st = streams[jb.stream_id];
+        st.s = &c->streams.at(jb.stream_id);
+        const double each = (double)st.s->n / st.s->K, N = jb.len;
+        st.edges += (double)jb.m * (N - 1);
+        hits += jb.m * N * each * events_in_interval(c, *st.s);
+        work += jb.m * N * N * each;
+        m += jb.m;
+        longest[jb.len] = std::max(longest[jb.len], N * std::min(each, 16.0 * CHUNK / st.s->K));
+    }
+    double tables = 105 + 2.5e-6 * hits + 1.6e-3 * m, block = 0, dense = 0;
+    for (const auto &kv : streams) {
+        const StreamDev &s = *kv.second.s;
+        const double K = s.K, n = (double)s.n, in = events_in_interval(c, s);
+        const double groups = std::min(1.0, kv.second.edges * std::min(K, 32.0) / (K * K));
+        const double used = std::min(1.0, kv.second.edges / (K * K * std::max(nI, 1u)));
+        tables += n * K * (8.1e-6 * groups + 3.5e-5 * used * in) + 2.7e-5 * s.n_chunks * K * K * groups;
+        block = std::max(block, 0.05 * K * K * groups);
+        dense = std::max(dense, 9.4e-3 * std::min<double>(n, CHUNK) * K * used * in);
+    }
+    double others = 3.1e-3 * m + 7.4e-7 * work;
+    for (double l : longest)
+        if (l > 0) others += 57 + 0.25 * l;
+    return 0.9 * (tables + block + dense) < others;
+}
+
 // Plans a batch over hit tables and runs it once; *ok = false, with its memory given back,
 // where tables do not apply to one of the streams or their memory would pass an eighth of
 // the device's (or the context's budget).
@@ -2913,6 +2956,7 @@ int batch_plan_hits(fem_batch *b, cudaStream_t st, bool *ok) {
     fem_ctx *c = b->ctx;
     BatchHits &h = b->hits;
     const uint32_t nI = b->nI;
+    if (!batch_over_tables(c, b->jobs, nI)) return FEM_OK;
     size_t free_bytes = 0, total_bytes = 0;
     CK(cudaMemGetInfo(&free_bytes, &total_bytes));
     const uint64_t most = std::min(total_bytes / 8, free_bytes / 2);

@@ -21,7 +21,7 @@ def recording():
 
 def job(torch, sid, cands, theta):
     m = len(cands[0])
-    return dict(stream_id=sid, len=8, theta=theta, cands=torch.from_numpy(fem.pack_episodes(*cands)).cuda(),
+    return dict(stream_id=sid, len=int(cands[0][0]), theta=theta, cands=torch.from_numpy(fem.pack_episodes(*cands)).cuda(),
                 exact_out=torch.zeros(m, dtype=torch.int32, device="cuda"),
                 survived_out=torch.zeros(m, dtype=torch.uint8, device="cuda"))
 
@@ -37,9 +37,10 @@ def test_only_the_flagged_jobs_are_counted_again(monkeypatch, capfd):
         m = 20
         flagged = (np.full(m, 8), np.stack([rng.permutation(8) for _ in range(m)]),
                    np.ones((m, 7), int))
-        quiet = [(np.full(50 + k, 8),
-                  np.stack([8 + rng.permutation(K - 8)[:8] for _ in range(50 + k)]),
-                  rng.integers(0, 2, (50 + k, 7))) for k in range(24)]
+        # (lengths 6 and 7, counted by the same launch)
+        quiet = [(np.full(50 + k, 6 + k % 2),
+                  np.stack([8 + rng.permutation(K - 8)[:8] for _ in range(50 + k)]) * (np.arange(8) < 6 + k % 2),
+                  rng.integers(0, 2, (50 + k, 7)) * (np.arange(7) < 5 + k % 2)) for k in range(24)]
         launches = []
         for sets in (quiet, [flagged] + quiet[:1], quiet[:-1] + [flagged] + quiet[-1:]):
             jobs = [job(torch, sid, c, 1) for c in sets]
