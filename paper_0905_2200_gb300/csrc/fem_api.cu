@@ -1441,12 +1441,22 @@ int level_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
 // 340 / 127.  At level 2 (every type pair or most of them) the other kernels fill the device
 // from about 1,000 candidates on: 239 pairs of 16 types, 4,000 events 290 / 96; 810 of 18,
 // 6,200 events 155 / 112; 952 of 19, 64,000 events 155 / 146; 1,397 of 39, 101,000 events
-// 95 / 172; 3,435 of 40, 20,000 events 104 / 144; 6,593 of 61, 179,000 events 145 / 192.  With a segment count configured, level 2 keeps its kernels.
-bool level_by_hits(const fem_ctx *c, const StreamDev &s, uint32_t N, uint32_t m, uint32_t nI) {
+// 95 / 172; 3,435 of 40, 20,000 events 104 / 144; 6,593 of 61, 179,000 events 145 / 192.  With a segment
+// count configured, level 2 keeps its kernels.  (On recordings without structure the others
+// need no recounts, and up to 64 candidates take 20 to 80 us there and 80 to 110 over tables; on
+// those with embedded chains that choice made whole searches up to 1.6 times slower, 841 to 1,351
+// us for one of 10 s.)  Large relaxed sets of four nodes and more, whose prefixes the
+// latest-chain kernel shares: 4.9 million on 80,000 events of 48 types 17.2 ms / 53.1, 1.3
+// million on 10,000 of 32 0.86 / 2.54, 57,000 on 406,000 of 64 1.28 / 2.10; from a thousand
+// million (candidates x events) on the difference is more than the recounts.  Type pairs and
+// intervals beyond 16,384 add a plan's time (548 episodes on 1,500 events of 200 types 88 / 285).
+bool level_by_hits(const fem_ctx *c, const StreamDev &s, uint32_t N, int pass, uint32_t m, uint32_t nI) {
     if (!hits_eligible(c, s, nI) || m == 0) return false;
-    const double cells = (double)s.n * s.K;
+    const double cells = (double)s.n * s.K, work = (double)m * N * (double)s.n / s.K;
     if (N == 2) return !c->cfg.segments && m <= 1000 && cells <= 1.5e6;
-    return 13 * cells <= 40e6 + (double)m * N * (double)s.n / s.K;
+    if (N >= 4 && pass == FEM_PASS_RELAXED && m >= kChainLargeSet && work >= 1e9) return false;
+    const double edges = (double)s.K * s.K * nI;
+    return 13 * cells + 2.3e3 * std::max(0.0, edges - 16384) <= 40e6 + work;
 }
 
 // Level 3 joins all pairs of frequent pairs from this many candidates on, with at most so
@@ -2516,7 +2526,7 @@ int fem_mine_levelwise_ex(fem_ctx *c, int32_t id, const fem_interval *I, uint32_
         bool use = false;
         const bool join = N == 3 && m >= kJoinCandidates && hits_eligible(c, s, nI) &&
                           (uint64_t)s.K * s.K * nI * s.K * nI <= kJoinCells;
-        if (tables() && (join || (!(N == 2 && pairs_level2) && level_by_hits(c, s, N, m, nI)))) {
+        if (tables() && (join || (!(N == 2 && pairs_level2) && level_by_hits(c, s, N, FEM_PASS_RELAXED, m, nI)))) {
             RETF(chosen(join, false, nullptr, m, FEM_PASS_RELAXED, rel, &use));
             if (use) RETF(over_tables(join, false, nullptr, m, FEM_PASS_RELAXED, rel, &plr, &counted));
             joined = join && counted;
@@ -2553,7 +2563,7 @@ int fem_mine_levelwise_ex(fem_ctx *c, int32_t id, const fem_interval *I, uint32_
         cudaEventRecord(c->ev[6], st);
         counted = false;
         const bool again = joined && ms >= kJoinCandidates / 2;
-        if (again || (tables() && level_by_hits(c, s, N, ms, nI))) {
+        if (again || (tables() && level_by_hits(c, s, N, FEM_PASS_EXACT, ms, nI))) {
             RETF(chosen(again, true, idx_s, ms, FEM_PASS_EXACT, ex, &use));
             if (use) RETF(over_tables(again, true, idx_s, ms, FEM_PASS_EXACT, ex, &plx, &counted));
         }
