@@ -874,8 +874,8 @@ int count_pass(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const u
 // eight slabs or more (a segment first goes through the window before it) unless that
 // would leave SMs without a block.  And segments whose tables stay in a part of the L2
 // cache while the blocks of all candidates, which run next to each other, read them (the
-// hour-long recording, 481 KB a slab: 168 ms with 240 segments,
-// 300 with eight).
+// hour-long recording, 481 KB a slab, with 240 segments 147 ms; while it took 168 so, with
+// eight it took 300).
 constexpr uint64_t kHitSegmentBytes = 24ull << 20;
 uint32_t hit_segments(const fem_ctx *c, uint32_t n_slabs, uint32_t n_chunks, uint32_t m,
                       uint64_t slab_bytes) {
@@ -1460,11 +1460,13 @@ bool level_by_hits(const fem_ctx *c, const StreamDev &s, uint32_t N, int pass, u
 }
 
 // Level 3 joins all pairs of frequent pairs from this many candidates on, with at most so
-// many cells of (pair, pair) counts (512 MB).  Its cost is that of the pairs: over tables by
-// candidate, 31,000 candidates of 29 types and 30,000 events take 256 us, 45,000 of 36 types
-// and 186,000 events 913, 76,000 of 46 types and 159,000 events 1,081; joined 210, 872 and
-// 696.  9,800 candidates of 22 types and 147,000 events are better counted one by one (456
-// against 899 us: a few hundred warps that walk the whole stream).
+// many cells of (pair, pair) counts (512 MB).  Its cost is that of the pairs and their lists'
+// entries; the candidates stand in for them here, since both grow with the frequent pairs.
+// Over tables by candidate / joined, us: 9,800 candidates of 22 types and 147,000 events 456 /
+// 899 (a few hundred warps that walk the whole stream); 31,000 of 29 types and 30,000 events 256
+// / 210; 45,000 of 36 and 186,000 events 913 / 872; 76,000 of 46 and 159,000 events 1,081 / 696.
+// On streams of a chunk or two the other kernels are as fast (74,500 of 64 types, 2,500 events
+// 57 / joined 111).
 constexpr uint32_t kJoinCandidates = 40000;
 constexpr uint64_t kJoinCells = 1ull << 27;
 

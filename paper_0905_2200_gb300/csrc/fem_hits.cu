@@ -268,7 +268,7 @@ __global__ void k_publish_count(const unsigned long long *src, Publish pub) {
 // back as the longest interval reaches, a few steps down the row, give the masks of four
 // edges.  The warp reserves room for its hits in the table, and the ranges are found again:
 // by each lane for its own hits where these are few, else event by event for all four
-// intervals.  What bounds it: issue slots, two thirds of them used, half the lanes in the
+// intervals.  What bounds it: issue slots, 62% of them used, half the lanes in the
 // walks.  Measured on the 406,000 events of 64 types at 20 Hz, all 16,128 edges, exact pass:
 // 258 us (48 recordings, 16 to 64 types: 3.1 ms exact, 3.3 relaxed; bursts of 64 types,
 // 635 us).  Lanes on the events of a few y, all x one after the other, with ballots for the

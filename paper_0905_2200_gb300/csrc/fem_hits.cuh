@@ -11,11 +11,12 @@
 // them different.  So the passes run in two steps:
 //
 //   * The stream is cut into slabs in which no type has more than 32 events, so that a
-//     set of a type's events in a slab is a word.  k_hit_build, one block per slab and one
-//     thread per edge at a time, walks the edge's two event lists once with two cursors
-//     and writes the edge's hits: a mask of the c events that have a b event in the
-//     interval, and per such event the range of those b events (as bits of a 64-bit
-//     word: the 32 events before the slab, then the slab's own) and the latest of them.
+//     set of a type's events in a slab is a word.  k_hit_build, one block per slab (several
+//     where there are few), gives a warp to a next type and a lane to each earlier type; the
+//     lane goes through the next type's events and from each a few steps back down its own
+//     type's, and writes every edge's hits: a mask of the next type's events that have one of
+//     the earlier type in the interval, and per such event the range of those (as bits of a
+//     64-bit word: the 32 events before the slab, then the slab's own) and the latest of them.
 //   * k_hit_count, one thread per (episode, segment), goes through the slabs with the
 //     admitted events of every node as a 64-bit word.  A node's admitted events are those
 //     of its edge's hits whose range meets the node before's word; the highest bit of the
@@ -24,14 +25,14 @@
 // A thread therefore does work only for hits (a tenth to a third of the events), where the
 // per-thread machine spends 60 to 150 issue slots on every event of every node, and the cost
 // of an episode hardly grows with its length: a node after one without admitted events is
-// passed over.  Measured (two-pass and single-pass counts, start of the change -> now): an
+// passed over.  Measured (two-pass and single-pass counts, without tables -> over them): an
 // hour of 64 types at 50 Hz, 100,000 episodes of 3-5 nodes, 332 -> 147 ms; 20,011 episodes
-// of 2-8 nodes on 196,000 events, 6.02 -> 1.56 ms; a bursting recording 31.4 -> 7.3 ms (no
+// of 2-8 nodes on 196,000 events, 6.02 -> 1.54 ms; a bursting recording 31.4 -> 6.8 ms (no
 // rings, and twice the entry classes in the first try); 100 episodes on 3,400 events, 0.95 ->
-// 0.26 ms (all lengths planned in one host wait).  What bounds it: in the count, warp issue
-// slots (41-54% used at 15 to 31 warps per SM, a third to a half of the lanes active: lanes
-// wait for the one with the most hits, so the candidates are ordered by their last three
-// intervals) and the latency of the tables' L2 reads; in the build, issue slots (two thirds used).
+// 0.27 ms (all lengths planned in one host wait).  What bounds it: in the count, the latency
+// of the tables' L2 reads and warp issue slots (35-45% used at 15 to 22 warps per SM, about
+// half of the lanes active: lanes wait for the one with the most hits, so the candidates are
+// ordered by their last three intervals); in the build, issue slots (62% used).
 //
 // MapConcatenate (template flag MC): the entry classes and transfer tables are those of
 // the other counting kernels, so the same stitch composes them; segments are runs of

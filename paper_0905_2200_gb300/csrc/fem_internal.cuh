@@ -322,7 +322,7 @@ struct HitBuild {
     uint32_t *err;                // ERR_DENSE
     uint32_t *dense;              // per type the shortest reach that was too dense, lowered
 };
-// ranges that a build of n_slabs slabs may reserve beyond its hits
+// the tables of n_slabs slabs and their numbers, places and index
 cudaError_t launch_hit_build(int pass, uint32_t n_slabs, const HitBuild &b, int sm_count,
                              cudaStream_t st);
 // for a batch: streams[j]'s slabs are blocks first[j] .. first[j + 1] (device arrays; host:

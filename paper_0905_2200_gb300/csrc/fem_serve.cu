@@ -368,7 +368,8 @@ int finish_enqueue(fem_server *v, Request &r, ServeStream &ss) {
 }
 
 // A one-shot's next attempt, enqueued on its lane after a capacity guard tripped (the last
-// attempt has finished): over the candidates whose flags the first attempt left, or over all
+// attempt has finished; the host waits for its flags, behind what else the lane holds, and not
+// for the recount): over the candidates whose flags the first attempt left, or over all
 // where those are more than half, or the guard left none.
 int enqueue_recount(fem_server *v, Request &r, ServeStream &ss) {
     cudaStream_t st = r.lane;
