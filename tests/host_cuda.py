@@ -27,20 +27,18 @@ def link(tmp):
     objs = [os.path.join(fembuild.OUT_DIR, n) for n in names]
     if not all(os.path.exists(o) for o in objs):
         pytest.skip("the build's objects are not kept here")
-    rt, lib = os.path.join(tmp, "libhostcuda.so"), os.path.join(tmp, "libfem_host.so")
-    subprocess.check_call(["gcc", "-shared", "-fPIC", "-O1", "-o", rt, os.path.join(HERE, "host_cuda.c")])
-    subprocess.check_call(["g++", "-shared", "-o", lib] + objs +
-                          [rt, f"-Wl,-rpath,{tmp}", "-Wl,--wrap=_Znwm"])
-    return lib, rt
+    # (one library that binds to itself: a process may hold the real runtime's names)
+    rt, lib = os.path.join(tmp, "host_cuda.o"), os.path.join(tmp, "libfem_host.so")
+    subprocess.check_call(["gcc", "-c", "-fPIC", "-O1", "-o", rt, os.path.join(HERE, "host_cuda.c")])
+    subprocess.check_call(["g++", "-shared", "-Wl,-Bsymbolic", "-Wl,--wrap=_Znwm", "-o", lib] + objs + [rt])
+    return lib
 
 
 class Host:
-    """The loaded pair; `launches` are the names of the kernels launched so far."""
+    """The loaded library; `launches` are the names of the kernels launched so far."""
 
     def __init__(self, tmp):
-        lib, rt = link(tmp)
-        self.rt = ctypes.CDLL(rt)
-        self.lib = ctypes.CDLL(lib)
+        self.lib = self.rt = ctypes.CDLL(link(tmp))
         self.launches = []
         self.plan = {}     # words of the next plans
         self.error = 0     # error word that the next counts publish
