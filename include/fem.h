@@ -89,11 +89,13 @@ typedef struct {
  * two types' events; with AUTO also fem_mine_levelwise's level-2 relaxed pass over two
  * to four intervals.  HITS (not a configuration value): tables of every edge's (type,
  * interval, next type) events with an event in the interval before them, built per slab of
- * the stream, and episodes counted over them in 64-bit words of events; with AUTO the
- * counts of sets that do not come in prefix runs, batches, window frequencies, and the
- * levels of fem_mine_levelwise whose work is large for the stream's events times types
- * (where a slab's words hold the events, K K n_intervals <= 262,144, and the tables fit
- * beside the stream); level 3 over 40,000 or more candidates joins them all at once.  AUTO
+ * the stream, and episodes counted over them in 64-bit words of events; with AUTO, where
+ * they are estimated to be the faster way, the counts of sets that do not come in prefix
+ * runs, batches, window frequencies, and the levels of fem_mine_levelwise whose work is large
+ * for the stream's events times types (where a slab's words hold the events, K K n_intervals
+ * <= 262,144, and the tables fit beside the stream; they have no segments or block sizes of
+ * fem_config's beyond the number of segments); level 3 over 40,000 or more candidates joins them
+ * all at once.  AUTO
  * otherwise: chosen by measurement when tuning is on; else CHAIN for the exact pass over
  * 256 or more candidates that come in runs of shared prefixes or over at most 64
  * candidates of three or more nodes, CHAIN for the relaxed pass over 32,768 or more such
@@ -299,8 +301,9 @@ void fem_result_free(fem_result *res);
  * pass (a device queue of (job, episode tile, segment) items, longest first);
  * the whole sequence (relaxed pass, per-job elimination at the job's theta,
  * exact pass on the survivors, scatter) runs without a host round trip and is
- * captured once in a CUDA graph that fem_batch_run replays.  Same results as
- * fem_count_two_pass on each job alone (Algorithm 4, Section 5.3.2).
+ * captured once in a CUDA graph that fem_batch_run replays.  Where that is estimated to be
+ * faster, all lengths go over hit tables (FEM_KERNEL_HITS), built in every run.  Same results
+ * as fem_count_two_pass on each job alone (Algorithm 4, Section 5.3.2).
  */
 typedef struct {
     int32_t stream_id;          /* a resident stream of this context */
@@ -421,9 +424,10 @@ int fem_mine_levelwise_ex(fem_ctx *ctx, int32_t stream_id, const fem_interval *i
  * integer window starts s (microseconds) such that the window [s, s + window_us)
  * holds every event of some occurrence of candidate i (first event at or after s,
  * last event before s + window_us).  Divide by (t[n-1] - t[0] + window_us) for the
- * fraction of windows.  One thread per episode; candidates must have distinct
- * types (FEM_EINVAL otherwise); window_us > 0.  counts_out: uint64[m], device if
- * counts_on_device.  FEM_EOVERFLOW if an edge held more than 32 pending entries.
+ * fraction of windows.  One thread per episode, or per episode and segment over hit
+ * tables (FEM_KERNEL_HITS); candidates must have distinct types (FEM_EINVAL otherwise);
+ * window_us > 0.  counts_out: uint64[m], device if counts_on_device.  FEM_EOVERFLOW if an
+ * edge held more than 32 pending entries where the tables do not apply.
  */
 int fem_count_windows(fem_ctx *ctx, int32_t stream_id, const fem_episode *cands, uint32_t m,
                       int cands_on_device, const fem_interval *intervals, uint32_t n_intervals,
