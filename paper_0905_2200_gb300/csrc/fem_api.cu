@@ -1301,10 +1301,12 @@ int windows_hits(fem_ctx *c, const StreamDev &s, const fem_episode *cands, uint3
 // hour-long recording's, 10 GB, are).
 int or_no_room(fem_ctx *c, int rc, bool *done, cudaStream_t st) {
     c->hits_busy = false;
-    size_t kept = 0;
-    for (const auto &kv : c->bufs)
-        if (kv.first.compare(0, 4, "hit_") == 0) kept += kv.second.cap;
-    if (kept > c->mem_device / 16) release_hits(c);
+    if (c->mem_used > c->mem_device / 16) {
+        size_t kept = 0;
+        for (const auto &kv : c->bufs)
+            if (kv.first.compare(0, 4, "hit_") == 0) kept += kv.second.cap;
+        if (kept > c->mem_device / 16) release_hits(c);
+    }
     if (rc != FEM_ENOMEM) return rc;
     *done = false;
     release_hits(c);
@@ -1324,6 +1326,9 @@ bool hits_eligible(const fem_ctx *c, const StreamDev &s, uint32_t nI) {
            (uint64_t)s.K * s.K * nI <= kHitMaxEdges && (s.n_chunks == 1 || s.least_span > max_hi) &&
            (double)s.n * (double)max_hi <= 8.0 * s.K * (double)std::max(s.t_max - s.t_min, 1u);
 }
+
+// Whether anything is or may be measured (else no key needs to be looked up).
+bool tune_used(const fem_ctx *c) { return c->tune_on || !c->tune.empty(); }
 
 // Whether a set that the rule sends over the hit tables goes there (*use): as measured for its
 // class, or, with tuning on and nothing measured, as two counts of either kind tell, each of
@@ -1525,7 +1530,7 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
     // too, and saves it a wait); where they turn out not to apply, the plan's words are the
     // validation's (100 episodes with repeated types 338 us with a validation after the plan, 320
     // so, 315 without tables; 200 on a stream with chunks of 5 ms 513, 322 and 338)
-    if (!hits || !plan_first(c, s, m, nI, pass) || !s.dense_hi.empty() || c->tune_on || !c->tune.empty()) {
+    if (!hits || !plan_first(c, s, m, nI, pass) || !s.dense_hi.empty() || tune_used(c)) {
         RET(validate(c, s, cands, gather, m, nI, info, st));
         known = true;
         hits = hits && !info[1] && !known_dense(c, s, info + 3);
@@ -1540,7 +1545,7 @@ int count_any(fem_ctx *c, const StreamDev &s, const fem_episode *cands, const ui
                                   known ? nullptr : info);
         return or_no_room(c, rc, done, st);
     };
-    if (hits && known) {
+    if (hits && known && tune_used(c)) {
         const int N = __builtin_popcount(info[0]) == 1 ? __builtin_ctz(info[0]) : 0;
         RET(tuned_route(c, tune_key(N, pass, kTuneSet, m, s.n_chunks, s.K), st, &hits,
                         [&] { return count_validated(c, s, cands, gather, m, d_ivl, nI, pass, out, info, st); },
@@ -2510,6 +2515,7 @@ int fem_mine_levelwise_ex(fem_ctx *c, int32_t id, const fem_interval *I, uint32_
         auto chosen = [&](bool join, bool planned, const uint32_t *g, uint32_t mm, int pass, uint32_t *o,
                           bool *use) -> int {
             *use = true;
+            if (!tune_used(c)) return FEM_OK;
             const std::string key = tune_key((int)N, pass, kTuneLevel, mm, s.n_chunks, s.K);
             if (!c->tune.count(key) && c->tune.count(tune_key((int)N, pass, 1, mm, s.n_chunks, s.K))) {
                 *use = false;

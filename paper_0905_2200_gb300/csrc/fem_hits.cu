@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256) k_plan_bins(const PlanArgs a) {
     }
     rep = __reduce_add_sync(0xffffffffu, rep);
     bad = __reduce_or_sync(0xffffffffu, bad);
-    brk = __reduce_add_sync(0xffffffffu, brk);
+    if (a.runs) brk = __reduce_add_sync(0xffffffffu, brk);
     if ((threadIdx.x & 31) == 0) {
         if (rep) atomicAdd(&a.words[PLAN_REP], rep);
         if (brk) atomicAdd(&a.words[PLAN_RUNS], brk);
@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(256) k_hit_cuts(const uint2 *bev, const uint16
 __global__ void __launch_bounds__(1024) k_plan_scan(const PlanArgs a, uint32_t bins, uint32_t edges,
                                                     Publish pub) {
     const uint32_t tid = threadIdx.x;
+    const bool too_dense = tid < a.K && a.dense[tid] <= a.max_hi;
     uint32_t total, n_edges, n_slabs, per;
     scan_words(a.hist, bins, &total, [](uint32_t v) { return v; },
                [&](uint32_t i, uint32_t, uint32_t at) { a.hist[i] = at; });
@@ -209,7 +210,7 @@ __global__ void __launch_bounds__(1024) k_plan_scan(const PlanArgs a, uint32_t b
     __syncthreads();
     if ((tid & 31) == 0) atomicMin(&least, fewest);
     // whether an edge in use leads from a type that is too dense (else none is told)
-    if (__syncthreads_or(tid < a.K && a.dense[tid] <= a.max_hi)) {
+    if (__syncthreads_or(too_dense)) {
         for (uint32_t i = tid; i < edges; i += 1024)
             if (a.edge_id[i] != ~0u && a.dense[i / a.n_ivl % a.K] <= a.max_hi) dense = 1;
         __syncthreads();

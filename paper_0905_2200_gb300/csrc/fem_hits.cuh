@@ -408,10 +408,8 @@ __global__ void __launch_bounds__(128) k_hit_windows(const CountParams p, const 
                                                      uint32_t w, unsigned long long *out) {
     const uint32_t ci = blockIdx.x * blockDim.x + threadIdx.x, seg = blockIdx.y;
     const HitTables &h = p.hits;
-    const uint32_t e0 = *reinterpret_cast<const volatile uint32_t *>(p.err);
     HitEpisode<NMAX> ep;
     const bool ok = ep.load(p, ci);
-    if (e0 & ERR_DENSE) return;  // (as in hit_count_tile)
     const uint32_t s0 = seg * p.cps, s1 = min(s0 + p.cps, h.n_slabs);
     uint32_t s_w = s0;
     if (ok) {
