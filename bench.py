@@ -47,9 +47,9 @@ NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum -k regex:"k_count|k_chain|k_pairs"
     # -c 5 over the first mining step with the rule's kernels and shapes (--no-tune; the
     # tuned step runs the same kernels), per launch
-    "598ebb585edf4a42": {
-        "single_recording_64types_300s": {"2/relaxed": 22733312, "2/exact": 4160256,
-                                          "3/relaxed": 12792320, "3/exact": 3917568},
+    "799479e92e85daa5": {
+        "single_recording_64types_300s": {"2/relaxed": 22711040, "2/exact": 4090112,
+                                          "3/relaxed": 12834560, "3/exact": 3915008},
     },
 }
 
